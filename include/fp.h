@@ -293,7 +293,7 @@ fp_status fp_design_layers(int32_t n_depths, const double *depths, const double 
  * 2^{#cycles(sigma^-1 tau)} -- the statistical-mechanics model behind the
  * paper's Eq. theory_eq (Sec. "Frame potential").  The sum over all pairings
  * runs as a transfer-matrix sweep over the bonds on the device, in FP64, with
- * a state of (k!)^{2(l-1)} entries (k = 3, l = 7: 17.4 GB) allocated for the
+ * a state of (k!)^{2(l-1)-1} entries (k = 3, l = 7: 2.9 GB) allocated for the
  * call and freed before it returns.  A variance-free reference for the Monte
  * Carlo estimates of F^(2) and F^(3).
  *   n >= 2; l in [2, 12] for k = 2, [2, 7] for k = 3 (FP_ERR_ARG otherwise);

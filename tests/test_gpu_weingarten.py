@@ -83,3 +83,54 @@ def test_exact_fk_argument_checks(fp):
             fp.exact_brickwork_fk(n, l, k)
     with pytest.raises(fp.FpError):
         fp.exact_brickwork_fk(8, 3, 2, q=1)
+
+
+def full_state_fk(n, l, k, q):
+    """The same sum over all (k!)^{2(l-1)} entries in numpy: nothing reduced by symmetry,
+    the link and Weingarten matrices from permutations (the latter as the Gram matrix's inverse)."""
+    import itertools
+    perms = list(itertools.permutations(range(k)))
+    s, P = len(perms), 2 * (l - 1)
+
+    def gram(d):
+        out = np.zeros((s, s))
+        for i, a in enumerate(perms):
+            for j, b in enumerate(perms):
+                c = [a.index(b[x]) for x in range(k)]        # a^-1 b
+                seen, n_cyc = set(), 0
+                for x in range(k):
+                    n_cyc += x not in seen
+                    while x not in seen:
+                        seen.add(x)
+                        x = c[x]
+                out[i, j] = float(d) ** n_cyc
+        return out
+
+    link, wg = gram(q), np.linalg.inv(gram(q * q))
+
+    def times(v, t, u, M):
+        shape = [1] * P
+        shape[t] = shape[u] = s
+        return v * (M if t < u else M.T).reshape(shape)
+
+    v = np.ones([s] * P)
+    for t in range(1, P, 2):
+        v = times(times(v, t, t - 1, wg), t, (t + 1) % P, link)
+    for b in range(1, n - 1):
+        for t in range(P):
+            v = np.moveaxis(np.tensordot(link, v, axes=(0, t)), 0, t)
+        for t in range((b + 1) % 2, P, 2):
+            v = times(v, t, (t - 1) % P, wg)
+    for t in range((n - 1) % 2, P, 2):
+        v = times(v, t, (t + 1) % P, link)
+    return v.sum()
+
+
+# kept slots 2l - 3: one CTA (k = 2 up to 9, k = 3 up to 3), shared-memory tiles alone, and each
+# number of slots left for the register passes
+@pytest.mark.parametrize("n,l,k,q", [(5, 6, 2, 2), (4, 7, 2, 2), (5, 8, 2, 3), (4, 9, 2, 2), (5, 10, 2, 2), (4, 11, 2, 2),
+                                     (4, 12, 2, 2), (5, 3, 3, 2), (4, 4, 3, 2), (5, 4, 3, 3), (4, 5, 3, 2),
+                                     (5, 5, 3, 2)])
+def test_exact_fk_matches_full_state(fp, n, l, k, q):
+    ref = full_state_fk(n, l, k, q)
+    assert abs(fp.exact_brickwork_fk(n, l, k, q=q) - ref) <= TOL * abs(ref)
