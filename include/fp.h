@@ -375,7 +375,8 @@ fp_status fp_set_wait_limit_ns(uint64_t ns);
  * out[2] = threads per CTA, out[3] = pass kind (0: FP32/FP64 FMA tile passes,
  * 1: persistent double-buffered FMA passes, 3: tensor-core passes with the
  * tile's operand in shared memory, 4: tensor-core passes with the tile's
- * operand in tensor memory, persistent over the tiles).  The autotuner
+ * operand in tensor memory, persistent over the tiles, 5: the HEA's phase and
+ * Hadamard sweep of boundaries up to 14 bits).  The autotuner
  * chooses it the first time the ensemble contracts that depth at that
  * precision (FP_PREC_FP32 and FP_PREC_FP32_RAW share one choice,
  * FP_PREC_TF32X3 has its own); before that the call returns FP_ERR_ARG.  `out`

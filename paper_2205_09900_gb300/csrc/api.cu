@@ -528,6 +528,11 @@ int brick_key(int l, int prec) {
 fp_status make_brick_cache(fp_ensemble *E, int l, bool fp32, int K, int R, int TH, int persist,
                            std::unique_ptr<BrickCache> &out) {
     auto bc = std::make_unique<BrickCache>();
+    if (persist == 5) {   // the HEA sweep: its shape follows from the boundary
+        K = 99;
+        if (E->d.kind != FP_HEA || !hea_shape(2 * (l - 1), fp32, &R, &TH))
+            return fail(FP_ERR_ARG, "the HEA sweep needs an HEA boundary of at most 14 bits");
+    }
     bc->variant[0] = K; bc->variant[1] = R; bc->variant[2] = TH; bc->variant[3] = persist;
     // K > N: shared-memory sweep, K == N: one tile
     // arcs hold the 5 (FP32) or 4 (FP64) lowest bits, so that tile loads read contiguous runs;
@@ -594,13 +599,18 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
         cands.push_back({kTcTile, kMaxWin, 256, 3});   // the tile's operand in shared memory
         cands.push_back({kTcTile, kMaxWin, 256, 4});   // in tensor memory, persistent over the tiles
     }
+    // P = 5: the HEA's own sweep, the fastest of all wherever it applies (kernels_hea.cu), so
+    // there is nothing to time; FP_PREC_TF32X3 keeps to the tensor cores where they apply
+    int heaR = 0, heaT = 0;
+    if (d.kind == FP_HEA && !(prec == FP_PREC_TF32X3 && N >= kTcTile + 2) && hea_shape(N, fp32, &heaR, &heaT))
+        cands.assign(1, {99, heaR, heaT, 5});
     const int kmin = 10;   // boundaries up to 2^10: shared-memory sweep, nothing to tune
     char ckey[256];
     // the HEA's ring has its own plans: its entries carry the kind after the precision
     snprintf(ckey, sizeof ckey, "%s n=%d l=%d %s%s", E->gpu_name.c_str(), d.n, l,
              !fp32 ? "fp64" : (prec == FP_PREC_TF32X3 && N >= kTcTile + 2) ? "tf32x3" : "fp32",
              d.kind == FP_HEA ? " hea" : "");
-    int bestK = cands[0].K, bestR = cands[0].R, bestT = cands[0].TH, bestP = 0;
+    int bestK = cands[0].K, bestR = cands[0].R, bestT = cands[0].TH, bestP = cands[0].P;
     bool have = false;
     const char *cache = getenv("FP_AUTOTUNE_CACHE");
     if (N <= kmin) {
@@ -625,7 +635,13 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
         have = false;   // a cache entry this depth cannot run (another build's file): tune instead
         cached.reset();
     }
-    if (!have && !idx.empty()) {
+    if (!have && cands.size() == 1) {
+        bestK = cands[0].K; bestR = cands[0].R; bestT = cands[0].TH; bestP = cands[0].P;
+        if (cache) {
+            FILE *f = fopen(cache, "a");
+            if (f) { fprintf(f, "%s|%d %d %d %d\n", ckey, bestK, bestR, bestT, bestP); fclose(f); }
+        }
+    } else if (!have && !idx.empty()) {
         const uint64_t nt = std::min<uint64_t>(idx.size(), 192);   // several waves of tiles per variant
         const int n_raw = d.kind == FP_HEA ? l * d.n : (int)layout_brickwork(d.n, l).size();
         const int n_maps = (d.kind == FP_HEA ? 2 * d.n : d.n - 1) * (l - 1);
@@ -718,10 +734,11 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
     const size_t celem = fp32 ? sizeof(float2) : sizeof(double2);
     const size_t S = (size_t)1 << N;
     const int n_raw = d.kind == FP_HEA ? l * d.n : (int)layout_brickwork(d.n, l).size();
-    const size_t per_raw = (size_t)2 * n_raw * 16 * sizeof(double2);
-    const size_t per_map = (size_t)maps_per_pair(bd) * 16 * celem;
+    const bool hea = it->second->dp.persist == 5;   // slot factors in place of raw gates and maps
+    const size_t per_raw = hea ? 0 : (size_t)2 * n_raw * 16 * sizeof(double2);
+    const size_t per_map = hea ? (size_t)d.n * N * 4 * celem : (size_t)maps_per_pair(bd) * 16 * celem;
     bool both = false;
-    if (bd.tile_bits == 0) brick_smem_bytes(bd, fp32, &both);
+    if (bd.tile_bits == 0 && !hea) brick_smem_bytes(bd, fp32, &both);
     const size_t per_state = bd.tile_bits ? 2 * S * celem + it->second->extra_per_pair : (both ? 0 : S * celem);
     const size_t per_pair = per_raw + per_map + per_state;
     uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(65535, E->ws_budget / per_pair));
@@ -743,7 +760,7 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
             pinfo[i].out = (int64_t)idx[done + i];
         }
         CK(upload(E->d_pairs, pinfo, E->st));
-        CK(E->d_raw.reserve(nb * per_raw));
+        CK(E->d_raw.reserve(std::max<size_t>(16, nb * per_raw)));
         CK(E->d_maps.reserve(nb * per_map));
         CK(E->d_states.reserve(std::max<size_t>(16, nb * per_state)));
         const double G = (double)std::max(bd.n_layers[0], bd.n_layers[1]) * bd.m;
@@ -754,6 +771,19 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         // pair records; the first sub-batch of a shape runs directly (it also
         // sets the kernels' shared-memory attributes outside any capture).
         const bool use_graph = !E->timing && !(d.flags & FP_FLAG_NO_GRAPHS);
+        auto sample = [&](cudaStream_t st) {
+            return hea ? launch_hea_slots(sp, E->d_pairs.as<PairInfo>(), (int)nb, l, E->d_maps.p, fp32, st)
+                       : launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), st);
+        };
+        auto sweep = [&](cudaStream_t st, int *nl) {
+            if (!hea)
+                return launch_brick(bd, bp.passes.data(), it->second->dp, E->d_pairs.as<PairInfo>(), (int)nb,
+                                    E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, err_scale, tr, kappa, err,
+                                    st, nl);
+            *nl = 1;
+            return launch_hea_sweep(bd, E->d_pairs.as<PairInfo>(), (int)nb, E->d_maps.p, E->d_states.p, fp32, err_scale,
+                                    tr, kappa, err, st);
+        };
         GraphKey gk{key, nb, E->d_pairs.p, E->d_raw.p, E->d_maps.p, E->d_states.p, tr, kappa, err};
         auto git = use_graph ? E->graphs.find(gk) : E->graphs.end();
         CK(cudaEventRecord(E->ev0, E->st));
@@ -767,15 +797,13 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         } else {
             {
                 KTimer t(E, FP_K_SAMPLE);
-                CK(launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), E->st));
+                CK(sample(E->st));
                 CK(t.stop((double)nb, sample_launch_count(E->raw_kind)));
             }
             {
                 KTimer t(E, FP_K_BRICK);
                 int nl = 0;
-                CK(launch_brick(bd, bp.passes.data(), it->second->dp, E->d_pairs.as<PairInfo>(), (int)nb,
-                                E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, err_scale, tr, kappa, err,
-                                E->st, &nl));
+                CK(sweep(E->st, &nl));
                 CK(t.stop(cmac_pair * (double)nb));
                 if (E->timing) {
                     E->kst.launches[FP_K_BRICK] += (uint64_t)(nl - 1);
@@ -790,12 +818,9 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
                 cudaGraph_t graph = nullptr;
                 cudaGraphExec_t exec = nullptr;
                 CK(cudaStreamBeginCapture(E->gst, cudaStreamCaptureModeThreadLocal));
-                cudaError_t ce = launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), E->gst);
+                cudaError_t ce = sample(E->gst);
                 int nl = 0;
-                if (ce == cudaSuccess)
-                    ce = launch_brick(bd, bp.passes.data(), it->second->dp, E->d_pairs.as<PairInfo>(), (int)nb,
-                                      E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, err_scale, tr, kappa,
-                                      err, E->gst, &nl);
+                if (ce == cudaSuccess) ce = sweep(E->gst, &nl);
                 cudaError_t ee = cudaStreamEndCapture(E->gst, &graph);
                 if (ce == cudaSuccess && ee == cudaSuccess && graph) {
                     ce = cudaGraphInstantiate(&exec, graph, 0);

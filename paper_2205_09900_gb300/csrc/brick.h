@@ -130,7 +130,8 @@ struct BrickDevPlan {
     int *err_flag;          // persist >= 2: raised by a kernel whose bounded wait ran out
     int win_bits;
     int threads;
-    int persist;        // 1: persistent double-buffered tile passes; 3, 4: tensor-core windows (fp_brick_variant)
+    int persist;        // 1: persistent double-buffered tile passes; 3, 4: tensor-core windows; 5: HEA sweep
+                        // (fp_brick_variant)
 };
 
 struct BrickHostPlan {

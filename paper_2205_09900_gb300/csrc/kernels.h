@@ -20,6 +20,15 @@ struct SampleParams {
 int sample_launch_count(int raw_kind);
 cudaError_t launch_sample(const SampleParams &sp, const PairInfo *pairs, int npairs, int max_raw,
                           double2 *raw, cudaStream_t st);
+// HEA boundary sweep for boundaries of N = 2L-2 <= 14 bits (kernels_hea.cu): the
+// sampled and merged 2x2 slot factors ([pair][qubit][slot][4] of C), then the
+// sweep and meet (`states`: one boundary per pair).  hea_shape: window bits and
+// threads per CTA of the sweep; false where it does not apply.
+cudaError_t launch_hea_slots(const SampleParams &sp, const PairInfo *pairs, int npairs, int L, void *slots, bool fp32,
+                             cudaStream_t st);
+bool hea_shape(int N, bool fp32, int *win_bits, int *threads);
+cudaError_t launch_hea_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, const void *slots, void *states,
+                             bool fp32, double err_scale, double *tr, double *kappa, double *err, cudaStream_t st);
 // Merged gates: ordered products of raw gates (FP64).
 cudaError_t launch_merge(const PairInfo *pairs, int npairs, int max_merged, const DevPlan *plans,
                          const MergeItem *items, const MergeRef *refs, const double2 *raw,

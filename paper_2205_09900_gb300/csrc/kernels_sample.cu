@@ -244,6 +244,67 @@ __global__ void sample_kernel(SampleParams sp, const PairInfo *__restrict__ pair
     }
 }
 
+// The 2x2 factors of the HEA boundary sweep (kernels_hea.cu), sampled and merged in
+// one pass: slot s of qubit q (brick.h), entry 2 y_s + y_{s-1}, at
+// slots[((p n + q) N + s) 4].  One thread per slot, the lanes of a warp over the
+// qubits of one slot (with the slots over the lanes every warp would run all three
+// branches: 3.9 ms against 1.4 ms for 12,500 pairs at n = 50, L = 8); only the two
+// merged slots sample both circuits.
+__device__ __forceinline__ void hea_rotation(uint64_t seed, uint64_t pair, int w, int t, int q, double2 (&m)[4]) {
+    const U64x4 x = philox(seed, (uint64_t)t, (uint64_t)q, pair, (uint64_t)w);
+    double sth, cth, sph, cph;   // of theta/2 and phi/2
+    sincospi_tab((double)(x.x[0] >> 11) * 0x1.0p-53, &sth, &cth);
+    sincospi_tab((double)(x.x[1] >> 11) * 0x1.0p-53, &sph, &cph);
+    m[0] = make_double2(cth * cph, -cth * sph);
+    m[1] = make_double2(-sth * cph, -sth * sph);
+    m[2] = make_double2(sth * cph, -sth * sph);
+    m[3] = make_double2(cth * cph, cth * sph);
+}
+
+template <typename C>
+__global__ void __launch_bounds__(128) hea_slots_kernel(SampleParams sp, const PairInfo *__restrict__ pairs, int npairs,
+                                                        int L, C *__restrict__ slots) {
+    const int N = 2 * L - 2, per = sp.n * N;
+    const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (id >= (int64_t)npairs * per) return;
+    const int p = (int)(id / per), r = (int)(id - (int64_t)p * per), s = r / sp.n, q = r - s * sp.n;
+    const uint64_t pair = pairs[p].pair;
+    const int wv = sp.self_pair ? 0 : 1;
+    double2 R[4];
+    if (s == 0 || s == L - 1) {   // R_1^V R_1^U^dagger; R_L^U^dagger R_L^V
+        double2 A[4], B[4];
+        hea_rotation(sp.seed, pair, 0, s, q, A);
+        hea_rotation(sp.seed, pair, wv, s, q, B);
+#pragma unroll
+        for (int r2 = 0; r2 < 2; ++r2)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                double2 acc = make_double2(0, 0);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const double2 t = s == 0 ? cmul(B[2 * r2 + k], cconj(A[2 * c + k]))
+                                             : cmul(cconj(A[2 * k + r2]), B[2 * k + c]);
+                    acc.x += t.x;
+                    acc.y += t.y;
+                }
+                R[2 * r2 + c] = acc;
+            }
+    } else if (s < L - 1) {
+        hea_rotation(sp.seed, pair, wv, s, q, R);
+    } else {
+        double2 A[4];
+        hea_rotation(sp.seed, pair, 0, 2 * L - 2 - s, q, A);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) R[e] = cconj(A[2 * (e & 1) + (e >> 1)]);
+    }
+    C *out = slots + ((int64_t)p * per + q * N + s) * 4;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        out[e].x = R[e].x;
+        out[e].y = R[e].y;
+    }
+}
+
 __global__ void merge_kernel(const PairInfo *__restrict__ pairs, const DevPlan *__restrict__ plans,
                              const MergeItem *__restrict__ items, const MergeRef *__restrict__ refs,
                              const double2 *__restrict__ raw, double2 *__restrict__ merged) {
@@ -329,6 +390,16 @@ cudaError_t launch_sample(const SampleParams &sp, const PairInfo *pairs, int npa
     }
     dim3 grid((2 * max_raw + 127) / 128, npairs);
     sample_kernel<<<grid, 128, 0, st>>>(sp, pairs, raw);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hea_slots(const SampleParams &sp, const PairInfo *pairs, int npairs, int L, void *slots, bool fp32,
+                             cudaStream_t st) {
+    if (npairs <= 0) return cudaSuccess;
+    const int64_t total = (int64_t)npairs * sp.n * (2 * L - 2);
+    const unsigned grid = (unsigned)((total + 127) / 128);
+    if (fp32) hea_slots_kernel<float2><<<grid, 128, 0, st>>>(sp, pairs, npairs, L, (float2 *)slots);
+    else hea_slots_kernel<double2><<<grid, 128, 0, st>>>(sp, pairs, npairs, L, (double2 *)slots);
     return cudaGetLastError();
 }
 

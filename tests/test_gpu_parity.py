@@ -359,6 +359,20 @@ def test_hea_small_and_odd_chains(fp, n, L):
     assert rel_err(tr, ref).max() <= TOL64
 
 
+# every boundary size of the phase-and-Hadamard sweep (2L - 2 = 2..14 bits): one to eight pairs a
+# CTA with the last one ragged, chains whose halves have an equal and an unequal number of qubits
+@pytest.mark.parametrize("n,L,count", [(3, 2, 131), (2, 3, 130), (5, 4, 19), (2, 4, 17), (6, 5, 9), (9, 5, 17), (7, 6, 5),
+                                       (4, 6, 1), (3, 7, 3), (6, 7, 4), (4, 8, 3), (5, 8, 2), (2, 8, 1)])
+def test_hea_sweep_every_size(fp, n, L, count):
+    ens, od = make(fp, "hea", n, L, seed=n * 11 + L)
+    ref = O.trace_batch(od, 5, count, "auto", threads=8)
+    t64, _, _ = ens.trace_batch(5, count, fp.PREC_FP64)
+    assert rel_err(t64, ref).max() <= TOL64
+    t32, _, _, e32 = ens.trace_batch(5, count, fp.PREC_FP32_RAW, with_err=True)
+    assert np.all(np.abs(t32 - t64) <= e32)   # the estimate that decides the FP64 recontraction bounds the error
+    assert ens.brick_variant(L, fp.PREC_FP64)[3] == 5 and ens.brick_variant(L, fp.PREC_FP32)[3] == 5
+
+
 def test_hea_self_pair_full_size(fp):
     ens, _ = make(fp, "hea", 50, 8, seed=3, flags=1)
     for prec, tol in ((0, 1e-10), (1, 1e-5)):
