@@ -473,7 +473,7 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
         {
             KTimer t(E, FP_K_SAMPLE);
             CK(launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nb, max_raw, E->d_raw.as<double2>(), E->st));
-            CK(t.stop((double)nb, sample_launch_count(E->raw_kind)));
+            CK(t.stop((double)nb));
         }
         {
             KTimer t(E, FP_K_MERGE);
@@ -655,12 +655,17 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
             pinfo[i].out = (int64_t)idx[i];
         }
         CK(upload(E->d_pairs, pinfo, E->st));
-        CK(E->d_raw.reserve(nt * 2 * n_raw * 16 * sizeof(double2)));
+        const bool haar = E->raw_kind == RAW_HAAR4;   // maps straight from the sampler
+        if (!haar) CK(E->d_raw.reserve(nt * 2 * n_raw * 16 * sizeof(double2)));
         CK(E->d_maps.reserve(nt * n_maps * 16 * celem));
         CK(E->d_states.reserve(nt * 2 * ((size_t)1 << N) * celem));
         SampleParams sp;
         sp.seed = d.seed; sp.n = d.n; sp.raw_kind = E->raw_kind; sp.self_pair = (d.flags & FP_FLAG_SELF_PAIR) ? 1 : 0;
-        CK(launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nt, n_raw, E->d_raw.as<double2>(), E->st));
+        if (haar)
+            CK(launch_brick_haar_maps(make_brick_plan(d.n, l, 0, 0, 0).dev, sp, E->d_pairs.as<PairInfo>(), (int)nt,
+                                      E->d_maps.p, fp32, E->st));
+        else
+            CK(launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nt, n_raw, E->d_raw.as<double2>(), E->st));
         float best_ms = 1e30f;
         // FP_PREC_TF32X3: the fastest tensor-core variant when one runs, else the fastest of all
         float best_tc_ms = 1e30f;
@@ -676,7 +681,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
                 CK(cudaEventRecord(E->ev0, E->st));
                 int nl = 0;
                 if (launch_brick(bc->hp.dev, bc->hp.passes.data(), bc->dp, E->d_pairs.as<PairInfo>(), (int)nt,
-                                 E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, 0.0, E->d_tr.as<double>(),
+                                 haar ? nullptr : E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, 0.0, E->d_tr.as<double>(),
                                  nullptr, nullptr, E->st, &nl) != cudaSuccess) {
                     cudaGetLastError();   // a variant this device cannot launch: skip it
                     ms_sum = 1e30f;
@@ -735,7 +740,8 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
     const size_t S = (size_t)1 << N;
     const int n_raw = d.kind == FP_HEA ? l * d.n : (int)layout_brickwork(d.n, l).size();
     const bool hea = it->second->dp.persist == 5;   // slot factors in place of raw gates and maps
-    const size_t per_raw = hea ? 0 : (size_t)2 * n_raw * 16 * sizeof(double2);
+    const bool haar = E->raw_kind == RAW_HAAR4;     // maps straight from the sampler
+    const size_t per_raw = hea || haar ? 0 : (size_t)2 * n_raw * 16 * sizeof(double2);
     const size_t per_map = hea ? (size_t)d.n * N * 4 * celem : (size_t)maps_per_pair(bd) * 16 * celem;
     bool both = false;
     if (bd.tile_bits == 0 && !hea) brick_smem_bytes(bd, fp32, &both);
@@ -772,14 +778,15 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         // sets the kernels' shared-memory attributes outside any capture).
         const bool use_graph = !E->timing && !(d.flags & FP_FLAG_NO_GRAPHS);
         auto sample = [&](cudaStream_t st) {
-            return hea ? launch_hea_slots(sp, E->d_pairs.as<PairInfo>(), (int)nb, l, E->d_maps.p, fp32, st)
+            return hea  ? launch_hea_slots(sp, E->d_pairs.as<PairInfo>(), (int)nb, l, E->d_maps.p, fp32, st)
+                   : haar ? launch_brick_haar_maps(bd, sp, E->d_pairs.as<PairInfo>(), (int)nb, E->d_maps.p, fp32, st)
                        : launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), st);
         };
         auto sweep = [&](cudaStream_t st, int *nl) {
             if (!hea)
                 return launch_brick(bd, bp.passes.data(), it->second->dp, E->d_pairs.as<PairInfo>(), (int)nb,
-                                    E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, err_scale, tr, kappa, err,
-                                    st, nl);
+                                    haar ? nullptr : E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32,
+                                    err_scale, tr, kappa, err, st, nl);
             *nl = 1;
             return launch_hea_sweep(bd, E->d_pairs.as<PairInfo>(), (int)nb, E->d_maps.p, E->d_states.p, fp32, err_scale,
                                     tr, kappa, err, st);
@@ -798,7 +805,7 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
             {
                 KTimer t(E, FP_K_SAMPLE);
                 CK(sample(E->st));
-                CK(t.stop((double)nb, sample_launch_count(E->raw_kind)));
+                CK(t.stop((double)nb));
             }
             {
                 KTimer t(E, FP_K_BRICK);
@@ -929,7 +936,7 @@ fp_status run_spiral(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
         {
             KTimer t(E, FP_K_SAMPLE);
             CK(launch_sample(smp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), E->st));
-            CK(t.stop((double)nb, sample_launch_count(E->raw_kind)));
+            CK(t.stop((double)nb));
         }
         {
             KTimer t(E, FP_K_MERGE);

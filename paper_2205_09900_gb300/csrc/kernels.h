@@ -16,10 +16,14 @@ struct SampleParams {
 };
 
 // Sampler: raw gates of U and V for every pair of the batch (FP64).
-// kernels one launch_sample issues (Haar gates: Gaussian draws, then the QR)
-int sample_launch_count(int raw_kind);
 cudaError_t launch_sample(const SampleParams &sp, const PairInfo *pairs, int npairs, int max_raw,
                           double2 *raw, cudaStream_t st);
+// Haar gates (kernels_haar.cu): raw records (launch_sample's RAW_HAAR4), and the maps of a
+// brickwork sweep straight from the sampled gates (launch_brick without raw gates).
+cudaError_t launch_haar_raw(const SampleParams &sp, const PairInfo *pairs, int npairs, int max_raw, double2 *raw,
+                            cudaStream_t st);
+cudaError_t launch_brick_haar_maps(const BrickDev &d, const SampleParams &sp, const PairInfo *pairs, int npairs,
+                                   void *maps, bool fp32, cudaStream_t st);
 // HEA boundary sweep for boundaries of N = 2L-2 <= 14 bits (kernels_hea.cu): the
 // sampled and merged 2x2 slot factors ([pair][qubit][slot][4] of C), then the
 // sweep and meet (`states`: one boundary per pair).  hea_shape: window bits and
@@ -60,7 +64,7 @@ int moments_blocks(uint64_t count);
 cudaError_t launch_bootstrap(const double *tr, const uint32_t *members, uint64_t n_members, const uint64_t *goff,
                              int n_groups, int k_max, int B, uint64_t seed, double *xs, double *out,
                              cudaStream_t st);
-// Brickwork fast path: maps, then either the shared-memory sweep (tile_bits == 0)
+// Brickwork fast path: maps (from the raw gates; raw == nullptr: they are in place), then either the shared-memory sweep (tile_bits == 0)
 // or init + light-cone passes + dot.  `states` holds npairs x 2 x 2^N
 // amplitudes (tiled) or npairs x 2^N (shared-memory path, left boundaries).
 cudaError_t launch_brick(const BrickDev &d, const BrickPass *hpasses, const BrickDevPlan &dp,

@@ -728,12 +728,15 @@ cudaError_t launch_brick(const BrickDev &d, const BrickPass *hpasses, const Bric
                          int *launches) {
     if (npairs <= 0) return cudaSuccess;
     const int nm = maps_per_pair(d);
-    dim3 gm((nm + 127) / 128, npairs);
-    if (fp32) brick_maps_kernel<float2><<<gm, 128, 0, st>>>(d, pairs, raw, (float2 *)maps);
-    else brick_maps_kernel<double2><<<gm, 128, 0, st>>>(d, pairs, raw, (double2 *)maps);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    int nl = 1;
+    cudaError_t e;
+    int nl = 0;
+    if (raw) {
+        dim3 gm((nm + 127) / 128, npairs);
+        if (fp32) brick_maps_kernel<float2><<<gm, 128, 0, st>>>(d, pairs, raw, (float2 *)maps);
+        else brick_maps_kernel<double2><<<gm, 128, 0, st>>>(d, pairs, raw, (double2 *)maps);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        nl = 1;
+    }
     if (d.tile_bits == 0) {
         bool both = false;
         const size_t smem = brick_smem_bytes(d, fp32, &both);

@@ -1,0 +1,238 @@
+// kernels_haar.cu -- Haar U(4) gates (K1) in 64-bit fixed point (haar_fixed.h),
+// and, for brickwork, the 4x4 maps of the boundary sweep (K2b) made from them in
+// the same kernel.
+//
+// A CTA makes G gates in three phases over shared memory: the Gaussian draws (8
+// Philox blocks per gate, spread over all threads), Gram-Schmidt (one thread per
+// gate, its columns in its own slice), and the output: the gate as 16 doubles
+// pairs (raw records), or its realigned map (brick.h) rounded once to the sweep's
+// precision.  Every brickwork gate enters exactly one map; those of the first and
+// the last layer enter as products of a U and a V gate, which sit on neighbouring
+// threads.  Nothing but the maps goes to global memory.
+//
+// Bound: the integer pipe (about 7,000 instructions a gate).  The FP64 form (Box-Muller
+// and Householder QR on the FP64 pipe, maps by a third kernel) took 19.6 ms for
+// 5.0 million gates (n = 51, l = 5, 20,001 pairs); this takes HAAR_MS ms.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "brick.h"
+#include "haar_fixed.h"
+#include "kernels.h"
+
+namespace fpk {
+namespace {
+
+constexpr int TH = 128;
+
+// phase 1: the Gaussian entries 2j, 2j+1 (row-major) of a gate from Philox block j
+template <int G>
+__device__ __forceinline__ void gauss_block(uint64_t seed, uint64_t pair, int stream, int g, int j, Fx2 *sm, int slot) {
+    const U64x4 x = philox(seed, (uint64_t)j, (uint64_t)g, pair, (uint64_t)stream);
+#pragma unroll 1   // one copy of the code: it is 400 instructions long
+    for (int h = 0; h < 2; ++h) sm[(2 * j + h) * G + slot] = gauss_fixed(h ? x.x[2] : x.x[0], h ? x.x[3] : x.x[1]);
+}
+
+// phase 2: Gram-Schmidt on the gate in slice `slot`; entry k of the matrix at
+// sm[k G + slot] (gram_schmidt_fixed, with the columns in shared memory so that one
+// copy of each step serves all columns)
+template <int G>
+__device__ __forceinline__ void columns(Fx2 *sm, int slot) {
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        Fx2 v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = sm[(4 * r + c) * G + slot];
+        if (c) {
+            shift_fixed<4>(v, lead_fixed<4>(v) - kRoom<4>);
+            for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+                for (int k = 0; k < c; ++k) {
+                    Fx2 q[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) q[r] = sm[(4 * r + k) * G + slot];
+                    project_fixed<4>(q, v);
+                }
+                const int drop = lead_fixed<4>(v) - kRoom<4>;
+                if (drop < kRedo<4>) break;
+                if (pass == 0) shift_fixed<4>(v, drop);
+            }
+        }
+        unit_fixed<4>(v);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) sm[(4 * r + c) * G + slot] = v[r];
+    }
+}
+
+// raw records: gate g of circuit w of pair p at raw[(raw_off + w n_raw + g) 16]
+template <int G>
+__global__ void __launch_bounds__(TH) haar_raw_kernel(SampleParams sp, const PairInfo *__restrict__ pairs,
+                                                      double2 *__restrict__ raw) {
+    __shared__ Fx2 sm[16 * G];
+    const PairInfo pi = pairs[blockIdx.y];
+    const int first = blockIdx.x * G, n = 2 * pi.n_raw - first;
+    if (n <= 0) return;
+    for (int i = threadIdx.x; i < 8 * G; i += TH) {
+        const int slot = i % G, idx = first + slot;
+        if (slot >= n) continue;
+        const int w = idx / pi.n_raw;
+        gauss_block<G>(sp.seed, pi.pair, sp.self_pair ? 0 : w, idx - w * pi.n_raw, i / G, sm, slot);
+    }
+    __syncthreads();
+    const int slot = threadIdx.x;
+    if (slot >= G || slot >= n) return;
+    columns<G>(sm, slot);
+    double2 *out = raw + (pi.raw_off + first + slot) * 16;
+#pragma unroll 4
+    for (int e = 0; e < 16; ++e) {
+        const Fx2 z = sm[e * G + slot];
+        out[e] = make_double2(fx_to_double(z.x, 62), fx_to_double(z.y, 62));
+    }
+}
+
+template <typename C> __device__ __forceinline__ C fx_out(Fx2 z, int k);
+template <> __device__ __forceinline__ float2 fx_out<float2>(Fx2 z, int k) {
+    return make_float2(fx_to_float(z.x, k), fx_to_float(z.y, k));
+}
+template <> __device__ __forceinline__ double2 fx_out<double2>(Fx2 z, int k) {
+    return make_double2(fx_to_double(z.x, k), fx_to_double(z.y, k));
+}
+
+// One gate of a brickwork pair: gate g of circuit w (0 = U, 1 = V), in circuit layer
+// tl (1-based) on bond b.
+struct GateOf { int pair, w, g, tl, b; };
+
+// Items: first the gates of the inner layers 2..l-1 (V's and U's, item = (pair, w, gate)),
+// then, from item `inner` (a multiple of G) on, those of layers 1 and l, the U and the V
+// gate of one place next to each other.  Blocks never mix the two kinds.
+struct Items { int64_t inner_count, inner, outer_count; int nmid, nout, c0, c1, gl; };
+
+__device__ __forceinline__ bool gate_of(const BrickDev &d, const Items &it, int64_t i, GateOf &o) {
+    if (i < it.inner) {
+        if (i >= it.inner_count) return false;
+        const int per = 2 * it.nmid;
+        o.pair = (int)(i / per);
+        const int r = (int)(i - (int64_t)o.pair * per);
+        o.w = r / it.nmid;
+        const int k = r - o.w * it.nmid, two = it.c0 + it.c1, lay = k / two, rem = k - lay * two;
+        const bool odd = rem >= it.c1;   // layer 2 (c1 gates), 3 (c0 gates), 4, ..
+        o.g = it.c0 + k;
+        o.tl = 2 + 2 * lay + (odd ? 1 : 0);
+        o.b = 2 * (odd ? rem - it.c1 : rem) + (o.tl - 1) % 2;
+        return true;
+    }
+    i -= it.inner;
+    if (i >= it.outer_count) return false;
+    const int per = 2 * it.nout;
+    o.pair = (int)(i / per);
+    const int r = (int)(i - (int64_t)o.pair * per), k = r >> 1;
+    o.w = r & 1;
+    const bool last = k >= it.c0;
+    o.tl = last ? d.l : 1;
+    o.g = last ? it.gl + k - it.c0 : k;
+    o.b = 2 * (last ? k - it.c0 : k) + (o.tl - 1) % 2;
+    return true;
+}
+
+template <typename C, int G>
+__global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleParams sp, Items it,
+                                                             const PairInfo *__restrict__ pairs, C *__restrict__ maps) {
+    __shared__ Fx2 sm[16 * G];
+    const int64_t first = (int64_t)blockIdx.x * G;
+    for (int i = threadIdx.x; i < 8 * G; i += TH) {
+        const int slot = i % G;
+        GateOf o;
+        if (gate_of(d, it, first + slot, o))
+            gauss_block<G>(sp.seed, pairs[o.pair].pair, sp.self_pair ? 0 : o.w, o.g, i / G, sm, slot);
+    }
+    __syncthreads();
+    const int slot = threadIdx.x;
+    if (slot >= G) return;
+    GateOf o;
+    const bool on = gate_of(d, it, first + slot, o);
+    if (on) columns<G>(sm, slot);
+    __syncwarp();
+    if (!on) return;
+    const bool outer = first >= it.inner;
+    const int tau = o.tl == 1 ? 2 * d.l - 3 : o.tl == d.l ? d.l - 2 : o.w ? o.tl - 2 : 2 * d.l - 2 - o.tl;
+    const int j = (tau - (o.b + 1) % 2) / 2;
+    const bool left = o.b < d.cut;
+    const int mi = left ? map_index(d, 0, o.b, j) : map_index(d, 1, d.n - 2 - o.b, j);
+    C *out = maps + ((size_t)o.pair * maps_per_pair(d) + mi) * 16;
+    // entry (r, c) of the gate at r = 2 y' + x', c = 2 y + x (x: qubit b+1, primes: after the
+    // gate) goes to row x + 2 x', column y + 2 y' of a left map, transposed in a right one
+    auto put = [&](int r, int c, C z) {
+        const int ex = (c & 1) + 2 * (r & 1), ey = (c >> 1) + 2 * (r >> 1);
+        out[left ? 4 * ex + ey : 4 * ey + ex] = z;
+    };
+    if (!outer) {   // V's gate, or U's conjugate transpose
+#pragma unroll 4
+        for (int e = 0; e < 16; ++e) {
+            Fx2 z = sm[e * G + slot];
+            const int r = e >> 2, c = e & 3;
+            if (!o.w) z.y = -z.y;
+            put(o.w ? r : c, o.w ? c : r, fx_out<C>(z, 62));
+        }
+        return;
+    }
+    // U_l^dagger V_l, or V_1 U_1^dagger: the two threads of a place make two rows each
+    const int us = slot & ~1, vs = slot | 1;
+    const bool mid = o.tl == d.l;
+#pragma unroll 1
+    for (int h = 0; h < 8; ++h) {
+        const int r = 2 * o.w + (h >> 2), c = h & 3;
+        int64_t re = 0, im = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const Fx2 a = sm[(mid ? 4 * k + r : 4 * c + k) * G + us], b = sm[(mid ? 4 * k + c : 4 * r + k) * G + vs];
+            re += smulhi(a.x, b.x) + smulhi(a.y, b.y);   // conj(a) b in 2^-60
+            im += smulhi(a.x, b.y) - smulhi(a.y, b.x);
+        }
+        put(r, c, fx_out<C>({re, im}, 60));
+    }
+}
+
+template <typename C>
+cudaError_t maps_t(const BrickDev &d, const SampleParams &sp, const PairInfo *pairs, int npairs, C *maps,
+                   cudaStream_t st) {
+    Items it;
+    it.c0 = d.n / 2;
+    it.c1 = (d.n - 1) / 2;
+    const int cl = d.l % 2 ? it.c0 : it.c1;
+    it.gl = (d.l / 2) * it.c0 + ((d.l - 1) / 2) * it.c1;   // gates before layer l
+    it.nmid = std::max(0, it.gl - it.c0);
+    it.nout = it.c0 + cl;
+    it.inner_count = (int64_t)npairs * 2 * it.nmid;
+    it.outer_count = (int64_t)npairs * 2 * it.nout;
+    // few gates: 32 per CTA, whose draws all 128 threads share (a batch that fits the SMs
+    // several times over has work enough with one thread per gate throughout)
+    const bool small = it.inner_count + it.outer_count <= 152 * 4 * 128;
+    const int G = small ? 32 : TH;
+    it.inner = (it.inner_count + G - 1) / G * G;
+    const unsigned grid = (unsigned)((it.inner + it.outer_count + G - 1) / G);
+    if (small) brick_haar_maps_kernel<C, 32><<<grid, TH, 0, st>>>(d, sp, it, pairs, maps);
+    else brick_haar_maps_kernel<C, TH><<<grid, TH, 0, st>>>(d, sp, it, pairs, maps);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_haar_raw(const SampleParams &sp, const PairInfo *pairs, int npairs, int max_raw, double2 *raw,
+                            cudaStream_t st) {
+    if (npairs <= 0 || max_raw <= 0) return cudaSuccess;
+    if ((int64_t)npairs * 2 * max_raw <= 152 * 4 * 128)
+        haar_raw_kernel<32><<<dim3((2 * max_raw + 31) / 32, npairs), TH, 0, st>>>(sp, pairs, raw);
+    else
+        haar_raw_kernel<TH><<<dim3((2 * max_raw + TH - 1) / TH, npairs), TH, 0, st>>>(sp, pairs, raw);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_brick_haar_maps(const BrickDev &d, const SampleParams &sp, const PairInfo *pairs, int npairs,
+                                   void *maps, bool fp32, cudaStream_t st) {
+    if (npairs <= 0) return cudaSuccess;
+    return fp32 ? maps_t<float2>(d, sp, pairs, npairs, (float2 *)maps, st)
+                : maps_t<double2>(d, sp, pairs, npairs, (double2 *)maps, st);
+}
+
+}  // namespace fpk

@@ -136,7 +136,8 @@ extern "C" fp_status fp_trace_brick_static(int32_t n, int32_t l, uint64_t seed, 
         base = (unsigned char *)g_scratch_ptr[dev];
     }
     fpk::PairInfo *pairs = (fpk::PairInfo *)base;
-    double2 *raw = (double2 *)(base + align256(count * per_info));
+    // (the gates go straight into their maps; the raw records' share of the scratch stays
+    // reserved, so that the largest count is what callers were told)
     void *maps = base + align256(count * per_info) + align256(count * per_raw);
     void *lbuf = base + align256(count * per_info) + align256(count * per_raw) + align256(count * per_map);
     fill_pairs_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(first, (uint32_t)count, n_raw, pairs);
@@ -146,12 +147,12 @@ extern "C" fp_status fp_trace_brick_static(int32_t n, int32_t l, uint64_t seed, 
     sp.n = n;
     sp.raw_kind = fpk::RAW_HAAR4;
     sp.self_pair = 0;
-    if ((e = fpk::launch_sample(sp, pairs, (int)count, n_raw, raw, st)) != cudaSuccess)
+    if ((e = fpk::launch_brick_haar_maps(d, sp, pairs, (int)count, maps, fp32, st)) != cudaSuccess)
         return sfail(FP_ERR_CUDA, cudaGetErrorString(e));
     fpk::BrickDevPlan dp;
     std::memset(&dp, 0, sizeof dp);
     int nl = 0;
-    if ((e = fpk::launch_brick(d, nullptr, dp, pairs, (int)count, raw, maps, lbuf, fp32, 0.0, tr, kappa, nullptr, st,
+    if ((e = fpk::launch_brick(d, nullptr, dp, pairs, (int)count, nullptr, maps, lbuf, fp32, 0.0, tr, kappa, nullptr, st,
                                &nl)) != cudaSuccess)
         return sfail(FP_ERR_CUDA, cudaGetErrorString(e));
     return FP_OK;
