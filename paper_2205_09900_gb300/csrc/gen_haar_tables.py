@@ -4,7 +4,7 @@ Run once, from this directory:
     python gen_haar_tables.py > haar_tables.h
 
 Values are computed at 60 significant digits (sympy) and rounded to the nearest integer:
-  cos, sin(2 pi k / 512) in units of 2^-62, k = 0..511
+  cos, sin(2 pi k / 512) in units of 2^-60 as 30-bit halves (h, l: h 2^30 + l), k = 0..511
   r_j = 1 / (3/4 + j/512) in units of 2^-63 and ln r_j (of the rounded r_j) in units of
   2^-62, j = 0..384 (r_128 = 1)
 """
@@ -21,11 +21,12 @@ def main():
     out = ["// haar_tables.h -- generated by gen_haar_tables.py (do not edit): tables of the",
            "// fixed-point Haar sampler.",
            "#pragma once", "#include <cstdint>", ""]
-    out.append("// cos, sin(2 pi k / 512) in units of 2^-62, k = 0..511")
-    out.append("FP_TABLE int64_t kCosSin[1024] = {")
+    out.append("// cos, sin(2 pi k / 512) in units of 2^-60 as 30-bit halves, k = 0..511")
+    out.append("FP_TABLE int32_t kCosSin[2048] = {")
     for k in range(512):
         a = sp.pi * sp.Rational(k, 256)
-        out.append(f"    {fix(sp.cos(a).evalf(DIG), 62)}LL, {fix(sp.sin(a).evalf(DIG), 62)}LL,")
+        c, s = fix(sp.cos(a).evalf(DIG), 60), fix(sp.sin(a).evalf(DIG), 60)
+        out.append(f"    {c >> 30}, {c & 0x3FFFFFFF}, {s >> 30}, {s & 0x3FFFFFFF},")
     out.append("};")
     out.append("")
     out.append("// r_j = 1 / (3/4 + j/512) in units of 2^-63, ln r_j in units of 2^-62, j = 0..384")

@@ -2,10 +2,11 @@
 // Gram-Schmidt columns on the integer pipe.
 //
 // GB300 issues 77 FP32 or integer operations in the time of one FP64 operation
-// per lane, and a 64 x 64 -> high-64 product is about ten integer instructions:
-// the same steps in fixed point take a seventh of the FP64 pipe's time and carry
-// 59 to 62 significant bits where a double carries 53.  All values below are
-// integers with the stated unit; products keep the high word, truncated.
+// per lane.  Values are integers of up to 60 bits with the stated unit ("Q60": units
+// of 2^-60); a product takes 30-bit halves, three 32 x 32 -> 64 multiply-adds (the
+// product of the low halves, below the last place, is left out and its mean added
+// where sums would collect it) and sums of products share their shifts.  The errors
+// are a few 2^-58, where a double carries 2^-53.
 //
 // The same functions compile for the host (tests/cpp/haar_fixed_check.cpp measures
 // their errors against extended precision).
@@ -28,13 +29,6 @@ FP_HD uint64_t umulhi(uint64_t a, uint64_t b) {
     return __umul64hi(a, b);
 #else
     return (uint64_t)(((unsigned __int128)a * b) >> 64);
-#endif
-}
-FP_HD int64_t smulhi(int64_t a, int64_t b) {
-#if defined(__CUDA_ARCH__)
-    return __mul64hi(a, b);
-#else
-    return (int64_t)(((__int128)a * b) >> 64);
 #endif
 }
 FP_HD int clz64(uint64_t x) {   // x != 0
@@ -63,11 +57,37 @@ FP_HD void table_pair(const int64_t *t, int k, int64_t &a, int64_t &b) {
 }
 
 struct Fx2 { int64_t x, y; };   // a complex fixed-point value
+struct Half { int32_t h, l; };  // h 2^30 + l, 0 <= l < 2^30
 
-constexpr uint64_t kOne62 = 1ull << 62;
+FP_HD Half halves(int64_t a) { return {(int32_t)(a >> 30), (int32_t)a & 0x3FFFFFFF}; }   // |a| <= 2^60
+FP_HD int64_t wide(int32_t a, int32_t b) { return (int64_t)a * b; }
+// a b 2^-60 rounded (|a|, |b| <= 2^60)
+FP_HD int64_t mul60(Half a, Half b) {
+    return wide(a.h, b.h) + ((wide(a.h, b.l) + wide(a.l, b.h) + (1ll << 29)) >> 30);
+}
+FP_HD int32_t mulhi32(int32_t a, int32_t b) {
+#if defined(__CUDA_ARCH__)
+    return __mulhi(a, b);
+#else
+    return (int32_t)(((int64_t)a * b) >> 32);
+#endif
+}
+
+FP_HD void table_halves(const int32_t *t, int k, Half &a, Half &b) {
+#if defined(__CUDA_ARCH__)
+    const int4 v = __ldg(reinterpret_cast<const int4 *>(t) + k);
+    a = {v.x, v.y};
+    b = {v.z, v.w};
+#else
+    a = {t[4 * k], t[4 * k + 1]};
+    b = {t[4 * k + 2], t[4 * k + 3]};
+#endif
+}
+
 constexpr uint64_t kLn2Q58 = 199786072581291495ull;        // ln 2 in 2^-58
-constexpr int64_t kTwoPiQ60 = 7244019458077122842ll;       // 2 pi in 2^-60
-FP_HD constexpr int64_t rec62(int64_t n) { return (int64_t)((kOne62 + (uint64_t)n / 2) / (uint64_t)n); }   // 1/n in 2^-62
+constexpr int64_t kTwoPiQ57 = 905502432259640355ll;        // 2 pi in 2^-57
+constexpr int64_t kOne60 = 1ll << 60;
+FP_HD constexpr int64_t rec(int n, int q) { return ((1ll << q) + n / 2) / n; }   // 1/n in 2^-q
 
 // 1/sqrt(a) for a in [2^62, 2^64) (units of 2^-64): the seed y0 in 2^-30 and
 // e = 1 - a y0^2 in 2^-60, |e| < 2^-20, with
@@ -80,7 +100,7 @@ FP_HD int64_t rsqrt_step(uint64_t a, uint32_t &y0) {
     return ((e >> 1) + ((3 * ((eh * eh) >> 40)) >> 3)) << 20;
 }
 
-// One complex Gaussian (E|Z|^2 = 1) from two Philox words, in units of 2^-59:
+// One complex Gaussian (E|Z|^2 = 1) from two Philox words, in units of 2^-57:
 // Z = sqrt(-ln u1) e^{2 pi i u2}, u1 = ((xa >> 11) + 1) 2^-53, u2 = (xb >> 11) 2^-53
 // (keying in fp.h).
 FP_HD Fx2 gauss_fixed(uint64_t xa, uint64_t xb) {
@@ -98,28 +118,31 @@ FP_HD Fx2 gauss_fixed(uint64_t xa, uint64_t xb) {
     int64_t rj, tj;
     table_pair(kRecLog, j, rj, tj);
     const uint64_t hi = umulhi(z, (uint64_t)rj), lo = z * (uint64_t)rj;
-    const int64_t y = (int64_t)((hi - (1ull << 62)) << 10) | (int64_t)(lo >> 54);   // 2^-72
-    const int64_t y64 = y >> 8;
-    int64_t p = rec62(6);                     // log1p(y) = y P, P = 1 - y/2 + y^2/3 - .. - y^5/6
-    p = rec62(5) - smulhi(y64, p);
-    p = rec62(4) - smulhi(y64, p);
-    p = rec62(3) - smulhi(y64, p);
-    p = rec62(2) - smulhi(y64, p);
-    p = (int64_t)kOne62 - smulhi(y64, p);
+    const int64_t y = (int64_t)((hi - (1ull << 62)) << 10) | (int64_t)(lo >> 54);   // Q72
+    // log1p(y) = y P, P = 1 - y/2 + y^2/3 - .. - y^5/6: each coefficient to the bits that
+    // its power of y leaves it
+    const int32_t y40 = (int32_t)(y >> 32);
+    const Half yh = halves(y >> 2);           // Q70
+    int32_t p = (int32_t)rec(5, 31) - (mulhi32(y40, (int32_t)rec(6, 31)) >> 8);       // Q31
+    p = (int32_t)rec(4, 32) - (mulhi32(y40, p) >> 7);                                 // Q32
+    int64_t P = rec(3, 60) - (wide(y40, p) >> 12);                                    // Q60
+    P = rec(2, 60) - (mul60(yh, halves(P)) >> 10);
+    P = kOne60 - (mul60(yh, halves(P)) >> 10);
     uint64_t L;
     int s;                                    // unit of L: 2^-s
-    if (K > 0) {
-        L = (uint64_t)K * kLn2Q58 + (uint64_t)((tj - (smulhi(y, p) >> 8)) >> 4);
-        s = 58;
-    } else if (j != 128) {
-        L = (uint64_t)(tj - (smulhi(y, p) >> 8));
-        s = 62;
-    } else {                                  // r = 1: L = -y P keeps its relative accuracy as u1 -> 1
-        const uint64_t d = (uint64_t)-y;      // y <= 0 here when L matters; y > 0 cannot occur with K = 0, z <= 1
+    if (K == 0 && j == 128) {                 // r = 1: L = -y P keeps its relative accuracy as u1 -> 1
+        const uint64_t d = (uint64_t)-y;      // z <= 1 here
         if (d == 0) return {0, 0};            // u1 = 1
         const int sh = clz64(d) - 1;
-        L = umulhi(d << sh, (uint64_t)p << 1);
+        L = umulhi(d << sh, (uint64_t)P << 3);
         s = 71 + sh;
+    } else {
+        L = (uint64_t)(tj - (mul60(yh, halves(P)) >> 8));   // Q62
+        s = 62;
+        if (K > 0) {
+            L = (uint64_t)K * kLn2Q58 + (uint64_t)((int64_t)L >> 4);
+            s = 58;
+        }
     }
     // rad = sqrt(L): L = a 2^E, a in [1/4, 1) in 2^-64, E even
     const int lzl = clz64(L);
@@ -130,26 +153,31 @@ FP_HD Fx2 gauss_fixed(uint64_t xa, uint64_t xb) {
         E += 1;
     }
     uint32_t y0;
-    const int64_t c1 = rsqrt_step(a, y0);     // 2^-80
-    int64_t rad = (int64_t)umulhi(a, (uint64_t)y0 << 32);      // sqrt(a) (1 - c) in 2^-62
-    rad += smulhi(rad, c1) >> 16;
+    const int64_t c1 = rsqrt_step(a, y0);     // Q80
+    int64_t rad = (int64_t)(((a >> 32) * y0 + (((uint64_t)(uint32_t)a * y0) >> 32)) >> 2);   // sqrt(a) (1 - c) in Q60
+    rad += mul60(halves(rad), halves(c1)) >> 20;
     // cos, sin of 2 pi u2: u2 = k/512 + t, |t| <= 2^-10 turns
     const uint64_t ph = xb & ~0x7FFull;       // turns in 2^-64
     const uint64_t kk = (ph + (1ull << 54)) >> 55;
     const int64_t t = (int64_t)(ph - (kk << 55));
-    int64_t ck, sk;
-    table_pair(kCosSin, (int)(kk & 511), ck, sk);
-    const int64_t x = smulhi(t << 8, kTwoPiQ60);   // radians in 2^-68
-    const int64_t x2 = smulhi(x, x);               // 2^-72
-    const int64_t sn = smulhi(x, (int64_t)kOne62 - (smulhi(x2, rec62(6) - (smulhi(x2, rec62(120)) >> 8)) >> 8)) >> 2;   // 2^-64
-    const int64_t cs = (int64_t)kOne62 -
-                       (smulhi(x2, rec62(2) - (smulhi(x2, rec62(24) - (smulhi(x2, rec62(720)) >> 8)) >> 8)) >> 8);      // 2^-62
-    const int64_t c = smulhi(ck, cs) * 4 - (smulhi(sk, sn)), d = smulhi(sk, cs) * 4 + (smulhi(ck, sn));                 // 2^-62
+    Half ck, sk;
+    table_halves(kCosSin, (int)(kk & 511), ck, sk);
+    const Half x = halves(mul60(halves(t << 6), halves(kTwoPiQ57)));   // radians in Q67
+    const int64_t x2 = mul60(x, x);                                    // Q74
+    const Half x2h = halves(x2);
+    const int64_t sv = kOne60 - (mul60(x2h, halves(rec(6, 60) - (wide(x2h.h, (int32_t)rec(120, 37)) >> 21))) >> 14);
+    const int32_t cw = (int32_t)rec(24, 35) - (mulhi32(x2h.h, (int32_t)rec(720, 40)) >> 17);
+    const Half cs = halves(kOne60 - (mul60(x2h, halves(rec(2, 60) - (wide(x2h.h, cw) >> 19))) >> 14));   // Q60
+    const Half sn = halves(mul60(x, halves(sv)) >> 7);                                                   // Q60
+    const Half c = halves(wide(ck.h, cs.h) - wide(sk.h, sn.h) +
+                          ((wide(ck.h, cs.l) + wide(ck.l, cs.h) - wide(sk.h, sn.l) - wide(sk.l, sn.h) + (1ll << 29)) >> 30));
+    const Half d = halves(wide(sk.h, cs.h) + wide(ck.h, sn.h) +
+                          ((wide(sk.h, cs.l) + wide(sk.l, cs.h) + wide(ck.h, sn.l) + wide(ck.l, sn.h) + (1ll << 30)) >> 30));
     // E <= 6: |rad 2^(E/2)| <= 6.06
-    const int half = E / 2 - 1;               // to units of 2^-59
-    const int64_t zr = smulhi(rad, c), zi = smulhi(rad, d);    // 2^-60
-    return half >= 0 ? Fx2{(int64_t)((uint64_t)zr << half), (int64_t)((uint64_t)zi << half)}
-                     : Fx2{half > -64 ? zr >> -half : 0, half > -64 ? zi >> -half : 0};
+    const Half rh = halves(rad);
+    const int64_t zr = mul60(rh, c), zi = mul60(rh, d);   // Q60
+    const int half = 3 - E / 2;               // to units of 2^-57
+    return {half < 64 ? zr >> half : 0, half < 64 ? zi >> half : 0};
 }
 
 // leading zero bits of the largest entry (63 for a zero vector)
@@ -169,64 +197,94 @@ FP_HD void shift_fixed(Fx2 (&v)[D], int sh) {
     }
 }
 
-// v (any scale, D entries) becomes v/|v| in units of 2^-62; a zero vector stays zero
+// v (any scale, D entries) becomes v/|v| in Q60; a zero vector stays zero
 template <int D>
 FP_HD void unit_fixed(Fx2 (&v)[D]) {
-    constexpr int room = D <= 4 ? 2 : 3;      // |entries| < 2^(64 - room): 2 D squares fit 64 bits
+    constexpr int room = D <= 4 ? 5 : 6;      // |entries| < 2^(64 - room): the sums below fit 63 bits
     shift_fixed<D>(v, lead_fixed<D>(v) - room);
-    uint64_t n2 = 0;                          // |v|^2 2^-64
+    int64_t sq = 0, cross = 1ll << 28;        // |v|^2 2^-60
 #pragma unroll
-    for (int i = 0; i < D; ++i) n2 += (uint64_t)smulhi(v[i].x, v[i].x) + (uint64_t)smulhi(v[i].y, v[i].y);
+    for (int i = 0; i < D; ++i) {
+        const Half x = halves(v[i].x), y = halves(v[i].y);
+        sq += wide(x.h, x.h) + wide(y.h, y.h);
+        cross += wide(x.h, x.l) + wide(y.h, y.l);
+    }
+    const uint64_t n2 = (uint64_t)(sq + (cross >> 29));
     const int lz = n2 ? clz64(n2) & ~1 : 0;
     const uint64_t a = n2 << lz;              // [2^62, 2^64)
     uint32_t y0;
     const int64_t c1 = a ? rsqrt_step(a, y0) : (y0 = 0, 0);
-    // 1/sqrt(a) in (1, 2], units of 2^-62 (2^-61 of room: values up to 2)
-    int64_t y = (int64_t)((uint64_t)y0 << 31);
-    y += smulhi(y, c1) >> 16;                 // 2^-61
-    // |v| = sqrt(a) 2^(32 - lz/2) with a read as a fraction: v/|v| 2^62 = v y_real 2^(lz/2 - 2)
-    const int h = lz / 2;
+    int64_t y = (int64_t)((uint64_t)y0 << 29);   // 1/sqrt(a) in (1, 2], Q59
+    y += mul60(halves(y), halves(c1)) >> 20;
+    // |v| = sqrt(a) 2^(62 - lz/2) with a read as a fraction: v/|v| 2^60 = v y 2^(lz/2 - 2), lz >= 2
+    const Half yh = halves(y);
+    const int h = lz / 2 - 1;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        v[i].x = (int64_t)((uint64_t)smulhi((int64_t)((uint64_t)v[i].x << 1), y) << h);
-        v[i].y = (int64_t)((uint64_t)smulhi((int64_t)((uint64_t)v[i].y << 1), y) << h);
+        v[i].x = (int64_t)((uint64_t)mul60(halves(v[i].x), yh) << h);
+        v[i].y = (int64_t)((uint64_t)mul60(halves(v[i].y), yh) << h);
     }
 }
 
-// v <- v - q <q, v>, q a unit vector in 2^-62, v in any unit with |v| < 2^63
+constexpr int kRoom = 6;   // leading zeros of a vector to project: entries below 2^58
+
+// v <- v - q <q, v>, q a unit vector in Q60, v in any unit with entries below 2^58.  The
+// cross sums stay below 2^63: sqrt(2 D) 2^60 and 2 D 2^58, in two parts for D > 4.
 template <int D>
 FP_HD void project_fixed(const Fx2 (&q)[D], Fx2 (&v)[D]) {
-    int64_t hr = D, hi = 0;                   // <q, v> / 4 in v's unit; D: half of each truncated bit of 2 D terms
+    constexpr int64_t r = 1ll << 29;          // rounds; a left-out product of low halves has mean 2^28
+    int64_t ah = 0, ac = r + D * r, al = 0, bh = 0, bc = r, bl = 0;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        hr += smulhi(q[i].x, v[i].x) + smulhi(q[i].y, v[i].y);
-        hi += smulhi(q[i].x, v[i].y) - smulhi(q[i].y, v[i].x);
+        const Half qx = halves(q[i].x), qy = halves(q[i].y), x = halves(v[i].x), y = halves(v[i].y);
+        ah += wide(qx.h, x.h) + wide(qy.h, y.h);
+        bh += wide(qx.h, y.h) - wide(qy.h, x.h);
+        ac += wide(qx.h, x.l) + wide(qy.h, y.l);
+        bc += wide(qx.h, y.l) - wide(qy.h, x.l);
+        (D > 4 ? al : ac) += wide(qx.l, x.h) + wide(qy.l, y.h);
+        (D > 4 ? bl : bc) += wide(qx.l, y.h) - wide(qy.l, x.h);
     }
-    hr *= 4;
-    hi *= 4;
+    const Half hr = halves(ah + (ac >> 30) + (D > 4 ? al >> 30 : 0)), hi = halves(bh + (bc >> 30) + (D > 4 ? bl >> 30 : 0));
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        v[i].x -= 4 * (smulhi(q[i].x, hr) - smulhi(q[i].y, hi));
-        v[i].y -= 4 * (smulhi(q[i].x, hi) + smulhi(q[i].y, hr) + 1);
+        const Half qx = halves(q[i].x), qy = halves(q[i].y);
+        v[i].x -= wide(qx.h, hr.h) - wide(qy.h, hi.h) +
+                  ((wide(qx.h, hr.l) + wide(qx.l, hr.h) - wide(qy.h, hi.l) - wide(qy.l, hi.h) + r) >> 30);
+        v[i].y -= wide(qx.h, hi.h) + wide(qy.h, hr.h) +
+                  ((wide(qx.h, hi.l) + wide(qx.l, hi.h) + wide(qy.h, hr.l) + wide(qy.l, hr.h) + 2 * r) >> 30);
     }
 }
 
-// A column that its projections shortened 2^kRedo-fold (16, or 8) or more keeps too few bits
+// conj(a) b summed over D entries (unit vectors in Q60), in Q60
+template <int D>
+FP_HD Fx2 dot_fixed(const Fx2 (&q)[D], const Fx2 (&v)[D]) {
+    constexpr int64_t r = 1ll << 29;
+    int64_t ah = 0, ac = r + D * r, bh = 0, bc = r;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        const Half qx = halves(q[i].x), qy = halves(q[i].y), x = halves(v[i].x), y = halves(v[i].y);
+        ah += wide(qx.h, x.h) + wide(qy.h, y.h);
+        bh += wide(qx.h, y.h) - wide(qy.h, x.h);
+        ac += (wide(qx.h, x.l) + wide(qx.l, x.h)) + (wide(qy.h, y.l) + wide(qy.l, y.h));
+        bc += (wide(qx.h, y.l) + wide(qx.l, y.h)) - (wide(qy.h, x.l) + wide(qy.l, x.h));
+    }
+    return {ah + (ac >> 30), bh + (bc >> 30)};
+}
+
+// A column that its projections shortened 2^kRedo-fold (16, or 4) or more keeps too few bits
 // clear of their rounding: it is scaled up and projected once more.
-template <int D> constexpr int kRedo = D <= 9 ? 4 : 3;
-// leading zeros that keep |v| below 2^63: entries below 2^(64 - room), 2 D of them
-template <int D> constexpr int kRoom = D <= 4 ? 3 : 4;
+template <int D> constexpr int kRedo = D <= 4 ? 4 : 2;
 
 // the columns v[c] of a matrix become the columns of its unitary factor (R's
-// diagonal positive), in units of 2^-62
+// diagonal positive), in Q60
 template <int D>
 FP_HD void gram_schmidt_fixed(Fx2 (&v)[D][D]) {
 #pragma unroll
     for (int c = 0; c < D; ++c) {
-        if (c) shift_fixed<D>(v[c], lead_fixed<D>(v[c]) - kRoom<D>);   // |v| < 2^63
+        if (c) shift_fixed<D>(v[c], lead_fixed<D>(v[c]) - kRoom);   // entries below 2^58
 #pragma unroll
         for (int k = 0; k < c; ++k) project_fixed<D>(v[k], v[c]);
-        const int drop = c ? lead_fixed<D>(v[c]) - kRoom<D> : 0;
+        const int drop = c ? lead_fixed<D>(v[c]) - kRoom : 0;
         if (drop >= kRedo<D>) {
             shift_fixed<D>(v[c], drop);
 #pragma unroll

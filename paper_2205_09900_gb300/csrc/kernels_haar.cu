@@ -10,9 +10,9 @@
 // the last layer enter as products of a U and a V gate, which sit on neighbouring
 // threads.  Nothing but the maps goes to global memory.
 //
-// Bound: the integer pipe (about 7,000 instructions a gate).  The FP64 form (Box-Muller
+// Bound: the integer pipe (about 17,000 instructions a gate, the 32 x 32 -> 64 products above all).  The FP64 form (Box-Muller
 // and Householder QR on the FP64 pipe, maps by a third kernel) took 19.6 ms for
-// 5.0 million gates (n = 51, l = 5, 20,001 pairs); this takes HAAR_MS ms.
+// 5.0 million gates (n = 51, l = 5, 20,001 pairs); this takes 3.4 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,7 +45,7 @@ __device__ __forceinline__ void columns(Fx2 *sm, int slot) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) v[r] = sm[(4 * r + c) * G + slot];
         if (c) {
-            shift_fixed<4>(v, lead_fixed<4>(v) - kRoom<4>);
+            shift_fixed<4>(v, lead_fixed<4>(v) - kRoom);
             for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll 1
                 for (int k = 0; k < c; ++k) {
@@ -54,7 +54,7 @@ __device__ __forceinline__ void columns(Fx2 *sm, int slot) {
                     for (int r = 0; r < 4; ++r) q[r] = sm[(4 * r + k) * G + slot];
                     project_fixed<4>(q, v);
                 }
-                const int drop = lead_fixed<4>(v) - kRoom<4>;
+                const int drop = lead_fixed<4>(v) - kRoom;
                 if (drop < kRedo<4>) break;
                 if (pass == 0) shift_fixed<4>(v, drop);
             }
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(TH) haar_raw_kernel(SampleParams sp, const Pai
 #pragma unroll 4
     for (int e = 0; e < 16; ++e) {
         const Fx2 z = sm[e * G + slot];
-        out[e] = make_double2(fx_to_double(z.x, 62), fx_to_double(z.y, 62));
+        out[e] = make_double2(fx_to_double(z.x, 60), fx_to_double(z.y, 60));
     }
 }
 
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleP
             Fx2 z = sm[e * G + slot];
             const int r = e >> 2, c = e & 3;
             if (!o.w) z.y = -z.y;
-            put(o.w ? r : c, o.w ? c : r, fx_out<C>(z, 62));
+            put(o.w ? r : c, o.w ? c : r, fx_out<C>(z, 60));
         }
         return;
     }
@@ -182,14 +182,13 @@ __global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleP
 #pragma unroll 1
     for (int h = 0; h < 8; ++h) {
         const int r = 2 * o.w + (h >> 2), c = h & 3;
-        int64_t re = 0, im = 0;
+        Fx2 x[4], y[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const Fx2 a = sm[(mid ? 4 * k + r : 4 * c + k) * G + us], b = sm[(mid ? 4 * k + c : 4 * r + k) * G + vs];
-            re += smulhi(a.x, b.x) + smulhi(a.y, b.y);   // conj(a) b in 2^-60
-            im += smulhi(a.x, b.y) - smulhi(a.y, b.x);
+            x[k] = sm[(mid ? 4 * k + r : 4 * c + k) * G + us];
+            y[k] = sm[(mid ? 4 * k + c : 4 * r + k) * G + vs];
         }
-        put(r, c, fx_out<C>({re, im}, 60));
+        put(r, c, fx_out<C>(dot_fixed<4>(x, y), 60));
     }
 }
 

@@ -85,7 +85,7 @@ static void check_qr(std::mt19937_64 &g, int count) {
         for (int r = 0; r < D; ++r)
             for (int c = 0; c < D; ++c) {
                 v[c][r] = gauss_fixed(g(), g());
-                A[r * D + c] = {ldexpl((ld)v[c][r].x, -59), ldexpl((ld)v[c][r].y, -59)};
+                A[r * D + c] = {ldexpl((ld)v[c][r].x, -57), ldexpl((ld)v[c][r].y, -57)};
                 Ad[r * D + c] = {(double)A[r * D + c].real(), (double)A[r * D + c].imag()};
             }
         gram_schmidt_fixed<D>(v);
@@ -95,7 +95,7 @@ static void check_qr(std::mt19937_64 &g, int count) {
         dc U[D * D];
         for (int r = 0; r < D; ++r)
             for (int c = 0; c < D; ++c) {
-                U[r * D + c] = {fx_to_double(v[c][r].x, 62), fx_to_double(v[c][r].y, 62)};
+                U[r * D + c] = {fx_to_double(v[c][r].x, 60), fx_to_double(v[c][r].y, 60)};
                 e += std::norm(lc(U[r * D + c]) - Q[r * D + c]);
                 ed += std::norm(lc(Qd[r * D + c]) - Q[r * D + c]);
             }
@@ -126,7 +126,7 @@ int main(int argc, char **argv) {
     auto one = [&](uint64_t xa, uint64_t xb) {
         const Fx2 z = gauss_fixed(xa, xb);
         const lc w = gauss_ld(xa, xb);
-        worst = std::max(worst, std::abs(lc(ldexpl((ld)z.x, -59), ldexpl((ld)z.y, -59)) - w));
+        worst = std::max(worst, std::abs(lc(ldexpl((ld)z.x, -57), ldexpl((ld)z.y, -57)) - w));
     };
     for (int i = 0; i < count; ++i) one(g(), g());
     printf("gauss random %.3Le\n", worst);
