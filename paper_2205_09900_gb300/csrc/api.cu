@@ -998,7 +998,7 @@ fp_status run_qudit(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         return fail(FP_ERR_INFEASIBLE, "qudit depth %d: boundary of %d^%d amplitudes exceeds 2^%d", l, d.q, bd.N,
                     FP_MAX_STATE_BITS);
     const int n_raw = (int)layout_brickwork(d.n, l).size();
-    const size_t per_pair = qudit_workspace_per_pair(d.q, bd, n_raw, fp32);
+    const size_t per_pair = qudit_workspace_per_pair(d.q, bd, fp32);
     const uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(65535, E->ws_budget / per_pair));
     const double G = (double)std::max(bd.n_layers[0], bd.n_layers[1]) * bd.m;
     const double err_scale = FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53) * std::sqrt(G);
@@ -1017,10 +1017,10 @@ fp_status run_qudit(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         CK(cudaEventRecord(E->ev0, E->st));
         {
             KTimer t(E, FP_K_BRICK);
-            CK(launch_qudit(d.q, bd, d.seed, E->d_pairs.as<PairInfo>(), (int)nb, n_raw,
+            CK(launch_qudit(d.q, bd, d.seed, E->d_pairs.as<PairInfo>(), (int)nb,
                             (d.flags & FP_FLAG_SELF_PAIR) ? 1 : 0, fp32, E->d_states.p, err_scale, tr, kappa, err,
                             E->st));
-            CK(t.stop(cmac_pair * (double)nb, 3));
+            CK(t.stop(cmac_pair * (double)nb, 2));
         }
         CK(cudaEventRecord(E->ev1, E->st));
         CK(cudaEventSynchronize(E->ev1));

@@ -180,95 +180,115 @@ FP_HD Fx2 gauss_fixed(uint64_t xa, uint64_t xb) {
     return {half < 64 ? zr >> half : 0, half < 64 ? zi >> half : 0};
 }
 
-// leading zero bits of the largest entry (63 for a zero vector)
+// Pieces of the column steps, one entry at a time (a lane may hold one row):
+// conj(q) v 2^-60 rounded, q in Q60
+FP_HD Fx2 dot1_fixed(Fx2 q, Fx2 v) {
+    constexpr int64_t r = 1ll << 29;          // rounds; a left-out product of low halves has mean 2^28
+    const Half qx = halves(q.x), qy = halves(q.y), x = halves(v.x), y = halves(v.y);
+    return {wide(qx.h, x.h) + wide(qy.h, y.h) +
+                ((wide(qx.h, x.l) + wide(qx.l, x.h) + wide(qy.h, y.l) + wide(qy.l, y.h) + 2 * r) >> 30),
+            wide(qx.h, y.h) - wide(qy.h, x.h) +
+                ((wide(qx.h, y.l) + wide(qx.l, y.h) - wide(qy.h, x.l) - wide(qy.l, x.h) + r) >> 30)};
+}
+// v <- v - q h
+FP_HD void sub1_fixed(Fx2 &v, Fx2 q, Half hr, Half hi) {
+    constexpr int64_t r = 1ll << 29;
+    const Half qx = halves(q.x), qy = halves(q.y);
+    v.x -= wide(qx.h, hr.h) - wide(qy.h, hi.h) +
+           ((wide(qx.h, hr.l) + wide(qx.l, hr.h) - wide(qy.h, hi.l) - wide(qy.l, hi.h) + r) >> 30);
+    v.y -= wide(qx.h, hi.h) + wide(qy.h, hr.h) +
+           ((wide(qx.h, hi.l) + wide(qx.l, hi.h) + wide(qy.h, hr.l) + wide(qy.l, hr.h) + 2 * r) >> 30);
+}
+FP_HD int lead1_fixed(Fx2 v) {
+    return clz64((uint64_t)(v.x ^ (v.x >> 63)) | (uint64_t)(v.y ^ (v.y >> 63)) | 1);
+}
+FP_HD void shift1_fixed(Fx2 &v, int sh) {
+    v.x = sh >= 0 ? (int64_t)((uint64_t)v.x << sh) : v.x >> -sh;
+    v.y = sh >= 0 ? (int64_t)((uint64_t)v.y << sh) : v.y >> -sh;
+}
+// |v|^2 2^-60 of one entry
+FP_HD int64_t norm1_fixed(Fx2 v) {
+    const Half x = halves(v.x), y = halves(v.y);
+    return wide(x.h, x.h) + wide(y.h, y.h) + ((wide(x.h, x.l) + wide(y.h, y.l) + (1ll << 28)) >> 29);
+}
+// 1/|v| from n2 = |v|^2 2^-60: v/|v| in Q60 is (v y 2^-60) 2^h (scale1_fixed)
+FP_HD Half inv_norm_fixed(uint64_t n2, int &h) {
+    const int lz = n2 ? clz64(n2) & ~1 : 2;
+    const uint64_t a = n2 << lz;              // [2^62, 2^64)
+    uint32_t y0 = 0;
+    const int64_t c1 = a ? rsqrt_step(a, y0) : 0;
+    int64_t y = (int64_t)((uint64_t)y0 << 29);   // 1/sqrt(a) in (1, 2], Q59
+    y += mul60(halves(y), halves(c1)) >> 20;
+    // |v| = sqrt(a) 2^(62 - lz/2) with a read as a fraction: v/|v| 2^60 = v y 2^(lz/2 - 2), lz >= 2
+    h = lz / 2 - 1;
+    return halves(y);
+}
+FP_HD void scale1_fixed(Fx2 &v, Half y, int h) {
+    v.x = (int64_t)((uint64_t)mul60(halves(v.x), y) << h);
+    v.y = (int64_t)((uint64_t)mul60(halves(v.y), y) << h);
+}
+
 template <int D>
-FP_HD int lead_fixed(const Fx2 (&v)[D]) {
-    uint64_t o = 1;
+FP_HD int lead_fixed(const Fx2 (&v)[D]) {     // leading zero bits of the largest entry
+    int l = 63;
 #pragma unroll
-    for (int i = 0; i < D; ++i) o |= (uint64_t)(v[i].x ^ (v[i].x >> 63)) | (uint64_t)(v[i].y ^ (v[i].y >> 63));
-    return clz64(o);
+    for (int i = 0; i < D; ++i) {
+        const int m = lead1_fixed(v[i]);
+        l = m < l ? m : l;
+    }
+    return l;
 }
 template <int D>
 FP_HD void shift_fixed(Fx2 (&v)[D], int sh) {
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        v[i].x = sh >= 0 ? (int64_t)((uint64_t)v[i].x << sh) : v[i].x >> -sh;
-        v[i].y = sh >= 0 ? (int64_t)((uint64_t)v[i].y << sh) : v[i].y >> -sh;
-    }
+    for (int i = 0; i < D; ++i) shift1_fixed(v[i], sh);
 }
 
+// leading zeros before the norm: entries below 2^(64 - room), so that 2 D squares fit 63 bits
+template <int D> constexpr int kUnitRoom = D <= 4 ? 5 : 6;
 // v (any scale, D entries) becomes v/|v| in Q60; a zero vector stays zero
 template <int D>
 FP_HD void unit_fixed(Fx2 (&v)[D]) {
-    constexpr int room = D <= 4 ? 5 : 6;      // |entries| < 2^(64 - room): the sums below fit 63 bits
-    shift_fixed<D>(v, lead_fixed<D>(v) - room);
-    int64_t sq = 0, cross = 1ll << 28;        // |v|^2 2^-60
+    shift_fixed<D>(v, lead_fixed<D>(v) - kUnitRoom<D>);
+    int64_t n2 = 0;
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        const Half x = halves(v[i].x), y = halves(v[i].y);
-        sq += wide(x.h, x.h) + wide(y.h, y.h);
-        cross += wide(x.h, x.l) + wide(y.h, y.l);
-    }
-    const uint64_t n2 = (uint64_t)(sq + (cross >> 29));
-    const int lz = n2 ? clz64(n2) & ~1 : 0;
-    const uint64_t a = n2 << lz;              // [2^62, 2^64)
-    uint32_t y0;
-    const int64_t c1 = a ? rsqrt_step(a, y0) : (y0 = 0, 0);
-    int64_t y = (int64_t)((uint64_t)y0 << 29);   // 1/sqrt(a) in (1, 2], Q59
-    y += mul60(halves(y), halves(c1)) >> 20;
-    // |v| = sqrt(a) 2^(62 - lz/2) with a read as a fraction: v/|v| 2^60 = v y 2^(lz/2 - 2), lz >= 2
-    const Half yh = halves(y);
-    const int h = lz / 2 - 1;
+    for (int i = 0; i < D; ++i) n2 += norm1_fixed(v[i]);
+    int h;
+    const Half y = inv_norm_fixed((uint64_t)n2, h);
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        v[i].x = (int64_t)((uint64_t)mul60(halves(v[i].x), yh) << h);
-        v[i].y = (int64_t)((uint64_t)mul60(halves(v[i].y), yh) << h);
-    }
+    for (int i = 0; i < D; ++i) scale1_fixed(v[i], y, h);
 }
 
 constexpr int kRoom = 6;   // leading zeros of a vector to project: entries below 2^58
 
-// v <- v - q <q, v>, q a unit vector in Q60, v in any unit with entries below 2^58.  The
-// cross sums stay below 2^63: sqrt(2 D) 2^60 and 2 D 2^58, in two parts for D > 4.
+// v <- v - q <q, v>, q a unit vector in Q60, v in any unit with entries below 2^58.
 template <int D>
 FP_HD void project_fixed(const Fx2 (&q)[D], Fx2 (&v)[D]) {
-    constexpr int64_t r = 1ll << 29;          // rounds; a left-out product of low halves has mean 2^28
-    int64_t ah = 0, ac = r + D * r, al = 0, bh = 0, bc = r, bl = 0;
+    int64_t hr = 0, hi = 0;
+    if (D <= 4) {   // one shift for the whole sum: the cross sums stay below sqrt(2 D) 2^60 + 2 D 2^58 < 2^63
+        constexpr int64_t r = 1ll << 29;
+        int64_t ac = r + D * r, bc = r;
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        const Half qx = halves(q[i].x), qy = halves(q[i].y), x = halves(v[i].x), y = halves(v[i].y);
-        ah += wide(qx.h, x.h) + wide(qy.h, y.h);
-        bh += wide(qx.h, y.h) - wide(qy.h, x.h);
-        ac += wide(qx.h, x.l) + wide(qy.h, y.l);
-        bc += wide(qx.h, y.l) - wide(qy.h, x.l);
-        (D > 4 ? al : ac) += wide(qx.l, x.h) + wide(qy.l, y.h);
-        (D > 4 ? bl : bc) += wide(qx.l, y.h) - wide(qy.l, x.h);
-    }
-    const Half hr = halves(ah + (ac >> 30) + (D > 4 ? al >> 30 : 0)), hi = halves(bh + (bc >> 30) + (D > 4 ? bl >> 30 : 0));
+        for (int i = 0; i < D; ++i) {
+            const Half qx = halves(q[i].x), qy = halves(q[i].y), x = halves(v[i].x), y = halves(v[i].y);
+            hr += wide(qx.h, x.h) + wide(qy.h, y.h);
+            hi += wide(qx.h, y.h) - wide(qy.h, x.h);
+            ac += wide(qx.h, x.l) + wide(qy.h, y.l) + wide(qx.l, x.h) + wide(qy.l, y.h);
+            bc += wide(qx.h, y.l) - wide(qy.h, x.l) + wide(qx.l, y.h) - wide(qy.l, x.h);
+        }
+        hr += ac >> 30;
+        hi += bc >> 30;
+    } else {
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        const Half qx = halves(q[i].x), qy = halves(q[i].y);
-        v[i].x -= wide(qx.h, hr.h) - wide(qy.h, hi.h) +
-                  ((wide(qx.h, hr.l) + wide(qx.l, hr.h) - wide(qy.h, hi.l) - wide(qy.l, hi.h) + r) >> 30);
-        v[i].y -= wide(qx.h, hi.h) + wide(qy.h, hr.h) +
-                  ((wide(qx.h, hi.l) + wide(qx.l, hi.h) + wide(qy.h, hr.l) + wide(qy.l, hr.h) + 2 * r) >> 30);
+        for (int i = 0; i < D; ++i) {
+            const Fx2 t = dot1_fixed(q[i], v[i]);
+            hr += t.x;
+            hi += t.y;
+        }
     }
-}
-
-// conj(a) b summed over D entries (unit vectors in Q60), in Q60
-template <int D>
-FP_HD Fx2 dot_fixed(const Fx2 (&q)[D], const Fx2 (&v)[D]) {
-    constexpr int64_t r = 1ll << 29;
-    int64_t ah = 0, ac = r + D * r, bh = 0, bc = r;
+    const Half a = halves(hr), b = halves(hi);
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        const Half qx = halves(q[i].x), qy = halves(q[i].y), x = halves(v[i].x), y = halves(v[i].y);
-        ah += wide(qx.h, x.h) + wide(qy.h, y.h);
-        bh += wide(qx.h, y.h) - wide(qy.h, x.h);
-        ac += (wide(qx.h, x.l) + wide(qx.l, x.h)) + (wide(qy.h, y.l) + wide(qy.l, y.h));
-        bc += (wide(qx.h, y.l) + wide(qx.l, y.h)) - (wide(qy.h, x.l) + wide(qy.l, x.h));
-    }
-    return {ah + (ac >> 30), bh + (bc >> 30)};
+    for (int i = 0; i < D; ++i) sub1_fixed(v[i], q[i], a, b);
 }
 
 // A column that its projections shortened 2^kRedo-fold (16, or 4) or more keeps too few bits

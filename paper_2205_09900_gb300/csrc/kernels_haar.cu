@@ -15,10 +15,8 @@
 // 5.0 million gates (n = 51, l = 5, 20,001 pairs); this takes 3.4 ms.
 #include <cuda_runtime.h>
 
-#include <algorithm>
-
 #include "brick.h"
-#include "haar_fixed.h"
+#include "haar_items.h"
 #include "kernels.h"
 
 namespace fpk {
@@ -91,50 +89,6 @@ __global__ void __launch_bounds__(TH) haar_raw_kernel(SampleParams sp, const Pai
     }
 }
 
-template <typename C> __device__ __forceinline__ C fx_out(Fx2 z, int k);
-template <> __device__ __forceinline__ float2 fx_out<float2>(Fx2 z, int k) {
-    return make_float2(fx_to_float(z.x, k), fx_to_float(z.y, k));
-}
-template <> __device__ __forceinline__ double2 fx_out<double2>(Fx2 z, int k) {
-    return make_double2(fx_to_double(z.x, k), fx_to_double(z.y, k));
-}
-
-// One gate of a brickwork pair: gate g of circuit w (0 = U, 1 = V), in circuit layer
-// tl (1-based) on bond b.
-struct GateOf { int pair, w, g, tl, b; };
-
-// Items: first the gates of the inner layers 2..l-1 (V's and U's, item = (pair, w, gate)),
-// then, from item `inner` (a multiple of G) on, those of layers 1 and l, the U and the V
-// gate of one place next to each other.  Blocks never mix the two kinds.
-struct Items { int64_t inner_count, inner, outer_count; int nmid, nout, c0, c1, gl; };
-
-__device__ __forceinline__ bool gate_of(const BrickDev &d, const Items &it, int64_t i, GateOf &o) {
-    if (i < it.inner) {
-        if (i >= it.inner_count) return false;
-        const int per = 2 * it.nmid;
-        o.pair = (int)(i / per);
-        const int r = (int)(i - (int64_t)o.pair * per);
-        o.w = r / it.nmid;
-        const int k = r - o.w * it.nmid, two = it.c0 + it.c1, lay = k / two, rem = k - lay * two;
-        const bool odd = rem >= it.c1;   // layer 2 (c1 gates), 3 (c0 gates), 4, ..
-        o.g = it.c0 + k;
-        o.tl = 2 + 2 * lay + (odd ? 1 : 0);
-        o.b = 2 * (odd ? rem - it.c1 : rem) + (o.tl - 1) % 2;
-        return true;
-    }
-    i -= it.inner;
-    if (i >= it.outer_count) return false;
-    const int per = 2 * it.nout;
-    o.pair = (int)(i / per);
-    const int r = (int)(i - (int64_t)o.pair * per), k = r >> 1;
-    o.w = r & 1;
-    const bool last = k >= it.c0;
-    o.tl = last ? d.l : 1;
-    o.g = last ? it.gl + k - it.c0 : k;
-    o.b = 2 * (last ? k - it.c0 : k) + (o.tl - 1) % 2;
-    return true;
-}
-
 template <typename C, int G>
 __global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleParams sp, Items it,
                                                              const PairInfo *__restrict__ pairs, C *__restrict__ maps) {
@@ -155,11 +109,8 @@ __global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleP
     __syncwarp();
     if (!on) return;
     const bool outer = first >= it.inner;
-    const int tau = o.tl == 1 ? 2 * d.l - 3 : o.tl == d.l ? d.l - 2 : o.w ? o.tl - 2 : 2 * d.l - 2 - o.tl;
-    const int j = (tau - (o.b + 1) % 2) / 2;
     const bool left = o.b < d.cut;
-    const int mi = left ? map_index(d, 0, o.b, j) : map_index(d, 1, d.n - 2 - o.b, j);
-    C *out = maps + ((size_t)o.pair * maps_per_pair(d) + mi) * 16;
+    C *out = maps + ((size_t)o.pair * maps_per_pair(d) + map_of(d, o)) * 16;
     // entry (r, c) of the gate at r = 2 y' + x', c = 2 y + x (x: qubit b+1, primes: after the
     // gate) goes to row x + 2 x', column y + 2 y' of a left map, transposed in a right one
     auto put = [&](int r, int c, C z) {
@@ -182,33 +133,25 @@ __global__ void __launch_bounds__(TH) brick_haar_maps_kernel(BrickDev d, SampleP
 #pragma unroll 1
     for (int h = 0; h < 8; ++h) {
         const int r = 2 * o.w + (h >> 2), c = h & 3;
-        Fx2 x[4], y[4];
+        Fx2 z = {0, 0};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            x[k] = sm[(mid ? 4 * k + r : 4 * c + k) * G + us];
-            y[k] = sm[(mid ? 4 * k + c : 4 * r + k) * G + vs];
+            const Fx2 t = dot1_fixed(sm[(mid ? 4 * k + r : 4 * c + k) * G + us], sm[(mid ? 4 * k + c : 4 * r + k) * G + vs]);
+            z.x += t.x;
+            z.y += t.y;
         }
-        put(r, c, fx_out<C>(dot_fixed<4>(x, y), 60));
+        put(r, c, fx_out<C>(z, 60));
     }
 }
 
 template <typename C>
 cudaError_t maps_t(const BrickDev &d, const SampleParams &sp, const PairInfo *pairs, int npairs, C *maps,
                    cudaStream_t st) {
-    Items it;
-    it.c0 = d.n / 2;
-    it.c1 = (d.n - 1) / 2;
-    const int cl = d.l % 2 ? it.c0 : it.c1;
-    it.gl = (d.l / 2) * it.c0 + ((d.l - 1) / 2) * it.c1;   // gates before layer l
-    it.nmid = std::max(0, it.gl - it.c0);
-    it.nout = it.c0 + cl;
-    it.inner_count = (int64_t)npairs * 2 * it.nmid;
-    it.outer_count = (int64_t)npairs * 2 * it.nout;
     // few gates: 32 per CTA, whose draws all 128 threads share (a batch that fits the SMs
     // several times over has work enough with one thread per gate throughout)
-    const bool small = it.inner_count + it.outer_count <= 152 * 4 * 128;
+    const bool small = brick_gates(d, npairs) <= 152 * 4 * 128;
     const int G = small ? 32 : TH;
-    it.inner = (it.inner_count + G - 1) / G * G;
+    const Items it = make_items(d, npairs, G);
     const unsigned grid = (unsigned)((it.inner + it.outer_count + G - 1) / G);
     if (small) brick_haar_maps_kernel<C, 32><<<grid, TH, 0, st>>>(d, sp, it, pairs, maps);
     else brick_haar_maps_kernel<C, TH><<<grid, TH, 0, st>>>(d, sp, it, pairs, maps);

@@ -5,12 +5,14 @@
 // its generalised-Hadamard formula serves only the ancilla form, which this
 // direct trace contraction does not use.
 //
-// K1q  qudit_sample:  Haar U(q^2) gates, one thread per gate: q^4 complex
-//                     Gaussians (Philox block k/2 for entry k, Box-Muller),
-//                     Householder QR, columns rotated so that R's diagonal is
-//                     positive real.
-// K2q  qudit_maps:    per (bond, position) the merged gate realigned into the
-//                     q^2 x q^2 map the sweep applies (FP64, stored FP32/FP64).
+// K1q  qudit_haar_maps: Haar U(q^2) gates in 64-bit fixed point (haar_fixed.h) and, in
+//                     the same kernel, the q^2 x q^2 maps the sweep applies: Gaussian
+//                     draws by all threads, Gram-Schmidt with a lane per row (3 or 2
+//                     gates a warp, sums over the rows by shuffles), the maps entry by
+//                     entry.  Bound: the integer pipe.  With FP64 Householder QR by a
+//                     thread per gate (its 9 x 9 arrays in local memory) and a separate
+//                     map kernel 500 pairs of l = 2 at n = 50, q = 3, nearly all of it
+//                     this kernel, took 2.5 ms; they take 0.48.
 // K3q  qudit_sweep:   one CTA per pair: the boundary over the 2m segment digits
 //                     of one qudit (q^{2m} amplitudes, in shared memory when it
 //                     fits, else in a per-pair global slot), both chain halves,
@@ -18,134 +20,154 @@
 //                     error estimate.
 #include <cuda_runtime.h>
 
-#include "brick.h"
+#include <algorithm>
+
+#include "haar_items.h"
 #include "kernels.h"
+#include "meet.h"
 
 namespace fpk {
 namespace {
 
-__device__ __forceinline__ double2 qmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 qconj(double2 a) { return make_double2(a.x, -a.y); }
+constexpr size_t kQuditSmem = 200 * 1024;   // shared memory of a boundary's two copies
 
-template <int Q>
-__global__ void __launch_bounds__(64) qudit_sample_kernel(uint64_t seed, const PairInfo *__restrict__ pairs, int npairs,
-                                                           int n_raw, int self_pair, double2 *__restrict__ raw) {
-    constexpr int D = Q * Q;
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= npairs * 2 * n_raw) return;
-    const int p = id / (2 * n_raw), w = (id / n_raw) % 2, g = id % n_raw;
-    const uint64_t pair = pairs[p].pair;
-    const int ws = self_pair ? 0 : w;
-    double2 A[D][D], Qm[D][D];
-    for (int k = 0; k < D * D; k += 2) {
-        U64x4 x = philox(seed, (uint64_t)(k / 2), (uint64_t)g, pair, (uint64_t)ws);
-        for (int h = 0; h < 2 && k + h < D * D; ++h) {
-            const uint64_t xa = x.x[2 * h], xb = x.x[2 * h + 1];
-            const double u1 = (double)((xa >> 11) + 1) * 0x1.0p-53;
-            const double u2 = (double)(xb >> 11) * 0x1.0p-53;
-            const double rad = sqrt(-2.0 * log(u1)) * 0.70710678118654752440;
-            double s, c;
-            sincospi(2.0 * u2, &s, &c);
-            A[(k + h) / D][(k + h) % D] = make_double2(rad * c, rad * s);
-        }
-    }
-    for (int r = 0; r < D; ++r)
-        for (int c = 0; c < D; ++c) Qm[r][c] = make_double2(r == c ? 1.0 : 0.0, 0.0);
-    for (int k = 0; k < D - 1; ++k) {
-        double nrm2 = 0;
-        for (int r = k; r < D; ++r) nrm2 += A[r][k].x * A[r][k].x + A[r][k].y * A[r][k].y;
-        const double nrm = sqrt(nrm2), a0 = hypot(A[k][k].x, A[k][k].y);
-        const double2 ph = a0 > 0 ? make_double2(A[k][k].x / a0, A[k][k].y / a0) : make_double2(1.0, 0.0);
-        double2 v[D];
-        for (int r = 0; r < D; ++r) v[r] = r < k ? make_double2(0, 0) : A[r][k];
-        v[k].x += ph.x * nrm;
-        v[k].y += ph.y * nrm;
-        double vn2 = 0;
-        for (int r = k; r < D; ++r) vn2 += v[r].x * v[r].x + v[r].y * v[r].y;
-        if (vn2 == 0) continue;
-        const double f = 2.0 / vn2;
-        for (int c = 0; c < D; ++c) {   // A <- (I - f v v^H) A
-            double2 s = make_double2(0, 0);
-            for (int r = k; r < D; ++r) { const double2 t = qmul(qconj(v[r]), A[r][c]); s.x += t.x; s.y += t.y; }
-            for (int r = k; r < D; ++r) { const double2 t = qmul(v[r], s); A[r][c].x -= f * t.x; A[r][c].y -= f * t.y; }
-        }
-        for (int r = 0; r < D; ++r) {   // Q <- Q (I - f v v^H)
-            double2 s = make_double2(0, 0);
-            for (int j = k; j < D; ++j) { const double2 t = qmul(Qm[r][j], v[j]); s.x += t.x; s.y += t.y; }
-            for (int j = k; j < D; ++j) { const double2 t = qmul(s, qconj(v[j])); Qm[r][j].x -= f * t.x; Qm[r][j].y -= f * t.y; }
-        }
-    }
-    // Z = Q R: rotate column j of Q by the phase of R_jj so that R's diagonal is positive real
-    double2 *out = raw + (size_t)id * D * D;
-    for (int j = 0; j < D; ++j) {
-        const double m = hypot(A[j][j].x, A[j][j].y);
-        const double2 ph = m > 0 ? make_double2(A[j][j].x / m, A[j][j].y / m) : make_double2(1.0, 0.0);
-        for (int r = 0; r < D; ++r) out[r * D + j] = qmul(Qm[r][j], ph);
-    }
+// A stored map entry: FP64 the complex entry; FP32 the pairs (re, re), (-im, im), so that a
+// complex multiply-add is two packed FMAs on (x.re, x.im) and (x.im, x.re).
+struct alignas(16) Pair2 { float2 r, i; };
+template <typename C> struct Entry;
+template <> struct Entry<float2> { using T = Pair2; };
+template <> struct Entry<double2> { using T = double2; };
+template <typename C> using EntryT = typename Entry<C>::T;
+__device__ __forceinline__ void put_entry(double2 *out, Fx2 z) { *out = fx_out<double2>(z, 60); }
+__device__ __forceinline__ void put_entry(Pair2 *out, Fx2 z) {
+    const float2 v = fx_out<float2>(z, 60);
+    *out = {make_float2(v.x, v.x), make_float2(-v.y, v.y)};
 }
 
-template <typename C> __device__ __forceinline__ C to_c(double2 z);
-template <> __device__ __forceinline__ double2 to_c<double2>(double2 z) { return z; }
-template <> __device__ __forceinline__ float2 to_c<float2>(double2 z) { return make_float2((float)z.x, (float)z.y); }
+template <int Q> constexpr int kGates = 4 * (32 / (Q * Q));   // gates per CTA: 12 (q = 3), 8 (q = 4)
 
-// one map per thread: (pair, side, layer t, gate j)
 template <int Q, typename C>
-__global__ void qudit_maps_kernel(BrickDev d, int npairs, int n_raw, const double2 *__restrict__ raw,
-                                  C *__restrict__ maps) {
-    constexpr int D = Q * Q;
-    const int per = maps_per_pair(d);
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= npairs * per) return;
-    const int p = id / per, mi = id % per, g = mi / d.m, j = mi % d.m, l = d.l;
-    const int side = g < d.n_layers[0] ? 0 : 1, t = side ? g - d.n_layers[0] : g;
-    const double2 *U = raw + (size_t)p * 2 * n_raw * D * D, *V = U + (size_t)n_raw * D * D;
-    const int b = brick_bond(d, side, t);
-    const int tau = 2 * j + (b + 1) % 2;
-    const int c0 = d.n / 2, c1 = (d.n - 1) / 2;
-    auto gidx = [&](int tl) {   // circuit gate index of layer tl (1-based) on bond b
-        const int tm = tl - 1;
-        return ((tm + 1) / 2) * c0 + (tm / 2) * c1 + (b - tm % 2) / 2;
-    };
-    // the merged gate at position tau (as for qubits: V's layers, the middle and
-    // cyclic merges, U's layers daggered), computed entry by entry
-    auto G = [&](int r, int c) -> double2 {
-        if (tau <= l - 3) return V[(size_t)gidx(tau + 2) * D * D + r * D + c];
-        if (tau == l - 2 || tau == 2 * l - 3) {
-            const int tl = tau == l - 2 ? l : 1;
-            const double2 *A = U + (size_t)gidx(tl) * D * D, *B = V + (size_t)gidx(tl) * D * D;
-            double2 acc = make_double2(0, 0);
-            for (int k = 0; k < D; ++k) {   // tau = l-2: U_l^dagger V_l ; tau = 2l-3: V_1 U_1^dagger
-                const double2 x = tau == l - 2 ? qmul(qconj(A[k * D + r]), B[k * D + c]) : qmul(B[r * D + k], qconj(A[c * D + k]));
-                acc.x += x.x;
-                acc.y += x.y;
+__global__ void __launch_bounds__(128) qudit_haar_maps_kernel(BrickDev d, uint64_t seed, int self_pair, Items it,
+                                                              const PairInfo *__restrict__ pairs,
+                                                              EntryT<C> *__restrict__ maps) {
+    constexpr int D = Q * Q, G = kGates<Q>, GW = 32 / D, NB = (D * D + 1) / 2;
+    constexpr int RS = D | 1;   // row stride: odd, so that the rows of a column lie in different banks
+    __shared__ Fx2 sm[G][D * RS];
+    __shared__ GateOf gate[G];
+    __shared__ uint8_t on[G];
+    const int64_t first = (int64_t)blockIdx.x * G;
+    if (threadIdx.x < G) on[threadIdx.x] = gate_of(d, it, first + threadIdx.x, gate[threadIdx.x]) ? 1 : 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < G * NB; i += 128) {
+        const int g = i / NB, j = i - g * NB;
+        if (!on[g]) continue;
+        const GateOf &o = gate[g];
+        const U64x4 x = philox(seed, (uint64_t)j, (uint64_t)o.g, pairs[o.pair].pair, (uint64_t)(self_pair ? 0 : o.w));
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h)
+            if (const int e = 2 * j + h; e < D * D)
+                sm[g][e / D * RS + e % D] = gauss_fixed(h ? x.x[2] : x.x[0], h ? x.x[3] : x.x[1]);
+    }
+    __syncthreads();
+    {
+        // lane = (gate of the warp, row); spare lanes repeat row 0 of the warp's first gate and
+        // write nothing.  Every lane runs every step, so the shuffles are warp-wide.
+        const int lane = threadIdx.x & 31;
+        const bool act = lane < GW * D;
+        const int gw = act ? lane / D : 0, r = act ? lane - gw * D : 0, g = (threadIdx.x >> 5) * GW + gw;
+        auto src = [&](int k) { return act ? gw * D + (r + k) % D : lane; };
+        const int s1 = src(1), s2 = src(2), s3 = src(3), s6 = src(6);
+        // over the rows of a gate: threes of threes (D = 9) or halves (D = 16)
+        auto rows = [&](auto x, auto op) {
+            if constexpr (D == 9) {
+                x = op(op(x, __shfl_sync(0xffffffffu, x, s3)), __shfl_sync(0xffffffffu, x, s6));
+                return op(op(x, __shfl_sync(0xffffffffu, x, s1)), __shfl_sync(0xffffffffu, x, s2));
+            } else {
+#pragma unroll
+                for (int k = 8; k > 0; k >>= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, k));
+                return x;
             }
-            return acc;
-        }
-        return qconj(U[(size_t)gidx(2 * l - 2 - tau) * D * D + c * D + r]);
-    };
-    C *out = maps + (size_t)id * D * D;
-    const bool left = side == 0;
-    // gate index (a_b q + a_{b+1}); segment tau (in) and tau+1 (out) of qudits y = b, x = b+1;
-    // map index e = w_tau + q w_{tau+1}: left M[ex][ey], right M[ey][ex]
-    for (int yt = 0; yt < Q; ++yt)
-        for (int xt = 0; xt < Q; ++xt)
-            for (int yt1 = 0; yt1 < Q; ++yt1)
-                for (int xt1 = 0; xt1 < Q; ++xt1) {
-                    const double2 gv = G(yt1 * Q + xt1, yt * Q + xt);
-                    const int ex = xt + Q * xt1, ey = yt + Q * yt1;
-                    out[left ? ex * D + ey : ey * D + ex] = to_c<C>(gv);
+        };
+        auto sum = [&](int64_t x) {
+            return (int64_t)rows((long long)x, [](long long a, long long b) { return a + b; });
+        };
+        auto lead = [&](Fx2 v) { return rows(lead1_fixed(v), [](int a, int b) { return min(a, b); }); };
+#pragma unroll 1
+        for (int c = 0; c < D; ++c) {
+            Fx2 v = sm[g][r * RS + c];
+            if (c) {
+                shift1_fixed(v, lead(v) - kRoom);
+                for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+                    for (int k = 0; k < c; ++k) {
+                        const Fx2 q = sm[g][r * RS + k], t = dot1_fixed(q, v);
+                        sub1_fixed(v, q, halves(sum(t.x)), halves(sum(t.y)));
+                    }
+                    const int drop = lead(v) - kRoom;
+                    if (pass == 1 || !__any_sync(0xffffffffu, drop >= kRedo<D>)) break;
+                    shift1_fixed(v, drop);   // (a second pass that a gate did not need does no harm)
                 }
+            }
+            shift1_fixed(v, lead(v) - kUnitRoom<D>);
+            int h;
+            const Half y = inv_norm_fixed((uint64_t)sum(norm1_fixed(v)), h);
+            scale1_fixed(v, y, h);
+            if (act) sm[g][r * RS + c] = v;
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    // maps, coalesced: entry e = row D + column; index e = w_tau + q w_tau+1 of the qudit's
+    // segments, rows the neighbour's (x) in a left map, columns in a right one
+    const bool outer = first >= it.inner;
+    for (int i = threadIdx.x; i < (outer ? G / 2 : G) * D * D; i += 128) {
+        const int p = i / (D * D), e = i - p * D * D, g = outer ? 2 * p : p;
+        if (!on[g]) continue;
+        const GateOf &o = gate[g];
+        const bool left = o.b < d.cut;
+        const int ex = left ? e / D : e % D, ey = left ? e % D : e / D;
+        const int r = (ey / Q) * Q + ex / Q, c = (ey % Q) * Q + ex % Q;   // gate row (after), column (before): q y + x
+        Fx2 z;
+        if (!outer) {
+            z = o.w ? sm[g][r * RS + c] : sm[g][c * RS + r];
+            if (!o.w) z.y = -z.y;
+        } else {   // U_l^dagger V_l, or V_1 U_1^dagger
+            const bool mid = o.tl == d.l;
+            z = {0, 0};
+#pragma unroll 1
+            for (int k = 0; k < D; ++k) {
+                const Fx2 t = dot1_fixed(sm[g][mid ? k * RS + r : c * RS + k], sm[g + 1][mid ? k * RS + c : r * RS + k]);
+                z.x += t.x;
+                z.y += t.y;
+            }
+        }
+        put_entry(&maps[((size_t)o.pair * maps_per_pair(d) + map_of(d, o)) * D * D + e], z);
+    }
 }
 
-template <typename C>
-__device__ __forceinline__ C cfmaq(C t, C x, C acc) {
+// acc + t x; the FP32 form takes x and its swapped copy xs
+__device__ __forceinline__ double2 cfmaq(double2 t, double2 x, double2, double2 acc) {
     acc.x = fma(t.x, x.x, acc.x);
     acc.x = fma(-t.y, x.y, acc.x);
     acc.y = fma(t.x, x.y, acc.y);
     acc.y = fma(t.y, x.x, acc.y);
     return acc;
+}
+__device__ __forceinline__ float2 cfmaq(const Pair2 &t, float2 x, float2 xs, float2 acc) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd, re;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "mov.b64 rd, {%8, %9};\n\tmov.b64 re, {%10, %11};\n\t"
+        "fma.rn.f32x2 re, ra, rc, re;\n\tfma.rn.f32x2 re, rb, rd, re;\n\tmov.b64 {%0, %1}, re;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(t.r.x), "f"(t.r.y), "f"(t.i.x), "f"(t.i.y), "f"(x.x), "f"(x.y), "f"(xs.x), "f"(xs.y), "f"(acc.x), "f"(acc.y));
+    return d;
+}
+template <typename C> __device__ __forceinline__ C swapped(C x) {
+    C s;
+    s.x = x.y;
+    s.y = x.x;
+    return s;
 }
 
 __device__ __forceinline__ double qsum(double v) {
@@ -154,25 +176,158 @@ __device__ __forceinline__ double qsum(double v) {
     return v;
 }
 
-// One CTA per pair.  The state lives at `st` (shared memory or the pair's
-// global slot), the left boundary at `lb`.  Maps are applied one at a time:
+// Results of a pair from the thread sums of its meet (all threads of the CTA).
+__device__ __forceinline__ void qudit_results(double sr, double si, double sa, double s2, const PairInfo &pi,
+                                              double err_scale, double *tr, double *kappa, double *err) {
+    __shared__ double red[4][8];
+    sr = qsum(sr); si = qsum(si); sa = qsum(sa); s2 = qsum(s2);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) { red[0][wid] = sr; red[1][wid] = si; red[2][wid] = sa; red[3][wid] = s2; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s[4] = {0, 0, 0, 0};
+        for (int c = 0; c < 4; ++c)
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s[c] += red[c][w];
+        write_meet(pi, s, err_scale, tr, kappa, err);
+    }
+}
+
+template <typename C>
+__device__ __forceinline__ void meet_term(C l, C r, double &sr, double &si, double &sa, double &s2) {
+    const double px = (double)l.x * r.x - (double)l.y * r.y, py = (double)l.x * r.y + (double)l.y * r.x;
+    sr += px;
+    si += py;
+    sa += sqrt(px * px + py * py);
+    s2 += px * px + py * py;
+}
+
+// Boundaries that fit shared memory twice (q^N <= 200 KB / 2): one CTA per pair, every map
+// read from one copy and written to the other, so that one barrier per map suffices.  A
+// work item is a group of q^2 amplitudes and q of its outputs (a boundary of 9^3 would keep
+// 81 of 256 threads busy with a group each), or, for BIG boundaries, two groups and all
+// their outputs, which reads every map entry from shared memory once for two products.
+// The next map arrives by cp.async meanwhile.  The left half waits in `lscr`.
+// Bound: FP32 issue.  500 pairs at n = 50, q = 3, FP32, sampler and maps included: l = 5 2.9 ms
+// against 8.0, l = 4 1.1 against 5.0 (a group per thread in place, two barriers per map).
+template <int Q, typename C, bool BIG>
+__global__ void __launch_bounds__(256) qudit_smem_kernel(BrickDev d, const PairInfo *__restrict__ pairs,
+                                                         const EntryT<C> *__restrict__ maps, C *__restrict__ lscr,
+                                                         double err_scale, double *__restrict__ tr,
+                                                         double *__restrict__ kappa, double *__restrict__ err) {
+    constexpr int D = Q * Q, GI = BIG ? 2 : 1, OI = BIG ? Q : 1;   // groups and output rows of an item
+    extern __shared__ __align__(16) unsigned char qsm[];
+    __shared__ __align__(16) EntryT<C> T[2][D * D];
+    const int p = blockIdx.x, N = d.N;
+    uint32_t S = 1;
+    for (int i = 0; i < N; ++i) S *= Q;
+    C *A = (C *)qsm, *B = A + S;
+    const EntryT<C> *mp = maps + (size_t)p * maps_per_pair(d) * D * D;
+    const int nmaps = maps_per_pair(d);   // side 0's maps, then side 1's, in sweep order
+    auto stage = [&](int k) {
+        if (k < nmaps)
+            for (int i = threadIdx.x; i < D * D; i += blockDim.x) cp_async<16>(&T[k & 1][i], &mp[(size_t)k * D * D + i]);
+    };
+    stage(0);
+    int k = 0;
+    for (int side = 0; side < 2; ++side) {
+        const int par = d.delta_par[side];
+        for (uint32_t w = threadIdx.x; w < S; w += blockDim.x) {
+            bool ok = true;
+            uint32_t x = w, prev = 0, w0 = 0;
+            for (int t = 0; t < N; ++t) {   // digits t and t+1 (mod N) equal for t of parity par
+                const uint32_t dig = x % Q;
+                x /= Q;
+                if (t == 0) w0 = dig;
+                else if (((t - 1) & 1) == par) ok = ok && dig == prev;
+                prev = dig;
+            }
+            if (((N - 1) & 1) == par) ok = ok && prev == w0;
+            C v;
+            v.x = ok ? 1 : 0;
+            v.y = 0;
+            A[w] = v;
+        }
+        for (int t = 0; t < d.n_layers[side]; ++t) {
+            const int par_t = layer_parity(d, side, t);
+            for (int j = 0; j < d.m; ++j, ++k) {
+                cp_async_wait_all();
+                __syncthreads();   // this map and the state are in place; the other buffers are free
+                stage(k + 1);
+                const EntryT<C> *Tk = T[k & 1];
+                const int pa = 2 * j + par_t, pb = (pa + 1) % N;
+                uint32_t sa = 1, sb = 1;   // powers of q
+                for (int i = 0; i < pa; ++i) sa *= Q;
+                for (int i = 0; i < pb; ++i) sb *= Q;
+                const uint32_t plo = pa < pb ? sa : sb, phi = pa < pb ? sb : sa;
+                const uint32_t ng = S / D, half = BIG ? (ng + 1) / 2 : ng;
+                for (uint32_t item = threadIdx.x; item < half * (BIG ? 1 : Q); item += blockDim.x) {
+                    const uint32_t og0 = item / half, g0 = item - og0 * half;
+                    uint32_t base[GI];
+                    C x[GI][D], xs[GI][D];
+#pragma unroll
+                    for (int u = 0; u < GI; ++u) {
+                        const uint32_t g = u == 0 || g0 + half < ng ? g0 + u * half : g0;   // (odd count: the middle one twice)
+                        const uint32_t r1 = g / plo, x1 = g + r1 * plo * (Q - 1);           // zero digits at the two positions
+                        const uint32_t r2 = x1 / phi;
+                        base[u] = x1 + r2 * phi * (Q - 1);
+#pragma unroll
+                        for (int e = 0; e < D; ++e) x[u][e] = A[base[u] + (e % Q) * sa + (e / Q) * sb], xs[u][e] = swapped(x[u][e]);
+                    }
+#pragma unroll 1
+                    for (int oi = 0; oi < OI; ++oi) {
+                        const uint32_t og = BIG ? (uint32_t)oi : og0;
+                        C acc[GI][Q];
+#pragma unroll
+                        for (int u = 0; u < GI; ++u)
+#pragma unroll
+                            for (int o = 0; o < Q; ++o) acc[u][o].x = 0, acc[u][o].y = 0;
+                        const EntryT<C> *row = Tk + og * Q * D;
+#pragma unroll
+                        for (int e = 0; e < D; ++e)
+#pragma unroll
+                            for (int o = 0; o < Q; ++o) {
+                                const EntryT<C> tv = row[o * D + e];
+#pragma unroll
+                                for (int u = 0; u < GI; ++u) acc[u][o] = cfmaq(tv, x[u][e], xs[u][e], acc[u][o]);
+                            }
+#pragma unroll
+                        for (int u = 0; u < GI; ++u)
+#pragma unroll
+                            for (int o = 0; o < Q; ++o) B[base[u] + o * sa + og * sb] = acc[u][o];   // output og q + o
+                    }
+                }
+                C *tmp = A;
+                A = B;
+                B = tmp;
+            }
+        }
+        __syncthreads();
+        if (side == 0)
+            for (uint32_t w = threadIdx.x; w < S; w += blockDim.x) lscr[(size_t)p * S + w] = A[w];
+        // (each thread reads back what it wrote, and rewrites A only where it has read it)
+    }
+    double sr = 0, si = 0, sa = 0, s2 = 0;
+    for (uint32_t w = threadIdx.x; w < S; w += blockDim.x) meet_term(lscr[(size_t)p * S + w], A[w], sr, si, sa, s2);
+    qudit_results(sr, si, sa, s2, pairs[p], err_scale, tr, kappa, err);
+}
+
+// Larger boundaries: one CTA per pair, the state and the left boundary in the pair's
+// global slot.  Maps are applied one at a time, in place:
 // every thread takes groups of q^2 amplitudes that differ only in digits
 // (tau, tau+1 mod N), one barrier per map.
 template <int Q, typename C>
 __global__ void __launch_bounds__(256) qudit_sweep_kernel(BrickDev d, const PairInfo *__restrict__ pairs,
-                                                           const C *__restrict__ maps, C *__restrict__ gstate,
-                                                           int in_smem, double err_scale, double *__restrict__ tr,
+                                                           const EntryT<C> *__restrict__ maps, C *__restrict__ gstate,
+                                                           double err_scale, double *__restrict__ tr,
                                                            double *__restrict__ kappa, double *__restrict__ err) {
     constexpr int D = Q * Q;
-    extern __shared__ __align__(16) unsigned char qsm[];
-    __shared__ double red[4][8];
-    __shared__ C T[D * D];
+    __shared__ EntryT<C> T[D * D];
     const int p = blockIdx.x, N = d.N;
     uint32_t S = 1;
     for (int i = 0; i < N; ++i) S *= Q;
-    C *st = in_smem ? (C *)qsm : gstate + (size_t)p * 2 * S;
-    C *lb = in_smem ? (C *)qsm + S : gstate + (size_t)p * 2 * S + S;
-    const C *mp = maps + (size_t)p * maps_per_pair(d) * D * D;
+    C *st = gstate + (size_t)p * 2 * S;
+    C *lb = st + S;
+    const EntryT<C> *mp = maps + (size_t)p * maps_per_pair(d) * D * D;
     uint32_t pw[32];
     pw[0] = 1;
     for (int i = 1; i <= N; ++i) pw[i] = pw[i - 1] * Q;
@@ -194,7 +349,7 @@ __global__ void __launch_bounds__(256) qudit_sweep_kernel(BrickDev d, const Pair
         for (int t = 0; t < d.n_layers[side]; ++t) {
             const int par_t = layer_parity(d, side, t);
             for (int j = 0; j < d.m; ++j) {
-                const C *src = mp + (size_t)map_index(d, side, t, j) * D * D;
+                const EntryT<C> *src = mp + (size_t)map_index(d, side, t, j) * D * D;
                 for (int i = threadIdx.x; i < D * D; i += blockDim.x) T[i] = src[i];
                 __syncthreads();
                 const int pa = 2 * j + par_t, pb = (pa + 1) % N;
@@ -206,20 +361,22 @@ __global__ void __launch_bounds__(256) qudit_sweep_kernel(BrickDev d, const Pair
                     const uint32_t x1 = a1 + r1 * pw[lo + 1];
                     const uint32_t a2 = x1 % pw[hi], r2 = x1 / pw[hi];
                     const uint32_t base = a2 + r2 * pw[hi + 1];
-                    C x[D], y[D];
+                    C x[D];
 #pragma unroll
                     for (int e = 0; e < D; ++e) x[e] = st[base + (e % Q) * sa + (e / Q) * sb];
+                    // q outputs at a time: with all q^2 in flight the FP64 and q = 4 forms spilled
+#pragma unroll 1
+                    for (int og = 0; og < Q; ++og) {
+                        C acc[Q];
 #pragma unroll
-                    for (int o = 0; o < D; ++o) {
-                        C acc;
-                        acc.x = 0;
-                        acc.y = 0;
+                        for (int o = 0; o < Q; ++o) acc[o].x = 0, acc[o].y = 0;
 #pragma unroll
-                        for (int e = 0; e < D; ++e) acc = cfmaq(T[o * D + e], x[e], acc);
-                        y[o] = acc;
+                        for (int e = 0; e < D; ++e)
+#pragma unroll
+                            for (int o = 0; o < Q; ++o) acc[o] = cfmaq(T[(og * Q + o) * D + e], x[e], swapped(x[e]), acc[o]);
+#pragma unroll
+                        for (int o = 0; o < Q; ++o) st[base + o * sa + og * sb] = acc[o];
                     }
-#pragma unroll
-                    for (int e = 0; e < D; ++e) st[base + (e % Q) * sa + (e / Q) * sb] = y[e];
                 }
                 __syncthreads();
             }
@@ -230,86 +387,55 @@ __global__ void __launch_bounds__(256) qudit_sweep_kernel(BrickDev d, const Pair
         }
     }
     double sr = 0, si = 0, sa = 0, s2 = 0;
-    for (uint32_t w = threadIdx.x; w < S; w += blockDim.x) {
-        const C l = lb[w], r = st[w];
-        const double px = (double)l.x * r.x - (double)l.y * r.y, py = (double)l.x * r.y + (double)l.y * r.x;
-        sr += px;
-        si += py;
-        sa += sqrt(px * px + py * py);
-        s2 += px * px + py * py;
-    }
-    sr = qsum(sr); si = qsum(si); sa = qsum(sa); s2 = qsum(s2);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { red[0][wid] = sr; red[1][wid] = si; red[2][wid] = sa; red[3][wid] = s2; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        sr = si = sa = s2 = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sr += red[0][w]; si += red[1][w]; sa += red[2][w]; s2 += red[3][w]; }
-        const int64_t o = pairs[p].out;
-        tr[2 * o] = sr;
-        tr[2 * o + 1] = si;
-        const double mag = sqrt(sr * sr + si * si);
-        if (kappa) kappa[o] = mag > 0 ? sa / mag : __longlong_as_double(0x7ff0000000000000LL);
-        if (err) err[o] = err_scale * (sqrt(s2) + mag);
-    }
+    for (uint32_t w = threadIdx.x; w < S; w += blockDim.x) meet_term(lb[w], st[w], sr, si, sa, s2);
+    qudit_results(sr, si, sa, s2, pairs[p], err_scale, tr, kappa, err);
 }
 
-template <int Q>
-cudaError_t run_qudit_t(const BrickDev &d, uint64_t seed, const PairInfo *pairs, int npairs, int n_raw, int self_pair,
-                        bool fp32, void *ws, double err_scale, double *tr, double *kappa, double *err, cudaStream_t st) {
+template <int Q, typename C>
+cudaError_t run_qc(const BrickDev &d, uint64_t seed, const PairInfo *pairs, int npairs, int self_pair, void *ws,
+                   double err_scale, double *tr, double *kappa, double *err, cudaStream_t st) {
     constexpr int D = Q * Q;
     size_t S = 1;
     for (int i = 0; i < d.N; ++i) S *= Q;
-    const size_t celem = fp32 ? sizeof(float2) : sizeof(double2);
-    double2 *raw = (double2 *)ws;
-    unsigned char *maps = (unsigned char *)(raw + (size_t)npairs * 2 * n_raw * D * D);
-    const size_t nmaps = (size_t)npairs * maps_per_pair(d);
-    unsigned char *gstate = maps + nmaps * D * D * celem;
-    const int total = npairs * 2 * n_raw;
-    qudit_sample_kernel<Q><<<(total + 63) / 64, 64, 0, st>>>(seed, pairs, npairs, n_raw, self_pair, raw);
+    EntryT<C> *maps = (EntryT<C> *)ws;
+    C *state = (C *)(maps + (size_t)npairs * maps_per_pair(d) * D * D);
+    const Items it = make_items(d, npairs, kGates<Q>);
+    const unsigned grid = (unsigned)((it.inner + it.outer_count + kGates<Q> - 1) / kGates<Q>);
+    qudit_haar_maps_kernel<Q, C><<<grid, 128, 0, st>>>(d, seed, self_pair, it, pairs, maps);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const unsigned mb = (unsigned)((nmaps + 127) / 128);
-    if (fp32) qudit_maps_kernel<Q, float2><<<mb, 128, 0, st>>>(d, npairs, n_raw, raw, (float2 *)maps);
-    else qudit_maps_kernel<Q, double2><<<mb, 128, 0, st>>>(d, npairs, n_raw, raw, (double2 *)maps);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t smem = 2 * S * celem;
-    const int in_smem = smem <= (size_t)200 * 1024 ? 1 : 0;
-    const size_t dyn = in_smem ? smem : 0;
-    if (fp32) {
-        if ((e = cudaFuncSetAttribute(qudit_sweep_kernel<Q, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)dyn)) != cudaSuccess)
-            return e;
-        qudit_sweep_kernel<Q, float2><<<npairs, 256, dyn, st>>>(d, pairs, (const float2 *)maps, (float2 *)gstate,
-                                                               in_smem, err_scale, tr, kappa, err);
+    const size_t smem = 2 * S * sizeof(C);
+    if (smem <= kQuditSmem) {
+        // two groups a thread from 512 groups up (q = 3, l = 5), where they still fill 192 threads twice
+        const bool big = S / D >= 512;
+        auto kern = big ? qudit_smem_kernel<Q, C, true> : qudit_smem_kernel<Q, C, false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        const int threads = big ? 192 : std::min(256, ((int)(S / Q) + 31) / 32 * 32);
+        kern<<<npairs, threads, smem, st>>>(d, pairs, maps, state, err_scale, tr, kappa, err);
     } else {
-        if ((e = cudaFuncSetAttribute(qudit_sweep_kernel<Q, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)dyn)) != cudaSuccess)
-            return e;
-        qudit_sweep_kernel<Q, double2><<<npairs, 256, dyn, st>>>(d, pairs, (const double2 *)maps,
-                                                                (double2 *)gstate, in_smem, err_scale, tr, kappa, err);
+        qudit_sweep_kernel<Q, C><<<npairs, 256, 0, st>>>(d, pairs, maps, state, err_scale, tr, kappa, err);
     }
     return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t qudit_workspace_per_pair(int q, const BrickDev &d, int n_raw, bool fp32) {
+size_t qudit_workspace_per_pair(int q, const BrickDev &d, bool fp32) {
     const size_t D = (size_t)q * q, celem = fp32 ? sizeof(float2) : sizeof(double2);
     size_t S = 1;
     for (int i = 0; i < d.N; ++i) S *= (size_t)q;
-    const bool in_smem = 2 * S * celem <= (size_t)200 * 1024;
-    return (size_t)2 * n_raw * D * D * sizeof(double2) + (size_t)maps_per_pair(d) * D * D * celem +
-           (in_smem ? 0 : 2 * S * celem);
+    return (size_t)maps_per_pair(d) * D * D * 16 + (2 * S * celem <= kQuditSmem ? S : 2 * S) * celem;
 }
 
-cudaError_t launch_qudit(int q, const BrickDev &d, uint64_t seed, const PairInfo *pairs, int npairs, int n_raw, int self_pair,
+cudaError_t launch_qudit(int q, const BrickDev &d, uint64_t seed, const PairInfo *pairs, int npairs, int self_pair,
                          bool fp32, void *ws, double err_scale, double *tr, double *kappa, double *err,
                          cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
     switch (q) {
-        case 3: return run_qudit_t<3>(d, seed, pairs, npairs, n_raw, self_pair, fp32, ws, err_scale, tr, kappa, err, st);
-        case 4: return run_qudit_t<4>(d, seed, pairs, npairs, n_raw, self_pair, fp32, ws, err_scale, tr, kappa, err, st);
+        case 3: return fp32 ? run_qc<3, float2>(d, seed, pairs, npairs, self_pair, ws, err_scale, tr, kappa, err, st)
+                            : run_qc<3, double2>(d, seed, pairs, npairs, self_pair, ws, err_scale, tr, kappa, err, st);
+        case 4: return fp32 ? run_qc<4, float2>(d, seed, pairs, npairs, self_pair, ws, err_scale, tr, kappa, err, st)
+                            : run_qc<4, double2>(d, seed, pairs, npairs, self_pair, ws, err_scale, tr, kappa, err, st);
         default: return cudaErrorInvalidValue;
     }
 }

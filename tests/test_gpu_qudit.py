@@ -51,6 +51,19 @@ def test_qudit_mixed_depths_and_global_state(fp):
     assert rel(t, ref).max() <= 1e-10
 
 
+# gates by the 12 (q = 3) and 8 (q = 4) of a CTA: fewer, exactly one CTA's, ragged; boundaries from
+# one group of q^2 amplitudes up to the largest shared-memory one and the smallest global one
+@pytest.mark.parametrize("q,n,l,count", [(3, 2, 2, 1), (3, 3, 3, 3), (3, 4, 5, 2), (3, 5, 2, 7), (4, 2, 2, 5), (4, 4, 2, 1),
+                                         (4, 3, 3, 3), (4, 5, 3, 2), (4, 4, 4, 2), (4, 3, 5, 1)])
+def test_qudit_every_shape(fp, q, n, l, count):
+    ens = fp.Ensemble(fp.PARALLEL, n, l, l, seed=47, q=q)
+    ref = np.array([O.trace_qudit(q, n, l, 47, 3 + p, "dense") for p in range(count)])
+    t64, _, _ = ens.trace_batch(3, count, fp.PREC_FP64)
+    assert rel(t64, ref).max() <= 1e-10
+    t32, _, _, e32 = ens.trace_batch(3, count, fp.PREC_FP32_RAW, with_err=True)
+    assert np.all(np.abs(t32 - t64) <= e32)
+
+
 def test_qudit_self_pair_is_dimension(fp):
     for l in (4, 6):
         ens = fp.Ensemble(fp.PARALLEL, 50, l, l, seed=44, q=3, flags=fp.FLAG_SELF_PAIR)
