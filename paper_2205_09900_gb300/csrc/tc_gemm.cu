@@ -3,16 +3,18 @@
 //
 //   C[M x N] = A[M x K] . Bt[N x K]^T (+ bias),  BF16 operands, FP32 accumulate
 //
-// One CTA (128 threads) owns a 128 x NT output tile (NT <= 256 columns) whose
-// FP32 accumulator lives in tensor memory (TMEM: NT columns x 128 lanes).  The
+// One CTA per SM walks 128 x NT output tiles (NT <= 256 columns).  The FP32
+// accumulators of two tiles live in tensor memory (TMEM: 2 x NT columns x 128
+// lanes), so that the epilogue of one tile runs beside the MMAs of the next.  The
 // K loop streams stages of 64 columns through a ring of TC_STAGES shared-memory
 // buffers, warp-specialised: one lane issues the TMA loads
 // (cp.async.bulk.tensor, completing on the stage's "full" mbarrier), one lane
 // waits for them and issues four tcgen05.mma (K = 16 each) and a
 // tcgen05.commit to the stage's "empty" mbarrier, which the loader waits on
-// before it refills the buffer.  A last commit signals the accumulator; the
-// epilogue reads it back with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31,
-// i.e. tile rows 32w..32w+31), adds the bias and applies one of
+// before it refills the buffer; the tile's last commit signals its accumulator.
+// Eight epilogue warps read it back with tcgen05.ld (warp w reaches TMEM lanes
+// 32 (w mod 4) .. + 31, i.e. those tile rows; two warps share them by columns),
+// add the bias and apply one of
 //   mode 0: identity,
 //   mode 1: GELU (the pre-activation optionally kept in Z),
 //   mode 2: multiply by GELU'(Z) (Z read: the backward pass of a GELU layer),
@@ -20,6 +22,8 @@
 // Tiles are 128-byte rows (64 BF16 of K) in the 128-byte swizzle, one TMA box
 // per operand and stage; rows and columns beyond the matrices are zero-filled
 // by the TMA unit.
+// Bound: 65536 x 256 x 2400 (80 GFLOP, 348 MB) is limited by HBM (51 us) and by the
+// weights' rereading from L2 (1.2 MB per tile).  GEMM_FIGURES
 // Every wait is bounded: on timeout the kernel raises the error flag, still
 // releases its TMEM, and returns; launches that find the flag raised return at
 // once.
@@ -28,8 +32,10 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
+#include <vector>
 
 #include "fp.h"
 #include "kernels.h"
@@ -37,7 +43,7 @@
 namespace fpk {
 namespace {
 
-constexpr int TC_BM = 128, TC_BK = 64, TC_THREADS = 128, TC_MAXN = 256, TC_STAGES = 4;
+constexpr int TC_BM = 128, TC_BK = 64, TC_EPI = 8, TC_THREADS = 64 + 32 * TC_EPI, TC_MAXN = 256, TC_STAGES = 4;
 constexpr uint64_t TC_DRAIN_NS = 1000000000ull;   // waits for work already issued (after a timeout)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -104,32 +110,36 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap *map, i
 // Shared memory per stage: the A tile [128 rows x 128 bytes] then the B tile
 // [boxn rows x 128 bytes], both written by the TMA unit with the 128-byte
 // swizzle that the MMA descriptors declare; stage bases 1024-byte aligned.
+// Warp 0: TMA producer, warp 1: MMA issuer, warps 2..9: epilogue.
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const __grid_constant__ CUtensorMap tmA,
-                                                                const __grid_constant__ CUtensorMap tmB, int boxn) {
+                                                                const __grid_constant__ CUtensorMap tmB, int boxn,
+                                                                int tiles_n, int tiles) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], done;
+    __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], tfull[2], tempty[2], done;
     __shared__ uint32_t taddr_sh;
-    __shared__ int abort_sh;
+    __shared__ volatile int abort_sh;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // an earlier launch timed out: do nothing (one read, so that the whole CTA agrees)
     if (tid == 0) abort_sh = g.err ? *(volatile const int *)g.err : 0;
     __syncthreads();
     if (abort_sh) return;
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int m0 = blockIdx.x * TC_BM, n0 = blockIdx.y * TC_MAXN;
-    const int NT = min(TC_MAXN, g.N - n0);   // a multiple of 16
-    const uint32_t ncols = NT <= 32 ? 32u : (NT <= 64 ? 64u : (NT <= 128 ? 128u : 256u));
+    const uint32_t ncols = boxn <= 32 ? 32u : (boxn <= 64 ? 64u : (boxn <= 128 ? 128u : 256u));   // per accumulator
     const uint32_t a_bytes = TC_BM * TC_BK * 2, b_bytes = (uint32_t)boxn * TC_BK * 2;
     const uint32_t stage_bytes = a_bytes + TC_MAXN * TC_BK * 2;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&taddr_sh)),
-                     "r"(ncols));
+                     "r"(2 * ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 32) {
         for (int s = 0; s < TC_STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&tfull[s], 1);
+            mbar_init(&tempty[s], TC_EPI);
         }
         mbar_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -142,130 +152,154 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
     const uint32_t taddr = taddr_sh;
     const int nk = (g.K + TC_BK - 1) / TC_BK;
     const uint32_t sbase = smem_u32(smem);
-    int issued = 0;   // producer: stages whose TMA loads were issued
     if (tid == 0) {
-        // producer: TMA loads of stage kt once the MMAs of stage kt - S have drained the buffer
-        for (int kt = 0; kt < nk; ++kt) {
-            const int s = kt % TC_STAGES, u = kt / TC_STAGES;
-            if (abort_sh || (u > 0 && !mbar_wait(smem_u32(&empty[s]), (uint32_t)(u - 1) & 1u, g.wait_ns))) {
-                abort_sh = 1;
-                break;
+        // producer: TMA loads of a stage once the MMAs TC_STAGES stages earlier have drained the buffer
+        int it = 0;
+        for (int t = blockIdx.x; t < tiles && !abort_sh; t += gridDim.x) {
+            const int m0 = t / tiles_n * TC_BM, n0 = t % tiles_n * TC_MAXN;
+            for (int kt = 0; kt < nk; ++kt, ++it) {
+                const int s = it % TC_STAGES, u = it / TC_STAGES;
+                if (abort_sh || (u > 0 && !mbar_wait(smem_u32(&empty[s]), (uint32_t)(u - 1) & 1u, g.wait_ns))) {
+                    abort_sh = 1;
+                    break;
+                }
+                const uint32_t fb = smem_u32(&full[s]);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(a_bytes + b_bytes)
+                             : "memory");
+                const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
+                tma_load(sa, &tmA, kt * TC_BK, m0, fb);
+                tma_load(sb, &tmB, kt * TC_BK, n0, fb);
             }
-            const uint32_t fb = smem_u32(&full[s]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(a_bytes + b_bytes)
-                         : "memory");
-            const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
-            tma_load(sa, &tmA, kt * TC_BK, m0, fb);
-            tma_load(sb, &tmB, kt * TC_BK, n0, fb);
-            ++issued;
         }
         // after a timeout: wait (bounded) for the loads still in flight, the last
         // issued phase of each stage buffer
         if (abort_sh)
-            for (int kt = (issued > TC_STAGES ? issued - TC_STAGES : 0); kt < issued; ++kt)
-                mbar_wait(smem_u32(&full[kt % TC_STAGES]), (uint32_t)(kt / TC_STAGES) & 1u, TC_DRAIN_NS);
+            for (int i = (it > TC_STAGES ? it - TC_STAGES : 0); i < it; ++i)
+                mbar_wait(smem_u32(&full[i % TC_STAGES]), (uint32_t)(i / TC_STAGES) & 1u, TC_DRAIN_NS);
     } else if (tid == 32) {
         // MMA issuer: four K = 16 steps per stage, then release the buffer
-        const uint32_t idesc = make_idesc(TC_BM, NT);
-        bool ok = true, any = false;
-        for (int kt = 0; kt < nk; ++kt) {
-            const int s = kt % TC_STAGES, u = kt / TC_STAGES;
-            if (abort_sh || !mbar_wait(smem_u32(&full[s]), (uint32_t)u & 1u, g.wait_ns)) {
-                ok = false;
+        bool any = false;
+        int it = 0, i = 0;   // stages and tiles so far
+        for (int t = blockIdx.x; t < tiles && !abort_sh; t += gridDim.x, ++i) {
+            const int acc = i & 1, n0 = t % tiles_n * TC_MAXN;
+            const uint32_t idesc = make_idesc(TC_BM, min(TC_MAXN, g.N - n0)), td = taddr + (uint32_t)acc * ncols;
+            // the accumulator's previous tile has been read
+            if (i >= 2 && !mbar_wait(smem_u32(&tempty[acc]), (uint32_t)(i / 2 - 1) & 1u, g.wait_ns)) {
+                abort_sh = 1;
                 break;
             }
-            any = true;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
+            for (int kt = 0; kt < nk; ++kt, ++it) {
+                const int s = it % TC_STAGES, u = it / TC_STAGES;
+                if (abort_sh || !mbar_wait(smem_u32(&full[s]), (uint32_t)u & 1u, g.wait_ns)) {
+                    abort_sh = 1;
+                    break;
+                }
+                any = true;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
 #pragma unroll
-            for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                const uint64_t ad = make_desc_sw128(sa + kk * 32);
-                const uint64_t bd = make_desc_sw128(sb + kk * 32);
-                const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.u32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(taddr),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+                for (int kk = 0; kk < TC_BK / 16; ++kk) {
+                    const uint64_t ad = make_desc_sw128(sa + kk * 32);
+                    const uint64_t bd = make_desc_sw128(sb + kk * 32);
+                    const uint32_t accum = (kt > 0 || kk > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n\t.reg .pred p;\n\t"
+                        "setp.ne.u32 p, %4, 0;\n\t"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(td),
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 smem_u32(&empty[s]))
+                             : "memory");
             }
+            if (abort_sh) break;
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&empty[s]))
+                             smem_u32(&tfull[acc]))
                          : "memory");
         }
-        if (!ok) abort_sh = 1;
-        // the last commit covers every MMA issued before it (also after a timeout,
-        // so that none is in flight when the tensor memory is released)
-        if (any)
+        // after a timeout: one more commit covers every MMA issued, so that none is in
+        // flight when the tensor memory is released
+        if (abort_sh && any) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              smem_u32(&done))
                          : "memory");
-        else
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&done)) : "memory");
-    }
-    __syncwarp();
-    // everyone: wait for the accumulator (or, after a timeout, for the MMAs in flight)
-    if (!mbar_wait(smem_u32(&done), 0u, abort_sh ? TC_DRAIN_NS : g.wait_ns)) {
-        abort_sh = 1;
-        mbar_wait(smem_u32(&done), 0u, TC_DRAIN_NS);   // every arrival on `done` is certain: drain
-    }
-    __syncthreads();
-    if (abort_sh) {
-        if (tid == 0 && g.err) atomicExch(g.err, 1);
-    } else {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int row = m0 + warp * 32 + lane;
-        const bool rv = row < g.M;
-        for (int c0 = 0; c0 < NT; c0 += 32) {
-            uint32_t r[32];
-            const uint32_t ta = taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-                "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                  "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-                  "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-                  "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                : "r"(ta));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (!rv) continue;
+            mbar_wait(smem_u32(&done), 0u, TC_DRAIN_NS);
+        }
+    } else if (warp >= 2) {
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        int i = 0;
+        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
+            const int acc = i & 1, m0 = t / tiles_n * TC_BM, n0 = t % tiles_n * TC_MAXN;
+            const int NT = min(TC_MAXN, g.N - n0);   // a multiple of 16
+            const bool ok = !abort_sh && mbar_wait(smem_u32(&tfull[acc]), (uint32_t)(i / 2) & 1u, g.wait_ns);
+            if (!__all_sync(0xffffffffu, ok)) {   // warp-uniform: the TMEM loads below are warp-collective
+                abort_sh = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int row = m0 + quarter * 32 + lane;
+            const bool rv = row < g.M;
+            for (int c0 = 32 * half; c0 < NT; c0 += 64) {
+                uint32_t r[32];
+                const uint32_t ta = taddr + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * ncols + (uint32_t)c0;
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                    "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                      "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                      "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                      "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                      "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                    : "r"(ta));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (!rv) continue;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (c0 + 4 * q >= NT) break;   // NT is a multiple of 16: groups of 4 are whole
-                const int col = n0 + c0 + 4 * q;
-                float v[4];
+                for (int q = 0; q < 8; ++q) {
+                    if (c0 + 4 * q >= NT) break;   // NT is a multiple of 16: groups of 4 are whole
+                    const int col = n0 + c0 + 4 * q;
+                    float v[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(r[4 * q + e]);
-                if (g.bias) {
-                    const float4 b = *(const float4 *)(g.bias + col);
-                    v[0] += b.x, v[1] += b.y, v[2] += b.z, v[3] += b.w;
-                }
-                if (g.mode == 1) {
-                    if (g.Z) *(float4 *)(g.Z + (size_t)row * g.ldz + col) = make_float4(v[0], v[1], v[2], v[3]);
+                    for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(r[4 * q + e]);
+                    if (g.bias) {
+                        const float4 b = *(const float4 *)(g.bias + col);
+                        v[0] += b.x, v[1] += b.y, v[2] += b.z, v[3] += b.w;
+                    }
+                    if (g.mode == 1) {
+                        if (g.Z) *(float4 *)(g.Z + (size_t)row * g.ldz + col) = make_float4(v[0], v[1], v[2], v[3]);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) v[e] = gelu_f(v[e]);
-                } else if (g.mode == 2) {
-                    const float4 z = *(const float4 *)(g.Z + (size_t)row * g.ldz + col);
-                    v[0] *= gelu_grad(z.x), v[1] *= gelu_grad(z.y), v[2] *= gelu_grad(z.z), v[3] *= gelu_grad(z.w);
-                }
-                if (g.Cf) *(float4 *)(g.Cf + (size_t)row * g.ldcf + col) = make_float4(v[0], v[1], v[2], v[3]);
-                if (g.Cb) {
-                    __nv_bfloat162 p0 = __floats2bfloat162_rn(v[0], v[1]), p1 = __floats2bfloat162_rn(v[2], v[3]);
-                    uint2 u;
-                    u.x = *(uint32_t *)&p0;
-                    u.y = *(uint32_t *)&p1;
-                    *(uint2 *)(g.Cb + (size_t)row * g.ldcb + col) = u;
-                }
-                if (g.Cbt) {
+                        for (int e = 0; e < 4; ++e) v[e] = gelu_f(v[e]);
+                    } else if (g.mode == 2) {
+                        const float4 z = *(const float4 *)(g.Z + (size_t)row * g.ldz + col);
+                        v[0] *= gelu_grad(z.x), v[1] *= gelu_grad(z.y), v[2] *= gelu_grad(z.z), v[3] *= gelu_grad(z.w);
+                    }
+                    if (g.Cf) *(float4 *)(g.Cf + (size_t)row * g.ldcf + col) = make_float4(v[0], v[1], v[2], v[3]);
+                    if (g.Cb) {
+                        __nv_bfloat162 p0 = __floats2bfloat162_rn(v[0], v[1]), p1 = __floats2bfloat162_rn(v[2], v[3]);
+                        uint2 u;
+                        u.x = *(uint32_t *)&p0;
+                        u.y = *(uint32_t *)&p1;
+                        *(uint2 *)(g.Cb + (size_t)row * g.ldcb + col) = u;
+                    }
+                    if (g.Cbt) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) g.Cbt[(size_t)(col + e) * g.ldct + row] = __float2bfloat16(v[e]);
+                        for (int e = 0; e < 4; ++e) g.Cbt[(size_t)(col + e) * g.ldct + row] = __float2bfloat16(v[e]);
+                    }
                 }
             }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[acc])) : "memory");
         }
     }
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
+    if (abort_sh && tid == 0 && g.err) atomicExch_system(g.err, 1);
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(2 * ncols));
+    }
 }
 
 bool aligned(const void *p, uintptr_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
@@ -342,13 +376,79 @@ cudaError_t launch_tc_gemm(const TcGemm &g, cudaStream_t st) {
         e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid((g.M + TC_BM - 1) / TC_BM, (g.N + TC_MAXN - 1) / TC_MAXN);
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const int tiles_n = (g.N + TC_MAXN - 1) / TC_MAXN, tiles = (g.M + TC_BM - 1) / TC_BM * tiles_n;
     TcGemm gk = g;
     gk.wait_ns = wait_limit_ns();
-    tc_gemm_kernel<<<grid, TC_THREADS, smem, st>>>(gk, ma, mb, boxn);
+    tc_gemm_kernel<<<std::min(tiles, sms), TC_THREADS, smem, st>>>(gk, ma, mb, boxn, tiles_n, tiles);
     return cudaGetLastError();
 }
 
+}  // namespace fpk
+
+namespace fpk {
+namespace {
+
+// An error flag of one call in pinned host memory that the kernel reaches through its
+// mapped address: nothing to clear, copy or allocate per call (an int from
+// cudaMallocAsync, cleared, copied back and freed, took 180 us of a 326 us call).  Flags
+// come from a free list that grows to the largest number of calls in flight at once
+// (each call waits for its kernel, so a returned flag is idle), at most kMaxFlags; the
+// list is portable over devices and threads.
+struct ErrorFlag {
+    static constexpr size_t kMaxFlags = 256;
+    volatile int *host = nullptr;
+    int *device = nullptr;
+    bool lost = false;   // lost: a kernel may still write it
+
+    static std::mutex &mu() { static std::mutex m; return m; }
+    static std::vector<int *> &pool() { static std::vector<int *> *v = new std::vector<int *>(); return *v; }
+
+    ErrorFlag() {
+        int *p = nullptr;
+        {
+            std::lock_guard<std::mutex> lk(mu());
+            if (!pool().empty()) {
+                p = pool().back();
+                pool().pop_back();
+            }
+        }
+        if (!p && cudaHostAlloc((void **)&p, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        void *d = nullptr;
+        if (cudaHostGetDevicePointer(&d, p, 0) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFreeHost(p);
+            return;
+        }
+        *p = 0;
+        host = p;
+        device = (int *)d;
+    }
+    ~ErrorFlag() {
+        if (!host || lost) return;
+        int *p = const_cast<int *>(host);
+        {
+            std::lock_guard<std::mutex> lk(mu());
+            if (pool().size() < kMaxFlags) {
+                try {
+                    pool().push_back(p);
+                    p = nullptr;
+                } catch (...) {
+                }
+            }
+        }
+        if (p) cudaFreeHost(p);
+    }
+    ErrorFlag(const ErrorFlag &) = delete;
+    ErrorFlag &operator=(const ErrorFlag &) = delete;
+};
+
+}  // namespace
 }  // namespace fpk
 
 extern "C" fp_status fp_gemm_bf16(int32_t M, int32_t N, int32_t K, const void *A, int32_t lda, const void *Bt,
@@ -366,17 +466,15 @@ extern "C" fp_status fp_gemm_bf16(int32_t M, int32_t N, int32_t K, const void *A
     if (const char *why = fpk::tc_gemm_check(g)) return fpk::api_fail(FP_ERR_ARG, why);
     if (M == 0) return FP_OK;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    int *derr = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&derr, sizeof(int), st);
-    if (e != cudaSuccess) return fpk::api_fail(FP_ERR_OOM, cudaGetErrorString(e));
-    g.err = derr;
-    int herr = 0;
-    e = cudaMemsetAsync(derr, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = fpk::launch_tc_gemm(g, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(derr, st);
+    fpk::ErrorFlag flag;
+    if (!flag.host) return fpk::api_fail(FP_ERR_OOM, "no pinned memory for the error flag");
+    g.err = flag.device;
+    cudaError_t e = fpk::launch_tc_gemm(g, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fpk::api_fail(FP_ERR_CUDA, cudaGetErrorString(e));
-    if (herr) return fpk::api_fail(FP_ERR_TIMEOUT, "tcgen05 GEMM: an mbarrier wait ran out");
+    if (e != cudaSuccess) {
+        flag.lost = true;
+        return fpk::api_fail(FP_ERR_CUDA, cudaGetErrorString(e));
+    }
+    if (*flag.host) return fpk::api_fail(FP_ERR_TIMEOUT, "tcgen05 GEMM: an mbarrier wait ran out");
     return FP_OK;
 }
