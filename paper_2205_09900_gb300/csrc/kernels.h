@@ -59,11 +59,11 @@ cudaError_t launch_moments(const double *tr, const int32_t *group, uint64_t coun
                            int n_groups, double *partials, int nblocks, double *out,
                            cudaStream_t st);
 int moments_blocks(uint64_t count);
-// Bootstrap of F^(k): members lists the pairs of group g at [goff[g], goff[g+1]);
-// xs (n_members doubles) is scratch; out[(g*k_max + k-1)*B + b].
-cudaError_t launch_bootstrap(const double *tr, const uint32_t *members, uint64_t n_members, const uint64_t *goff,
-                             int n_groups, int k_max, int B, uint64_t seed, double *xs, double *out,
-                             cudaStream_t st);
+// Bootstrap of F^(k): tr [2 count], group [count] on the device; scratch of
+// bootstrap_scratch bytes; out[(g*k_max + k-1)*B + b].  Waits for the group sizes.
+size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max);
+cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t count, int n_groups, int k_max, int B,
+                             uint64_t seed, void *scratch, double *out, cudaStream_t st);
 // Brickwork fast path: maps (from the raw gates; raw == nullptr: they are in place), then either the shared-memory sweep (tile_bits == 0)
 // or init + light-cone passes + dot.  `states` holds npairs x 2 x 2^N
 // amplitudes (tiled) or npairs x 2^N (shared-memory path, left boundaries).

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "kernels.h"
 
@@ -76,26 +77,241 @@ __global__ void moments_pass2(const double *__restrict__ partials, int nblocks, 
     out[t] = s + c;
 }
 
-// xs[j] = |Tr|^2 of pair members[j] (pairs listed group by group)
-__global__ void abs2_gather_kernel(const double *__restrict__ tr, const uint32_t *__restrict__ members, uint64_t n,
-                                   double *__restrict__ xs) {
-    for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t i = members[j];
-        xs[j] = tr[2 * i] * tr[2 * i] + tr[2 * i + 1] * tr[2 * i + 1];
+// Members of every group in increasing pair order, on the device: counts per chunk of
+// pairs, offsets, and xs = |Tr|^2 of the members group by group.  A CTA takes one (chunk,
+// group) and places its members by a scan; the group ids stay in L2 (one CTA per group
+// over all 200,000 pairs took 520 us, a counting sort on the host and its copies as much).
+constexpr int GT = 256, GP = 4, kChunk = GT * GP;
+__device__ __forceinline__ uint32_t group_scan(uint32_t v, uint32_t *total, uint32_t (&sh)[GT / 32]) {   // exclusive
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) sh[wid] = x;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+    for (int w = 0; w < GT / 32; ++w) {
+        if (w < wid) before += sh[w];
+        all += sh[w];
+    }
+    *total = all;
+    return before + x - v;
+}
+
+// cnt[g nchunks + c]: members of group g = blockIdx.y in chunk c = blockIdx.x (`per` pairs)
+__global__ void __launch_bounds__(GT) group_count_kernel(const int32_t *__restrict__ group, uint64_t count, uint64_t per,
+                                                         uint32_t *__restrict__ cnt) {
+    __shared__ uint32_t sh[GT / 32];
+    const uint64_t lo = blockIdx.x * per, hi = lo + per < count ? lo + per : count;
+    uint32_t n = 0, all;
+    for (uint64_t i = lo + threadIdx.x; i < hi; i += GT) n += group[i] == (int)blockIdx.y;
+    group_scan(n, &all, sh);
+    if (threadIdx.x == 0) cnt[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = all;
+}
+
+// off[g] = first member of group g, off[n_groups] = all members; xoff: the same over the
+// groups of at most max_n members (the ones that are counted in shared memory); cnt: from
+// counts to the chunk's first position in its group; exp2 cleared
+constexpr int kNoScale = 1 << 20;
+__global__ void __launch_bounds__(1024) group_offsets_kernel(uint32_t *__restrict__ cnt, int nchunks, int n_groups,
+                                                             uint32_t max_n, uint64_t *__restrict__ off,
+                                                             uint64_t *__restrict__ xoff, int *__restrict__ exp2) {
+    const int lane = threadIdx.x & 31;
+    for (int g = threadIdx.x >> 5; g < n_groups; g += 32) {   // a warp per group
+        uint64_t s = 0;
+        for (int c = lane; c - lane < nchunks; c += 32) {
+            const uint32_t v = c < nchunks ? cnt[(size_t)g * nchunks + c] : 0;
+            uint32_t x = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (c < nchunks) cnt[(size_t)g * nchunks + c] = (uint32_t)s + x - v;
+            s += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) off[g + 1] = s, exp2[g] = -kNoScale;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    uint64_t s = 0, x = 0;
+    off[0] = xoff[0] = 0;
+    for (int g = 0; g < n_groups; ++g) {
+        const uint64_t n = off[g + 1];
+        off[g + 1] = s += n;
+        xoff[g + 1] = x += n <= max_n ? n : 0;
     }
 }
 
-// Block (b, g): resample b of group g.  Draw i takes position
+// xs of the members, and the group's scale: exp2[g] = e with every x < 2^e, or kNoScale
+// when a power x^k_max is not finite (such a group takes the FP64 sums below)
+__global__ void __launch_bounds__(GT) group_place_kernel(const double *__restrict__ tr, const int32_t *__restrict__ group,
+                                                         uint64_t count, uint64_t per, const uint64_t *__restrict__ off,
+                                                         const uint32_t *__restrict__ cnt, int k_max,
+                                                         double *__restrict__ xs, int *__restrict__ exp2) {
+    __shared__ uint32_t sh[GT / 32];
+    const uint64_t lo = blockIdx.x * per, hi = lo + per < count ? lo + per : count;
+    uint64_t at = off[blockIdx.y] + cnt[(size_t)blockIdx.y * gridDim.x + blockIdx.x];
+    int e = -kNoScale;
+    for (uint64_t i0 = lo; i0 < hi; i0 += kChunk) {
+        const uint64_t i = i0 + (uint64_t)threadIdx.x * GP;
+        bool in[GP];
+        uint32_t n = 0, all;
+#pragma unroll
+        for (int j = 0; j < GP; ++j) {
+            in[j] = i + j < hi && group[i + j] == (int)blockIdx.y;
+            n += in[j];
+        }
+        uint32_t pos = group_scan(n, &all, sh);
+#pragma unroll
+        for (int j = 0; j < GP; ++j) {
+            if (!in[j]) continue;
+            const double a = tr[2 * (i + j)], b = tr[2 * (i + j) + 1], x = a * a + b * b;
+            xs[at + pos++] = x;
+            double p = x;
+            for (int k = 1; k < k_max; ++k) p *= x;
+            e = max(e, isfinite(p) ? (x > 0 ? ilogb(x) + 1 : -kNoScale) : kNoScale);
+        }
+        at += all;
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0 && e > -kNoScale) atomicMax(&exp2[blockIdx.y], e);
+}
+
+// The powers of every member in fixed point: limbs (low first) of floor(x^k 2^(96 - k e))
+// for group scale e, at xf[((k - 1) n + j) 3], j over the members of the groups of xoff.
+// x^k is the product of doubles that the FP64 sums use.
+__global__ void powers_kernel(const double *__restrict__ xs, const uint64_t *__restrict__ off,
+                              const uint64_t *__restrict__ xoff, int n_groups, int k_max, const int *__restrict__ exp2,
+                              uint32_t *__restrict__ xf) {
+    const uint64_t n = xoff[n_groups], j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    int g = 0, top = n_groups;   // the last g with xoff[g] <= j
+    while (top - g > 1) {
+        const int mid = (g + top) / 2;
+        (xoff[mid] <= j ? g : top) = mid;
+    }
+    const int e = exp2[g];
+    if (e >= kNoScale) return;
+    const double x = xs[off[g] + (j - xoff[g])];
+    double p = 1.0;
+    for (int k = 1; k <= k_max; ++k) {
+        p *= x;
+        uint32_t l0 = 0, l1 = 0, l2 = 0;
+        if (p > 0 && e > -kNoScale) {
+            int pe;
+            const uint64_t m = (uint64_t)(frexp(p, &pe) * 0x1.0p53);   // p = m 2^(pe - 53), pe <= k e
+            const int sh = 96 + pe - 53 - k * e;                       // <= 43
+            if (sh >= 0) {   // m 2^sh over three limbs
+                const uint64_t lo = sh < 64 ? m << sh : 0, hi = sh ? m >> (64 - sh) : 0;
+                l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), l2 = (uint32_t)hi;
+            } else if (sh > -64) {
+                const uint64_t lo = m >> -sh;
+                l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32);
+            }
+        }
+        uint32_t *o = xf + ((uint64_t)(k - 1) * n + j) * 3;
+        o[0] = l0, o[1] = l1, o[2] = l2;
+    }
+}
+
+// RB resamples of one group per CTA.  A resample's draws are counted per member in
+// shared memory (bytes: a count above 255 in N draws of N members has probability
+// below 1/256! for N > 255 and cannot occur for fewer), then F^(k) = sum of count x^k / N
+// is summed exactly in fixed point: one 32 x 32 -> 64 multiply-add per limb where the
+// FP64 pipe, 77 times slower, took a multiplication and an addition per draw and k
+// (the whole call, 300 resamples of 200,000 traces, 9 groups, k <= 4: BOOT_FIGURES).
+// Bound: the Philox rounds.
+constexpr int CT = 512, RB = 4;
+__global__ void __launch_bounds__(CT) bootstrap_count_kernel(const uint32_t *__restrict__ xf,
+                                                             const uint64_t *__restrict__ off,
+                                                             const uint64_t *__restrict__ xoff, int n_groups, int k_max,
+                                                             int B, uint64_t seed, const int *__restrict__ exp2,
+                                                             uint32_t max_n, double *__restrict__ out) {
+    extern __shared__ uint32_t cnt[];   // [words][RB]: word w holds the counts of members 4w .. 4w+3
+    __shared__ uint64_t red[CT / 32][RB][3];
+    const int g = blockIdx.y, b0 = blockIdx.x * RB;
+    const uint64_t N = off[g + 1] - off[g], o = xoff[g], n = xoff[n_groups];
+    if (N == 0 || N > max_n || exp2[g] >= kNoScale) return;   // bootstrap_kernel takes these
+    const uint32_t words = (uint32_t)((N + 3) / 4);
+    for (uint32_t i = threadIdx.x; i < words * RB; i += CT) cnt[i] = 0;
+    __syncthreads();
+    const uint32_t nq = words, Nn = (uint32_t)N;   // draws come in fours
+    for (uint32_t i = threadIdx.x; i < nq * RB; i += CT) {
+        const uint32_t r = i / nq, q = i - r * nq;
+        if (b0 + (int)r >= B) break;
+        const U64x4 x = philox(seed, (uint64_t)(b0 + r), q, (uint64_t)g, 5);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (4 * q + w >= Nn) break;
+            const uint32_t pos = __umulhi((uint32_t)(x.x[w] >> 32), Nn);
+            atomicAdd(&cnt[(pos >> 2) * RB + r], 1u << (8 * (pos & 3)));
+        }
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int k = 0; k < k_max; ++k) {
+        uint64_t s[RB][3];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) s[r][0] = s[r][1] = s[r][2] = 0;
+        const uint32_t *xk = xf + ((uint64_t)k * n + o) * 3;
+        for (uint32_t w = threadIdx.x; w < words; w += CT) {
+            uint32_t c[RB];
+#pragma unroll
+            for (int r = 0; r < RB; ++r) c[r] = cnt[w * RB + r];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const uint32_t j = 4 * w + m;
+                if (j >= Nn) break;
+                const uint32_t l0 = xk[3 * (uint64_t)j], l1 = xk[3 * (uint64_t)j + 1], l2 = xk[3 * (uint64_t)j + 2];
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    const uint32_t cr = (c[r] >> (8 * m)) & 255u;
+                    s[r][0] += (uint64_t)cr * l0;
+                    s[r][1] += (uint64_t)cr * l1;
+                    s[r][2] += (uint64_t)cr * l2;
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                for (int d = 16; d > 0; d >>= 1) s[r][l] += __shfl_down_sync(0xffffffffu, s[r][l], d);
+                if (lane == 0) red[wid][r][l] = s[r][l];
+            }
+        __syncthreads();
+        if (threadIdx.x < RB && b0 + (int)threadIdx.x < B) {
+            uint64_t t[3] = {0, 0, 0};
+            for (int w = 0; w < CT / 32; ++w)
+                for (int l = 0; l < 3; ++l) t[l] += red[w][threadIdx.x][l];
+            // t0 + t1 2^32 + t2 2^64, as a high and a low part that double holds to 2^-106
+            const uint64_t mid = t[1] + (t[0] >> 32);                  // (< 2^63)
+            const uint64_t hi = t[2] + (mid >> 32), lo = (mid << 32) | (t[0] & 0xffffffffu);
+            const double v = ((double)hi * 0x1.0p64 + (double)lo) / (double)N;
+            out[((size_t)g * k_max + k) * B + b0 + threadIdx.x] =
+                exp2[g] > -kNoScale ? ldexp(v, (k + 1) * exp2[g] - 96) : 0.0;
+        }
+        __syncthreads();
+    }
+}
+
+// The groups the counts do not take (empty, too large for shared memory, powers that
+// are not finite), in FP64.  Block (b, g): resample b of group g.  Draw i takes position
 // ((x >> 32) N_g) >> 32 of the group, x = word i % 4 of Philox block
 // {b, i / 4, g, 5} (key {seed, 0}); F^(k) of the resample = mean of a^k over
 // the draws.  Fixed thread-to-draw mapping and tree: deterministic.
 constexpr int BT = 256;
 __global__ void __launch_bounds__(BT) bootstrap_kernel(const double *__restrict__ xs,
                                                        const uint64_t *__restrict__ goff, int k_max, int B,
-                                                       uint64_t seed, double *__restrict__ out) {
+                                                       uint64_t seed, const int *__restrict__ exp2, uint32_t max_n,
+                                                       double *__restrict__ out) {
     __shared__ double sh[FP_MAX_KMAX][BT / 32];
     const int b = blockIdx.x, g = blockIdx.y;
     const uint64_t off = goff[g], N = goff[g + 1] - off;
+    if (N > 0 && N <= max_n && exp2[g] < kNoScale) return;   // bootstrap_count_kernel's
     double s[FP_MAX_KMAX];
 #pragma unroll
     for (int k = 0; k < FP_MAX_KMAX; ++k) s[k] = 0.0;
@@ -135,16 +351,62 @@ __global__ void __launch_bounds__(BT) bootstrap_kernel(const double *__restrict_
 
 }  // namespace
 
-cudaError_t launch_bootstrap(const double *tr, const uint32_t *members, uint64_t n_members, const uint64_t *goff,
-                             int n_groups, int k_max, int B, uint64_t seed, double *xs, double *out,
-                             cudaStream_t st) {
-    if (n_members > 0) {
-        abs2_gather_kernel<<<(unsigned)std::min<uint64_t>((n_members + 255) / 256, 4096), 256, 0, st>>>(
-            tr, members, n_members, xs);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+namespace {
+constexpr uint32_t kMaxCounted = 200 * 1024 / RB;   // members whose counts fit shared memory
+uint64_t counted_members(uint64_t count, int n_groups) {
+    return std::min<uint64_t>(count, (uint64_t)n_groups * kMaxCounted);
+}
+size_t up16(size_t b) { return (b + 15) / 16 * 16; }
+// pairs per chunk: whole passes of a CTA, at most 4096 chunks
+uint64_t chunk_pairs(uint64_t count) { return ((count + 4095) / 4096 + kChunk - 1) / kChunk * kChunk; }
+int chunks(uint64_t count) { return count ? (int)((count + chunk_pairs(count) - 1) / chunk_pairs(count)) : 0; }
+}  // namespace
+
+size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max) {
+    return up16((size_t)count * 8) + up16((size_t)(2 * n_groups + 2) * 8) + up16((size_t)n_groups * 4) +
+           up16((size_t)n_groups * chunks(count) * 4) + (size_t)counted_members(count, n_groups) * k_max * 12;
+}
+
+cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t count, int n_groups, int k_max, int B,
+                             uint64_t seed, void *scratch, double *out, cudaStream_t st) {
+    char *at = (char *)scratch;
+    double *xs = (double *)at;
+    at += up16((size_t)count * 8);
+    uint64_t *off = (uint64_t *)at, *xoff = off + n_groups + 1;
+    at += up16((size_t)(2 * n_groups + 2) * 8);
+    int *exp2 = (int *)at;
+    at += up16((size_t)n_groups * 4);
+    uint32_t *cnt = (uint32_t *)at;
+    const int nc = chunks(count);
+    uint32_t *xf = (uint32_t *)(at + up16((size_t)n_groups * nc * 4));
+    cudaError_t e;
+    const dim3 cg((unsigned)nc, (unsigned)n_groups);
+    if (n_groups > 65535) return cudaErrorInvalidValue;
+    if (nc > 0) {
+        group_count_kernel<<<cg, GT, 0, st>>>(group, count, chunk_pairs(count), cnt);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    bootstrap_kernel<<<dim3((unsigned)B, (unsigned)n_groups), BT, 0, st>>>(xs, goff, k_max, B, seed, out);
+    group_offsets_kernel<<<1, 1024, 0, st>>>(cnt, nc, n_groups, kMaxCounted, off, xoff, exp2);
+    if (nc > 0) group_place_kernel<<<cg, GT, 0, st>>>(tr, group, count, chunk_pairs(count), off, cnt, k_max, xs, exp2);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const uint64_t nx = counted_members(count, n_groups);
+    if (nx > 0) {
+        // the largest counted group's size sets the shared memory (two CTAs per SM up to 25,600 members)
+        uint64_t largest = 0;
+        std::vector<uint64_t> h((size_t)n_groups + 1);
+        if ((e = cudaMemcpyAsync(h.data(), off, h.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+        powers_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(xs, off, xoff, n_groups, k_max, exp2, xf);
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        for (int g = 0; g < n_groups; ++g)
+            if (h[g + 1] - h[g] <= kMaxCounted) largest = std::max(largest, h[g + 1] - h[g]);
+        const size_t smem = (size_t)((largest + 3) / 4) * 4 * RB;
+        if ((e = cudaFuncSetAttribute(bootstrap_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return e;
+        if (largest > 0)
+            bootstrap_count_kernel<<<dim3((unsigned)((B + RB - 1) / RB), (unsigned)n_groups), CT, smem, st>>>(
+                xf, off, xoff, n_groups, k_max, B, seed, exp2, kMaxCounted, out);
+    }
+    bootstrap_kernel<<<dim3((unsigned)B, (unsigned)n_groups), BT, 0, st>>>(xs, off, k_max, B, seed, exp2, kMaxCounted, out);
     return cudaGetLastError();
 }
 

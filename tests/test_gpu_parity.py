@@ -520,6 +520,31 @@ def test_bootstrap_matches_oracle(fp):
     assert np.array_equal(ens.bootstrap(t, grp, N, K, B, seed=23), got, equal_nan=True)
 
 
+# groups around the counters' words (four members), of the largest counted size and above it, empty,
+# all zero, with values over 60 orders of magnitude, and with infinite and NaN traces; resamples that
+# do not fill the last CTA
+@pytest.mark.parametrize("k_max,B", [(1, 1), (3, 6), (8, 5)])
+def test_bootstrap_group_shapes(fp, k_max, B):
+    rng = np.random.default_rng(k_max)
+    sizes = [1, 2, 3, 4, 5, 255, 256, 257, 5000, 0, 51_200, 51_201, 300, 300, 300, 40]
+    grp = np.repeat(np.arange(len(sizes), dtype=np.int32), sizes)
+    rng.shuffle(grp)
+    z = (rng.normal(size=len(grp)) + 1j * rng.normal(size=len(grp))) * np.sqrt(0.5)
+    z[grp == 12] = 0
+    wide = grp == 13
+    z[wide] *= 10.0 ** rng.uniform(-15, 15, wide.sum())
+    z[np.flatnonzero(grp == 14)[7]] = np.inf
+    z[np.flatnonzero(grp == 15)[3]] = np.nan
+    ens = fp.Ensemble(fp.PARALLEL, 8, 2, 1 + len(sizes), seed=1)
+    t = np.ascontiguousarray(np.stack([z.real, z.imag], axis=1).reshape(-1))
+    got = ens.bootstrap(t, grp, len(grp), k_max, B, seed=5)
+    with np.errstate(all="ignore"):
+        ref = O.bootstrap(z, grp, len(sizes), k_max, B, seed=5)
+    ref[14][np.isnan(ref[14])] = np.inf   # |inf + 0i|^2: infinite here, NaN in the oracle's complex product
+    # the oracle adds up to 51,201 non-negative terms one by one: relative rounding below 51,201 x 2^-53
+    assert np.allclose(got, ref, rtol=6e-12, atol=0, equal_nan=True)
+
+
 # ---------------------------------------------------------------------------
 # Local circuits at T = 100 (the deepest T of the local workload): the pairs
 # whose boundaries reach 2^18-2^24 amplitudes and run on 4- and 16-CTA
