@@ -150,6 +150,7 @@ struct fp_ensemble {
     std::map<int, std::unique_ptr<SpiralCache>> spiral_plans;
     DBuf d_spiral_scratch;
     DBuf d_maps, d_states;
+    DBuf d_step_items, d_step_which, d_step_pairs, d_step_meet, d_step_part;   // lock-step sweep
     DBuf d_flag;               // device error flag of kernels with bounded waits (zero when clear)
     std::atomic<int> cancel{0};   // fp_cancel: checked by the Monte Carlo driver between batches
     std::string gpu_name;
@@ -317,6 +318,98 @@ struct KTimer {
     }
 };
 
+// Lock-step sweep (kernels_step.cu): pairs of at least 2^kStepBits amplitudes.  Below it a
+// pair's boundary fits an SM's caches and one CTA per pair is faster (STEPBITS).
+constexpr int kStepBits = 14;
+// amplitudes of one buffer of each side (whole 16-byte words)
+void step_sides(const HostPlan &h, size_t *left, size_t *right) {
+    int b[2] = {0, 0};
+    for (size_t k = 0; k < h.ops.size(); ++k) {
+        int &m = b[(int)k < h.n_left ? 0 : 1];
+        m = std::max(m, (int)h.ops[k].b_out);
+    }
+    *left = std::max<size_t>(16, (size_t)1 << b[0]);
+    *right = std::max<size_t>(16, (size_t)1 << b[1]);
+}
+
+// Work lists of a lock-step batch, uploaded; plans: the uploaded DevPlans by pinfo[i].plan.
+template <typename F>
+fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<PairInfo> &pinfo,
+                      const std::vector<DevPlan> &plans, StepBatch &out) {
+    std::vector<StepPair> sp(nb);
+    size_t n_steps = 0, at = 0, n_items = 0;
+    for (uint64_t i = 0; i < nb; ++i) n_steps = std::max(n_steps, (size_t)std::max(plan(i).n_left, plan(i).n_right));
+    std::vector<uint32_t> count(n_steps + 1, 0), blocks(n_steps, 0);
+    for (uint64_t i = 0; i < nb; ++i)
+        for (int s = 0; s < 2; ++s)
+            for (int k = 0; k < (s ? plan(i).n_right : plan(i).n_left); ++k) ++count[k + 1];
+    for (size_t k = 0; k < n_steps; ++k) count[k + 1] += count[k];   // first item of each step
+    n_items = count[n_steps];
+    std::vector<uint32_t> fill(count.begin(), count.end() - 1);
+    std::vector<StepItem> items(n_items);
+    uint32_t meet = 0;
+    std::vector<uint32_t> meet_which;
+    for (uint64_t r = nb; r-- > 0;) {   // largest boundaries first: the small ones fill the launch's tail
+        const HostPlan &h = plan(r);
+        size_t side[2];
+        step_sides(h, &side[0], &side[1]);
+        for (int s = 0; s < 2; ++s) {
+            const uint64_t buf[2] = {at, at + side[s]};
+            at += 2 * side[s];
+            sp[r].base[s] = buf[0];
+            int cur = 0;
+            for (int k = 0; k < (s ? h.n_right : h.n_left); ++k) {
+                const int local = s ? h.n_left + k : k;
+                const DevOp &op = h.ops[local];
+                StepItem &it = items[fill[k]++];
+                std::memset(&it, 0, sizeof it);
+                const bool flat = op.nk == 0;
+                it.form = op.inplace2 ? STEP_IN_PLACE
+                        : flat && op.nc == 1 && op.nn == 3 ? STEP_1_3
+                        : flat && op.nc == 3 && op.nn == 1 ? STEP_3_1
+                        : flat && op.nc == 0 && op.nn == 4 ? STEP_0_4
+                        : flat && op.nc == 4 && op.nn == 0 ? STEP_4_0 : STEP_ANY;
+                it.units = it.form == STEP_IN_PLACE ? 1u << (op.b_out - 2)
+                         : it.form == STEP_ANY ? 1u << op.b_out : 1u << (op.b_in - op.nc);
+                it.log_units = it.units >= (1u << 16) ? 12 : 10;
+                it.in = buf[cur];
+                if (it.form != STEP_IN_PLACE) cur ^= 1;
+                it.out = buf[cur];
+                it.op = plans[pinfo[r].plan].ops_off + local;
+                it.table = pinfo[r].table_off + local;
+                it.first = blocks[k];
+                blocks[k] += std::max(1u, it.units >> it.log_units);
+            }
+            sp[r].final[s] = buf[cur];
+        }
+        sp[r].first = meet;
+        const uint32_t mb = h.bits_final > kMeetChunk ? 1u << (h.bits_final - kMeetChunk) : 1u;
+        meet_which.insert(meet_which.end(), mb, (uint32_t)r);
+        meet += mb;
+    }
+    out.step_first.assign(n_steps + 1, 0);
+    for (size_t k = 0; k < n_steps; ++k) out.step_first[k + 1] = out.step_first[k] + blocks[k];
+    std::vector<uint32_t> which(out.step_first[n_steps]);
+    for (size_t k = 0; k < n_steps; ++k)
+        for (uint32_t j = count[k]; j < count[k + 1]; ++j) {
+            const uint32_t first = out.step_first[k] + items[j].first;
+            std::fill_n(which.begin() + first, std::max(1u, items[j].units >> items[j].log_units), j);
+        }
+    CK(upload(E->d_step_items, items, E->st));
+    CK(upload(E->d_step_which, which, E->st));
+    CK(upload(E->d_step_pairs, sp, E->st));
+    CK(upload(E->d_step_meet, meet_which, E->st));
+    CK(E->d_step_part.reserve((size_t)meet * 4 * sizeof(double)));
+    CK(cudaStreamSynchronize(E->st));   // the host lists end here
+    out.items = E->d_step_items.as<StepItem>();
+    out.which = E->d_step_which.as<uint32_t>();
+    out.pairs = E->d_step_pairs.as<StepPair>();
+    out.meet_which = E->d_step_meet.as<uint32_t>();
+    out.partials = E->d_step_part.p;
+    out.meet_blocks = meet;
+    return FP_OK;
+}
+
 // Generic path over a subset of pairs: outputs go to slots idx[i] of the
 // device arrays (pairs first + idx[i]).
 fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> &idx_in,
@@ -397,6 +490,7 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
     }
     const uint64_t count = kept.size();
     if (count == 0) return FP_OK;
+    const std::vector<DevPlan> &dev_plans = pools.plans;   // (local circuits: filled above)
     const std::vector<uint64_t> &idx = kept;
     auto hp = [&](uint64_t i) -> const HostPlan & { return local ? local_plans[i] : E->plans[plan_idx[i]]; };
     const bool fp32 = prec != FP_PREC_FP64;
@@ -414,21 +508,33 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
         }
         return std::make_pair(1, E->sms * 2);
     };
+    // local-circuit pairs of 2^14 amplitudes and more go in lock-step (kernels_step.cu), each with
+    // its own boundaries; they are the last ones in the order by size
+    const bool lockstep = local && !sweep_cluster_forced();
+    auto in_steps = [&](uint64_t i) { return lockstep && hp(i).bits_max >= kStepBits; };
     uint64_t done = 0;
     while (done < count) {
         uint64_t nb = 0;
-        size_t raw_b = 0, mer_b = 0, tab_b = 0;
+        size_t raw_b = 0, mer_b = 0, tab_b = 0, step_b = 0;
         int bits_max = 0, max_raw = 0, max_mer = 0, max_ops = 0;
+        const bool steps = in_steps(done);
         while (done + nb < count && nb < 65535) {
             const HostPlan &h = hp(done + nb);
+            if (in_steps(done + nb) != steps) break;
             size_t r = (size_t)2 * h.n_raw * 16 * sizeof(double2);
             size_t m = h.merges.size() * 16 * sizeof(double2);
             size_t t = h.ops.size() * 16 * sizeof(double2);
             int bm = std::max(bits_max, h.bits_max);
             const int slots_full = cluster_of(bm).second;
             size_t ws = (size_t)std::min<uint64_t>(slots_full, nb + 1) * 3 * ((size_t)1 << bm) * sizeof(double2);
-            if (nb > 0 && raw_b + r + mer_b + m + tab_b + t + ws > E->ws_budget) break;
-            raw_b += r; mer_b += m; tab_b += t; bits_max = bm;
+            size_t own = 0;
+            if (steps) {
+                size_t sl, sr;
+                step_sides(h, &sl, &sr);
+                own = 2 * (sl + sr) * celem;
+            }
+            if (nb > 0 && raw_b + r + mer_b + m + tab_b + t + (steps ? step_b + own : ws) > E->ws_budget) break;
+            raw_b += r; mer_b += m; tab_b += t; step_b += own; bits_max = bm;
             max_raw = std::max(max_raw, h.n_raw);
             max_mer = std::max<int>(max_mer, (int)h.merges.size());
             max_ops = std::max<int>(max_ops, (int)h.ops.size());
@@ -459,11 +565,17 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
         const int ctas = slots * cl.first;
         size_t ws_elems = (size_t)1 << bits_max;
         CK(upload(E->d_pairs, pinfo, E->st));
-        CK(upload(E->d_order, order, E->st));
+        StepBatch sb;
+        if (steps) {
+            fp_status bs = build_steps(E, nb, [&](uint64_t i) -> const HostPlan & { return hp(done + i); }, pinfo, dev_plans, sb);
+            if (bs != FP_OK) return bs;
+        } else {
+            CK(upload(E->d_order, order, E->st));
+        }
         CK(E->d_raw.reserve(std::max<size_t>(16, ro * 16 * sizeof(double2))));
         CK(E->d_merged.reserve(std::max<size_t>(16, mo * 16 * sizeof(double2))));
         CK(E->d_tables.reserve(std::max<size_t>(16, to * 16 * sizeof(double2))));
-        CK(E->d_ws.reserve((size_t)slots * 3 * ws_elems * celem));
+        CK(E->d_ws.reserve(steps ? step_b : (size_t)slots * 3 * ws_elems * celem));
         SampleParams sp;
         sp.seed = d.seed;
         sp.n = d.n;
@@ -490,11 +602,18 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
         }
         {
             KTimer t(E, FP_K_SWEEP);
+            if (steps) {
+                CK(launch_steps(sb, E->d_pairs.as<PairInfo>(), (int)nb, E->d_plans.as<DevPlan>(), E->d_ops.as<DevOp>(),
+                                E->d_tables.p, fp32, E->d_ws.p, FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53), tr,
+                                kappa, err, E->st));
+                CK(t.stop(cmacs, (int)sb.step_first.size() + 2));
+            } else {
             CK(launch_sweep_generic(E->d_pairs.as<PairInfo>(), E->d_order.as<int32_t>(), (int)nb, E->d_plans.as<DevPlan>(),
                                     E->d_ops.as<DevOp>(), E->d_tables.p, fp32, E->d_ws.p, ws_elems, ctas,
                                     cl.first, E->d_ticket.as<int>(), FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53), tr,
                                     kappa, err, E->st));
             CK(t.stop(cmacs));
+            }
         }
         CK(cudaEventRecord(E->ev1, E->st));
         CK(cudaEventSynchronize(E->ev1));

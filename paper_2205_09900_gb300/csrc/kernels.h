@@ -3,6 +3,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "brick.h"
 #include "fp_internal.h"
 
@@ -50,6 +52,40 @@ cudaError_t launch_sweep_generic(const PairInfo *pairs, const int32_t *order, in
                                  bool fp32, void *workspace, size_t ws_elems_per_cta, int ctas, int cs,
                                  int *ticket, double err_unit, double *tr, double *kappa, double *err,
                                  cudaStream_t st);
+// Lock-step sweep of local-circuit pairs (kernels_step.cu).  Step k of the batch applies
+// operation k of both sides of every pair: block i of the launch works on item
+// which[step_first[k] + i], on its outputs or groups of outputs ("units")
+// (i - first) << log_units and the 2^log_units - 1 after it.
+enum StepForm : uint8_t { STEP_IN_PLACE, STEP_1_3, STEP_3_1, STEP_0_4, STEP_4_0, STEP_ANY };
+constexpr int kMeetChunk = 14;
+struct StepItem {
+    uint64_t in, out;        // first amplitudes of the operation's buffers in the workspace
+    int64_t table;           // its table
+    int32_t op;              // its DevOp
+    uint32_t first, units;   // first block of the step's launch; units in all
+    uint8_t form, log_units; // StepForm
+    uint16_t pad;
+};
+struct StepPair {
+    uint64_t base[2];        // start amplitude of each side
+    uint64_t final[2];       // final boundary of each side
+    uint32_t first;          // first block of its meet
+    uint32_t pad;
+};
+struct StepBatch {
+    const StepItem *items;                 // device
+    const uint32_t *which;                 // device
+    const StepPair *pairs;                 // device
+    const uint32_t *meet_which;            // device
+    void *partials;                        // device: 4 doubles per meet block
+    std::vector<uint32_t> step_first;      // host: first block of each step, and the end
+    uint32_t meet_blocks;
+};
+cudaError_t launch_steps(const StepBatch &b, const PairInfo *pairs, int npairs, const DevPlan *plans, const DevOp *ops,
+                         const void *tables, bool fp32, void *ws, double err_unit, double *tr, double *kappa, double *err,
+                         cudaStream_t st);
+// Whether FP_SWEEP_CLUSTER fixes the cluster size of the generic sweep.
+bool sweep_cluster_forced();
 // Cluster size for a batch whose largest boundary has `bits` bits, and how many
 // such clusters can be resident (0 if clusters of that size cannot launch).
 int sweep_cluster_size(int bits);

@@ -239,11 +239,14 @@ cudaError_t launch_c(int cs, int ctas, cudaStream_t st, const PairInfo *pairs, c
 // Boundaries up to 2^13 amplitudes (64 KB in FP32) stay with one CTA; up to
 // 2^17 a cluster of 4 CTAs; larger ones a cluster of 16.  The environment
 // variable FP_SWEEP_CLUSTER (1, 4, 8 or 16) overrides the choice.
+static int forced_cluster() {
+    const char *e = getenv("FP_SWEEP_CLUSTER");
+    const int v = e ? atoi(e) : 0;
+    return v == 1 || v == 4 || v == 8 || v == 16 ? v : 0;
+}
+bool sweep_cluster_forced() { return forced_cluster() != 0; }
 int sweep_cluster_size(int bits) {
-    if (const char *e = getenv("FP_SWEEP_CLUSTER")) {
-        const int v = atoi(e);
-        if (v == 1 || v == 4 || v == 8 || v == 16) return v;
-    }
+    if (const int v = forced_cluster()) return v;
     return bits <= 13 ? 1 : (bits <= 17 ? 4 : 16);
 }
 

@@ -520,6 +520,33 @@ def test_bootstrap_matches_oracle(fp):
     assert np.array_equal(ens.bootstrap(t, grp, N, K, B, seed=23), got, equal_nan=True)
 
 
+# the lock-step sweep of large local boundaries (2^14 amplitudes up) against the ticket-queue sweep
+# (FP_SWEEP_CLUSTER set): random and diagonal gates, odd chains, one batch and several (64 MB of
+# workspace), every operation shape these circuits produce
+@pytest.mark.parametrize("n,T,flags,ws,count", [(20, (60, 90, 10), 0, 0, 24), (13, (70, 80, 5), 0, 64 << 20, 40),
+                                                (9, (60, 60, 1), 0, 0, 30), (16, (60, 60, 1), 2, 0, 24),
+                                                (20, (60, 60, 1), 1, 0, 16)])
+def test_local_lockstep_matches_ticket_sweep(fp, n, T, flags, ws, count, monkeypatch):
+    def run(prec):
+        ens = fp.Ensemble(fp.LOCAL, n, 1, 1, *T, seed=n, flags=flags | fp.FLAG_SKIP_INFEASIBLE, workspace_bytes=ws)
+        out = ens.trace_batch(100, count, prec, with_err=True)
+        ens.close()
+        return out
+    t64, k64, g64, e64 = run(fp.PREC_FP64)
+    t32, k32, g32, e32 = run(fp.PREC_FP32_RAW)
+    monkeypatch.setenv("FP_SWEEP_CLUSTER", "16")
+    r64, rk, rg, re = run(fp.PREC_FP64)
+    assert np.array_equal(g64, rg) and np.array_equal(g32, rg)
+    ok = rg >= 0
+    assert ok.sum() >= count - 4
+    assert rel_err(t64[ok], r64[ok]).max() <= 1e-11
+    assert np.allclose(e64[ok], re[ok], rtol=1e-9)
+    well = ok & (rk < 1e6)
+    assert np.allclose(k64[well], rk[well], rtol=1e-8)
+    assert np.all(np.abs(t32[ok] - t64[ok]) <= e32[ok])
+    assert np.allclose(e32[ok], e64[ok] * 2.0 ** 29, rtol=1e-3)
+
+
 # groups around the counters' words (four members), of the largest counted size and above it, empty,
 # all zero, with values over 60 orders of magnitude, and with infinite and NaN traces; resamples that
 # do not fill the last CTA
