@@ -253,30 +253,46 @@ struct PlanPools {
     std::vector<DevRecipe> recipes;
     std::vector<MergeItem> items;
     std::vector<MergeRef> refs;
-    void add(const HostPlan &h) {
-        DevPlan p;
-        std::memset(&p, 0, sizeof p);
-        p.n_left = h.n_left;
-        p.n_right = h.n_right;
-        p.ops_off = (int)ops.size();
-        p.rec_off = (int)recipes.size();
-        p.merge_off = (int)items.size();
-        p.n_merged = (int)h.merges.size();
-        p.ref_off = (int)refs.size();
-        p.n_raw = h.n_raw;
-        p.raw_kind = h.raw_kind;
-        p.bits_max = h.bits_max;
-        p.bits_final = h.bits_final;
-        p.left_final_buf = h.left_final_buf;
-        for (int k = 0; k < FP_MAX_STATE_BITS; ++k) p.dot_perm[k] = h.dot_perm[k];
-        p.prefactor = h.prefactor;
-        p.cost = h.cost;
-        p.sqrt_ops = std::sqrt((double)std::max(1, std::max(h.n_left, h.n_right)));
-        ops.insert(ops.end(), h.ops.begin(), h.ops.end());
-        recipes.insert(recipes.end(), h.recipes.begin(), h.recipes.end());
-        items.insert(items.end(), h.merges.begin(), h.merges.end());
-        refs.insert(refs.end(), h.refs.begin(), h.refs.end());
-        plans.push_back(p);
+    // plan(i), i in [0, count): sizes first, then the copies on the host cores
+    template <typename F>
+    void fill(size_t count, F plan) {
+        plans.resize(count);
+        size_t no = 0, ni = 0, nr = 0;
+        for (size_t i = 0; i < count; ++i) {
+            const HostPlan &h = plan(i);
+            DevPlan &p = plans[i];
+            std::memset(&p, 0, sizeof p);
+            p.ops_off = p.rec_off = (int)no;
+            p.merge_off = (int)ni;
+            p.ref_off = (int)nr;
+            no += h.ops.size();
+            ni += h.merges.size();
+            nr += h.refs.size();
+        }
+        ops.resize(no);
+        recipes.resize(no);
+        items.resize(ni);
+        refs.resize(nr);
+        parallel_for(count, [&](uint64_t i) {
+            const HostPlan &h = plan(i);
+            DevPlan &p = plans[i];
+            p.n_left = h.n_left;
+            p.n_right = h.n_right;
+            p.n_merged = (int)h.merges.size();
+            p.n_raw = h.n_raw;
+            p.raw_kind = h.raw_kind;
+            p.bits_max = h.bits_max;
+            p.bits_final = h.bits_final;
+            p.left_final_buf = h.left_final_buf;
+            for (int k = 0; k < FP_MAX_STATE_BITS && k < (int)h.dot_perm.size(); ++k) p.dot_perm[k] = h.dot_perm[k];
+            p.prefactor = h.prefactor;
+            p.cost = h.cost;
+            p.sqrt_ops = std::sqrt((double)std::max(1, std::max(h.n_left, h.n_right)));
+            std::copy(h.ops.begin(), h.ops.end(), ops.begin() + p.ops_off);
+            std::copy(h.recipes.begin(), h.recipes.end(), recipes.begin() + p.rec_off);
+            std::copy(h.merges.begin(), h.merges.end(), items.begin() + p.merge_off);
+            std::copy(h.refs.begin(), h.refs.end(), refs.begin() + p.ref_off);
+        });
     }
 };
 
@@ -445,7 +461,7 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
             kept.push_back(slot);
         }
         if (E->dev_plans_dirty) {
-            for (const auto &h : E->plans) pools.add(h);
+            pools.fill(E->plans.size(), [&](size_t i) -> const HostPlan & { return E->plans[i]; });
             fp_status s = upload_pools(E, pools);
             if (s != FP_OK) return s;
             E->dev_plans_dirty = false;
@@ -478,10 +494,8 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
             local_plans.push_back(std::move(all[i]));
             kept.push_back(idx_in[i]);
         }
-        for (uint64_t i = 0; i < local_plans.size(); ++i) {
-            pools.add(local_plans[i]);
-            plan_idx.push_back((int)i);
-        }
+        for (uint64_t i = 0; i < local_plans.size(); ++i) plan_idx.push_back((int)i);
+        pools.fill(local_plans.size(), [&](size_t i) -> const HostPlan & { return local_plans[i]; });
         if (!local_plans.empty()) {
             fp_status s = upload_pools(E, pools);
             if (s != FP_OK) return s;

@@ -87,14 +87,14 @@ struct DevOp {
     uint8_t new_pos[4];    // ascending positions in the output layout
 };
 
-// How to fill one op's table (16 entries, index e = cons | keep<<nc | new<<(nc+nk)).
+// How to fill one op's table (16 entries, index e = cons | keep<<nc | new<<(nc+nk)):
+// entry e is the sum of up to 4 slots of the merged gate, src[e][s] = slot, plus 64 for
+// a slot that enters with a minus sign (a fused CZ), -1 for none; merged = -1: the
+// constant src[e][0] (sums of CZ signs are small integers).
 struct DevRecipe {
     int32_t merged;        // merged gate id, or -1 for constants
     int32_t nent;          // 2^(nc+nk+nn)
-    int8_t src[16][4];     // merged-gate slots summed into entry e (-1: unused)
-    int8_t sgn[16][4];     // +1 / -1 weight of each summed slot (a fused CZ sign)
-    double cre[16];        // constant entries (merged == -1)
-    double cim[16];
+    int8_t src[16][4];
 };
 
 // One 4x4 map of the spiral sweep (planner.cpp: make_spiral_plan).

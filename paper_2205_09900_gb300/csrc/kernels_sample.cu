@@ -215,12 +215,14 @@ __global__ void table_kernel(const PairInfo *__restrict__ pairs, const DevPlan *
         if (e < r.nent) {
             if (M) {
                 for (int s = 0; s < 4; ++s) {
-                    int k = r.src[e][s];
-                    if (k >= 0) { re += r.sgn[e][s] * M[k].x; im += r.sgn[e][s] * M[k].y; }
+                    const int k = r.src[e][s];
+                    if (k < 0) continue;
+                    const double2 m = M[k & 15];
+                    re += k & 64 ? -m.x : m.x;
+                    im += k & 64 ? -m.y : m.y;
                 }
             } else {
-                re = r.cre[e];
-                im = r.cim[e];
+                re = r.src[e][0];
             }
         }
         out[e] = to_c<C>(re, im);

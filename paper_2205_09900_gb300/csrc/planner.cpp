@@ -23,6 +23,7 @@
 #include "planner.h"
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -64,17 +65,40 @@ std::vector<GateSlot> layout_hea_pauli(int n, int L, bool cz) {
 std::vector<GateSlot> layout_local(int n, const std::vector<int> &bonds) {
     (void)n;
     std::vector<GateSlot> g;
+    g.reserve(bonds.size());
     for (size_t i = 0; i < bonds.size(); ++i) g.push_back({0, bonds[i], (int)i});
     return g;
 }
 
 namespace {
 
+// Gates multiplied into one operator, in application order (nearly always one or two:
+// no allocation for them).
+struct Chain {
+    static constexpr int kSmall = 4;
+    MergeRef small[kSmall];
+    std::vector<MergeRef> big;   // all of them, once they are more than kSmall
+    int n = 0;
+    void push_back(const MergeRef &r) {
+        if (n < kSmall) {
+            small[n++] = r;
+            return;
+        }
+        if (n == kSmall) big.assign(small, small + kSmall);
+        big.push_back(r);
+        ++n;
+    }
+    const MergeRef *begin() const { return n > kSmall ? big.data() : small; }
+    const MergeRef *end() const { return begin() + n; }
+    size_t size() const { return (size_t)n; }
+    const MergeRef &operator[](size_t i) const { return begin()[i]; }
+};
+
 struct SeqEl {
     int kind;                       // 0 gate2 (data), 1 gate1 (data), 2 constant diagonal
     int q;
     bool invol = false;             // a lone constant involution (GateSlot kind 3)
-    std::vector<MergeRef> chain;    // application order
+    Chain chain;                    // application order
     double dre[4], dim[4];          // kind 2 entries
 };
 
@@ -140,8 +164,8 @@ void merge_sequence(std::vector<SeqEl> &seq) {
             } else {
                 // application order: seq[i]'s chain first, then m's
                 m.invol = false;
-                std::vector<MergeRef> c = std::move(seq[i].chain);
-                c.insert(c.end(), m.chain.begin(), m.chain.end());
+                Chain c = std::move(seq[i].chain);
+                for (const MergeRef &r : m.chain) c.push_back(r);
                 m.chain = std::move(c);
             }
             unlink(i);
@@ -488,13 +512,16 @@ HostPlan make_plan(int n, const std::vector<GateSlot> &U, const std::vector<Gate
         } else {
             e.chain.push_back({which, g.raw, dagger, e.kind == 1 ? 2 : dim});
         }
-        seq.push_back(e);
+        seq.push_back(std::move(e));
     };
+    seq.reserve(U.size() + V.size());
     for (const auto &g : V) push(g, 1, 0);
     for (auto it = U.rbegin(); it != U.rend(); ++it) push(*it, 0, 1);
 
     // 2. merges
     merge_sequence(seq);
+    P.merges.reserve(seq.size());
+    P.refs.reserve(U.size() + V.size());
     for (auto &e : seq) {
         if (e.kind == 2) continue;
         MergeItem mi;
@@ -506,19 +533,20 @@ HostPlan make_plan(int n, const std::vector<GateSlot> &U, const std::vector<Gate
 
     // 3. segments and factors
     std::vector<int> s(n, 0), base(n + 1, 0);
-    std::vector<std::vector<int>> posq(seq.size());
+    std::vector<std::array<int, 2>> posq(seq.size());
     for (size_t t = 0; t < seq.size(); ++t) {
         const SeqEl &e = seq[t];
         int nq = e.kind == 1 ? 1 : 2;
         for (int i = 0; i < nq; ++i) {
             int q = e.q + i;
-            if (e.kind == 2) posq[t].push_back(s[q] - 1);
-            else posq[t].push_back(s[q]++);
+            if (e.kind == 2) posq[t][i] = s[q] - 1;
+            else posq[t][i] = s[q]++;
         }
     }
     for (int q = 0; q < n; ++q) base[q + 1] = base[q] + std::max(s[q], 1);
     const int nvars = base[n];
     std::vector<Factor> fs;
+    fs.reserve(2 * seq.size());   // (a fused pair appends one more)
     int merged_id = 0;
     for (size_t t = 0; t < seq.size(); ++t) {
         const SeqEl &e = seq[t];
@@ -575,13 +603,14 @@ HostPlan make_plan(int n, const std::vector<GateSlot> &U, const std::vector<Gate
     // processing orders
     std::vector<int> order[2];
     for (int side = 0; side < 2; ++side) {
-        std::vector<std::pair<std::pair<int, int>, int>> key;
+        std::vector<std::pair<int, int>> key;   // (distance from the chain end, factor)
+        key.reserve(fs.size());
         for (size_t i = 0; i < fs.size(); ++i) {
             if (fs[i].side != side) continue;
-            int sk = side == 0 ? fs[i].site : (n - 1 - fs[i].site);
-            key.push_back({{sk, (int)i}, (int)i});
+            key.push_back({side == 0 ? fs[i].site : (n - 1 - fs[i].site), (int)i});
         }
         std::sort(key.begin(), key.end());
+        order[side].reserve(key.size());
         for (auto &k : key) order[side].push_back(k.second);
     }
 
@@ -589,7 +618,9 @@ HostPlan make_plan(int n, const std::vector<GateSlot> &U, const std::vector<Gate
     // segment in the processing order becomes one factor over their <= 3 segments.
     // The CZ otherwise opens the neighbour's segment while the shared segment is
     // still waiting for the 1-qubit op that closes it, one boundary bit more.
-    for (int side = 0; side < 2; ++side) {
+    bool one_qubit = false;
+    for (const Factor &f : fs) one_qubit = one_qubit || f.kind == 1;
+    for (int side = 0; side < 2 && one_qubit; ++side) {
         std::vector<int> fused;
         const std::vector<int> &ord = order[side];
         for (size_t p = 0; p < ord.size(); ++p) {
@@ -617,111 +648,112 @@ HostPlan make_plan(int n, const std::vector<GateSlot> &U, const std::vector<Gate
         order[side] = fused;
     }
 
-    // 4. sweep programs
-    std::vector<int> final_layout[2];
+    // 4. sweep programs.  `at[v]`: bit position of variable v in the boundary (-1: not
+    // in it); `layout`: the variable at each position
+    std::vector<int> final_layout[2], at(nvars), last(nvars);
+    P.ops.reserve(order[0].size() + order[1].size());
+    P.recipes.reserve(order[0].size() + order[1].size());
     int bits_max = 0;
     for (int side = 0; side < 2; ++side) {
-        std::vector<int> last(nvars, -1);
+        std::fill(last.begin(), last.end(), -1);
+        std::fill(at.begin(), at.end(), -1);
         for (size_t p = 0; p < order[side].size(); ++p) {
             const Factor &f = fs[order[side][p]];
             for (int k = 0; k < f.nslots; ++k) last[f.slot_var[k]] = (int)p;
         }
         std::vector<int> layout;   // var at each bit position
+        layout.reserve(FP_MAX_STATE_BITS + 4);
         for (size_t p = 0; p < order[side].size(); ++p) {
             const Factor &f = fs[order[side][p]];
-            int dv[4], nd = 0;
+            // the factor's variables: summed here (`cons`, by position), kept, new; variables
+            // that occur in no other factor are summed inside the table (`sumv`)
+            int cons[4], keep[4], nw[4], sumv[4], npos[4], nc = 0, nk = 0, nn = 0, nsum = 0, seen[4], nd = 0;
             for (int k = 0; k < f.nslots; ++k) {
-                int v = f.slot_var[k];
+                const int v = f.slot_var[k];
                 bool dup = false;
-                for (int z = 0; z < nd; ++z) dup |= dv[z] == v;
-                if (!dup) dv[nd++] = v;
+                for (int z = 0; z < nd; ++z) dup |= seen[z] == v;
+                if (dup) continue;
+                seen[nd++] = v;
+                const bool is_last = last[v] == (int)p && side_mask[v] != 3;
+                if (at[v] >= 0) (is_last ? cons[nc++] : keep[nk++]) = v;
+                else (is_last ? sumv[nsum++] : nw[nn++]) = v;
             }
-            std::vector<int> cons, keep, nw, sumv;
-            for (int z = 0; z < nd; ++z) {
-                int v = dv[z];
-                bool present = std::find(layout.begin(), layout.end(), v) != layout.end();
-                bool is_last = last[v] == (int)p && side_mask[v] != 3;
-                if (present) (is_last ? cons : keep).push_back(v);
-                else (is_last ? sumv : nw).push_back(v);
-            }
-            std::vector<int> cpos;
-            for (int v : cons) cpos.push_back((int)(std::find(layout.begin(), layout.end(), v) - layout.begin()));
-            // sort consumed by position
-            std::vector<int> ci(cons.size());
-            for (size_t z = 0; z < ci.size(); ++z) ci[z] = (int)z;
-            std::sort(ci.begin(), ci.end(), [&](int a, int b) { return cpos[a] < cpos[b]; });
-            std::vector<int> cons_s, cpos_s;
-            for (int z : ci) { cons_s.push_back(cons[z]); cpos_s.push_back(cpos[z]); }
-            std::vector<int> out;
-            std::vector<int> npos;
-            if (!cons_s.empty() && nw.size() == cons_s.size()) {
-                out = layout;
-                for (size_t z = 0; z < nw.size(); ++z) { out[cpos_s[z]] = nw[z]; npos.push_back(cpos_s[z]); }
-            } else {
-                for (int v : layout)
-                    if (std::find(cons_s.begin(), cons_s.end(), v) == cons_s.end()) out.push_back(v);
-                for (int v : nw) { npos.push_back((int)out.size()); out.push_back(v); }
-            }
-            if ((int)std::max(layout.size(), out.size()) > max_bits) {
-                P.infeasible = true;
-                P.error = "boundary of " + std::to_string(std::max(layout.size(), out.size())) +
-                          " bits exceeds the limit of " + std::to_string(max_bits);
-                return P;
-            }
-            bits_max = std::max<int>(bits_max, (int)std::max(layout.size(), out.size()));
+            for (int z = 1; z < nc; ++z)   // ascending positions
+                for (int y = z; y > 0 && at[cons[y - 1]] > at[cons[y]]; --y) std::swap(cons[y - 1], cons[y]);
             DevOp op;
             std::memset(&op, 0, sizeof op);
-            op.nc = (uint8_t)cons_s.size();
-            op.nk = (uint8_t)keep.size();
-            op.nn = (uint8_t)nw.size();
+            op.nc = (uint8_t)nc;
+            op.nk = (uint8_t)nk;
+            op.nn = (uint8_t)nn;
             op.b_in = (uint8_t)layout.size();
-            op.b_out = (uint8_t)out.size();
-            for (size_t z = 0; z < cons_s.size(); ++z) op.cons_pos[z] = (uint8_t)cpos_s[z];
-            for (size_t z = 0; z < keep.size(); ++z)
-                op.keep_pos[z] = (uint8_t)(std::find(out.begin(), out.end(), keep[z]) - out.begin());
-            for (size_t z = 0; z < nw.size(); ++z) op.new_pos[z] = (uint8_t)npos[z];
+            const size_t out_bits = layout.size() - nc + nn, wide = std::max(layout.size(), out_bits);
+            if ((int)wide > max_bits) {
+                P.infeasible = true;
+                P.error = "boundary of " + std::to_string(wide) + " bits exceeds the limit of " + std::to_string(max_bits);
+                return P;
+            }
+            bits_max = std::max<int>(bits_max, (int)wide);
+            for (int z = 0; z < nc; ++z) op.cons_pos[z] = (uint8_t)at[cons[z]];
+            if (nc > 0 && nn == nc) {   // the new variables take the summed ones' places
+                for (int z = 0; z < nc; ++z) {
+                    npos[z] = at[cons[z]];
+                    layout[npos[z]] = nw[z];
+                    at[nw[z]] = npos[z];
+                    at[cons[z]] = -1;
+                }
+            } else {                    // the rest closes up, the new ones come on top
+                for (int z = 0; z < nc; ++z) at[cons[z]] = -1;
+                if (nc) {
+                    size_t w = 0;
+                    for (int v : layout)
+                        if (at[v] >= 0) {
+                            at[v] = (int)w;
+                            layout[w++] = v;
+                        }
+                    layout.resize(w);
+                }
+                for (int z = 0; z < nn; ++z) {
+                    npos[z] = at[nw[z]] = (int)layout.size();
+                    layout.push_back(nw[z]);
+                }
+            }
+            op.b_out = (uint8_t)layout.size();
+            for (int z = 0; z < nk; ++z) op.keep_pos[z] = (uint8_t)at[keep[z]];
+            for (int z = 0; z < nn; ++z) op.new_pos[z] = (uint8_t)npos[z];
             op.inplace2 = (op.nc == 2 && op.nn == 2 && op.nk == 0 && op.b_in == op.b_out &&
                            op.new_pos[0] == op.cons_pos[0] && op.new_pos[1] == op.cons_pos[1]);
-            // recipe
+            // recipe: slot k of the factor reads bit from[k] of (table index | summed bits << 4)
             DevRecipe r;
-            std::memset(&r, 0, sizeof r);
             r.merged = f.merged;
-            int nbits = op.nc + op.nk + op.nn;
+            const int nbits = nc + nk + nn;
             r.nent = 1 << nbits;
-            for (int e = 0; e < 16; ++e)
-                for (int z = 0; z < 4; ++z) { r.src[e][z] = -1; r.sgn[e][z] = 1; }
-            std::vector<int> ivars;   // var of each table-index bit
-            for (int v : cons_s) ivars.push_back(v);
-            for (int v : keep) ivars.push_back(v);
-            for (int v : nw) ivars.push_back(v);
-            int nsum = (int)sumv.size();
+            std::memset(r.src, -1, sizeof r.src);
+            int from[4];
+            for (int k = 0; k < f.nslots; ++k) {
+                const int v = f.slot_var[k];
+                for (int z = 0; z < nc; ++z) if (cons[z] == v) from[k] = z;
+                for (int z = 0; z < nk; ++z) if (keep[z] == v) from[k] = nc + z;
+                for (int z = 0; z < nn; ++z) if (nw[z] == v) from[k] = nc + nk + z;
+                for (int z = 0; z < nsum; ++z) if (sumv[z] == v) from[k] = 4 + z;
+            }
             for (int e = 0; e < r.nent; ++e) {
                 int ns = 0;
-                double cre = 0, cim = 0;
+                double constant = 0;
                 for (int sv = 0; sv < (1 << nsum); ++sv) {
+                    const int word = e | (sv << 4);
                     int val[4];
-                    for (int k = 0; k < f.nslots; ++k) {
-                        int v = f.slot_var[k], x = -1;
-                        for (int z = 0; z < nbits; ++z) if (ivars[z] == v) x = (e >> z) & 1;
-                        for (int z = 0; z < nsum; ++z) if (sumv[z] == v) x = (sv >> z) & 1;
-                        val[k] = x;
-                    }
-                    int ent = slot_entry(f, val);
-                    if (f.kind == 2) { cre += f.dre[ent]; cim += f.dim[ent]; }
-                    else if (f.kind == 3) {   // 2x2 slot times the diagonal's sign
-                        r.sgn[e][ns] = (int8_t)f.dre[val[2] * 2 + val[3]];
-                        r.src[e][ns++] = (int8_t)ent;
-                    } else {
-                        r.src[e][ns++] = (int8_t)ent;   // 4x4 slots 0..15, 2x2 slots 0..3
-                    }
+                    for (int k = 0; k < f.nslots; ++k) val[k] = (word >> from[k]) & 1;
+                    const int ent = slot_entry(f, val);
+                    if (f.kind == 2) constant += f.dre[ent];
+                    else if (f.kind == 3)   // 2x2 slot times the diagonal's sign
+                        r.src[e][ns++] = (int8_t)(ent + (f.dre[val[2] * 2 + val[3]] < 0 ? 64 : 0));
+                    else r.src[e][ns++] = (int8_t)ent;   // 4x4 slots 0..15, 2x2 slots 0..3
                 }
-                r.cre[e] = cre;
-                r.cim[e] = cim;
+                if (f.kind == 2) r.src[e][0] = (int8_t)constant;
             }
             P.ops.push_back(op);
             P.recipes.push_back(r);
             P.cost += (double)(1u << op.b_out) * (double)(1u << op.nc);
-            layout = out;
         }
         final_layout[side] = layout;
         (side == 0 ? P.n_left : P.n_right) = (int)order[side].size();
