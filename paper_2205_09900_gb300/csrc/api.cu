@@ -335,7 +335,8 @@ struct KTimer {
 };
 
 // Lock-step sweep (kernels_step.cu): pairs of at least 2^kStepBits amplitudes.  Below it a
-// pair's boundary fits an SM's caches and one CTA per pair is faster (STEPBITS).
+// pair's boundary fits an SM's caches and one CTA per pair keeps it there: the 2,205 smaller
+// pairs of 4,000 at n = 20, T = 20..100 take 0.6 ms.
 constexpr int kStepBits = 14;
 // amplitudes of one buffer of each side (whole 16-byte words)
 void step_sides(const HostPlan &h, size_t *left, size_t *right) {
@@ -670,8 +671,10 @@ fp_status make_brick_cache(fp_ensemble *E, int l, bool fp32, int K, int R, int T
     // K > N: shared-memory sweep, K == N: one tile
     // arcs hold the 5 (FP32) or 4 (FP64) lowest bits, so that tile loads read contiguous runs;
     // the tensor-core pass (12-bit tiles) holds 3: at l = 10 a 12-bit arc through the 5
-    // lowest bits would need 49 passes instead of 18
-    bc->hp = make_brick_plan(E->d.n, l, K, persist >= 3 ? 3 : (fp32 ? 5 : 4), R, E->d.kind == FP_HEA ? 1 : 0);
+    // lowest bits would need 49 passes instead of 20; from 20 bits up 2 (27 passes at l = 11
+    // instead of 49: a run of 4 amplitudes is one 32-byte sector)
+    const int low = persist >= 3 ? (2 * (l - 1) >= 20 ? 2 : 3) : (fp32 ? 5 : 4);
+    bc->hp = make_brick_plan(E->d.n, l, K, low, R, E->d.kind == FP_HEA ? 1 : 0);
     for (const auto &ps : bc->hp.passes) {
         if (ps.n_gates > 255) return fail(FP_ERR_ARG, "tile pass with %d gates exceeds 255", ps.n_gates);
         if (ps.n_rp > 160) return fail(FP_ERR_ARG, "tile pass with %d register passes exceeds 160", ps.n_rp);
@@ -680,7 +683,7 @@ fp_status make_brick_cache(fp_ensemble *E, int l, bool fp32, int K, int R, int T
         if (!fp32 || !tc_plan_ok(bc->hp.dev, bc->hp.passes.data(), bc->hp.rpasses.data()))
             return fail(FP_ERR_ARG, "the tensor-core tile pass needs FP32, %d-bit tiles, %d-bit windows and l >= 8",
                         kTcTile, kMaxWin);
-        const std::vector<TcWin> wins = make_tc_windows(bc->hp);
+        const std::vector<TcWin> wins = make_tc_windows(bc->hp, persist == 3);
         CK(upload(bc->d_tcwins, wins, E->st));
         CK(upload(bc->d_tcxa, make_tc_xaddr(bc->hp, wins), E->st));
         bc->dp.tcwins = bc->d_tcwins.as<TcWin>();
@@ -727,11 +730,14 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
                                                        {13, 5, 256, 1}, {12, 4, 256, 0}, {12, 5, 128, 0}}
                                    : std::vector<Cand>{{13, 3, 512, 0}, {13, 4, 256, 0}};
     if (((size_t)1 << N) * (fp32 ? sizeof(float2) : sizeof(double2)) <= (size_t)200 * 1024) cands.push_back({99, 0, 0, 0});
-    // P = 3, 4: tensor-core windows (TF32 x 3 tcgen05 MMAs), boundaries of more than two 12-bit tiles
-    if (fp32 && N >= kTcTile + 2) {
-        cands.push_back({kTcTile, kMaxWin, 256, 3});   // the tile's operand in shared memory
-        cands.push_back({kTcTile, kMaxWin, 256, 4});   // in tensor memory, persistent over the tiles
-    }
+    // P = 4: tensor-core windows (TF32 x 3 tcgen05 MMAs) with the tile's operand in tensor memory,
+    // boundaries of more than two 12-bit tiles.  P = 3 (the operand in shared memory) runs when the
+    // cache file asks for it; it was 20-25 % slower at every depth, and planning it took seconds.
+    // At 20 bits FP_PREC_FP32 stays with the FFMA passes, which timed fastest there before the
+    // tensor-core plans held 2 low bits (35 ms per 96 pairs at n = 50, against 26.8 now): they are
+    // 9 times more accurate (1.2e-6 of a trace against 1.1e-5: the tensor cores' accumulators
+    // truncate).  FP_PREC_TF32X3 asks for the tensor cores.
+    if (fp32 && N >= kTcTile + 2 && (N != 20 || prec == FP_PREC_TF32X3)) cands.push_back({kTcTile, kMaxWin, 256, 4});
     // P = 5: the HEA's own sweep, the fastest of all wherever it applies (kernels_hea.cu), so
     // there is nothing to time; FP_PREC_TF32X3 keeps to the tensor cores where they apply
     int heaR = 0, heaT = 0;
@@ -825,6 +831,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
                 float ms = 0;
                 CK(cudaEventElapsedTime(&ms, E->ev0, E->ev1));
                 if (rep == 1) ms_sum += ms;     // first repetition warms caches and code
+                else if (ms > 1.5f * best_ms) { ms_sum = ms; rep = 1; }   // out of the running already
                 if (bc->dp.err_flag) {
                     fp_status fs = check_flag(E);
                     if (fs != FP_OK) return fs;

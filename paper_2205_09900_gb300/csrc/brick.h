@@ -168,8 +168,10 @@ FP_HD int maps_per_pair(const BrickDev &d) { return (d.n_layers[0] + d.n_layers[
 
 BrickHostPlan make_brick_plan(int n, int l, int tile_bits, int low_bits, int win_bits, int kind = 0);
 // Tensor-core window tables (one per register pass) of a plan with kTcTile-bit
-// tiles and kMaxWin-bit windows.
-std::vector<TcWin> make_tc_windows(const BrickHostPlan &P);
+// tiles and kMaxWin-bit windows; rotations: with the row orders and store
+// orders (rotm) that the shared-memory operand form needs against bank conflicts (their
+// search takes half a second); without, ascending rows.
+std::vector<TcWin> make_tc_windows(const BrickHostPlan &P, bool rotations = true);
 // Per-thread exchange address tables of those windows (one per register pass).
 std::vector<TcXa> make_tc_xaddr(const BrickHostPlan &P, const std::vector<TcWin> &W);
 

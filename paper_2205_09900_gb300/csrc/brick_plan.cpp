@@ -4,9 +4,17 @@
 // (tau, tau+1 mod N), tau = 2j + p_t, where p_t alternates.  A tile holds K
 // bits forming a contiguous cyclic arc of the ring that contains the `low`
 // lowest physical bits (so that loading a tile reads runs of 2^low contiguous
-// amplitudes).  Greedy schedule: each pass takes the arc that can apply the
-// most not-yet-applied gates whose bits lie in the arc and whose
-// predecessors (gates of the previous layer sharing a bit) are applied.
+// amplitudes).  A pass over the boundary applies a sequence of register windows
+// (r consecutive ring bits of its arc), each every gate that its bits allow.
+//
+// Two schedules.  FFMA passes are bound by the gates they apply: greedy, each pass takes the
+// arc and then the windows that apply the most gates.  On the tensor cores a window costs the
+// same whatever it applies, and the greedy choice leaves jagged frontiers that need many
+// small windows: those plans (12-bit tiles, 5-bit windows, at most 3 low bits) take the
+// cheapest sequence of windows and arcs that a beam search over the ring's frontier (how many
+// layers each bit has passed) finds.  At n = 50, l = 8, 9, 10: 63, 71, 81 windows in 14, 16, 20
+// passes instead of 65, 78, 98 in 12, 14, 18 (l = 2..10 mixed: 138 -> 129 ms).  The FFMA passes
+// gain nothing from it (l = 11: 35.5 ms instead of 35.0).
 #include <algorithm>
 #include <array>
 #include <cstring>
@@ -125,6 +133,123 @@ static void choose_swizzle(const BrickHostPlan &P, BrickPass &ps, int K) {
     }
 }
 
+namespace {
+
+// One side's schedule: per pass the arc's first ring bit and its windows' offsets in the arc.
+struct SidePass {
+    int arc;
+    std::vector<int> windows;
+};
+
+struct Frontier {
+    std::array<uint8_t, FP_MAX_STATE_BITS> h;   // layers applied to each bit
+    bool operator==(const Frontier &o) const { return h == o.h; }
+};
+
+// every gate that bits start .. start+cnt-1 (mod N) allow; calls f(layer, first bit)
+template <typename F>
+int apply_window(Frontier &fr, int N, int L, int par0, int start, int cnt, F f) {
+    int got = 0;
+    for (bool more = true; more;) {
+        more = false;
+        for (int i = 0; i + 1 < cnt; ++i) {
+            const int a = (start + i) % N, b = (start + i + 1) % N, t = fr.h[a];
+            if (t != fr.h[b] || t >= L || (a & 1) != ((par0 + t) & 1)) continue;
+            f(t, a);
+            ++fr.h[a];
+            ++fr.h[b];
+            ++got;
+            more = true;
+        }
+    }
+    return got;
+}
+
+// A new arc costs about 0.7 of a window (the tile's load and store), one without the low
+// bits 3 more (strided rows); a window applies about 5.5 gates in the long run.
+constexpr double kArcCost = 0.7, kFarArcCost = 3.7, kGatesPerWindow = 5.5;
+constexpr size_t kBeam = 48;
+
+std::vector<SidePass> beam_schedule(int N, int L, int par0, int K, int r, uint32_t low_mask) {
+    struct Node {
+        Frontier fr;
+        int arc, win, parent, gates;
+        double cost, score;
+    };
+    const int nwin = K - r + 1, total = L * N / 2;
+    std::vector<char> near(N);
+    for (int a = 0; a < N; ++a) {
+        uint32_t mask = 0;
+        for (int i = 0; i < K; ++i) mask |= 1u << ((a + i) % N);
+        near[a] = (mask & low_mask) == low_mask;
+    }
+    std::vector<Node> all(1);
+    all[0].fr.h.fill(0);
+    all[0].arc = all[0].parent = -1;
+    all[0].gates = 0;
+    all[0].cost = 0;
+    std::vector<int> cur{0};
+    int best = -1;
+    std::vector<Node> next;
+    std::vector<std::pair<double, int>> order;
+    auto nop = [](int, int) {};
+    while (!cur.empty()) {
+        next.clear();
+        for (int id : cur) {
+            const Node nd = all[id];
+            if (best >= 0 && nd.cost >= all[best].cost) continue;
+            for (int a = 0; a < N; ++a) {
+                const bool same = a == nd.arc;
+                for (int o = 0; o < nwin; ++o) {
+                    Node k = nd;
+                    const int g = apply_window(k.fr, N, L, par0, a + o, r, nop);
+                    if (g == 0) continue;
+                    k.arc = a;
+                    k.win = o;
+                    k.parent = id;
+                    k.gates += g;
+                    k.cost += 1.0 + (same ? 0.0 : near[a] ? kArcCost : kFarArcCost);
+                    k.score = k.cost - k.gates / kGatesPerWindow;
+                    next.push_back(k);
+                }
+            }
+        }
+        // the kBeam best with different frontiers or arcs (ties in order: deterministic)
+        order.resize(next.size());
+        for (size_t i = 0; i < next.size(); ++i) {
+            order[i] = {next[i].score, (int)i};
+            if (next[i].gates == total && (best < 0 || next[i].cost < all[best].cost)) {
+                all.push_back(next[i]);
+                best = (int)all.size() - 1;
+            }
+        }
+        const size_t top = std::min(order.size(), 8 * kBeam);
+        std::partial_sort(order.begin(), order.begin() + (long)top, order.end());
+        const size_t first = all.size();
+        cur.clear();
+        for (size_t i = 0; i < top && cur.size() < kBeam; ++i) {
+            const Node &k = next[(size_t)order[i].second];
+            if (k.gates == total) continue;
+            bool dup = false;
+            for (size_t j = first; j < all.size() && !dup; ++j) dup = all[j].arc == k.arc && all[j].fr == k.fr;
+            if (dup) continue;
+            all.push_back(k);
+            cur.push_back((int)all.size() - 1);
+        }
+    }
+    std::vector<SidePass> out;
+    std::vector<int> path;
+    for (int id = best; id > 0; id = all[id].parent) path.push_back(id);
+    for (size_t i = path.size(); i-- > 0;) {
+        const Node &k = all[path[i]];
+        if (out.empty() || out.back().arc != k.arc) out.push_back({k.arc, {}});
+        out.back().windows.push_back(k.win);
+    }
+    return out;
+}
+
+}  // namespace
+
 BrickHostPlan make_brick_plan(int n, int l, int tile_bits, int low_bits, int win_bits, int kind) {
     BrickHostPlan P;
     BrickDev &d = P.dev;
@@ -145,6 +270,7 @@ BrickHostPlan make_brick_plan(int n, int l, int tile_bits, int low_bits, int win
     if (d.tile_bits == 0) return P;
     const int K = tile_bits;
     const bool whole = K == N;
+    const bool tc = !whole && K == kTcTile && win_bits == kMaxWin && low_bits <= 3;
     // candidate arcs: those holding the low bits first (coalesced tile loads);
     // every arc when none of those can make progress
     std::vector<uint32_t> arcs, all_arcs;
@@ -165,7 +291,45 @@ BrickHostPlan make_brick_plan(int n, int l, int tile_bits, int low_bits, int win
             return (1u << tau) | (1u << ((tau + 1) % N));
         };
         size_t left = (size_t)L * m;
-        while (left > 0) {
+        Frontier fr;
+        fr.h.fill(0);
+        const int r = std::min(win_bits, K);
+        std::vector<SidePass> beam;
+        if (tc) beam = beam_schedule(N, L, par(0), K, r, (1u << low_bits) - 1u);
+        for (const SidePass &sp : beam) {
+            BrickPass ps;
+            std::memset(&ps, 0, sizeof ps);
+            ps.gate_off = (int)P.gates.size();
+            ps.rp_off = (int)P.rpasses.size();
+            ps.rg_off = (int)P.rgates.size();
+            for (int i = 0; i < K; ++i) ps.smask |= 1u << ((sp.arc + i) % N);
+            int loc[32];
+            for (int b = 0, k = 0; b < N; ++b) if (ps.smask & (1u << b)) loc[b] = k++;
+            for (int o : sp.windows) {
+                RegPass rp;
+                std::memset(&rp, 0, sizeof rp);
+                rp.r = (uint8_t)r;
+                for (int i = 0; i < r; ++i) rp.win[i] = rp.srt[i] = (uint8_t)loc[(sp.arc + o + i) % N];
+                std::sort(rp.srt, rp.srt + r);
+                rp.gate_off = (int16_t)P.rgates.size();
+                left -= (size_t)apply_window(fr, N, L, par(0), sp.arc + o, r, [&](int t, int a) {
+                    BrickGate g;
+                    g.layer = (uint8_t)t;
+                    g.j = (uint8_t)((a - par(t)) / 2);
+                    g.a = (uint8_t)loc[a];
+                    g.b = (uint8_t)loc[(a + 1) % N];
+                    P.rgates.push_back({(uint8_t)((a - sp.arc - o + 2 * N) % N), (uint8_t)(P.gates.size() - ps.gate_off)});
+                    P.gates.push_back(g);
+                    ++rp.n_gates;
+                });
+                P.rpasses.push_back(rp);
+            }
+            ps.n_gates = (int)P.gates.size() - ps.gate_off;
+            ps.n_rp = (int)P.rpasses.size() - ps.rp_off;
+            choose_swizzle(P, ps, K);
+            P.passes.push_back(ps);
+        }
+        while (left > 0) {   // greedy, or no complete schedule found
             uint32_t best_mask = 0;
             std::vector<int> best;
             for (int round = 0; round < 2 && best.empty(); ++round)
@@ -316,7 +480,7 @@ static void tc_exchange(uint32_t *xcb, const uint8_t *u, const uint8_t *v) {
     }
 }
 
-std::vector<TcWin> make_tc_windows(const BrickHostPlan &P) {
+std::vector<TcWin> make_tc_windows(const BrickHostPlan &P, bool rotations) {
     std::vector<TcWin> out(P.rpasses.size());
     for (const BrickPass &ps : P.passes) {
         // Row orders of the pass's windows.  The 16 lanes of a half-warp drain the
@@ -363,9 +527,11 @@ std::vector<TcWin> make_tc_windows(const BrickHostPlan &P) {
                 if (rowbits[w][pre[pi][r]] == b) return 1u << (r + 1);
             return 0u;
         };
-        std::vector<std::vector<int>> cost(nw, std::vector<int>(np, 0)), from(nw, std::vector<int>(np, -1));
+        // (the tensor-memory form exchanges through its own conflict-free maps whatever the rows:
+        // ascending ones, `pre[0]`, then also store a pass's last window in the longest runs)
+        std::vector<std::vector<int>> cost(nw, std::vector<int>(np, 0)), from(nw, std::vector<int>(np, 0));
         std::vector<uint32_t> bk((size_t)np * kTcTile);
-        for (int w = 1; w < nw; ++w) {
+        for (int w = 1; rotations && w < nw; ++w) {
             for (int q = 0; q < np; ++q)
                 for (int b = 0; b < kTcTile; ++b) bk[(size_t)q * kTcTile + b] = bank(w, q, b);
             // the transition depends on the previous prefix only through its 4 lane bits
@@ -396,7 +562,7 @@ std::vector<TcWin> make_tc_windows(const BrickHostPlan &P) {
             rows_of(w, choice[w], rows);
             tc_layout(out[ps.rp_off + w], P.rpasses[ps.rp_off + w], rows);
         }
-        for (int w = 0; w + 1 < nw; ++w) out[ps.rp_off + w].rotm = tc_rotation(out[ps.rp_off + w], out[ps.rp_off + w + 1]);
+        for (int w = 0; rotations && w + 1 < nw; ++w) out[ps.rp_off + w].rotm = tc_rotation(out[ps.rp_off + w], out[ps.rp_off + w + 1]);
         const uint8_t first[4] = {0, 1, 2, 3};   // the tile load: lanes store consecutive tile indices
         for (int w = 0; w < nw; ++w)
             tc_exchange(out[ps.rp_off + w].xcb, w ? out[ps.rp_off + w - 1].row : first, out[ps.rp_off + w].row);
