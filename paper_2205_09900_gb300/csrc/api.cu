@@ -118,7 +118,7 @@ struct SpiralCache {        // one depth of the paper's HEA on the spiral sweep
     // variants: FP64, FP32, FP64 spread over a 4-CTA cluster (small batches:
     // the FP64 recontraction of a few flagged pairs)
     SpiralConfig cfg[3];
-    DBuf d_wins[3], d_ij[3];   // register windows of cfg[p]
+    DBuf d_wins[3];   // register windows of cfg[p]
     int nwins[3] = {0, 0, 0}, h[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};
 };
 
@@ -1021,8 +1021,7 @@ SpiralCache *spiral_plan(fp_ensemble *E, int L) {
             std::vector<uint8_t> ij;
             spiral_windows(sc->sp, sc->cfg[p].R, sc->cfg[p].split, wins, ij, sc->h[p]);
             sc->nwins[p] = (int)wins.size();
-            if (upload(sc->d_wins[p], wins, E->st) != cudaSuccess || upload(sc->d_ij[p], ij, E->st) != cudaSuccess)
-                sc.reset();
+            if (upload(sc->d_wins[p], wins, E->st) != cudaSuccess) sc.reset();
         }
     }
     SpiralCache *out = sc.get();
@@ -1096,7 +1095,7 @@ fp_status run_spiral(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
             const bool use_win = cf.R > 0;
             CK(launch_spiral(E->d_pairs.as<PairInfo>(), (int)nb, sc->d_maps.as<SpiralMap>(), nmaps, sp.bits,
                              sp.first_bit, cf, use_win ? sc->d_wins[p].as<SpiralWin>() : nullptr,
-                             use_win ? sc->nwins[p] : 0, use_win ? sc->d_ij[p].as<uint8_t>() : nullptr, sc->h[p],
+                             use_win ? sc->nwins[p] : 0, sc->h[p],
                              E->d_merged.as<double2>(), E->d_maps.p, E->d_spiral_scratch.p, fp32, err_scale, tr,
                              kappa, err, E->st));
             CK(t.stop(cmac_pair * (double)nb));

@@ -117,7 +117,13 @@ struct SpiralMap {
 };
 // A register window of the spiral sweep: maps [first, first + n_maps) act only
 // on the window's nb state bits (ascending); map k acts on window bits
-// (ij[k] & 15, ij[k] >> 4) as its (low, high) index bits.
+// (ij[k] & 15, ij[k] >> 4) as its (low, high) index bits.  The maps walk: each starts on the
+// bit that the last one ended on, so map k of a window acts on bits walk[k], walk[k + 1]
+// (indices into `bits`; the padding bits follow).
+// half: a bit that an SP_LL map freed lies outside the window; its zero half needs no
+// work and its position is the highest of the CTA's own, so the CTA takes the lower half of
+// its groups (what the other half holds is not read before an SP_RR map, which reads
+// the zero half's partner alone, has written it).
 // The state is split over s = 0, 1 or 2 cluster bits h0 < h1: amplitude x
 // lives in CTA rank (x_h0 + 2 x_h1) of a 2^s-CTA cluster at local index
 // y = x without those bits, stored at the swizzled slot
@@ -128,7 +134,7 @@ struct SpiralMap {
 // at slot sw(base) ^ (XOR of off[k] over the set bits k of i) in CTA
 // rank(base) ^ (XOR of ctab[k]).
 constexpr int kSpiralMaxWin = 5;
-constexpr int kSpiralWinMaxMaps = 16;   // maps per window (staged in shared memory)
+constexpr int kSpiralWinMaxMaps = kSpiralMaxWin - 1;   // maps per window (staged in shared memory)
 constexpr int kSpiralMaxPos = 24;
 struct SpiralWin {
     uint8_t bits[kSpiralMaxWin];   // state bits of the window, ascending
@@ -136,10 +142,14 @@ struct SpiralWin {
     uint8_t n_maps;
     uint8_t cross;                 // 1: the window holds a cluster bit
     uint8_t n_pos;                 // bits - nb
+    uint8_t half;                  // 1: the upper half of the CTA's groups is a freed bit's zero half
+    uint8_t walk[kSpiralMaxWin];   // window bits in the order the maps walk them
     uint8_t ctab[kSpiralMaxWin];   // rank contribution of each window bit (cluster bits)
     uint8_t pos[kSpiralMaxPos];
     uint16_t off[kSpiralMaxWin];   // sw(local unit vector) of each window bit (0: cluster bit)
     int32_t first;
+    // what the kernel reads: slot | rank << 16 of the walk's bits and of the bits of t'
+    uint32_t vx[kSpiralMaxWin], gx[kSpiralMaxPos];
 };
 
 // One pair of a batch.

@@ -132,7 +132,7 @@ struct SpiralConfig {
 SpiralConfig spiral_config(int bits, bool fp32, int min_split = 0);   // split >= min_split (<= 2)
 size_t spiral_map_elems(bool fp32);
 cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm, int nmaps, int bits, int first_bit,
-                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const uint8_t *ij, const int *h,
+                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const int *h,
                           const double2 *merged, void *maps, void *scratch, bool fp32, double err_scale, double *tr,
                           double *kappa, double *err, cudaStream_t st);
 // Qudit brickwork (kernels_qudit.cu): sampler, maps and sweep of pairs

@@ -4,10 +4,10 @@
 // wires are rings of segments, each tapped by one CZ, into a sequence of
 // in-place 4x4 maps on a state of 2^bits amplitudes (one bit per CZ of a bond
 // plus an auxiliary bit).  Per pair:
-//   spiral_maps_kernel   builds every map from the pair's merged 1-qubit
-//                        operators (FP64 products, stored in C; FP32 maps as
+//   spiral_maps_kernel   the coefficients of every map from the pair's merged
+//                        1-qubit operators (FP64 products, stored in C; FP32 as
 //                        broadcast pairs for packed FMAs);
-//   spiral_win_kernel    register windows: consecutive maps on at most R
+//   spiral_win_kernel    register windows: consecutive maps that walk at most R
 //                        state bits run on 2^R amplitudes per thread in
 //                        registers, one barrier per window.  The state sits
 //                        in shared memory (swizzled), in one CTA or split
@@ -16,6 +16,15 @@
 //                        for four CTAs: a per-pair global slice).
 // Both sweeps start from delta(aux, first bit) and end with the FP64 sum of
 // the state = Tr, its cancellation ratio and rounding-error estimate.
+//
+// Arithmetic bounds the windows (the FMA pipe in FP32, the FP64 pipe at 1/77 of
+// its rate in FP64), so a map is applied by its type, not as 16 entries: the
+// coupling H as two additions, then 2 products per output (SP_MID, the bulk) or
+// 1, in place of 4 products (SP_MID: 20 packed operations instead of 32, RL, LL
+// 12, DIAG 8).  And no window touches a freed bit's zero half (SpiralWin::half).
+// n = 50, about 2,000 pairs per depth: FP32 L = 8 (two CTAs) 36.8 ms instead of 47, L = 7 (one
+// CTA) 4.5 ms instead of 7.0; FP64 with few pairs (four CTAs) 20.9 ms instead of 44.  The two-CTA
+// form is held back by its cross windows and barriers (31 % of the issue slots, 16 warps).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -48,49 +57,37 @@ __device__ __forceinline__ double2 zm(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Entries per stored map: FP64 keeps the 16 complex entries; FP32 keeps each
-// entry t as the pairs (tr, tr) and (-ti, ti), so that acc += t x is two
-// packed FMAs: (tr, tr) * (xr, xi) + (-ti, ti) * (xi, xr).
-template <typename C> struct MapW { static constexpr int w = 16; };
-template <> struct MapW<float2> { static constexpr int w = 32; };
+// Coefficients of a stored map: 8 (entry 4 ia + 2 ob + oa of the types with two 1-qubit
+// operators) or 4 (entry 2 ob + ia), see spiral_maps_kernel.  FP64 keeps them as they are;
+// FP32 keeps a coefficient t as the pairs (tr, tr) and (-ti, ti), so that acc += t x is
+// two packed FMAs: (tr, tr) * (xr, xi) + (-ti, ti) * (xi, xr).
+constexpr int kCoefs = 8;
+template <typename C> struct MapW { static constexpr int w = kCoefs; };
+template <> struct MapW<float2> { static constexpr int w = 2 * kCoefs; };
 
-template <typename C> __device__ __forceinline__ void put_entry(C *dst, int e, double2 t) { dst[e] = mk<C>(t.x, t.y); }
-template <> __device__ __forceinline__ void put_entry<float2>(float2 *dst, int e, double2 t) {   // one 16-byte store
+__device__ __forceinline__ void put_entry(double2 *dst, int e, double2 t) { dst[e] = t; }
+__device__ __forceinline__ void put_entry(float2 *dst, int e, double2 t) {   // one 16-byte store
     *reinterpret_cast<float4 *>(dst + 2 * e) = make_float4((float)t.x, (float)t.x, (float)-t.y, (float)t.y);
 }
 
-// Entry T[4 o + f] of every map, o = o_a + 2 o_b, f = i_a + 2 i_b (SpiralType):
-// one thread per entry, so the 16 threads of a map store its record contiguously.
+// One thread per coefficient, so the 8 threads of a map store its record contiguously.
+//   SP_MID, SP_MID_AUX, SP_MID_RR: F[o_a][i_a] G[o_b][o_a] at 4 i_a + 2 o_b + o_a
+//   the others (but SP_START):     G[o_b][i_a] at 2 o_b + i_a
 template <typename C>
 __global__ void spiral_maps_kernel(const PairInfo *__restrict__ pairs, int npairs, const SpiralMap *__restrict__ sm,
                                    int nmaps, const double2 *__restrict__ merged, C *__restrict__ maps) {
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int m = gid >> 4, e = gid & 15;
+    const int m = gid / kCoefs, e = gid % kCoefs;
     if (m >= nmaps) return;
     const SpiralMap s = sm[m];
-    const int o = e >> 2, f = e & 3;
-    const int oa = o & 1, ob = o >> 1, ia = f & 1, ib = f >> 1;
-    const double h = (ob & ib) ? -1.0 : 1.0;   // H[o_b][i_b] = (-1)^{o_b i_b}
+    if (s.type == SP_START || (s.f < 0 && e >= 4)) return;
     for (int p = blockIdx.y; p < npairs; p += gridDim.y) {   // grid.y is capped at 65535
         const int64_t mo = pairs[p].merged_off;
-        // entry (r, c) of merged item k (the identity when k < 0)
-        auto mat = [&](int k, int r, int c) {
-            return k >= 0 ? merged[(mo + k) * 16 + 2 * r + c] : make_double2(r == c ? 1.0 : 0.0, 0.0);
-        };
-        double2 v = make_double2(0, 0);
-        switch (s.type) {
-            case SP_DIAG_BA: if (o == f) v = mat(s.g, ib, ia); break;
-            case SP_START: if (oa == ob) v = make_double2(h, 0); break;
-            case SP_MID: v = zm(mat(s.f, oa, ia), mat(s.g, ob, oa)); v.x *= h; v.y *= h; break;
-            case SP_MID_AUX: if (ob == ib) v = zm(mat(s.f, oa, ia), mat(s.g, ob, oa)); break;
-            case SP_RL: if (oa == ia) { v = mat(s.g, ob, ia); v.x *= h; v.y *= h; } break;
-            case SP_MID_RR: if (ib == 0) v = zm(mat(s.f, oa, ia), mat(s.g, ob, oa)); break;
-            case SP_RR: if (oa == ia && ib == 0) v = mat(s.g, ob, ia); break;
-            case SP_LL: if (oa == 0) { v = mat(s.g, ob, ia); v.x *= h; v.y *= h; } break;
-            case SP_LL_AUX: if (oa == 0 && ob == ib) v = mat(s.g, ib, ia); break;
-            default: break;
-        }
-        put_entry<C>(maps + ((size_t)p * nmaps + m) * MapW<C>::w, e, v);
+        auto mat = [&](int k, int r, int c) { return merged[(mo + k) * 16 + 2 * r + c]; };
+        const int a = e & 1, ob = (e >> 1) & 1;
+        double2 v = mat(s.g, ob, a);
+        if (s.f >= 0) v = zm(mat(s.f, a, e >> 2), v);
+        put_entry(maps + ((size_t)p * nmaps + m) * MapW<C>::w, e, v);
     }
 }
 
@@ -103,56 +100,120 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {   // a *
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 
-__device__ __forceinline__ double2 cmac(double2 t, double2 x, double2 acc) {
-    acc.x = fma(t.x, x.x, acc.x);
-    acc.x = fma(-t.y, x.y, acc.x);
-    acc.y = fma(t.x, x.y, acc.y);
-    acc.y = fma(t.y, x.x, acc.y);
+// complex sum, difference and t0 x0 (+ t1 x1) for a stored coefficient t
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return fadd2(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return ffma2(b, make_float2(-1.f, -1.f), a); }   // exact product
+struct Coef64 { double2 t; };
+struct Coef32 { float2 r, i; };
+__device__ __forceinline__ Coef64 coef(const double2 *T, int e) { return {T[e]}; }
+__device__ __forceinline__ Coef32 coef(const float2 *T, int e) {
+    const float4 q = *reinterpret_cast<const float4 *>(T + 2 * e);
+    return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+}
+__device__ __forceinline__ double2 cmul(const Coef64 &c, double2 x) {
+    return make_double2(fma(-c.t.y, x.y, c.t.x * x.x), fma(c.t.y, x.x, c.t.x * x.y));
+}
+__device__ __forceinline__ double2 cmac(const Coef64 &c, double2 x, double2 acc) {
+    acc.x = fma(c.t.x, x.x, acc.x);
+    acc.x = fma(-c.t.y, x.y, acc.x);
+    acc.y = fma(c.t.x, x.y, acc.y);
+    acc.y = fma(c.t.y, x.x, acc.y);
     return acc;
 }
-
-// (x0, x1, x2, x3) <- T (x0, x1, x2, x3) for one stored map T
-__device__ __forceinline__ void quad(double2 &x0, double2 &x1, double2 &x2, double2 &x3, const double2 (&T)[16]) {
-    double2 y[4];
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        double2 acc = make_double2(0, 0);
-        acc = cmac(T[4 * o + 0], x0, acc);
-        acc = cmac(T[4 * o + 1], x1, acc);
-        acc = cmac(T[4 * o + 2], x2, acc);
-        acc = cmac(T[4 * o + 3], x3, acc);
-        y[o] = acc;
-    }
-    x0 = y[0]; x1 = y[1]; x2 = y[2]; x3 = y[3];
+__device__ __forceinline__ float2 cmul(const Coef32 &c, float2 x) {
+    return ffma2(c.i, make_float2(x.y, x.x), fmul2(c.r, x));
 }
-__device__ __forceinline__ void quad(float2 &x0, float2 &x1, float2 &x2, float2 &x3, const float2 (&T)[32]) {
-    const float2 x[4] = {x0, x1, x2, x3};
-    float2 acc[4];
-#pragma unroll
-    for (int o = 0; o < 4; ++o) acc[o] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {   // the four outputs accumulate side by side
-        const float2 xs = make_float2(x[f].y, x[f].x);
-#pragma unroll
-        for (int o = 0; o < 4; ++o) acc[o] = ffma2(T[2 * (4 * o + f)], x[f], acc[o]);
-#pragma unroll
-        for (int o = 0; o < 4; ++o) acc[o] = ffma2(T[2 * (4 * o + f) + 1], xs, acc[o]);
-    }
-    x0 = acc[0]; x1 = acc[1]; x2 = acc[2]; x3 = acc[3];
+__device__ __forceinline__ float2 cmac(const Coef32 &c, float2 x, float2 acc) {
+    return ffma2(c.i, make_float2(x.y, x.x), ffma2(c.r, x, acc));
 }
 
-__device__ __forceinline__ void load_map(double2 (&T)[16], const double2 *__restrict__ src) {
+// A map of SpiralType on the quads x[i_a][i_b] of a register block (or of one quad): first
+// PRE, what becomes of the input of bit b: 0 nothing, 1 the coupling H, 2 only i_b = 0 (a
+// freed bit); then CORE for each output bit o_b: 0 F and G (8 coefficients), 1 G with the
+// bit a kept (4), 2 G with i_a summed and the output bit a zero (4), 3 the start (a = b,
+// old a summed).  All quads pass one stage before the next, in place, so that the
+// coefficients of one o_b are live at a time: with all 8 a window of 32 amplitudes spills.
+template <typename C, int PRE, int CORE>
+struct TypedMap {
+    const C *T;
+    template <int N, int A, int B>
+    __device__ __forceinline__ void apply(C (&v)[N]) const {
+        if constexpr (PRE != 0) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) T[e] = src[e];
-}
-__device__ __forceinline__ void load_map(float2 (&T)[32], const float2 *__restrict__ src) {   // 16-byte loads
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
+            for (int x = 0; x < N; ++x) {
+                if (x & B) continue;
+                const C x0 = v[x], x1 = v[x | B];
+                if constexpr (PRE == 1) v[x] = cadd(x0, x1);
+                v[x | B] = PRE == 1 ? csub(x0, x1) : x0;
+            }
+        }
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const float4 q = s4[e];
-        T[2 * e] = make_float2(q.x, q.y);
-        T[2 * e + 1] = make_float2(q.z, q.w);
+        for (int ob = 0; ob < 2; ++ob) {
+            using K = decltype(coef(T, 0));
+            if constexpr (CORE == 3) {
+#pragma unroll
+                for (int x = 0; x < N; ++x) {
+                    if ((x & A) || ((x & B) != 0) != (ob != 0)) continue;
+                    const C y = cadd(v[x], v[x | A]);
+                    v[x] = ob == 0 ? y : mk<C>(0.0, 0.0);
+                    v[x | A] = ob == 0 ? mk<C>(0.0, 0.0) : y;
+                }
+            } else {
+                const K t00 = coef(T, 2 * ob), t01 = coef(T, 2 * ob + 1);
+                K t10 = t00, t11 = t00;
+                if constexpr (CORE == 0) { t10 = coef(T, 4 + 2 * ob); t11 = coef(T, 4 + 2 * ob + 1); }
+#pragma unroll
+                for (int x = 0; x < N; ++x) {
+                    if ((x & A) || ((x & B) != 0) != (ob != 0)) continue;
+                    const C u0 = v[x], u1 = v[x | A];
+                    if constexpr (CORE == 0) {
+                        v[x] = cmac(t10, u1, cmul(t00, u0));
+                        v[x | A] = cmac(t11, u1, cmul(t01, u0));
+                    } else if constexpr (CORE == 1) {
+                        v[x] = cmul(t00, u0);
+                        v[x | A] = cmul(t01, u1);
+                    } else {
+                        v[x] = cmac(t01, u1, cmul(t00, u0));
+                        v[x | A] = mk<C>(0.0, 0.0);
+                    }
+                }
+            }
+        }
+    }
+};
+
+// f(the map of this type)
+template <typename C, typename F>
+__device__ __forceinline__ void with_map(int type, const C *__restrict__ T, F f) {
+    switch (type) {
+        case SP_MID: f(TypedMap<C, 1, 0>{T}); break;
+        case SP_DIAG_BA: f(TypedMap<C, 0, 1>{T}); break;
+        case SP_START: f(TypedMap<C, 1, 3>{T}); break;
+        case SP_MID_AUX: f(TypedMap<C, 0, 0>{T}); break;
+        case SP_RL: f(TypedMap<C, 1, 1>{T}); break;
+        case SP_MID_RR: f(TypedMap<C, 2, 0>{T}); break;
+        case SP_RR: f(TypedMap<C, 2, 1>{T}); break;
+        case SP_LL: f(TypedMap<C, 1, 2>{T}); break;
+        default: f(TypedMap<C, 0, 2>{T}); break;   // SP_LL_AUX
     }
 }
 
@@ -218,19 +279,20 @@ __global__ void __launch_bounds__(512) spiral_sweep_kernel(const PairInfo *__res
     const C *mp = maps + (size_t)blockIdx.x * nmaps * MapW<C>::w;
     for (int k = 0; k < nmaps; ++k) {
         const SpiralMap s = sm[k];
-        C T[MapW<C>::w];
-        load_map(T, mp + (size_t)k * MapW<C>::w);
+        const C *T = mp + (size_t)k * MapW<C>::w;
         const int lo = s.a < s.b ? s.a : s.b, hi = s.a < s.b ? s.b : s.a;
         const uint32_t ia = 1u << s.a, ib = 1u << s.b;
-        for (uint32_t q = threadIdx.x; q < (S >> 2); q += blockDim.x) {
-            const uint32_t i0 = ins0s(ins0s(q, lo), hi);
-            C x0 = st[i0], x1 = st[i0 | ia], x2 = st[i0 | ib], x3 = st[i0 | ia | ib];
-            quad(x0, x1, x2, x3, T);
-            st[i0] = x0;
-            st[i0 | ia] = x1;
-            st[i0 | ib] = x2;
-            st[i0 | ia | ib] = x3;
-        }
+        with_map<C>(s.type, T, [&](const auto &map) {
+            for (uint32_t q = threadIdx.x; q < (S >> 2); q += blockDim.x) {
+                const uint32_t i0 = ins0s(ins0s(q, lo), hi);
+                C v[4] = {st[i0], st[i0 | ia], st[i0 | ib], st[i0 | ia | ib]};
+                map.template apply<4, 1, 2>(v);
+                st[i0] = v[0];
+                st[i0 | ia] = v[1];
+                st[i0 | ib] = v[2];
+                st[i0 | ia | ib] = v[3];
+            }
+        });
         __syncthreads();
     }
     double s[4];
@@ -238,37 +300,13 @@ __global__ void __launch_bounds__(512) spiral_sweep_kernel(const PairInfo *__res
     if (threadIdx.x == 0) write_result(pairs[blockIdx.x], s, err_scale, tr, kappa, err);
 }
 
-// One map on window bits (I, J) of a thread's 2^R register block.
-template <typename C, int I, int J, int R>
-__device__ __forceinline__ void win_map(C (&v)[1 << R], const C (&T)[MapW<C>::w]) {
-#pragma unroll
-    for (int x = 0; x < (1 << R); ++x) {
-        if (x & ((1 << I) | (1 << J))) continue;
-        quad(v[x], v[x | (1 << I)], v[x | (1 << J)], v[x | (1 << I) | (1 << J)], T);
-    }
-}
-
-template <typename C, int R, int I>
-__device__ __forceinline__ void win_map_j(int j, C (&v)[1 << R], const C (&T)[MapW<C>::w]) {
-    switch (j) {
-        case 0: if constexpr (I != 0) win_map<C, I, 0, R>(v, T); break;
-        case 1: if constexpr (I != 1) win_map<C, I, 1, R>(v, T); break;
-        case 2: if constexpr (I != 2 && R > 2) win_map<C, I, 2, R>(v, T); break;
-        case 3: if constexpr (I != 3 && R > 3) win_map<C, I, 3, R>(v, T); break;
-        case 4: if constexpr (I != 4 && R > 4) win_map<C, I, 4, R>(v, T); break;
-        default: break;
-    }
-}
-
-template <typename C, int R>
-__device__ __forceinline__ void win_map_ij(int i, int j, C (&v)[1 << R], const C (&T)[MapW<C>::w]) {
-    switch (i) {
-        case 0: win_map_j<C, R, 0>(j, v, T); break;
-        case 1: win_map_j<C, R, 1>(j, v, T); break;
-        case 2: if constexpr (R > 2) win_map_j<C, R, 2>(j, v, T); break;
-        case 3: if constexpr (R > 3) win_map_j<C, R, 3>(j, v, T); break;
-        case 4: if constexpr (R > 4) win_map_j<C, R, 4>(j, v, T); break;
-        default: break;
+// The window's maps: map k acts on its walk's bits k and k + 1.
+template <typename C, int R, int K = 0>
+__device__ __forceinline__ void win_maps(int n_maps, const SpiralMap *__restrict__ sm, C (&v)[1 << R], const C *T) {
+    if constexpr (K + 1 < R) {
+        if (K >= n_maps) return;
+        with_map<C>(sm[K].type, T + K * MapW<C>::w, [&](const auto &map) { map.template apply<(1 << R), 1 << K, 2 << K>(v); });
+        win_maps<C, R, K + 1>(n_maps, sm, v, T);
     }
 }
 
@@ -303,10 +341,6 @@ __device__ __forceinline__ void win_sync(bool cluster_wide) {
     __syncthreads();
 }
 
-__device__ __forceinline__ uint32_t del_bit(uint32_t x, int p) {   // remove bit p
-    return (x & ((1u << p) - 1u)) | ((x >> (p + 1)) << p);
-}
-
 template <int CL>
 __device__ __forceinline__ uint32_t pick_cta(const uint32_t (&ac)[CL], uint32_t r) {
     if constexpr (CL == 1) return ac[0];
@@ -326,9 +360,9 @@ template <typename C, int CL> struct WinThreads { static constexpr int n = 256; 
 template <> struct WinThreads<float2, 2> { static constexpr int n = 512; };
 
 template <typename C, int R, int CL>
-__global__ void __launch_bounds__(WinThreads<C, CL>::n) spiral_win_kernel(const PairInfo *__restrict__ pairs,
-                                                         const SpiralWin *__restrict__ wins, int nwins,
-                                                         const uint8_t *__restrict__ ij, int nmaps, int bits,
+__global__ void __launch_bounds__(WinThreads<C, CL>::n, sizeof(C) == 8 ? 512 / WinThreads<C, CL>::n : 1)
+    spiral_win_kernel(const PairInfo *__restrict__ pairs, const SpiralWin *__restrict__ wins, int nwins,
+                                                         const SpiralMap *__restrict__ sm, int nmaps, int bits,
                                                          int first_bit, int h0, int h1, const C *__restrict__ maps,
                                                          double err_scale, double *__restrict__ tr,
                                                          double *__restrict__ kappa, double *__restrict__ err) {
@@ -336,7 +370,7 @@ __global__ void __launch_bounds__(WinThreads<C, CL>::n) spiral_win_kernel(const 
     __shared__ double red[4][16];
     __shared__ double part[3][4];   // CL > 1: ranks 1.. write their sums into rank 0
     constexpr int c = CL == 4 ? 2 : (CL == 2 ? 1 : 0);
-    constexpr int MB = kSpiralWinMaxMaps * MapW<C>::w;   // elements of one staged window of maps
+    constexpr int MB = kSpiralWinMaxMaps * MapW<C>::w;   // elements of one staged window of coefficients
     C *st = (C *)smem_raw;
     const uint32_t SL = 1u << (bits - c);
     C *mbuf = st + SL;   // two windows of maps: this one and the next (cp.async)
@@ -371,64 +405,45 @@ __global__ void __launch_bounds__(WinThreads<C, CL>::n) spiral_win_kernel(const 
     win_sync<CL>(true);   // with CL > 1 also: every part exists before any remote access
     const uint32_t G = 1u << (bits - R - c);   // groups this CTA handles per window
     for (int w = 0; w < nwins; ++w) {
-        const SpiralWin &W = wins[w];   // uniform reads (read-only path)
-        const int n_pos = W.n_pos, first = W.first, n_maps = W.n_maps;
-        const bool cross = CL > 1 && W.cross;
+        const SpiralWin *W = wins + w;   // uniform reads (read-only path)
+        const int n_pos = W->n_pos, first = W->first, n_maps = W->n_maps;
+        const bool cross = CL > 1 && W->cross;
         if (w + 1 < nwins) stage(w + 1);   // lands while this window computes
         const C *mw = mbuf + (w & 1) * MB;
-        uint32_t off[R], ctab[R];
-#pragma unroll
-        for (int k = 0; k < R; ++k) { off[k] = W.off[k]; ctab[k] = W.ctab[k]; }
-        for (uint32_t t = threadIdx.x; t < G; t += blockDim.x) {
+        const uint32_t Gw = G >> W->half;   // without the groups of a freed bit's zero half
+        for (uint32_t t = threadIdx.x; t < Gw; t += blockDim.x) {
             const uint32_t tt = rank * G + t;
-            uint32_t b = 0;
-            for (int j = 0; j < n_pos; ++j) b |= ((tt >> j) & 1u) << W.pos[j];
-            uint32_t cb = 0, lb = b;
-            if constexpr (c == 2) { cb = ((b >> h0) & 1u) | (((b >> h1) & 1u) << 1); lb = del_bit(del_bit(b, h1), h0); }
-            if constexpr (c == 1) { cb = (b >> h0) & 1u; lb = del_bit(b, h0); }
-            uint32_t pb = swz(lb);
+            uint32_t base = 0;
+            for (int j = 0; j < n_pos; ++j) base ^= ((tt >> j) & 1u) ? W->gx[j] : 0u;
             C v[1 << R];
-            if (!cross) {
+            uint32_t vx[R];
 #pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    uint32_t a = pb;
+            for (int k = 0; k < R; ++k) vx[k] = W->vx[k];
+            auto at = [&](int i) {
+                uint32_t a = base;
 #pragma unroll
-                    for (int k = 0; k < R; ++k) if ((i >> k) & 1) a ^= off[k];
-                    v[i] = st[a];
-                }
+                for (int k = 0; k < R; ++k) if ((i >> k) & 1) a ^= vx[k];
+                return a;
+            };
+            auto remote = [&](uint32_t a) { return pick_cta<CL>(ac, a >> 16) + (a & 0xffffu) * (uint32_t)sizeof(C); };
+            if (!cross) {   // rank bits are its own
+#pragma unroll
+                for (int i = 0; i < (1 << R); ++i) v[i] = st[at(i) & 0xffffu];
             } else {
 #pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    uint32_t a = pb, r = cb;
+                for (int i = 0; i < (1 << R); ++i) v[i] = dsm_ld(remote(at(i)), C());
+            }
+            win_maps<C, R>(n_maps, sm + first, v, mw);
+            // the store addresses are rebuilt (not kept live across the maps)
+            asm volatile("" : "+r"(base), "+l"(W));
 #pragma unroll
-                    for (int k = 0; k < R; ++k) if ((i >> k) & 1) { a ^= off[k]; r ^= ctab[k]; }
-                    v[i] = dsm_ld(pick_cta<CL>(ac, r) + a * (uint32_t)sizeof(C), C());
-                }
-            }
-            for (int m = 0; m < n_maps; ++m) {
-                C T[MapW<C>::w];
-                load_map(T, mw + m * MapW<C>::w);
-                const int q = ij[first + m];
-                win_map_ij<C, R>(q & 15, q >> 4, v, T);
-            }
-            // the store addresses are rebuilt from pb (not kept live across the maps)
-            asm volatile("" : "+r"(pb), "+r"(cb));
+            for (int k = 0; k < R; ++k) vx[k] = W->vx[k];
             if (!cross) {
 #pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    uint32_t a = pb;
-#pragma unroll
-                    for (int k = 0; k < R; ++k) if ((i >> k) & 1) a ^= off[k];
-                    st[a] = v[i];
-                }
+                for (int i = 0; i < (1 << R); ++i) st[at(i) & 0xffffu] = v[i];
             } else {
 #pragma unroll
-                for (int i = 0; i < (1 << R); ++i) {
-                    uint32_t a = pb, r = cb;
-#pragma unroll
-                    for (int k = 0; k < R; ++k) if ((i >> k) & 1) { a ^= off[k]; r ^= ctab[k]; }
-                    dsm_st(pick_cta<CL>(ac, r) + a * (uint32_t)sizeof(C), v[i]);
-                }
+                for (int i = 0; i < (1 << R); ++i) dsm_st(remote(at(i)), v[i]);
             }
         }
         const bool next_cross = CL > 1 && w + 1 < nwins && wins[w + 1].cross;
@@ -452,7 +467,7 @@ __global__ void __launch_bounds__(WinThreads<C, CL>::n) spiral_win_kernel(const 
 }
 
 template <typename C, int R, int CL>
-cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int nwins, const uint8_t *ij, int nmaps,
+cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int nwins, const SpiralMap *sm, int nmaps,
                   int bits, int first_bit, const int *h, const void *maps, double err_scale, double *tr, double *kappa,
                   double *err, cudaStream_t st) {
     constexpr int c = CL == 4 ? 2 : (CL == 2 ? 1 : 0);
@@ -474,7 +489,7 @@ cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, pairs, wins, nwins, ij, nmaps, bits, first_bit, h[0], h[1], (const C *)maps,
+    return cudaLaunchKernelEx(&cfg, k, pairs, wins, nwins, sm, nmaps, bits, first_bit, h[0], h[1], (const C *)maps,
                               err_scale, tr, kappa, err);
 }
 
@@ -520,18 +535,18 @@ SpiralConfig spiral_config(int bits, bool fp32, int min_split) {
 }
 
 cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm, int nmaps, int bits, int first_bit,
-                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const uint8_t *ij, const int *h,
+                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const int *h,
                           const double2 *merged, void *maps, void *scratch, bool fp32, double err_scale, double *tr,
                           double *kappa, double *err, cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
-    dim3 gm((16 * nmaps + 255) / 256, std::min(npairs, 65535));
+    dim3 gm((kCoefs * nmaps + 255) / 256, std::min(npairs, 65535));
     if (fp32) spiral_maps_kernel<float2><<<gm, 256, 0, st>>>(pairs, npairs, sm, nmaps, merged, (float2 *)maps);
     else spiral_maps_kernel<double2><<<gm, 256, 0, st>>>(pairs, npairs, sm, nmaps, merged, (double2 *)maps);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (wins && cfg.R > 0) {
 #define FP_SPIRAL_WIN_CASE(C, R, CL)                                                                               \
-    return win_t<C, R, CL>(pairs, npairs, wins, nwins, ij, nmaps, bits, first_bit, h, maps, err_scale, tr, kappa, \
+    return win_t<C, R, CL>(pairs, npairs, wins, nwins, sm, nmaps, bits, first_bit, h, maps, err_scale, tr, kappa, \
                            err, st)
         const int CL = 1 << cfg.split;
         if (!fp32) {

@@ -410,20 +410,33 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
     wins.clear();
     ij.assign(P.maps.size(), 0);
     R = std::min(std::max(R, 2), std::min(kSpiralMaxWin, P.bits));
-    // runs of consecutive maps on at most R bits
+    // runs of consecutive maps that walk at most R different bits
     std::vector<uint32_t> sets;
     std::vector<std::pair<size_t, size_t>> runs;
     for (size_t k = 0; k < P.maps.size();) {
-        uint32_t set = 0;
+        uint32_t set = 1u << P.maps[k].a;
         size_t e = k;
-        for (; e < P.maps.size(); ++e) {
-            const uint32_t s2 = set | (1u << P.maps[e].a) | (1u << P.maps[e].b);
-            if (__builtin_popcount(s2) > R || e - k >= (size_t)kSpiralWinMaxMaps) break;
-            set = s2;
+        for (; e < P.maps.size() && e - k < (size_t)(R - 1); ++e) {
+            if (set >> P.maps[e].b & 1 || (e > k && P.maps[e].a != P.maps[e - 1].b)) break;
+            set |= 1u << P.maps[e].b;
         }
         sets.push_back(set);
         runs.push_back({k, e});
         k = e;
+    }
+    // the bits that are freed (SP_LL, SP_LL_AUX) and not taken again (SP_RR, SP_MID_RR) before
+    // a run starts, and stay so during it
+    std::vector<uint32_t> freed(runs.size(), 0);
+    {
+        uint32_t f = 0;
+        for (size_t i = 0; i < runs.size(); ++i) {
+            freed[i] = f & ~sets[i];
+            for (size_t m = runs[i].first; m < runs[i].second; ++m) {
+                const SpiralMap &mp = P.maps[m];
+                if (mp.type == SP_LL || mp.type == SP_LL_AUX) f |= 1u << mp.a;
+                if (mp.type == SP_RR || mp.type == SP_MID_RR) f &= ~(1u << mp.b);
+            }
+        }
     }
     // cluster bits: the state bits the fewest runs touch
     int hb[2] = {-1, -1};
@@ -454,8 +467,14 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
         w.nb = (uint8_t)nb;
         w.n_maps = (uint8_t)(runs[i].second - runs[i].first);
         w.first = (int32_t)runs[i].first;
-        for (size_t m = runs[i].first; m < runs[i].second; ++m)
+        int nw = 0;
+        w.walk[nw++] = (uint8_t)loc[P.maps[runs[i].first].a];
+        for (size_t m = runs[i].first; m < runs[i].second; ++m) {
             ij[m] = (uint8_t)(loc[P.maps[m].a] | (loc[P.maps[m].b] << 4));
+            w.walk[nw++] = (uint8_t)loc[P.maps[m].b];
+        }
+        for (int k = 0; k < nb; ++k)   // the padding bits
+            if (std::find(w.walk, w.walk + nw, (uint8_t)k) == w.walk + nw) w.walk[nw++] = (uint8_t)k;
         wins.push_back(w);
     }
     if (h_out) { h_out[0] = hb[0]; h_out[1] = hb[1]; }
@@ -472,7 +491,13 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
         // lane q: the free non-cluster bit of lowest local position with residue q mod 4
         // (16 lanes then touch 16 distinct slots of sw), else the lowest one left
         const uint32_t freem = ((1u << P.bits) - 1u) & ~set;
-        uint32_t lanes = 0;
+        // a freed bit takes the highest bit of a CTA's group index t
+        const int zpos = P.bits - R - split - 1;
+        int z = -1;
+        for (int b = 0; b < P.bits && zpos >= 0; ++b)
+            if ((freem & ~hmask & freed[i]) >> b & 1) z = b;
+        const uint32_t zm = z >= 0 ? 1u << z : 0u;
+        uint32_t lanes = zm;
         int n = 0;
         for (int q = 0; q < 4; ++q) {
             int pick = -1;
@@ -484,9 +509,21 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
         }
         for (int b = 0; b < P.bits; ++b)
             if ((freem & ~hmask & ~lanes) >> b & 1) w.pos[n++] = (uint8_t)b;
+        if (z >= 0) {
+            std::copy_backward(w.pos + zpos, w.pos + n, w.pos + n + 1);
+            w.pos[zpos] = (uint8_t)z;
+            ++n;
+        }
+        w.half = z >= 0;
         for (int b = 0; b < P.bits; ++b)
             if ((freem & hmask) >> b & 1) w.pos[n++] = (uint8_t)b;
         w.n_pos = (uint8_t)n;
+        auto slot = [&](int b) {
+            return hmask >> b & 1 ? (uint32_t)((b == hb[0] ? 1 : 0) | (b == hb[1] ? 2 : 0)) << 16
+                                  : spiral_swizzle(1u << local(b));
+        };
+        for (int k = 0; k < w.nb; ++k) w.vx[k] = slot(w.bits[w.walk[k]]);
+        for (int j = 0; j < n; ++j) w.gx[j] = slot(w.pos[j]);
     }
 }
 
