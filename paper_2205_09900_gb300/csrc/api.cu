@@ -115,14 +115,23 @@ struct BrickCache {
 struct SpiralCache {        // one depth of the paper's HEA on the spiral sweep
     SpiralPlan sp;
     DBuf d_maps, d_items, d_refs, d_plan;
-    // variants: FP64, FP32, FP64 spread over a 4-CTA cluster (small batches:
-    // the FP64 recontraction of a few flagged pairs)
-    SpiralConfig cfg[3];
-    DBuf d_wins[3];   // register windows of cfg[p]
-    int nwins[3] = {0, 0, 0}, h[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};
+    // variants: FP64 over 2^p CTAs (p <= kSpiralMaxSplit; R = 0: not for this size, but
+    // `base`, the smallest), then FP32
+    static constexpr int kFp32 = kSpiralMaxSplit + 1;
+    SpiralConfig cfg[kFp32 + 1];
+    DBuf d_wins[kFp32 + 1];   // register windows of cfg[p]
+    int nwins[kFp32 + 1] = {}, base = 0;
+    int resident[kFp32] = {};        // FP64 clusters of variant p on the device at a time
+    SpiralCut cut[kFp32 + 1];
+};
+
+struct SideStream {   // beside an ensemble's own stream, joined before its call goes on
+    cudaStream_t st = nullptr;
+    cudaEvent_t ev = nullptr;
 };
 
 struct fp_ensemble {
+    static constexpr size_t kSideStreams = 8;
     fp_ensemble_desc d;
     cudaStream_t st = nullptr;
     int device = 0;
@@ -149,6 +158,7 @@ struct fp_ensemble {
     // spiral sweep (the paper's HEA), per depth; null: the depth is not spiral-shaped
     std::map<int, std::unique_ptr<SpiralCache>> spiral_plans;
     DBuf d_spiral_scratch;
+    std::vector<SideStream> side;
     DBuf d_maps, d_states;
     DBuf d_step_items, d_step_which, d_step_pairs, d_step_meet, d_step_part;   // lock-step sweep
     DBuf d_flag;               // device error flag of kernels with bounded waits (zero when clear)
@@ -1014,13 +1024,17 @@ SpiralCache *spiral_plan(fp_ensemble *E, int L) {
             upload(sc->d_refs, sc->sp.refs, E->st) != cudaSuccess ||
             upload(sc->d_plan, std::vector<DevPlan>{pl}, E->st) != cudaSuccess)
             sc.reset();
-        for (int p = 0; sc && p < 3; ++p) {
-            sc->cfg[p] = spiral_config(sc->sp.bits, p == 1, p == 2 ? 2 : 0);
+        if (sc) sc->base = spiral_config(sc->sp.bits, false).split;
+        for (int p = 0; sc && p <= SpiralCache::kFp32; ++p) {
+            const bool fp32 = p == SpiralCache::kFp32;
+            if (!fp32 && p < sc->base) continue;
+            sc->cfg[p] = spiral_config(sc->sp.bits, fp32, fp32 ? 0 : p);
             if (sc->cfg[p].R == 0) continue;
             std::vector<SpiralWin> wins;
             std::vector<uint8_t> ij;
-            spiral_windows(sc->sp, sc->cfg[p].R, sc->cfg[p].split, wins, ij, sc->h[p]);
+            spiral_windows(sc->sp, sc->cfg[p].R, sc->cfg[p].split, wins, ij, sc->cut[p].h);
             sc->nwins[p] = (int)wins.size();
+            if (!fp32) sc->resident[p] = spiral_resident(sc->sp.bits, sc->cfg[p]);
             if (upload(sc->d_wins[p], wins, E->st) != cudaSuccess) sc.reset();
         }
     }
@@ -1029,85 +1043,183 @@ SpiralCache *spiral_plan(fp_ensemble *E, int L) {
     return out;
 }
 
-// Spiral sweep for pairs of one depth L (FP_HEA_PAULI with CNOT walls):
-// sampler, merged 1-qubit operators, maps, one CTA per pair; sub-batches
-// under the workspace budget.
-fp_status run_spiral(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> &idx, int L, SpiralCache *sc, int prec,
+// FP64 variant for nb pairs: the fewest microseconds per window over the waves of clusters
+// that nb pairs take (16 CTAs per pair for the few pairs that a recontraction usually has).
+int spiral_variant(const SpiralCache *sc, uint64_t nb, bool fp32) {
+    if (fp32) return SpiralCache::kFp32;
+    int best = sc->base;
+    double best_us = 1e300;
+    for (int p = sc->base; p < SpiralCache::kFp32; ++p) {
+        if (sc->cfg[p].R == 0 || sc->cfg[p].split != p || sc->resident[p] <= 0) continue;
+        const double us = std::ceil((double)nb / sc->resident[p]) * spiral_wave_us(sc->sp.bits, p);
+        if (us < best_us) { best_us = us; best = p; }
+    }
+    return best;
+}
+
+struct SpiralJob {   // pairs of one depth L
+    int L;
+    const std::vector<uint64_t> *idx;
+    SpiralCache *sc;
+    int variant, n_raw, n_merged, n_maps;
+    size_t scr, per_pair;         // amplitudes of global state and bytes per pair
+    uint64_t pair0 = 0;           // a batch's first pair, raw gate, merged item, map and state of the buffers
+    size_t raw0 = 0, merged0 = 0, map0 = 0, scr0 = 0;
+};
+
+// The batch [done, done + nb) of a job's pairs, from the host's descriptors to the traces, on `st`.
+fp_status spiral_batch(fp_ensemble *E, const SpiralJob &j, uint64_t nb, bool fp32, double *tr, double *kappa, double *err,
+                       cudaStream_t st) {
+    const SpiralCache *sc = j.sc;
+    const size_t celem = fp32 ? sizeof(float2) : sizeof(double2);
+    const PairInfo *pairs = E->d_pairs.as<PairInfo>() + j.pair0;
+    SampleParams smp;
+    smp.seed = E->d.seed;
+    smp.n = E->d.n;
+    smp.raw_kind = E->raw_kind;
+    smp.self_pair = (E->d.flags & FP_FLAG_SELF_PAIR) ? 1 : 0;
+    const double err_scale = FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53) * std::sqrt((double)j.n_maps);
+    {
+        KTimer t(E, FP_K_SAMPLE);
+        CK(launch_sample(smp, pairs, (int)nb, j.n_raw, E->d_raw.as<double2>(), st));
+        CK(t.stop((double)nb));
+    }
+    {
+        KTimer t(E, FP_K_MERGE);
+        CK(launch_merge(pairs, (int)nb, j.n_merged, sc->d_plan.as<DevPlan>(), sc->d_items.as<MergeItem>(),
+                        sc->d_refs.as<MergeRef>(), E->d_raw.as<double2>(), E->d_merged.as<double2>(), st));
+        CK(t.stop((double)nb));
+    }
+    {
+        KTimer t(E, FP_K_SPIRAL);
+        const int p = j.variant;
+        const SpiralConfig &cf = sc->cfg[p];
+        const bool use_win = cf.R > 0;
+        char *maps = E->d_maps.as<char>() + j.map0 * spiral_map_elems(fp32) * celem;
+        CK(launch_spiral(pairs, (int)nb, sc->d_maps.as<SpiralMap>(), j.n_maps, sc->sp.bits, sc->sp.first_bit, cf,
+                         use_win ? sc->d_wins[p].as<SpiralWin>() : nullptr, use_win ? sc->nwins[p] : 0, sc->cut[p],
+                         E->d_merged.as<double2>(), maps, E->d_spiral_scratch.as<char>() + j.scr0 * celem, fp32,
+                         err_scale, tr, kappa, err, st));
+        CK(t.stop(4.0 * (double)j.n_maps * (double)((size_t)1 << sc->sp.bits) * (double)nb));
+        if (E->timing) E->kst.launches[FP_K_SPIRAL] += 1;   // maps + sweep
+    }
+    return FP_OK;
+}
+
+// Spiral sweep for pairs of the depths in `by_depth` (FP_HEA_PAULI with CNOT walls):
+// sampler, merged 1-qubit operators, maps, a CTA or cluster per pair.  Depths that fit the
+// workspace budget together run side by side on a stream each, deepest first: the
+// recontracted pairs of one depth alone leave most SMs idle (n = 50, L = 2..8: their FP64
+// sweeps take 14.9 ms one after another, 5 side by side).  Otherwise (or to time the kernels) depth by depth, in sub-batches under the budget.
+fp_status run_spiral(fp_ensemble *E, uint64_t first, const std::map<int, std::vector<uint64_t>> &by_depth, int prec,
                      double *tr, double *kappa, double *err, float *gpu_ms) {
     const fp_ensemble_desc &d = E->d;
-    const SpiralPlan &sp = sc->sp;
     const bool fp32 = prec != FP_PREC_FP64;
     const size_t celem = fp32 ? sizeof(float2) : sizeof(double2);
-    const int n_raw = 1 + d.n + L * d.n;
-    const int n_merged = (int)sp.merges.size(), nmaps = (int)sp.maps.size();
-    const int pv = fp32 ? 1 : 0;
-    const SpiralConfig &cfg = sc->cfg[pv];
-    const size_t scr = cfg.scratch_elems, mw = spiral_map_elems(fp32);
-    const size_t per_pair = (size_t)2 * n_raw * 16 * sizeof(double2) + (size_t)n_merged * 16 * sizeof(double2) +
-                            (size_t)nmaps * mw * celem + scr * celem;
-    // sub-batches of at most 65535 pairs (the sampler and merge grids index pairs by grid.y)
-    const uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(65535, E->ws_budget / per_pair));
-    const double err_scale = FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53) * std::sqrt((double)nmaps);
-    const double cmac_pair = 4.0 * (double)nmaps * (double)((size_t)1 << sp.bits);
-    SampleParams smp;
-    smp.seed = d.seed;
-    smp.n = d.n;
-    smp.raw_kind = E->raw_kind;
-    smp.self_pair = (d.flags & FP_FLAG_SELF_PAIR) ? 1 : 0;
-    for (uint64_t done = 0; done < idx.size();) {
-        const uint64_t nb = std::min<uint64_t>(cap, idx.size() - done);
-        std::vector<PairInfo> pinfo(nb);
+    constexpr uint64_t kMaxBatch = 65535;   // the sampler and merge grids index pairs by grid.y
+    std::vector<SpiralJob> jobs;
+    size_t all = 0;
+    bool together = !E->timing;
+    for (auto it = by_depth.rbegin(); it != by_depth.rend(); ++it) {
+        SpiralJob j;
+        j.L = it->first;
+        j.idx = &it->second;
+        j.sc = E->spiral_plans[j.L].get();
+        j.n_raw = 1 + d.n + j.L * d.n;
+        j.n_merged = (int)j.sc->sp.merges.size();
+        j.n_maps = (int)j.sc->sp.maps.size();
+        j.scr = j.sc->cfg[fp32 ? SpiralCache::kFp32 : j.sc->base].scratch_elems;
+        j.per_pair = (size_t)2 * j.n_raw * 16 * sizeof(double2) + (size_t)j.n_merged * 16 * sizeof(double2) +
+                     (size_t)j.n_maps * spiral_map_elems(fp32) * celem + j.scr * celem;
+        all += j.idx->size() * j.per_pair;
+        together = together && j.idx->size() <= kMaxBatch;
+        jobs.push_back(j);
+    }
+    together = together && jobs.size() > 1 && all <= E->ws_budget;
+    // a launch set: one batch of one job, or every job's only batch
+    std::vector<PairInfo> pinfo;
+    auto place = [&](SpiralJob &j, uint64_t done, uint64_t nb, const SpiralJob *after, uint64_t nb_after) {
+        if (after) {
+            j.pair0 = after->pair0 + nb_after;
+            j.raw0 = after->raw0 + nb_after * 2 * after->n_raw;
+            j.merged0 = after->merged0 + nb_after * after->n_merged;
+            j.map0 = after->map0 + nb_after * after->n_maps;
+            j.scr0 = after->scr0 + nb_after * after->scr;
+        }
+        j.variant = spiral_variant(j.sc, nb, fp32);
         for (uint64_t i = 0; i < nb; ++i) {
-            std::memset(&pinfo[i], 0, sizeof(PairInfo));
-            pinfo[i].pair = first + idx[done + i];
-            pinfo[i].plan = 0;
-            pinfo[i].n_raw = n_raw;
-            pinfo[i].raw_off = (int64_t)i * 2 * n_raw;
-            pinfo[i].merged_off = (int64_t)i * n_merged;
-            pinfo[i].out = (int64_t)idx[done + i];
+            PairInfo pi;
+            std::memset(&pi, 0, sizeof pi);
+            pi.pair = first + (*j.idx)[done + i];
+            pi.n_raw = j.n_raw;
+            pi.raw_off = (int64_t)(j.raw0 + i * 2 * j.n_raw);
+            pi.merged_off = (int64_t)(j.merged0 + i * j.n_merged);
+            pi.out = (int64_t)(*j.idx)[done + i];
+            pinfo.push_back(pi);
         }
+    };
+    auto reserve = [&](const SpiralJob &j, uint64_t nb) -> fp_status {   // up to the end of j's batch of nb
         CK(upload(E->d_pairs, pinfo, E->st));
-        CK(E->d_raw.reserve(nb * 2 * n_raw * 16 * sizeof(double2)));
-        CK(E->d_merged.reserve(std::max<size_t>(16, nb * n_merged * 16 * sizeof(double2))));
-        CK(E->d_maps.reserve(nb * nmaps * mw * celem));
-        CK(E->d_spiral_scratch.reserve(std::max<size_t>(16, nb * scr * celem)));
-        CK(cudaEventRecord(E->ev0, E->st));
-        {
-            KTimer t(E, FP_K_SAMPLE);
-            CK(launch_sample(smp, E->d_pairs.as<PairInfo>(), (int)nb, n_raw, E->d_raw.as<double2>(), E->st));
-            CK(t.stop((double)nb));
-        }
-        {
-            KTimer t(E, FP_K_MERGE);
-            CK(launch_merge(E->d_pairs.as<PairInfo>(), (int)nb, n_merged, sc->d_plan.as<DevPlan>(),
-                            sc->d_items.as<MergeItem>(), sc->d_refs.as<MergeRef>(), E->d_raw.as<double2>(),
-                            E->d_merged.as<double2>(), E->st));
-            CK(t.stop((double)nb));
-        }
-        {
-            KTimer t(E, FP_K_SPIRAL);
-            // too few FP64 pairs to fill the SMs: the 4-CTA form (same windows, smaller parts)
-            int p = pv;
-            if (!fp32 && sc->cfg[2].R > 0 && sc->cfg[2].split > cfg.split &&
-                (int64_t)nb * (1 << cfg.split) < (int64_t)E->sms)
-                p = 2;
-            const SpiralConfig &cf = sc->cfg[p];
-            const bool use_win = cf.R > 0;
-            CK(launch_spiral(E->d_pairs.as<PairInfo>(), (int)nb, sc->d_maps.as<SpiralMap>(), nmaps, sp.bits,
-                             sp.first_bit, cf, use_win ? sc->d_wins[p].as<SpiralWin>() : nullptr,
-                             use_win ? sc->nwins[p] : 0, sc->h[p],
-                             E->d_merged.as<double2>(), E->d_maps.p, E->d_spiral_scratch.p, fp32, err_scale, tr,
-                             kappa, err, E->st));
-            CK(t.stop(cmac_pair * (double)nb));
-            if (E->timing) E->kst.launches[FP_K_SPIRAL] += 1;   // maps + sweep
-        }
+        CK(E->d_raw.reserve((j.raw0 + nb * 2 * j.n_raw) * 16 * sizeof(double2)));
+        CK(E->d_merged.reserve(std::max<size_t>(16, (j.merged0 + nb * j.n_merged) * 16 * sizeof(double2))));
+        CK(E->d_maps.reserve((j.map0 + nb * j.n_maps) * spiral_map_elems(fp32) * celem));
+        CK(E->d_spiral_scratch.reserve(std::max<size_t>(16, (j.scr0 + nb * j.scr) * celem)));
+        return FP_OK;
+    };
+    auto finish = [&](uint64_t pairs) -> fp_status {
         CK(cudaEventRecord(E->ev1, E->st));
         CK(cudaEventSynchronize(E->ev1));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, E->ev0, E->ev1));
         if (gpu_ms) *gpu_ms += ms;
-        E->kst.pairs += nb;
-        done += nb;
+        E->kst.pairs += pairs;
+        return FP_OK;
+    };
+    if (together) {
+        uint64_t total = 0;
+        for (size_t k = 0; k < jobs.size(); ++k) {
+            place(jobs[k], 0, jobs[k].idx->size(), k ? &jobs[k - 1] : nullptr, k ? jobs[k - 1].idx->size() : 0);
+            total += jobs[k].idx->size();
+        }
+        fp_status s = reserve(jobs.back(), jobs.back().idx->size());
+        if (s != FP_OK) return s;
+        while (E->side.size() < std::min(jobs.size(), fp_ensemble::kSideStreams)) {
+            SideStream x;
+            CK(cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking));
+            E->side.push_back(x);
+            CK(cudaEventCreateWithFlags(&E->side.back().ev, cudaEventDisableTiming));
+        }
+        CK(cudaEventRecord(E->ev0, E->st));
+        for (SideStream &x : E->side) CK(cudaStreamWaitEvent(x.st, E->ev0, 0));
+        for (size_t k = 0; k < jobs.size() && s == FP_OK; ++k)
+            s = spiral_batch(E, jobs[k], jobs[k].idx->size(), fp32, tr, kappa, err, E->side[k % E->side.size()].st);
+        cudaError_t joined = cudaSuccess;   // (after a failed launch too: what runs still uses the buffers)
+        for (SideStream &x : E->side) {
+            cudaError_t e = cudaEventRecord(x.ev, x.st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(E->st, x.ev, 0);
+            if (e != cudaSuccess) joined = e;
+        }
+        if (s != FP_OK || joined != cudaSuccess)
+            for (SideStream &x : E->side) cudaStreamSynchronize(x.st);
+        if (s != FP_OK) return s;
+        CK(joined);
+        return finish(total);
+    }
+    for (SpiralJob &j : jobs) {
+        const uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(kMaxBatch, E->ws_budget / j.per_pair));
+        for (uint64_t done = 0; done < j.idx->size();) {
+            const uint64_t nb = std::min<uint64_t>(cap, j.idx->size() - done);
+            pinfo.clear();
+            place(j, done, nb, nullptr, 0);
+            fp_status s = reserve(j, nb);
+            if (s != FP_OK) return s;
+            CK(cudaEventRecord(E->ev0, E->st));
+            s = spiral_batch(E, j, nb, fp32, tr, kappa, err, E->st);
+            if (s != FP_OK) return s;
+            s = finish(nb);
+            if (s != FP_OK) return s;
+            done += nb;
+        }
     }
     return FP_OK;
 }
@@ -1209,9 +1321,8 @@ fp_status route(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> &idx
         fp_status s = run_brick(E, first, it->second, it->first, prec, tr, kappa, err, gpu_ms);
         if (s != FP_OK) return s;
     }
-    for (auto it = spiral_depth.rbegin(); it != spiral_depth.rend(); ++it) {
-        fp_status s = run_spiral(E, first, it->second, it->first, E->spiral_plans[it->first].get(), prec, tr, kappa,
-                                 err, gpu_ms);
+    if (!spiral_depth.empty()) {
+        fp_status s = run_spiral(E, first, spiral_depth, prec, tr, kappa, err, gpu_ms);
         if (s != FP_OK) return s;
     }
     return run_generic(E, first, generic, depth, prec, tr, kappa, err, gpu_ms);
@@ -1369,6 +1480,10 @@ void fp_ensemble_destroy(fp_ensemble *ens) {
     for (auto &kv : ens->graphs) if (kv.second) cudaGraphExecDestroy(kv.second);
     for (int k = 0; k < 2; ++k) if (ens->gev[k]) cudaEventDestroy(ens->gev[k]);
     if (ens->gst) cudaStreamDestroy(ens->gst);
+    for (SideStream &x : ens->side) {
+        if (x.ev) cudaEventDestroy(x.ev);
+        cudaStreamDestroy(x.st);
+    }
     delete ens;
 }
 

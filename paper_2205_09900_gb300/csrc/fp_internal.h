@@ -124,8 +124,8 @@ struct SpiralMap {
 // work and its position is the highest of the CTA's own, so the CTA takes the lower half of
 // its groups (what the other half holds is not read before an SP_RR map, which reads
 // the zero half's partner alone, has written it).
-// The state is split over s = 0, 1 or 2 cluster bits h0 < h1: amplitude x
-// lives in CTA rank (x_h0 + 2 x_h1) of a 2^s-CTA cluster at local index
+// The state is split over s = 0 .. 4 cluster bits h0 < h1 < ..: amplitude x
+// lives in CTA rank (x_h0 + 2 x_h1 + ..) of a 2^s-CTA cluster at local index
 // y = x without those bits, stored at the swizzled slot
 // sw(y) = y ^ fold4(y >> 4) (fold4: XOR of the 4-bit chunks).  A CTA handles
 // the window's groups t' = rank * G + t; the group base takes bit j of t' at
@@ -136,6 +136,8 @@ struct SpiralMap {
 constexpr int kSpiralMaxWin = 5;
 constexpr int kSpiralWinMaxMaps = kSpiralMaxWin - 1;   // maps per window (staged in shared memory)
 constexpr int kSpiralMaxPos = 24;
+constexpr int kSpiralMaxSplit = 4;
+struct SpiralCut { int h[kSpiralMaxSplit]; };   // cluster bits, ascending (-1: unused)
 struct SpiralWin {
     uint8_t bits[kSpiralMaxWin];   // state bits of the window, ascending
     uint8_t nb;                    // window bits (the register block is 2^nb)

@@ -120,19 +120,23 @@ cudaError_t run_passes_tc(const BrickDev &d, const BrickPass *hpasses, const Bri
 // (spiral_map_elems(fp32) elements of C per map), then the sweep.  The
 // configuration of a state of 2^bits amplitudes: R = 0 applies one map per
 // pass (shared memory when it fits, else `scratch`, scratch_elems per pair);
-// R = 4 or 5 runs windows of R bits (spiral_windows with `split`; cluster bits
-// h[0], h[1]) over shared memory of one CTA (split = 0) or a 2^split-CTA
-// cluster (split = 1, 2).
+// R = 4 or 5 runs windows of R bits (spiral_windows with `split` cluster bits) over
+// shared memory of one CTA (split = 0) or a 2^split-CTA cluster (split <= 2, FP64 <= 4).
 constexpr size_t kSpiralSmemMax = 128 * 1024;
 struct SpiralConfig {
     int R = 0;
     int split = 0;
     size_t scratch_elems = 0;
 };
-SpiralConfig spiral_config(int bits, bool fp32, int min_split = 0);   // split >= min_split (<= 2)
+SpiralConfig spiral_config(int bits, bool fp32, int min_split = 0);   // split >= min_split where it applies
+// FP64 clusters of this form that the device holds at a time, and about what a window
+// takes them (us): 16-amplitude groups of 3 maps keep an SM quarter busy for 14.8 us per
+// warp (an FP64 instruction per 77 cycles), plus the barrier.
+int spiral_resident(int bits, const SpiralConfig &cfg);
+double spiral_wave_us(int bits, int split);
 size_t spiral_map_elems(bool fp32);
 cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm, int nmaps, int bits, int first_bit,
-                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const int *h,
+                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const SpiralCut &cut,
                           const double2 *merged, void *maps, void *scratch, bool fp32, double err_scale, double *tr,
                           double *kappa, double *err, cudaStream_t st);
 // Qudit brickwork (kernels_qudit.cu): sampler, maps and sweep of pairs

@@ -25,6 +25,7 @@
 // n = 50, about 2,000 pairs per depth: FP32 L = 8 (two CTAs) 36.8 ms instead of 47, L = 7 (one
 // CTA) 4.5 ms instead of 7.0; FP64 with few pairs (four CTAs) 20.9 ms instead of 44.  The two-CTA
 // form is held back by its cross windows and barriers (31 % of the issue slots, 16 warps).
+// FP64 L = 8, 4 pairs: 16 CTAs each 4.7 ms, 4 CTAs each 13.9.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -37,6 +38,9 @@ namespace cg = cooperative_groups;
 
 namespace fpk {
 namespace {
+
+template <int X> constexpr int kLog2 = 1 + kLog2<X / 2>;
+template <> constexpr int kLog2<1> = 0;
 
 __device__ __forceinline__ uint32_t ins0s(uint32_t x, int p) {   // insert a zero bit at position p
     return (x & ((1u << p) - 1u)) | ((x >> p) << (p + 1));
@@ -341,19 +345,34 @@ __device__ __forceinline__ void win_sync(bool cluster_wide) {
     __syncthreads();
 }
 
-template <int CL>
-__device__ __forceinline__ uint32_t pick_cta(const uint32_t (&ac)[CL], uint32_t r) {
-    if constexpr (CL == 1) return ac[0];
-    else if constexpr (CL == 2) return r ? ac[1] : ac[0];
-    else return (r & 2) ? ((r & 1) ? ac[3] : ac[2]) : ((r & 1) ? ac[1] : ac[0]);
-}
+// Address of rank r's part in the cluster window: kept for up to 4 ranks, else computed.
+template <int CL> struct CtaParts {
+    static constexpr int n = CL <= 4 ? CL : 1;
+    uint32_t ac[n];
+    __device__ __forceinline__ explicit CtaParts(const void *st) {
+#pragma unroll
+        for (int r = 0; r < n; ++r) ac[r] = CL == 1 ? 0u : CL <= 4 ? cluster_addr(st, r) : (uint32_t)__cvta_generic_to_shared(st);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t r) const {
+        if constexpr (CL == 1) return ac[0];
+        else if constexpr (CL == 2) return r ? ac[1] : ac[0];
+        else if constexpr (CL == 4) return (r & 2) ? ((r & 1) ? ac[3] : ac[2]) : ((r & 1) ? ac[1] : ac[0]);
+        else {
+            uint32_t a;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(ac[0]), "r"(r));
+            return a;
+        }
+    }
+};
 
-// Register windows over a state held in the shared memory of CL = 1, 2 or 4
-// CTAs (one pair per CTA or per cluster).  With CL > 1 the cluster bits h0
-// (and h1) of an amplitude give its CTA rank; a window holding one of them
+// Register windows over a state held in the shared memory of CL = 1, 2, 4, 8 or 16
+// CTAs (one pair per CTA or per cluster).  With CL > 1 the cluster bits h of an
+// amplitude give its CTA rank; a window holding one of them
 // ("cross" window) reads and writes other CTAs' parts through distributed
 // shared memory and is fenced by cluster barriers; the other windows stay in
-// their own CTA.  Addressing: SpiralWin.
+// their own CTA.  Addressing: SpiralWin.  8 and 16 CTAs serve FP64 batches of a few pairs
+// (spiral_split): an FP64 instruction occupies its SM quarter for about 77 cycles, so a
+// pair is as fast as the number of quarters that share it.
 // Threads per CTA: the FP32 two-CTA form runs one CTA per SM (its half of the
 // state fills the shared memory), so it takes as many warps as its registers allow.
 template <typename C, int CL> struct WinThreads { static constexpr int n = 256; };
@@ -363,33 +382,30 @@ template <typename C, int R, int CL>
 __global__ void __launch_bounds__(WinThreads<C, CL>::n, sizeof(C) == 8 ? 512 / WinThreads<C, CL>::n : 1)
     spiral_win_kernel(const PairInfo *__restrict__ pairs, const SpiralWin *__restrict__ wins, int nwins,
                                                          const SpiralMap *__restrict__ sm, int nmaps, int bits,
-                                                         int first_bit, int h0, int h1, const C *__restrict__ maps,
+                                                         int first_bit, SpiralCut cut, const C *__restrict__ maps,
                                                          double err_scale, double *__restrict__ tr,
                                                          double *__restrict__ kappa, double *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[4][16];
-    __shared__ double part[3][4];   // CL > 1: ranks 1.. write their sums into rank 0
-    constexpr int c = CL == 4 ? 2 : (CL == 2 ? 1 : 0);
+    __shared__ double part[CL][4];   // CL > 1: ranks 1.. write their sums into rank 0
+    constexpr int c = kLog2<CL>;
     constexpr int MB = kSpiralWinMaxMaps * MapW<C>::w;   // elements of one staged window of coefficients
     C *st = (C *)smem_raw;
     const uint32_t SL = 1u << (bits - c);
     C *mbuf = st + SL;   // two windows of maps: this one and the next (cp.async)
-    uint32_t rank = 0, ac[CL];   // ac[r]: rank r's part in the cluster window
+    uint32_t rank = 0;
+    const CtaParts<CL> cta(st);
     double *part0 = &part[0][0];
     if constexpr (CL > 1) {
         cg::cluster_group cl = cg::this_cluster();
         rank = cl.block_rank();
-#pragma unroll
-        for (int r = 0; r < CL; ++r) ac[r] = cluster_addr(st, r);
         part0 = cl.map_shared_rank(&part[0][0], 0);
-    } else {
-        ac[0] = 0;
     }
     const int aux = bits - 1;
     for (uint32_t y = threadIdx.x; y < SL; y += blockDim.x) {
         uint32_t x = y;
-        if constexpr (c >= 1) x = ins0s(x, h0) | ((rank & 1u) << h0);
-        if constexpr (c == 2) x = ins0s(x, h1) | (((rank >> 1) & 1u) << h1);
+#pragma unroll
+        for (int q = 0; q < c; ++q) x = ins0s(x, cut.h[q]) | (((rank >> q) & 1u) << cut.h[q]);
         st[swz(y)] = mk<C>((((x >> aux) ^ (x >> first_bit)) & 1u) ? 0.0 : 1.0, 0.0);
     }
     const C *mp = maps + (size_t)(blockIdx.x / CL) * nmaps * MapW<C>::w;
@@ -425,7 +441,7 @@ __global__ void __launch_bounds__(WinThreads<C, CL>::n, sizeof(C) == 8 ? 512 / W
                 for (int k = 0; k < R; ++k) if ((i >> k) & 1) a ^= vx[k];
                 return a;
             };
-            auto remote = [&](uint32_t a) { return pick_cta<CL>(ac, a >> 16) + (a & 0xffffu) * (uint32_t)sizeof(C); };
+            auto remote = [&](uint32_t a) { return cta(a >> 16) + (a & 0xffffu) * (uint32_t)sizeof(C); };
             if (!cross) {   // rank bits are its own
 #pragma unroll
                 for (int i = 0; i < (1 << R); ++i) v[i] = st[at(i) & 0xffffu];
@@ -467,30 +483,55 @@ __global__ void __launch_bounds__(WinThreads<C, CL>::n, sizeof(C) == 8 ? 512 / W
 }
 
 template <typename C, int R, int CL>
-cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int nwins, const SpiralMap *sm, int nmaps,
-                  int bits, int first_bit, const int *h, const void *maps, double err_scale, double *tr, double *kappa,
-                  double *err, cudaStream_t st) {
-    constexpr int c = CL == 4 ? 2 : (CL == 2 ? 1 : 0);
-    const size_t bytes = (((size_t)1 << (bits - c)) + 2 * kSpiralWinMaxMaps * MapW<C>::w) * sizeof(C);
+cudaLaunchConfig_t win_config(int npairs, int bits, cudaLaunchAttribute *attr, cudaStream_t st) {
+    constexpr int c = kLog2<CL>;
     const uint32_t G = 1u << (bits - R - c);
-    const int threads = (int)std::min<uint32_t>(WinThreads<C, CL>::n, std::max<uint32_t>(32u, G));
-    auto k = spiral_win_kernel<C, R, CL>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3((unsigned)(npairs * CL));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = bytes;
+    cfg.blockDim = dim3((unsigned)std::min<uint32_t>(WinThreads<C, CL>::n, std::max<uint32_t>(32u, G)));
+    cfg.dynamicSmemBytes = (((size_t)1 << (bits - c)) + 2 * kSpiralWinMaxMaps * MapW<C>::w) * sizeof(C);
     cfg.stream = st;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = CL;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, pairs, wins, nwins, sm, nmaps, bits, first_bit, h[0], h[1], (const C *)maps,
-                              err_scale, tr, kappa, err);
+    return cfg;
+}
+
+template <typename C, int R, int CL>
+cudaError_t win_prepare(size_t bytes) {
+    auto k = spiral_win_kernel<C, R, CL>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+// clusters of this form that the device holds at a time (0: it cannot run them)
+template <int CL>
+int resident_fp64(int bits) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = win_config<double2, 4, CL>(1, bits, attr, nullptr);
+    int n = 0;
+    if (win_prepare<double2, 4, CL>(cfg.dynamicSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, spiral_win_kernel<double2, 4, CL>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+template <typename C, int R, int CL>
+cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int nwins, const SpiralMap *sm, int nmaps,
+                  int bits, int first_bit, const SpiralCut &cut, const void *maps, double err_scale, double *tr, double *kappa,
+                  double *err, cudaStream_t st) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = win_config<C, R, CL>(npairs, bits, attr, st);
+    cudaError_t e = win_prepare<C, R, CL>(cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, spiral_win_kernel<C, R, CL>, pairs, wins, nwins, sm, nmaps, bits, first_bit, cut,
+                              (const C *)maps, err_scale, tr, kappa, err);
 }
 
 template <typename C>
@@ -521,7 +562,7 @@ SpiralConfig spiral_config(int bits, bool fp32, int min_split) {
     const size_t bytes = ((size_t)1 << bits) * (fp32 ? sizeof(float2) : sizeof(double2));
     c.split = bytes <= kSpiralSmemMax ? 0 : bytes <= 2 * kSpiralSmemMax ? 1 : bytes <= 4 * kSpiralSmemMax ? 2 : -1;
     if (const char *ev = std::getenv("FP_SPIRAL_SPLIT")) min_split = std::max(min_split, std::atoi(ev));   // tuning
-    if (c.split >= 0) c.split = std::max(c.split, std::min(min_split, 2));
+    if (c.split >= 0) c.split = std::max(c.split, std::min(min_split, fp32 ? 2 : kSpiralMaxSplit));
     // measured on GB300 (n = 50, depths 5..8): 5-bit windows from 2^13 FP32
     // amplitudes up, else 4
     c.R = fp32 && bits >= 13 ? 5 : 4;
@@ -534,8 +575,24 @@ SpiralConfig spiral_config(int bits, bool fp32, int min_split) {
     return c;
 }
 
+int spiral_resident(int bits, const SpiralConfig &cfg) {
+    if (cfg.R != 4) return 0;
+    switch (cfg.split) {
+        case 0: return resident_fp64<1>(bits);
+        case 1: return resident_fp64<2>(bits);
+        case 2: return resident_fp64<4>(bits);
+        case 3: return resident_fp64<8>(bits);
+        default: return resident_fp64<16>(bits);
+    }
+}
+
+double spiral_wave_us(int bits, int split) {
+    const int w = bits - 4 - 5 - split;   // log2 of a CTA's warps of groups
+    return 14.8 * (w > 2 ? 1 << (w - 2) : 1) + (split ? 2.5 : 0.7);
+}
+
 cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm, int nmaps, int bits, int first_bit,
-                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const int *h,
+                          const SpiralConfig &cfg, const SpiralWin *wins, int nwins, const SpiralCut &cut,
                           const double2 *merged, void *maps, void *scratch, bool fp32, double err_scale, double *tr,
                           double *kappa, double *err, cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
@@ -546,7 +603,7 @@ cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm
     if (e != cudaSuccess) return e;
     if (wins && cfg.R > 0) {
 #define FP_SPIRAL_WIN_CASE(C, R, CL)                                                                               \
-    return win_t<C, R, CL>(pairs, npairs, wins, nwins, sm, nmaps, bits, first_bit, h, maps, err_scale, tr, kappa, \
+    return win_t<C, R, CL>(pairs, npairs, wins, nwins, sm, nmaps, bits, first_bit, cut, maps, err_scale, tr, kappa, \
                            err, st)
         const int CL = 1 << cfg.split;
         if (!fp32) {
@@ -554,6 +611,8 @@ cudaError_t launch_spiral(const PairInfo *pairs, int npairs, const SpiralMap *sm
             if (CL == 1) FP_SPIRAL_WIN_CASE(double2, 4, 1);
             if (CL == 2) FP_SPIRAL_WIN_CASE(double2, 4, 2);
             if (CL == 4) FP_SPIRAL_WIN_CASE(double2, 4, 4);
+            if (CL == 8) FP_SPIRAL_WIN_CASE(double2, 4, 8);
+            if (CL == 16) FP_SPIRAL_WIN_CASE(double2, 4, 16);
         } else if (cfg.R == 4) {
             if (CL == 1) FP_SPIRAL_WIN_CASE(float2, 4, 1);
             if (CL == 2) FP_SPIRAL_WIN_CASE(float2, 4, 2);

@@ -406,7 +406,7 @@ static uint32_t spiral_swizzle(uint32_t y) {   // s(y) of the spiral window kern
 }
 
 void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin> &wins, std::vector<uint8_t> &ij,
-                    int h_out[2]) {
+                    int *h_out) {
     wins.clear();
     ij.assign(P.maps.size(), 0);
     R = std::min(std::max(R, 2), std::min(kSpiralMaxWin, P.bits));
@@ -439,7 +439,7 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
         }
     }
     // cluster bits: the state bits the fewest runs touch
-    int hb[2] = {-1, -1};
+    int hb[kSpiralMaxSplit] = {-1, -1, -1, -1};
     {
         std::vector<std::pair<int, int>> use;   // (runs touching the bit, bit)
         for (int b = 0; b < P.bits; ++b) {
@@ -448,11 +448,12 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
             use.push_back({c, b});
         }
         std::sort(use.begin(), use.end());
-        for (int q = 0; q < split && q < 2; ++q) hb[q] = use[q].second;
-        if (split == 2 && hb[0] > hb[1]) std::swap(hb[0], hb[1]);
+        split = std::min(split, std::min(kSpiralMaxSplit, P.bits));
+        for (int q = 0; q < split; ++q) hb[q] = use[q].second;
+        std::sort(hb, hb + split);
     }
     uint32_t hmask = 0;
-    for (int q = 0; q < 2; ++q) if (hb[q] >= 0) hmask |= 1u << hb[q];
+    for (int q = 0; q < split; ++q) hmask |= 1u << hb[q];
     for (size_t i = 0; i < runs.size(); ++i) {
         // pad to R bits with the lowest other non-cluster bits (every window moves 2^R amplitudes)
         uint32_t &set = sets[i];
@@ -477,7 +478,12 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
             if (std::find(w.walk, w.walk + nw, (uint8_t)k) == w.walk + nw) w.walk[nw++] = (uint8_t)k;
         wins.push_back(w);
     }
-    if (h_out) { h_out[0] = hb[0]; h_out[1] = hb[1]; }
+    for (int q = 0; h_out && q < std::max(split, 2); ++q) h_out[q] = hb[q];
+    auto rank_of = [&](int b) {   // rank contribution of a state bit
+        int r = 0;
+        for (int q = 0; q < split; ++q) if (hb[q] == b) r = 1 << q;
+        return r;
+    };
     auto local = [&](int b) { return b - __builtin_popcount(hmask & ((1u << b) - 1u)); };
     for (size_t i = 0; i < wins.size(); ++i) {
         SpiralWin &w = wins[i];
@@ -485,7 +491,7 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
         w.cross = (set & hmask) ? 1 : 0;
         for (int q = 0; q < w.nb; ++q) {
             const int b = w.bits[q];
-            w.ctab[q] = (uint8_t)((b == hb[0] ? 1 : 0) | (b == hb[1] ? 2 : 0));
+            w.ctab[q] = (uint8_t)rank_of(b);
             w.off[q] = (hmask >> b & 1) ? 0 : (uint16_t)spiral_swizzle(1u << local(b));
         }
         // lane q: the free non-cluster bit of lowest local position with residue q mod 4
@@ -519,8 +525,7 @@ void spiral_windows(const SpiralPlan &P, int R, int split, std::vector<SpiralWin
             if ((freem & hmask) >> b & 1) w.pos[n++] = (uint8_t)b;
         w.n_pos = (uint8_t)n;
         auto slot = [&](int b) {
-            return hmask >> b & 1 ? (uint32_t)((b == hb[0] ? 1 : 0) | (b == hb[1] ? 2 : 0)) << 16
-                                  : spiral_swizzle(1u << local(b));
+            return hmask >> b & 1 ? (uint32_t)rank_of(b) << 16 : spiral_swizzle(1u << local(b));
         };
         for (int k = 0; k < w.nb; ++k) w.vx[k] = slot(w.bits[w.walk[k]]);
         for (int j = 0; j < n; ++j) w.gx[j] = slot(w.pos[j]);
