@@ -100,6 +100,26 @@ FP_HD int64_t rsqrt_step(uint64_t a, uint32_t &y0) {
     return ((e >> 1) + ((3 * ((eh * eh) >> 40)) >> 3)) << 20;
 }
 
+// cos and sin of 2 pi ph 2^-64 in Q60
+FP_HD void cos_sin_fixed(uint64_t ph, Half &c, Half &d) {
+    // the angle is k/512 + t turns, |t| <= 2^-10
+    const uint64_t kk = (ph + (1ull << 54)) >> 55;
+    const int64_t t = (int64_t)(ph - (kk << 55));
+    Half ck, sk;
+    table_halves(kCosSin, (int)(kk & 511), ck, sk);
+    const Half x = halves(mul60(halves(t << 6), halves(kTwoPiQ57)));   // radians in Q67
+    const int64_t x2 = mul60(x, x);                                    // Q74
+    const Half x2h = halves(x2);
+    const int64_t sv = kOne60 - (mul60(x2h, halves(rec(6, 60) - (wide(x2h.h, (int32_t)rec(120, 37)) >> 21))) >> 14);
+    const int32_t cw = (int32_t)rec(24, 35) - (mulhi32(x2h.h, (int32_t)rec(720, 40)) >> 17);
+    const Half cs = halves(kOne60 - (mul60(x2h, halves(rec(2, 60) - (wide(x2h.h, cw) >> 19))) >> 14));   // Q60
+    const Half sn = halves(mul60(x, halves(sv)) >> 7);                                                   // Q60
+    c = halves(wide(ck.h, cs.h) - wide(sk.h, sn.h) +
+                          ((wide(ck.h, cs.l) + wide(ck.l, cs.h) - wide(sk.h, sn.l) - wide(sk.l, sn.h) + (1ll << 29)) >> 30));
+    d = halves(wide(sk.h, cs.h) + wide(ck.h, sn.h) +
+                          ((wide(sk.h, cs.l) + wide(sk.l, cs.h) + wide(ck.h, sn.l) + wide(ck.l, sn.h) + (1ll << 30)) >> 30));
+}
+
 // One complex Gaussian (E|Z|^2 = 1) from two Philox words, in units of 2^-57:
 // Z = sqrt(-ln u1) e^{2 pi i u2}, u1 = ((xa >> 11) + 1) 2^-53, u2 = (xb >> 11) 2^-53
 // (keying in fp.h).
@@ -156,23 +176,8 @@ FP_HD Fx2 gauss_fixed(uint64_t xa, uint64_t xb) {
     const int64_t c1 = rsqrt_step(a, y0);     // Q80
     int64_t rad = (int64_t)(((a >> 32) * y0 + (((uint64_t)(uint32_t)a * y0) >> 32)) >> 2);   // sqrt(a) (1 - c) in Q60
     rad += mul60(halves(rad), halves(c1)) >> 20;
-    // cos, sin of 2 pi u2: u2 = k/512 + t, |t| <= 2^-10 turns
-    const uint64_t ph = xb & ~0x7FFull;       // turns in 2^-64
-    const uint64_t kk = (ph + (1ull << 54)) >> 55;
-    const int64_t t = (int64_t)(ph - (kk << 55));
-    Half ck, sk;
-    table_halves(kCosSin, (int)(kk & 511), ck, sk);
-    const Half x = halves(mul60(halves(t << 6), halves(kTwoPiQ57)));   // radians in Q67
-    const int64_t x2 = mul60(x, x);                                    // Q74
-    const Half x2h = halves(x2);
-    const int64_t sv = kOne60 - (mul60(x2h, halves(rec(6, 60) - (wide(x2h.h, (int32_t)rec(120, 37)) >> 21))) >> 14);
-    const int32_t cw = (int32_t)rec(24, 35) - (mulhi32(x2h.h, (int32_t)rec(720, 40)) >> 17);
-    const Half cs = halves(kOne60 - (mul60(x2h, halves(rec(2, 60) - (wide(x2h.h, cw) >> 19))) >> 14));   // Q60
-    const Half sn = halves(mul60(x, halves(sv)) >> 7);                                                   // Q60
-    const Half c = halves(wide(ck.h, cs.h) - wide(sk.h, sn.h) +
-                          ((wide(ck.h, cs.l) + wide(ck.l, cs.h) - wide(sk.h, sn.l) - wide(sk.l, sn.h) + (1ll << 29)) >> 30));
-    const Half d = halves(wide(sk.h, cs.h) + wide(ck.h, sn.h) +
-                          ((wide(sk.h, cs.l) + wide(sk.l, cs.h) + wide(ck.h, sn.l) + wide(ck.l, sn.h) + (1ll << 30)) >> 30));
+    Half c, d;
+    cos_sin_fixed(xb & ~0x7FFull, c, d);
     // E <= 6: |rad 2^(E/2)| <= 6.06
     const Half rh = halves(rad);
     const int64_t zr = mul60(rh, c), zi = mul60(rh, d);   // Q60

@@ -23,15 +23,19 @@
 //
 // Bound: FP32 adds and FMAs (5,100 clocks per qubit at N = 14) beside the
 // exchange's shared-memory traffic (two 8-byte accesses per amplitude and
-// exchange, with the table reads 5,600); FP64: the FP64 pipe.  Measured per pair
+// exchange, with the table reads 5,600).  FP64 (N >= 6) computes in 64-bit integers
+// (fixed.h): bound by the integer pipes instead of the FP64 pipe.  Measured per pair
 // at n = 50 on a GB300, against dense 4x4 maps on the same boundary: L = 8 FP32
 // 1.6 us against 11.0 (tensor-core tile passes), L = 7 0.31 against 5.6, L = 6
-// 0.07 against 1.5 (one map per shared-memory pass); L = 8 FP64, 214 pairs, 76 us
-// against 320 (FMA tile passes).
+// 0.07 against 1.5 (one map per shared-memory pass); L = 8 FP64, 214 pairs, 76 us in FP64
+// arithmetic against 320 (FMA tile passes).  100,000 pairs, L = 1..8, of which about 700 go
+// through FP64: 61.5 ms with FP64 arithmetic, 46.7 with integers, 42.7 with the slots
+// sampled in fixed point too.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "brick.h"
+#include "fixed.h"
 #include "kernels.h"
 #include "meet.h"
 
@@ -46,11 +50,11 @@ template <> struct HeaShape<float2, 8> { static constexpr int R = 4, CLB = 0; };
 template <> struct HeaShape<float2, 10> { static constexpr int R = 5, CLB = 0; };
 template <> struct HeaShape<float2, 12> { static constexpr int R = 5, CLB = 0; };
 template <> struct HeaShape<float2, 14> { static constexpr int R = 5, CLB = 0; };
-template <> struct HeaShape<double2, 6> { static constexpr int R = 3, CLB = 0; };
-template <> struct HeaShape<double2, 8> { static constexpr int R = 4, CLB = 0; };
-template <> struct HeaShape<double2, 10> { static constexpr int R = 4, CLB = 0; };
-template <> struct HeaShape<double2, 12> { static constexpr int R = 4, CLB = 0; };
-template <> struct HeaShape<double2, 14> { static constexpr int R = 4, CLB = 1; };
+template <> struct HeaShape<longlong2, 6> { static constexpr int R = 3, CLB = 0; };
+template <> struct HeaShape<longlong2, 8> { static constexpr int R = 4, CLB = 0; };
+template <> struct HeaShape<longlong2, 10> { static constexpr int R = 4, CLB = 0; };
+template <> struct HeaShape<longlong2, 12> { static constexpr int R = 4, CLB = 0; };
+template <> struct HeaShape<longlong2, 14> { static constexpr int R = 4, CLB = 1; };
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -75,6 +79,10 @@ __device__ __forceinline__ void butterfly(double2 &a, double2 &b) {
     a = s;
     b = d;
 }
+
+// What a boundary of C needs: its coefficients, and its left half's amplitudes for the meet.
+template <typename C> struct HeaNum { using Coef = C; using Out = C; };
+template <> struct HeaNum<longlong2> { using Coef = int4; using Out = double2; };   // FP64 (fixed.h)
 
 // Geometry of the sweep, all compile-time.  Window w holds local bits
 // [lo(w), lo(w) + R) in registers and applies the Hadamards of bits
@@ -154,10 +162,15 @@ __host__ __device__ constexpr uint32_t hslot(uint32_t y) { return y ^ ((y >> R) 
 
 template <typename C, int N, int R, int CLB>
 __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>::kCta))   // at most 128 registers
-    hea_sweep_kernel(int n, int cut, const PairInfo *__restrict__ pairs, int npairs, const C *__restrict__ slots,
-                     C *__restrict__ lscr, double err_scale, double *__restrict__ tr, double *__restrict__ kappa,
+    hea_sweep_kernel(int n, int cut, const PairInfo *__restrict__ pairs, int npairs,
+                     const typename HeaNum<C>::Coef *__restrict__ slots, typename HeaNum<C>::Out *__restrict__ lscr,
+                     double err_scale, double *__restrict__ tr, double *__restrict__ kappa,
                      double *__restrict__ err) {
     using H = Hea<N, R, CLB>;
+    using Coef = typename HeaNum<C>::Coef;
+    using Out = typename HeaNum<C>::Out;
+    constexpr bool fix = std::is_same<C, longlong2>::value;
+    static_assert(sizeof(Coef) == sizeof(C), "the shared-memory layout");
     constexpr int T = H::T, NW = H::NW, V = 1 << R, NL = H::NL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int grp = threadIdx.x / T, t = threadIdx.x % T;
@@ -165,9 +178,9 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
     const int pw = (int)(CLB ? blockIdx.x >> 1 : blockIdx.x) * H::GP + grp;
     const int p = pw < npairs ? pw : npairs - 1;   // spare groups repeat the last pair and write nothing
     C *buf = (C *)smem_raw + (size_t)grp * H::kStride;
-    C *tabs = (C *)smem_raw + (size_t)H::GP * H::kStride + (size_t)grp * 3 * H::kTab;
-    C *sl = (C *)smem_raw + (size_t)H::GP * (H::kStride + 3 * H::kTab) + (size_t)grp * 8 * N;
-    const C *gs = slots + (size_t)p * n * N * 4;
+    Coef *tabs = (Coef *)smem_raw + (size_t)H::GP * H::kStride + (size_t)grp * 3 * H::kTab;
+    Coef *sl = (Coef *)smem_raw + (size_t)H::GP * (H::kStride + 3 * H::kTab) + (size_t)grp * 8 * N;
+    const Coef *gs = slots + (size_t)p * n * N * 4;
     auto sync = [] {
         if constexpr (T <= 32) __syncwarp();
         else __syncthreads();
@@ -186,7 +199,7 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
         if (CLB && b == N - 1) return rank;
         return b < H::lo(w) ? ((uint32_t)t >> b) & 1u : ((uint32_t)t >> (b - R)) & 1u;
     };
-    auto build_dir = [&](auto fc, const C *s, C *tab) {
+    auto build_dir = [&](auto fc, const Coef *s, Coef *tab) {
         constexpr bool fwd = decltype(fc)::value;
         static_for<NW>([&](auto wc) {
             constexpr int w = decltype(wc)::value;
@@ -196,11 +209,14 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
                 static_for<H::len(w, fwd) - 1>([&](auto jc) {
                     constexpr int j = decltype(jc)::value + 1;
                     const uint32_t cur = ((uint32_t)e >> H::pos(w, fwd, j)) & 1u;
-                    const C m = s[4 * H::bit(w, fwd, j) + 2 * cur + prev];
-                    f = j == 1 ? m : cmul(f, m);
+                    const Coef m = s[4 * H::bit(w, fwd, j) + 2 * cur + prev];
+                    if constexpr (j > 1) f = cmul(f, m);
+                    else if constexpr (fix) f = fix_join(m);
+                    else f = m;
                     prev = cur;
                 });
-                tab[H::off(w, fwd) + e] = f;
+                if constexpr (fix) tab[H::off(w, fwd) + e] = fix_coef(f);
+                else tab[H::off(w, fwd) + e] = f;
             }
         });
     };
@@ -209,12 +225,34 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
         else build_dir(std::false_type{}, sl + (k & 1) * 4 * N, tabs + (k % 3) * H::kTab);
     };
     C v[V];
+    int scale = 0;   // fixed point: amplitudes are v 2^scale
     auto ones = [&] {
+        if constexpr (fix) scale = 1 - kFixTop;
 #pragma unroll
-        for (int i = 0; i < V; ++i) v[i].x = 1, v[i].y = 0;
+        for (int i = 0; i < V; ++i) {
+            if constexpr (fix) v[i].x = 1ll << (kFixTop - 1);
+            else v[i].x = 1;
+            v[i].y = 0;
+        }
+    };
+    // Fixed point: every thread's block has its own scale, published beside the amplitudes.  A
+    // window's product and R Hadamards grow a component at most 16 sqrt(2) times and the CTAs'
+    // Hadamard doubles it, to below 2^63.  Four copies: between two writes of one copy
+    // lies an exchange with a barrier of the whole group (at most two in a row are a warp's).
+    __shared__ int scale_sh[fix ? 4 * H::kCta : 1];
+    [[maybe_unused]] int turn = 0;
+    auto scales = [&] { return scale_sh + (4 * grp + (turn & 3)) * T; };
+    // for the meet
+    auto result = [&](const C &a) -> Out {
+        if constexpr (fix) {
+            const double f = ldexp(1.0, scale);
+            return make_double2((double)a.x * f, (double)a.y * f);
+        } else {
+            return a;
+        }
     };
     // window w's factors, then its Hadamards
-    auto window = [&](auto wc, auto fc, const C *tab, bool ladder) {
+    auto window = [&](auto wc, auto fc, const Coef *tab, bool ladder) {
         constexpr int w = decltype(wc)::value;
         constexpr bool fwd = decltype(fc)::value;
         if constexpr (H::size(w, fwd) > 0) {
@@ -241,7 +279,7 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
     };
     auto pass_dir = [&](auto fc, int k, bool ladder) {
         constexpr bool fwd = decltype(fc)::value;
-        const C *tab = tabs + (k % 3) * H::kTab;
+        const Coef *tab = tabs + (k % 3) * H::kTab;
         static_for<NW>([&](auto kc) {
             constexpr int step = decltype(kc)::value, w = fwd ? step : NW - 1 - step;
             using WC = std::integral_constant<int, w>;
@@ -251,20 +289,36 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
                     const uint32_t a0 = base(WC{});
 #pragma unroll
                     for (int i = 0; i < V; ++i) buf[a0 ^ hslot<C, R>((uint32_t)i << H::lo(w))] = v[i];
+                    if constexpr (fix) scales()[t] = scale;
                     cg::this_cluster().sync();
                     const C *other = cg::this_cluster().map_shared_rank(buf, rank ^ 1u);
+                    [[maybe_unused]] int so = 0, top = 0;
+                    if constexpr (fix) {
+                        so = cg::this_cluster().map_shared_rank(scales(), rank ^ 1u)[t];
+                        top = max(scale, so);
+                        ++turn;
+                    }
 #pragma unroll
                     for (int i = 0; i < V; ++i) {
-                        const C u = other[a0 ^ hslot<C, R>((uint32_t)i << H::lo(w))];
+                        C u = other[a0 ^ hslot<C, R>((uint32_t)i << H::lo(w))];
+                        if constexpr (fix) {
+                            fix_align(u, so, top);
+                            fix_align(v[i], scale, top);
+                        }
                         v[i].x = rank ? u.x - v[i].x : v[i].x + u.x;
                         v[i].y = rank ? u.y - v[i].y : v[i].y + u.y;
                     }
+                    if constexpr (fix) scale = top;
                     cg::this_cluster().sync();   // read before either side writes again
                 }
             }
             if constexpr (step < NW - 1) {
                 constexpr int wn = fwd ? w + 1 : w - 1;
                 const uint32_t a0 = base(WC{}), a1 = base(std::integral_constant<int, wn>{});
+                if constexpr (fix) {
+                    fix_settle(v, scale);
+                    scales()[t] = scale;
+                }
 #pragma unroll
                 for (int i = 0; i < V; ++i) buf[a0 ^ hslot<C, R>((uint32_t)i << H::lo(w))] = v[i];
                 // tables k+1 (over those of pass k-2, which everyone has left) and the
@@ -277,6 +331,18 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
                 else __syncthreads();
 #pragma unroll
                 for (int i = 0; i < V; ++i) v[i] = buf[a1 ^ hslot<C, R>((uint32_t)i << H::lo(wn))];
+                if constexpr (fix) {
+                    // the thread that had register i's amplitude in window w
+                    auto had = [](uint32_t y) { return (y & ((1u << H::lo(w)) - 1u)) | ((y >> (H::lo(w) + R)) << H::lo(w)); };
+                    const int *e = scales() + had(((uint32_t)t & ((1u << H::lo(wn)) - 1u)) | (((uint32_t)t >> H::lo(wn)) << (H::lo(wn) + R)));
+                    int top = e[0];
+#pragma unroll
+                    for (int i = 1; i < V; ++i) top = max(top, e[had((uint32_t)i << H::lo(wn))]);
+#pragma unroll
+                    for (int i = 0; i < V; ++i) fix_align(v[i], e[had((uint32_t)i << H::lo(wn))], top);
+                    scale = top;
+                    ++turn;
+                }
             }
         });
     };
@@ -290,7 +356,7 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
     build(0);
     sync();
     ones();
-    C *lp = lscr + (((size_t)pw << N) | ((size_t)rank << NL));
+    Out *lp = lscr + (((size_t)pw << N) | ((size_t)rank << NL));
     for (int k = 0; k < n; ++k) {
         load_slots(k + 2);   // over pass k's matrices, whose tables are built
         commit();
@@ -299,16 +365,18 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
         if (k == cut - 1) {   // the left half is done; both halves end in the same window
             if (pw < npairs)
 #pragma unroll
-                for (int i = 0; i < V; ++i) lp[(size_t)i * T + t] = v[i];
+                for (int i = 0; i < V; ++i) lp[(size_t)i * T + t] = result(v[i]);
             ones();
             sync();   // the next pass may start in another window than this one ended in
+        } else if (k + 1 < n) {   // the next pass goes on in the same window
+            if constexpr (fix) fix_settle(v, scale);
         }
     }
-    MeetAcc<C> acc;
+    MeetAcc<Out> acc;
     if (pw < npairs) {
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-            acc.add(lp[(size_t)i * T + t], v[i]);
+            acc.add(lp[(size_t)i * T + t], result(v[i]));
             if ((i & 7) == 7) acc.flush();
         }
         acc.flush();
@@ -402,7 +470,8 @@ cudaError_t run_thread(const BrickDev &d, const PairInfo *pairs, int npairs, con
 }
 
 template <typename C, int N>
-cudaError_t run_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, const C *slots, C *lscr, double err_scale,
+cudaError_t run_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, const typename HeaNum<C>::Coef *slots,
+                      typename HeaNum<C>::Out *lscr, double err_scale,
                       double *tr, double *kappa, double *err, cudaStream_t st) {
     constexpr int R = HeaShape<C, N>::R, CLB = HeaShape<C, N>::CLB;
     using H = Hea<N, R, CLB>;
@@ -425,17 +494,21 @@ cudaError_t run_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, cons
     return cudaLaunchKernelEx(&cfg, k, d.n, d.cut, pairs, npairs, slots, lscr, err_scale, tr, kappa, err);
 }
 
-template <typename C>
-cudaError_t launch_t(const BrickDev &d, const PairInfo *pairs, int npairs, const C *slots, C *lscr, double err_scale,
+// C: FP32, or FP64 in its thread kernels; W: what the wider sweeps compute in
+template <typename C, typename W>
+cudaError_t launch_t(const BrickDev &d, const PairInfo *pairs, int npairs, const void *slots, void *lscr, double err_scale,
                      double *tr, double *kappa, double *err, cudaStream_t st) {
+    const C *ts = (const C *)slots;
+    const auto *ws = (const typename HeaNum<W>::Coef *)slots;
+    auto *ls = (typename HeaNum<W>::Out *)lscr;
     switch (d.N) {
-        case 2: return run_thread<C, 2>(d, pairs, npairs, slots, err_scale, tr, kappa, err, st);
-        case 4: return run_thread<C, 4>(d, pairs, npairs, slots, err_scale, tr, kappa, err, st);
-        case 6: return run_sweep<C, 6>(d, pairs, npairs, slots, lscr, err_scale, tr, kappa, err, st);
-        case 8: return run_sweep<C, 8>(d, pairs, npairs, slots, lscr, err_scale, tr, kappa, err, st);
-        case 10: return run_sweep<C, 10>(d, pairs, npairs, slots, lscr, err_scale, tr, kappa, err, st);
-        case 12: return run_sweep<C, 12>(d, pairs, npairs, slots, lscr, err_scale, tr, kappa, err, st);
-        case 14: return run_sweep<C, 14>(d, pairs, npairs, slots, lscr, err_scale, tr, kappa, err, st);
+        case 2: return run_thread<C, 2>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
+        case 4: return run_thread<C, 4>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
+        case 6: return run_sweep<W, 6>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
+        case 8: return run_sweep<W, 8>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
+        case 10: return run_sweep<W, 10>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
+        case 12: return run_sweep<W, 12>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
+        case 14: return run_sweep<W, 14>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -452,11 +525,11 @@ void shape_t(int *win_bits, int *threads) {
 bool hea_shape(int N, bool fp32, int *win_bits, int *threads) {
     switch (N) {
         case 2: case 4: *win_bits = N; *threads = 128; return true;
-        case 6: fp32 ? shape_t<float2, 6>(win_bits, threads) : shape_t<double2, 6>(win_bits, threads); return true;
-        case 8: fp32 ? shape_t<float2, 8>(win_bits, threads) : shape_t<double2, 8>(win_bits, threads); return true;
-        case 10: fp32 ? shape_t<float2, 10>(win_bits, threads) : shape_t<double2, 10>(win_bits, threads); return true;
-        case 12: fp32 ? shape_t<float2, 12>(win_bits, threads) : shape_t<double2, 12>(win_bits, threads); return true;
-        case 14: fp32 ? shape_t<float2, 14>(win_bits, threads) : shape_t<double2, 14>(win_bits, threads); return true;
+        case 6: fp32 ? shape_t<float2, 6>(win_bits, threads) : shape_t<longlong2, 6>(win_bits, threads); return true;
+        case 8: fp32 ? shape_t<float2, 8>(win_bits, threads) : shape_t<longlong2, 8>(win_bits, threads); return true;
+        case 10: fp32 ? shape_t<float2, 10>(win_bits, threads) : shape_t<longlong2, 10>(win_bits, threads); return true;
+        case 12: fp32 ? shape_t<float2, 12>(win_bits, threads) : shape_t<longlong2, 12>(win_bits, threads); return true;
+        case 14: fp32 ? shape_t<float2, 14>(win_bits, threads) : shape_t<longlong2, 14>(win_bits, threads); return true;
         default: return false;
     }
 }
@@ -464,9 +537,8 @@ bool hea_shape(int N, bool fp32, int *win_bits, int *threads) {
 cudaError_t launch_hea_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, const void *slots, void *states,
                              bool fp32, double err_scale, double *tr, double *kappa, double *err, cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
-    return fp32 ? launch_t<float2>(d, pairs, npairs, (const float2 *)slots, (float2 *)states, err_scale, tr, kappa, err, st)
-                : launch_t<double2>(d, pairs, npairs, (const double2 *)slots, (double2 *)states, err_scale, tr, kappa,
-                                    err, st);
+    return fp32 ? launch_t<float2, float2>(d, pairs, npairs, slots, states, err_scale, tr, kappa, err, st)
+                : launch_t<double2, longlong2>(d, pairs, npairs, slots, states, err_scale, tr, kappa, err, st);
 }
 
 }  // namespace fpk
