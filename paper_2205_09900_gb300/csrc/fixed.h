@@ -34,16 +34,33 @@ __device__ __forceinline__ int4 fix_coef(longlong2 q) {
 __device__ __forceinline__ longlong2 fix_join(int4 t) {
     return make_longlong2(((long long)t.x << 31) + t.y, ((long long)t.z << 31) + t.w);
 }
+// a double of magnitude at most 1 as such a coefficient's integer (no FP64 instruction)
+__device__ __forceinline__ long long fix_unit(double t) {
+    const long long b = __double_as_longlong(t);
+    const int ex = (int)(b >> 52) & 0x7FF, sh = ex - (1023 + 52 - kFixCoef);   // sh <= 9
+    const long long man = (b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll;
+    const long long q = ex == 0 ? 0 : sh >= 0 ? man << sh : sh > -54 ? (man + (1ll << (-sh - 1))) >> -sh : 0;
+    return b < 0 ? -q : q;
+}
+// sum of products v t of split amplitudes v = (2^31 a.x + a.y) + i (2^31 b.x + b.y)
+struct FixSum {
+    long long hr = 0, mr = 0, hi = 0, mi = 0;
+    __device__ __forceinline__ void add(int2 a, int2 b, int4 t) {
+        hr += (long long)a.x * t.x - (long long)b.x * t.z;
+        mr += (long long)a.x * t.y + (long long)a.y * t.x - (long long)b.x * t.w - (long long)b.y * t.z;
+        hi += (long long)a.x * t.z + (long long)b.x * t.x;
+        mi += (long long)a.x * t.w + (long long)a.y * t.z + (long long)b.x * t.y + (long long)b.y * t.x;
+    }
+    __device__ __forceinline__ longlong2 value() const {
+        constexpr int s = 62 - kFixCoef;
+        return make_longlong2((hr << s) + ((mr + (1ll << (30 - s))) >> (31 - s)),
+                              (hi << s) + ((mi + (1ll << (30 - s))) >> (31 - s)));
+    }
+};
 __device__ __forceinline__ longlong2 cmul(longlong2 v, int4 t) {
-    const int2 a = fix_split(v.x), b = fix_split(v.y);
-    const int nh = -b.x, nl = -b.y;
-    const long long hr = (long long)a.x * t.x + (long long)nh * t.z;
-    const long long mr = (long long)a.x * t.y + (long long)a.y * t.x + (long long)nh * t.w + (long long)nl * t.z;
-    const long long hi = (long long)a.x * t.z + (long long)b.x * t.x;
-    const long long mi = (long long)a.x * t.w + (long long)a.y * t.z + (long long)b.x * t.y + (long long)b.y * t.x;
-    constexpr int s = 62 - kFixCoef;
-    return make_longlong2((hr << s) + ((mr + (1ll << (30 - s))) >> (31 - s)),
-                          (hi << s) + ((mi + (1ll << (30 - s))) >> (31 - s)));
+    FixSum z;
+    z.add(fix_split(v.x), fix_split(v.y), t);
+    return z.value();
 }
 __device__ __forceinline__ void butterfly(longlong2 &a, longlong2 &b) {
     const longlong2 s = make_longlong2(a.x + b.x, a.y + b.y), d = make_longlong2(a.x - b.x, a.y - b.y);
