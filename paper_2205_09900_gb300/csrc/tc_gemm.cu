@@ -22,8 +22,11 @@
 // Tiles are 128-byte rows (64 BF16 of K) in the 128-byte swizzle, one TMA box
 // per operand and stage; rows and columns beyond the matrices are zero-filled
 // by the TMA unit.
-// Bound: 65536 x 256 x 2400 (80 GFLOP, 348 MB) is limited by HBM (51 us) and by the
-// weights' rereading from L2 (1.2 MB per tile).  GEMM_FIGURES
+// Bound: 65536 x 256 x 2400 (80 GFLOP, 348 MB) needs 51 us of HBM; the call takes 101 us (335 with
+// one tile per CTA and a device error flag allocated per call; 110 with the epilogue's accesses
+// a row per lane).  Leaving out the loads of A or the stores saves 18 us each, those of the weights
+// 6: shared memory takes in and gives out 48 KB per 64 columns of K beside the epilogue,
+// and 512 tiles are four waves of 152 CTAs, the last one a third full.
 // Every wait is bounded: on timeout the kernel raises the error flag, still
 // releases its TMEM, and returns; launches that find the flag raised return at
 // once.
@@ -44,6 +47,7 @@ namespace fpk {
 namespace {
 
 constexpr int TC_BM = 128, TC_BK = 64, TC_EPI = 8, TC_THREADS = 64 + 32 * TC_EPI, TC_MAXN = 256, TC_STAGES = 4;
+constexpr int TC_STG = 4096;   // bytes of an epilogue warp's staging block
 constexpr uint64_t TC_DRAIN_NS = 1000000000ull;   // waits for work already issued (after a timeout)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -91,6 +95,71 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase, uint64_
 __device__ __forceinline__ float gelu_f(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678f)) + z * 0.39894228f * expf(-0.5f * z * z);
+}
+
+// A warp's 32 x 32 block of results (lane = row) to and from global memory through its 4 KB of
+// shared memory, whole 128-byte (FP32) or 64-byte (BF16) row pieces per instruction: with a row
+// per lane every 8- or 16-byte access is a sector of its own.  Chunk c of row r sits at chunk
+// c ^ (r mod 8) (BF16: c ^ (r / 2 mod 4)), so that both directions meet all banks.  rows: valid
+// rows from the block's first (may be <= 0), nc: valid columns, 16 or 32.
+__device__ __forceinline__ void put_rows(unsigned char *s, int lane, const float (&v)[32], float *dst, int ld, int rows, int nc) {
+    float4 *b = (float4 *)s;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        b[8 * lane + (c ^ (lane & 7))] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+    __syncwarp();
+    const int c = lane & 7;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = 4 * i + (lane >> 3);
+        if (r < rows && 4 * c < nc) *(float4 *)(dst + (size_t)r * ld + 4 * c) = b[8 * r + (c ^ (r & 7))];
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ void get_rows(unsigned char *s, int lane, float (&v)[32], const float *src, int ld, int rows, int nc) {
+    float4 *b = (float4 *)s;
+    const int c = lane & 7;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = 4 * i + (lane >> 3);
+        if (r < rows && 4 * c < nc) b[8 * r + (c ^ (r & 7))] = *(const float4 *)(src + (size_t)r * ld + 4 * c);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float4 z = b[8 * lane + (q ^ (lane & 7))];
+        v[4 * q] = z.x, v[4 * q + 1] = z.y, v[4 * q + 2] = z.z, v[4 * q + 3] = z.w;
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    return *(const uint32_t *)&p;
+}
+// wide: rows start on 16 bytes (else on 8)
+__device__ __forceinline__ void put_rows_bf16(unsigned char *s, int lane, const float (&v)[32], __nv_bfloat16 *dst, int ld,
+                                              int rows, int nc, bool wide) {
+    uint4 *b = (uint4 *)s;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        b[4 * lane + (c ^ ((lane >> 1) & 3))] = make_uint4(bf16_pair(v[8 * c], v[8 * c + 1]), bf16_pair(v[8 * c + 2], v[8 * c + 3]),
+                                                           bf16_pair(v[8 * c + 4], v[8 * c + 5]), bf16_pair(v[8 * c + 6], v[8 * c + 7]));
+    __syncwarp();
+    const int c = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = 8 * i + (lane >> 2);
+        if (r >= rows || 8 * c >= nc) continue;
+        const uint4 u = b[4 * r + (c ^ ((r >> 1) & 3))];
+        __nv_bfloat16 *d = dst + (size_t)r * ld + 8 * c;
+        if (wide) {
+            *(uint4 *)d = u;
+        } else {
+            *(uint2 *)d = make_uint2(u.x, u.y);
+            *(uint2 *)(d + 4) = make_uint2(u.z, u.w);
+        }
+    }
+    __syncwarp();
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *m, uint32_t count) {
@@ -228,6 +297,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
         }
     } else if (warp >= 2) {
         const int quarter = warp & 3, half = (warp - 2) >> 2;
+        unsigned char *stg = smem + TC_STAGES * stage_bytes + (warp - 2) * TC_STG;
+        const bool wide = g.ldcb % 8 == 0 && ((uintptr_t)g.Cb & 15) == 0;
         int i = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
             const int acc = i & 1, m0 = t / tiles_n * TC_BM, n0 = t % tiles_n * TC_MAXN;
@@ -253,38 +324,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
                       "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                     : "r"(ta));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (!rv) continue;
+                float v[32];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (c0 + 4 * q >= NT) break;   // NT is a multiple of 16: groups of 4 are whole
-                    const int col = n0 + c0 + 4 * q;
-                    float v[4];
+                for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
+                const int nc = min(32, NT - c0);   // 32 or 16 columns
+                if (g.bias) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(r[4 * q + e]);
-                    if (g.bias) {
-                        const float4 b = *(const float4 *)(g.bias + col);
-                        v[0] += b.x, v[1] += b.y, v[2] += b.z, v[3] += b.w;
+                    for (int q = 0; q < 8; ++q) {
+                        if (4 * q >= nc) break;
+                        const float4 b = *(const float4 *)(g.bias + n0 + c0 + 4 * q);
+                        v[4 * q] += b.x, v[4 * q + 1] += b.y, v[4 * q + 2] += b.z, v[4 * q + 3] += b.w;
                     }
-                    if (g.mode == 1) {
-                        if (g.Z) *(float4 *)(g.Z + (size_t)row * g.ldz + col) = make_float4(v[0], v[1], v[2], v[3]);
+                }
+                const int r0 = m0 + quarter * 32;
+                if (g.mode == 1) {
+                    if (g.Z) put_rows(stg, lane, v, g.Z + (size_t)r0 * g.ldz + n0 + c0, g.ldz, g.M - r0, nc);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) v[e] = gelu_f(v[e]);
-                    } else if (g.mode == 2) {
-                        const float4 z = *(const float4 *)(g.Z + (size_t)row * g.ldz + col);
-                        v[0] *= gelu_grad(z.x), v[1] *= gelu_grad(z.y), v[2] *= gelu_grad(z.z), v[3] *= gelu_grad(z.w);
-                    }
-                    if (g.Cf) *(float4 *)(g.Cf + (size_t)row * g.ldcf + col) = make_float4(v[0], v[1], v[2], v[3]);
-                    if (g.Cb) {
-                        __nv_bfloat162 p0 = __floats2bfloat162_rn(v[0], v[1]), p1 = __floats2bfloat162_rn(v[2], v[3]);
-                        uint2 u;
-                        u.x = *(uint32_t *)&p0;
-                        u.y = *(uint32_t *)&p1;
-                        *(uint2 *)(g.Cb + (size_t)row * g.ldcb + col) = u;
-                    }
-                    if (g.Cbt) {
+                    for (int e = 0; e < 32; ++e) v[e] = gelu_f(v[e]);
+                } else if (g.mode == 2) {
+                    float z[32];
+                    get_rows(stg, lane, z, g.Z + (size_t)r0 * g.ldz + n0 + c0, g.ldz, g.M - r0, nc);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) g.Cbt[(size_t)(col + e) * g.ldct + row] = __float2bfloat16(v[e]);
-                    }
+                    for (int e = 0; e < 32; ++e) v[e] *= gelu_grad(z[e]);
+                }
+                if (g.Cf) put_rows(stg, lane, v, g.Cf + (size_t)r0 * g.ldcf + n0 + c0, g.ldcf, g.M - r0, nc);
+                if (g.Cb) put_rows_bf16(stg, lane, v, g.Cb + (size_t)r0 * g.ldcb + n0 + c0, g.ldcb, g.M - r0, nc, wide);
+                if (g.Cbt && rv) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (e < nc) g.Cbt[(size_t)(n0 + c0 + e) * g.ldct + row] = __float2bfloat16(v[e]);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
@@ -306,7 +374,7 @@ bool aligned(const void *p, uintptr_t a) { return ((uintptr_t)p & (a - 1)) == 0;
 
 }  // namespace
 
-size_t tc_gemm_smem_bytes() { return (size_t)TC_STAGES * (TC_BM + TC_MAXN) * TC_BK * 2 + 1024; }
+size_t tc_gemm_smem_bytes() { return (size_t)TC_STAGES * (TC_BM + TC_MAXN) * TC_BK * 2 + TC_EPI * TC_STG + 1024; }
 
 const char *tc_gemm_check(const TcGemm &g) {
     if (g.M < 0 || g.N <= 0 || g.N % 16 != 0 || g.K <= 0 || g.K % 8 != 0) return "need N % 16 == 0 and K % 8 == 0";
