@@ -27,9 +27,9 @@
 // a row per lane).  Leaving out the loads of A or the stores saves 18 us each, those of the weights
 // 6: shared memory takes in and gives out 48 KB per 64 columns of K beside the epilogue,
 // and 512 tiles are four waves of 152 CTAs, the last one a third full.
-// Every wait is bounded: on timeout the kernel raises the error flag, still
-// releases its TMEM, and returns; launches that find the flag raised return at
-// once.
+// Every wait is bounded: on timeout the kernel raises the error flag, waits (bounded)
+// for the loads and MMAs that it has in flight, releases its TMEM, and returns;
+// launches that find the flag raised return at once.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -221,9 +221,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
     const uint32_t taddr = taddr_sh;
     const int nk = (g.K + TC_BK - 1) / TC_BK;
     const uint32_t sbase = smem_u32(smem);
+    int it = 0;   // producer, issuer: stages whose loads, MMAs were issued
     if (tid == 0) {
         // producer: TMA loads of a stage once the MMAs TC_STAGES stages earlier have drained the buffer
-        int it = 0;
         for (int t = blockIdx.x; t < tiles && !abort_sh; t += gridDim.x) {
             const int m0 = t / tiles_n * TC_BM, n0 = t % tiles_n * TC_MAXN;
             for (int kt = 0; kt < nk; ++kt, ++it) {
@@ -240,15 +240,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
                 tma_load(sb, &tmB, kt * TC_BK, n0, fb);
             }
         }
-        // after a timeout: wait (bounded) for the loads still in flight, the last
-        // issued phase of each stage buffer
-        if (abort_sh)
-            for (int i = (it > TC_STAGES ? it - TC_STAGES : 0); i < it; ++i)
-                mbar_wait(smem_u32(&full[i % TC_STAGES]), (uint32_t)(i / TC_STAGES) & 1u, TC_DRAIN_NS);
     } else if (tid == 32) {
         // MMA issuer: four K = 16 steps per stage, then release the buffer
-        bool any = false;
-        int it = 0, i = 0;   // stages and tiles so far
+        int i = 0;   // tiles so far
         for (int t = blockIdx.x; t < tiles && !abort_sh; t += gridDim.x, ++i) {
             const int acc = i & 1, n0 = t % tiles_n * TC_MAXN;
             const uint32_t idesc = make_idesc(TC_BM, min(TC_MAXN, g.N - n0)), td = taddr + (uint32_t)acc * ncols;
@@ -264,7 +258,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
                     abort_sh = 1;
                     break;
                 }
-                any = true;
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
 #pragma unroll
@@ -286,14 +279,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              smem_u32(&tfull[acc]))
                          : "memory");
-        }
-        // after a timeout: one more commit covers every MMA issued, so that none is in
-        // flight when the tensor memory is released
-        if (abort_sh && any) {
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&done))
-                         : "memory");
-            mbar_wait(smem_u32(&done), 0u, TC_DRAIN_NS);
         }
     } else if (warp >= 2) {
         const int quarter = warp & 3, half = (warp - 2) >> 2;
@@ -363,7 +348,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(TcGemm g, const 
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (abort_sh && tid == 0 && g.err) atomicExch_system(g.err, 1);
+    // No role runs any more, so every thread reads the same abort_sh here.  Whichever role gave up,
+    // the others may have issued all they had to before they could see it (the epilogue waits for
+    // a whole tile, the issuer for a stage at a time), so the drain comes after the barrier: the
+    // loads of the last phase of each stage buffer, and one more commit, which covers every MMA,
+    // so that nothing is in flight when the tensor memory is released and the CTA ends.
+    if (abort_sh) {
+        if (tid == 0) {
+            for (int i = (it > TC_STAGES ? it - TC_STAGES : 0); i < it; ++i)
+                mbar_wait(smem_u32(&full[i % TC_STAGES]), (uint32_t)(i / TC_STAGES) & 1u, TC_DRAIN_NS);
+            if (g.err) atomicExch_system(g.err, 1);
+        } else if (tid == 32 && it > 0) {
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             smem_u32(&done))
+                         : "memory");
+            mbar_wait(smem_u32(&done), 0u, TC_DRAIN_NS);
+        }
+        __syncwarp();
+        __syncthreads();
+    }
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(2 * ncols));
