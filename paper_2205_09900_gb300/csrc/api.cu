@@ -1595,7 +1595,7 @@ fp_status fp_bootstrap(fp_ensemble *ens, const double *tr, const int32_t *group,
         if (count) CK(cudaMemcpyAsync(ens->d_boot_group.p, group, count * sizeof(int32_t), cudaMemcpyHostToDevice, ens->st));
         dgroup = ens->d_boot_group.as<int32_t>();
     }
-    CK(ens->d_boot_xs.reserve(bootstrap_scratch(count, ng, k_max)));
+    CK(ens->d_boot_xs.reserve(bootstrap_scratch(count, ng, k_max, n_resamples)));
     const size_t nout = (size_t)ng * k_max * n_resamples;
     CK(ens->d_boot_out.reserve(nout * sizeof(double)));
     {

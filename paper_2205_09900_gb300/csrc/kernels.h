@@ -97,7 +97,7 @@ cudaError_t launch_moments(const double *tr, const int32_t *group, uint64_t coun
 int moments_blocks(uint64_t count);
 // Bootstrap of F^(k): tr [2 count], group [count] on the device; scratch of
 // bootstrap_scratch bytes; out[(g*k_max + k-1)*B + b].  Waits for the group sizes.
-size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max);
+size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max, int B);
 cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t count, int n_groups, int k_max, int B,
                              uint64_t seed, void *scratch, double *out, cudaStream_t st);
 // Brickwork fast path: maps (from the raw gates; raw == nullptr: they are in place), then either the shared-memory sweep (tile_bits == 0)

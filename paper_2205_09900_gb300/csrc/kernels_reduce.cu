@@ -9,7 +9,9 @@
 // block partials by one thread in block order with Neumaier compensation.
 // The bootstrap (paper: Supplementary, "Bootstrapping for uncertainty
 // quantification") resamples each group's stored |Tr|^2 with replacement and
-// evaluates F^(k) on every resample, one CTA per (resample, group).
+// evaluates F^(k) on every resample: draws counted per member and summed in fixed
+// point, a few resamples of a group per CTA (bootstrap_count_kernel); the resamples and
+// powers that need it draw by draw in FP64 (bootstrap_kernel).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -114,11 +116,12 @@ __global__ void __launch_bounds__(GT) group_count_kernel(const int32_t *__restri
 
 // off[g] = first member of group g, off[n_groups] = all members; xoff: the same over the
 // groups of at most max_n members (the ones that are counted in shared memory); cnt: from
-// counts to the chunk's first position in its group; exp2 cleared
+// counts to the chunk's first position in its group; exp2 and the list `redo` cleared
 constexpr int kNoScale = 1 << 20;
 __global__ void __launch_bounds__(1024) group_offsets_kernel(uint32_t *__restrict__ cnt, int nchunks, int n_groups,
                                                              uint32_t max_n, uint64_t *__restrict__ off,
-                                                             uint64_t *__restrict__ xoff, int *__restrict__ exp2) {
+                                                             uint64_t *__restrict__ xoff, int *__restrict__ exp2,
+                                                             unsigned long long *__restrict__ redo) {
     const int lane = threadIdx.x & 31;
     for (int g = threadIdx.x >> 5; g < n_groups; g += 32) {   // a warp per group
         uint64_t s = 0;
@@ -136,6 +139,7 @@ __global__ void __launch_bounds__(1024) group_offsets_kernel(uint32_t *__restric
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
+    *redo = 0;
     uint64_t s = 0, x = 0;
     off[0] = xoff[0] = 0;
     for (int g = 0; g < n_groups; ++g) {
@@ -180,7 +184,7 @@ __global__ void __launch_bounds__(GT) group_place_kernel(const double *__restric
     if ((threadIdx.x & 31) == 0 && e > -kNoScale) atomicMax(&exp2[blockIdx.y], e);
 }
 
-// The powers of every member in fixed point: limbs (low first) of floor(x^k 2^(96 - k e))
+// The powers of every member in fixed point: limbs (low first) of x^k 2^(96 - k e), rounded,
 // for group scale e, at xf[((k - 1) n + j) 3], j over the members of the groups of xoff.
 // x^k is the product of doubles that the FP64 sums use.
 __global__ void powers_kernel(const double *__restrict__ xs, const uint64_t *__restrict__ off,
@@ -208,7 +212,7 @@ __global__ void powers_kernel(const double *__restrict__ xs, const uint64_t *__r
                 const uint64_t lo = sh < 64 ? m << sh : 0, hi = sh ? m >> (64 - sh) : 0;
                 l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32), l2 = (uint32_t)hi;
             } else if (sh > -64) {
-                const uint64_t lo = m >> -sh;
+                const uint64_t lo = (m + (1ull << (-sh - 1))) >> -sh;
                 l0 = (uint32_t)lo, l1 = (uint32_t)(lo >> 32);
             }
         }
@@ -220,22 +224,35 @@ __global__ void powers_kernel(const double *__restrict__ xs, const uint64_t *__r
 // RB resamples of one group per CTA.  A resample's draws are counted per member in
 // shared memory (bytes: a count above 255 in N draws of N members has probability
 // below 1/256! for N > 255 and cannot occur for fewer), then F^(k) = sum of count x^k / N
-// is summed exactly in fixed point: one 32 x 32 -> 64 multiply-add per limb where the
+// is summed in fixed point: one 32 x 32 -> 64 multiply-add per limb where the
 // FP64 pipe, 77 times slower, took a multiplication and an addition per draw and k
 // (the whole call, 300 resamples of 200,000 traces, 9 groups, k <= 4: 0.44 ms against
-// 2.06 ms with FP64 sums and host-built group lists).
+// 2.06 ms with FP64 sums and host-built group lists).  The sums of the integers are exact;
+// each term is rounded at half a unit, 2^-97 of the power of the group's largest member.  A
+// sum of N terms below N 2^53 units (a resample that missed members far above the rest) would
+// hold less than a double: that resample and k goes to bootstrap_kernel, so that every
+// F^(k) is within 2^-54 of the sum of its terms.
 // Bound: the Philox rounds.
 constexpr int CT = 512, RB = 4;
+static_assert(FP_MAX_KMAX <= 8, "a bit per power in an entry of the list");
+// list of bootstrap_kernel's work: redo[0] entries, entry (g B + b) << 8 | bit per k
+__device__ __forceinline__ void redo_add(unsigned long long *redo, uint64_t gb, uint32_t ks) {
+    redo[1 + atomicAdd(redo, 1ull)] = gb << 8 | ks;
+}
 __global__ void __launch_bounds__(CT) bootstrap_count_kernel(const uint32_t *__restrict__ xf,
                                                              const uint64_t *__restrict__ off,
                                                              const uint64_t *__restrict__ xoff, int n_groups, int k_max,
                                                              int B, uint64_t seed, const int *__restrict__ exp2,
-                                                             uint32_t max_n, double *__restrict__ out) {
+                                                             uint32_t max_n, unsigned long long *__restrict__ redo,
+                                                             double *__restrict__ out) {
     extern __shared__ uint32_t cnt[];   // [words][RB]: word w holds the counts of members 4w .. 4w+3
     __shared__ uint64_t red[CT / 32][RB][3];
     const int g = blockIdx.y, b0 = blockIdx.x * RB;
     const uint64_t N = off[g + 1] - off[g], o = xoff[g], n = xoff[n_groups];
-    if (N == 0 || N > max_n || exp2[g] >= kNoScale) return;   // bootstrap_kernel takes these
+    if (N == 0 || N > max_n || exp2[g] >= kNoScale) {   // bootstrap_kernel takes these
+        if (threadIdx.x < RB && b0 + (int)threadIdx.x < B) redo_add(redo, (uint64_t)g * B + b0 + threadIdx.x, 0xff);
+        return;
+    }
     const uint32_t words = (uint32_t)((N + 3) / 4);
     for (uint32_t i = threadIdx.x; i < words * RB; i += CT) cnt[i] = 0;
     __syncthreads();
@@ -253,6 +270,7 @@ __global__ void __launch_bounds__(CT) bootstrap_count_kernel(const uint32_t *__r
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t again = 0;   // threads below RB: the powers whose sum kept too few bits
     for (int k = 0; k < k_max; ++k) {
         uint64_t s[RB][3];
 #pragma unroll
@@ -294,59 +312,67 @@ __global__ void __launch_bounds__(CT) bootstrap_count_kernel(const uint32_t *__r
             const double v = ((double)hi * 0x1.0p64 + (double)lo) / (double)N;
             out[((size_t)g * k_max + k) * B + b0 + threadIdx.x] =
                 exp2[g] > -kNoScale ? ldexp(v, (k + 1) * exp2[g] - 96) : 0.0;
+            if (exp2[g] > -kNoScale && v < 0x1.0p53) again |= 1u << k;
         }
         __syncthreads();
     }
+    if (again) redo_add(redo, (uint64_t)g * B + b0 + threadIdx.x, again);
 }
 
-// The groups the counts do not take (empty, too large for shared memory, powers that
-// are not finite), in FP64.  Block (b, g): resample b of group g.  Draw i takes position
-// ((x >> 32) N_g) >> 32 of the group, x = word i % 4 of Philox block
+// In FP64, draw by draw: the groups that the counts do not take (empty, too large for
+// shared memory, powers that are not finite) and the sums that they could not hold; redo ==
+// nullptr: every resample of every group.  Entry (g, b): resample b of group g.  Draw i takes
+// position ((x >> 32) N_g) >> 32 of the group, x = word i % 4 of Philox block
 // {b, i / 4, g, 5} (key {seed, 0}); F^(k) of the resample = mean of a^k over
-// the draws.  Fixed thread-to-draw mapping and tree: deterministic.
+// the draws.  Fixed thread-to-draw mapping and tree: deterministic, whatever the list's order.
 constexpr int BT = 256;
 __global__ void __launch_bounds__(BT) bootstrap_kernel(const double *__restrict__ xs,
-                                                       const uint64_t *__restrict__ goff, int k_max, int B,
-                                                       uint64_t seed, const int *__restrict__ exp2, uint32_t max_n,
+                                                       const uint64_t *__restrict__ goff, int n_groups, int k_max, int B,
+                                                       uint64_t seed, const unsigned long long *__restrict__ redo,
                                                        double *__restrict__ out) {
     __shared__ double sh[FP_MAX_KMAX][BT / 32];
-    const int b = blockIdx.x, g = blockIdx.y;
-    const uint64_t off = goff[g], N = goff[g + 1] - off;
-    if (N > 0 && N <= max_n && exp2[g] < kNoScale) return;   // bootstrap_count_kernel's
-    double s[FP_MAX_KMAX];
+    const uint64_t entries = redo ? redo[0] : (uint64_t)n_groups * B;
+    for (uint64_t e = blockIdx.x; e < entries; e += gridDim.x) {
+        const uint64_t gb = redo ? redo[1 + e] >> 8 : e;
+        const uint32_t ks = redo ? (uint32_t)redo[1 + e] & 0xffu : 0xffu;
+        const int g = (int)(gb / (uint64_t)B), b = (int)(gb - (uint64_t)g * B);
+        const uint64_t off = goff[g], N = goff[g + 1] - off;
+        double s[FP_MAX_KMAX];
 #pragma unroll
-    for (int k = 0; k < FP_MAX_KMAX; ++k) s[k] = 0.0;
-    const uint64_t nq = (N + 3) / 4;
-    for (uint64_t q = threadIdx.x; q < nq; q += BT) {
-        const U64x4 x = philox(seed, (uint64_t)b, q, (uint64_t)g, 5);
+        for (int k = 0; k < FP_MAX_KMAX; ++k) s[k] = 0.0;
+        const uint64_t nq = (N + 3) / 4;
+        for (uint64_t q = threadIdx.x; q < nq; q += BT) {
+            const U64x4 x = philox(seed, (uint64_t)b, q, (uint64_t)g, 5);
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            if (4 * q + w >= N) break;
-            const uint64_t pos = ((x.x[w] >> 32) * N) >> 32;
-            const double a2 = xs[off + pos];
-            double p = 1.0;
+            for (int w = 0; w < 4; ++w) {
+                if (4 * q + w >= N) break;
+                const uint64_t pos = ((x.x[w] >> 32) * N) >> 32;
+                const double a2 = xs[off + pos];
+                double p = 1.0;
 #pragma unroll
-            for (int k = 0; k < FP_MAX_KMAX; ++k) {
-                if (k < k_max) {
-                    p *= a2;
-                    s[k] += p;
+                for (int k = 0; k < FP_MAX_KMAX; ++k) {
+                    if (k < k_max) {
+                        p *= a2;
+                        s[k] += p;
+                    }
                 }
             }
         }
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < FP_MAX_KMAX; ++k) {
-        double v = s[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[k][wid] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < k_max) {
-        const int k = threadIdx.x;
-        double v = 0;
-        for (int w = 0; w < BT / 32; ++w) v += sh[k][w];
-        out[((size_t)g * k_max + k) * B + b] = N ? v / (double)N : __longlong_as_double(0x7ff8000000000000LL);
+        for (int k = 0; k < FP_MAX_KMAX; ++k) {
+            double v = s[k];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) sh[k][wid] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < k_max && (ks >> threadIdx.x & 1)) {
+            const int k = threadIdx.x;
+            double v = 0;
+            for (int w = 0; w < BT / 32; ++w) v += sh[k][w];
+            out[((size_t)g * k_max + k) * B + b] = N ? v / (double)N : __longlong_as_double(0x7ff8000000000000LL);
+        }
+        __syncthreads();
     }
 }
 
@@ -363,9 +389,10 @@ uint64_t chunk_pairs(uint64_t count) { return ((count + 4095) / 4096 + kChunk - 
 int chunks(uint64_t count) { return count ? (int)((count + chunk_pairs(count) - 1) / chunk_pairs(count)) : 0; }
 }  // namespace
 
-size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max) {
+size_t bootstrap_scratch(uint64_t count, int n_groups, int k_max, int B) {
     return up16((size_t)count * 8) + up16((size_t)(2 * n_groups + 2) * 8) + up16((size_t)n_groups * 4) +
-           up16((size_t)n_groups * chunks(count) * 4) + (size_t)counted_members(count, n_groups) * k_max * 12;
+           up16((size_t)n_groups * chunks(count) * 4) + up16((size_t)counted_members(count, n_groups) * k_max * 12) +
+           ((size_t)n_groups * B + 1) * 8;
 }
 
 cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t count, int n_groups, int k_max, int B,
@@ -379,7 +406,10 @@ cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t co
     at += up16((size_t)n_groups * 4);
     uint32_t *cnt = (uint32_t *)at;
     const int nc = chunks(count);
-    uint32_t *xf = (uint32_t *)(at + up16((size_t)n_groups * nc * 4));
+    at += up16((size_t)n_groups * nc * 4);
+    const uint64_t nx = counted_members(count, n_groups);
+    uint32_t *xf = (uint32_t *)at;
+    unsigned long long *redo = (unsigned long long *)(at + up16((size_t)nx * k_max * 12));
     cudaError_t e;
     const dim3 cg((unsigned)nc, (unsigned)n_groups);
     if (n_groups > 65535) return cudaErrorInvalidValue;
@@ -387,13 +417,12 @@ cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t co
         group_count_kernel<<<cg, GT, 0, st>>>(group, count, chunk_pairs(count), cnt);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    group_offsets_kernel<<<1, 1024, 0, st>>>(cnt, nc, n_groups, kMaxCounted, off, xoff, exp2);
+    group_offsets_kernel<<<1, 1024, 0, st>>>(cnt, nc, n_groups, kMaxCounted, off, xoff, exp2, redo);
     if (nc > 0) group_place_kernel<<<cg, GT, 0, st>>>(tr, group, count, chunk_pairs(count), off, cnt, k_max, xs, exp2);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const uint64_t nx = counted_members(count, n_groups);
+    uint64_t largest = 0;   // of the groups that are counted
     if (nx > 0) {
         // the largest counted group's size sets the shared memory (two CTAs per SM up to 25,600 members)
-        uint64_t largest = 0;
         std::vector<uint64_t> h((size_t)n_groups + 1);
         if ((e = cudaMemcpyAsync(h.data(), off, h.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
         powers_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(xs, off, xoff, n_groups, k_max, exp2, xf);
@@ -405,9 +434,10 @@ cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t co
             return e;
         if (largest > 0)
             bootstrap_count_kernel<<<dim3((unsigned)((B + RB - 1) / RB), (unsigned)n_groups), CT, smem, st>>>(
-                xf, off, xoff, n_groups, k_max, B, seed, exp2, kMaxCounted, out);
+                xf, off, xoff, n_groups, k_max, B, seed, exp2, kMaxCounted, redo, out);
     }
-    bootstrap_kernel<<<dim3((unsigned)B, (unsigned)n_groups), BT, 0, st>>>(xs, off, k_max, B, seed, exp2, kMaxCounted, out);
+    const unsigned fgrid = (unsigned)std::min<uint64_t>((uint64_t)B * n_groups, 152 * 8);
+    bootstrap_kernel<<<fgrid, BT, 0, st>>>(xs, off, n_groups, k_max, B, seed, largest > 0 ? redo : nullptr, out);
     return cudaGetLastError();
 }
 
