@@ -17,6 +17,24 @@ struct SampleParams {
     int32_t self_pair;
 };
 
+// Let a kernel's launches take up to `most` bytes of dynamic shared memory.  The limit belongs to
+// the function, not to a call: `most` is the same for every call of a kernel, so that no host
+// thread lowers it between another's call and its launch.
+template <typename... A>
+inline cudaError_t allow_smem(void (*kernel)(A...), size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+// up to all that its static arrays leave of an SM's
+template <typename... A>
+inline cudaError_t allow_all_smem(void (*kernel)(A...)) {
+    cudaFuncAttributes fa;
+    int dev = 0, all = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e == cudaSuccess ? allow_smem(kernel, (size_t)all - fa.sharedSizeBytes) : e;
+}
+
 // Sampler: raw gates of U and V for every pair of the batch (FP64).
 cudaError_t launch_sample(const SampleParams &sp, const PairInfo *pairs, int npairs, int max_raw,
                           double2 *raw, cudaStream_t st);

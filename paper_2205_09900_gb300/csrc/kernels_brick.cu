@@ -780,7 +780,7 @@ cudaError_t run_passes(const BrickDev &d, const BrickPass *hpasses, const BrickD
     int maxg = 0;
     for (int i = 0; i < d.n_passes[0] + d.n_passes[1]; ++i) maxg = hpasses[i].n_gates > maxg ? hpasses[i].n_gates : maxg;
     const size_t smem = (((size_t)1 << K) + (size_t)maxg * MapSlot<C>::width) * sizeof(C);
-    cudaError_t e = cudaFuncSetAttribute(brick_pass_kernel<C, K, R, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_all_smem(brick_pass_kernel<C, K, R, TH>);
     if (e != cudaSuccess) return e;
     for (int side = 0; side < 2; ++side)
         for (int p = 0; p < d.n_passes[side]; ++p) {
@@ -799,7 +799,7 @@ cudaError_t run_passes_db(const BrickDev &d, const BrickPass *hpasses, const Bri
     for (int i = 0; i < d.n_passes[0] + d.n_passes[1]; ++i) maxg = hpasses[i].n_gates > maxg ? hpasses[i].n_gates : maxg;
     const size_t smem = ((size_t)2 * ((size_t)1 << K) + (size_t)maxg * (2 * 16 + MapSlot<C>::width)) * sizeof(C);
     auto kern = brick_pass_db_kernel<C, K, R, TH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -816,6 +816,8 @@ cudaError_t run_passes_db(const BrickDev &d, const BrickPass *hpasses, const Bri
         }
     return cudaSuccess;
 }
+
+constexpr size_t kSmemPair = 200 * 1024;   // a pair's boundary and maps in one CTA
 
 }  // namespace
 
@@ -844,11 +846,11 @@ cudaError_t launch_brick(const BrickDev &d, const BrickPass *hpasses, const Bric
     // Haar and diagonal gates' maps (entries of magnitude at most 1; the HEA's hold Hadamards) in FP64,
     // as far as both sides and the maps fit an SM
     const size_t fix = !fp32 && d.tile_bits == 0 && d.kind == 0 ? brick_fix_bytes(d) : 0;
-    if (fix && fix <= (size_t)200 * 1024) {
+    if (fix && fix <= kSmemPair) {
         const uint32_t items = 2u << (d.N - 2);
         const int gt = (int)std::min<uint32_t>(512, std::max<uint32_t>(32, items));
         const int gpc = gt == 32 ? (int)std::max<size_t>(1, std::min<size_t>(8, (size_t)72 * 1024 / fix)) : 1;
-        if ((e = cudaFuncSetAttribute(brick_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(fix * gpc))) != cudaSuccess) return e;
+        if ((e = allow_smem(brick_fix_kernel, kSmemPair)) != cudaSuccess) return e;
         brick_fix_kernel<<<(npairs + gpc - 1) / gpc, gt * gpc, fix * gpc, st>>>(d, pairs, npairs, (const double2 *)maps, gt,
                                                                                err_scale, tr, kappa, err);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -861,15 +863,15 @@ cudaError_t launch_brick(const BrickDev &d, const BrickPass *hpasses, const Bric
         int gpc = gt == 32 ? 8 : 1;
         // one pair per CTA: its maps go to shared memory too, when they fit
         const size_t map_bytes = (size_t)nm * 16 * (fp32 ? sizeof(float2) : sizeof(double2));
-        const int stage = gt > 32 && smem + map_bytes <= (size_t)200 * 1024 ? 1 : 0;
+        const int stage = gt > 32 && smem + map_bytes <= kSmemPair ? 1 : 0;
         size_t smem_cta = (smem + (stage ? map_bytes : 0)) * gpc;
         int grid = (npairs + gpc - 1) / gpc;
         if (fp32) {
-            if ((e = cudaFuncSetAttribute(brick_smem_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cta)) != cudaSuccess) return e;
+            if ((e = allow_smem(brick_smem_kernel<float2>, kSmemPair)) != cudaSuccess) return e;
             brick_smem_kernel<float2><<<grid, gt * gpc, smem_cta, st>>>(d, pairs, npairs, (const float2 *)maps,
                                                                          (float2 *)states, gt, both, stage, err_scale, tr, kappa, err);
         } else {
-            if ((e = cudaFuncSetAttribute(brick_smem_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cta)) != cudaSuccess) return e;
+            if ((e = allow_smem(brick_smem_kernel<double2>, kSmemPair)) != cudaSuccess) return e;
             brick_smem_kernel<double2><<<grid, gt * gpc, smem_cta, st>>>(d, pairs, npairs, (const double2 *)maps,
                                                                           (double2 *)states, gt, both, stage, err_scale, tr, kappa, err);
         }

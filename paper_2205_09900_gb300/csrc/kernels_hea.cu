@@ -477,7 +477,7 @@ cudaError_t run_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, cons
     using H = Hea<N, R, CLB>;
     auto k = hea_sweep_kernel<C, N, R, CLB>;
     const size_t smem = H::template smem<C>();
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];

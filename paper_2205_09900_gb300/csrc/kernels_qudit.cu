@@ -409,7 +409,7 @@ cudaError_t run_qc(const BrickDev &d, uint64_t seed, const PairInfo *pairs, int 
         // two groups a thread from 512 groups up (q = 3, l = 5), where they still fill 192 threads twice
         const bool big = S / D >= 512;
         auto kern = big ? qudit_smem_kernel<Q, C, true> : qudit_smem_kernel<Q, C, false>;
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(kern, kQuditSmem)) != cudaSuccess) return e;
         const int threads = big ? 192 : std::min(256, ((int)(S / Q) + 31) / 32 * 32);
         kern<<<npairs, threads, smem, st>>>(d, pairs, maps, state, err_scale, tr, kappa, err);
     } else {

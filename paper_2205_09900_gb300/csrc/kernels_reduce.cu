@@ -430,8 +430,7 @@ cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t co
         for (int g = 0; g < n_groups; ++g)
             if (h[g + 1] - h[g] <= kMaxCounted) largest = std::max(largest, h[g + 1] - h[g]);
         const size_t smem = (size_t)((largest + 3) / 4) * 4 * RB;
-        if ((e = cudaFuncSetAttribute(bootstrap_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = allow_smem(bootstrap_count_kernel, kMaxCounted * RB)) != cudaSuccess) return e;
         if (largest > 0)
             bootstrap_count_kernel<<<dim3((unsigned)((B + RB - 1) / RB), (unsigned)n_groups), CT, smem, st>>>(
                 xf, off, xoff, n_groups, k_max, B, seed, exp2, kMaxCounted, redo, out);

@@ -501,9 +501,9 @@ cudaLaunchConfig_t win_config(int npairs, int bits, cudaLaunchAttribute *attr, c
 }
 
 template <typename C, int R, int CL>
-cudaError_t win_prepare(size_t bytes) {
+cudaError_t win_prepare() {
     auto k = spiral_win_kernel<C, R, CL>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(k, kSpiralSmemMax + 2 * kSpiralWinMaxMaps * MapW<C>::w * sizeof(C));   // a CTA's part, two windows' maps
     if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
@@ -514,7 +514,7 @@ int resident_fp64(int bits) {
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = win_config<double2, 4, CL>(1, bits, attr, nullptr);
     int n = 0;
-    if (win_prepare<double2, 4, CL>(cfg.dynamicSmemBytes) != cudaSuccess ||
+    if (win_prepare<double2, 4, CL>() != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, spiral_win_kernel<double2, 4, CL>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -528,7 +528,7 @@ cudaError_t win_t(const PairInfo *pairs, int npairs, const SpiralWin *wins, int 
                   double *err, cudaStream_t st) {
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = win_config<C, R, CL>(npairs, bits, attr, st);
-    cudaError_t e = win_prepare<C, R, CL>(cfg.dynamicSmemBytes);
+    cudaError_t e = win_prepare<C, R, CL>();
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, spiral_win_kernel<C, R, CL>, pairs, wins, nwins, sm, nmaps, bits, first_bit, cut,
                               (const C *)maps, err_scale, tr, kappa, err);
@@ -542,7 +542,7 @@ cudaError_t sweep_t(const PairInfo *pairs, int npairs, const SpiralMap *sm, int 
     const int threads = bits >= 11 ? 512 : (bits >= 9 ? 128 : 32);
     if (bytes <= kSpiralSmemMax) {
         auto k = spiral_sweep_kernel<C, true>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        cudaError_t e = allow_smem(k, kSpiralSmemMax);
         if (e != cudaSuccess) return e;
         k<<<npairs, threads, bytes, st>>>(pairs, sm, nmaps, bits, first_bit, (const C *)maps, nullptr, err_scale, tr,
                                           kappa, err);
