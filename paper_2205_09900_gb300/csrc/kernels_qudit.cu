@@ -96,16 +96,25 @@ __global__ void __launch_bounds__(128) qudit_haar_maps_kernel(BrickDev d, uint64
         for (int c = 0; c < D; ++c) {
             Fx2 v = sm[g][r * RS + c];
             if (c) {
-                shift1_fixed(v, lead(v) - kRoom);
-                for (int pass = 0; pass < 2; ++pass) {
+                auto project = [&](Fx2 u) {
 #pragma unroll 1
                     for (int k = 0; k < c; ++k) {
-                        const Fx2 q = sm[g][r * RS + k], t = dot1_fixed(q, v);
-                        sub1_fixed(v, q, halves(sum(t.x)), halves(sum(t.y)));
+                        const Fx2 q = sm[g][r * RS + k], t = dot1_fixed(q, u);
+                        sub1_fixed(u, q, halves(sum(t.x)), halves(sum(t.y)));
                     }
-                    const int drop = lead(v) - kRoom;
-                    if (pass == 1 || !__any_sync(0xffffffffu, drop >= kRedo<D>)) break;
-                    shift1_fixed(v, drop);   // (a second pass that a gate did not need does no harm)
+                    return u;
+                };
+                shift1_fixed(v, lead(v) - kRoom);
+                v = project(v);
+                // a second time where this gate needs it; the warp's other gates go along and keep
+                // what they had, so that a gate is the same wherever in a batch it is made
+                const int drop = lead(v) - kRoom;
+                const bool again = act && on[g] && drop >= kRedo<D>;
+                if (__any_sync(0xffffffffu, again)) {
+                    Fx2 u = v;
+                    shift1_fixed(u, drop);
+                    u = project(u);
+                    if (again) v = u;
                 }
             }
             shift1_fixed(v, lead(v) - kUnitRoom<D>);
