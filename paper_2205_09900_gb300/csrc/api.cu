@@ -26,6 +26,7 @@
 #include "kernels.h"
 #include "brick.h"
 #include "planner.h"
+#include "tune.h"
 
 using namespace fpk;
 
@@ -815,42 +816,40 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
                                       E->d_maps.p, fp32, E->st));
         else
             CK(launch_sample(sp, E->d_pairs.as<PairInfo>(), (int)nt, n_raw, E->d_raw.as<double2>(), E->st));
-        float best_ms = 1e30f;
-        // FP_PREC_TF32X3: the fastest tensor-core variant when one runs, else the fastest of all
-        float best_tc_ms = 1e30f;
-        Cand best_tc{0, 0, 0, 0};
-        for (const Cand &c : cands) {
-            std::unique_ptr<BrickCache> bc;
-            if (c.K != 99 && c.K > N) continue;   // tiles larger than the boundary
-            fp_status s = make_brick_cache(E, l, fp32, c.K, c.R, c.TH, c.P, bc);
-            if (s != FP_OK) continue;
-            if (bc->extra_per_pair) CK(E->d_states.reserve(nt * (2 * ((size_t)1 << N) * celem + bc->extra_per_pair)));
-            float ms_sum = 0;
-            for (int rep = 0; rep < 2; ++rep) {
-                CK(cudaEventRecord(E->ev0, E->st));
-                int nl = 0;
-                if (launch_brick(bc->hp.dev, bc->hp.passes.data(), bc->dp, E->d_pairs.as<PairInfo>(), (int)nt,
-                                 haar ? nullptr : E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, 0.0, E->d_tr.as<double>(),
-                                 nullptr, nullptr, E->st, &nl) != cudaSuccess) {
-                    cudaGetLastError();   // a variant this device cannot launch: skip it
-                    ms_sum = 1e30f;
-                    break;
-                }
-                CK(cudaEventRecord(E->ev1, E->st));
-                CK(cudaEventSynchronize(E->ev1));
-                float ms = 0;
-                CK(cudaEventElapsedTime(&ms, E->ev0, E->ev1));
-                if (rep == 1) ms_sum += ms;     // first repetition warms caches and code
-                else if (ms > 1.5f * best_ms) { ms_sum = ms; rep = 1; }   // out of the running already
-                if (bc->dp.err_flag) {
-                    fp_status fs = check_flag(E);
-                    if (fs != FP_OK) return fs;
-                }
+        std::unique_ptr<BrickCache> bc;
+        auto run = [&](int i, float &ms) -> int {
+            const Cand &c = cands[(size_t)i];
+            if (c.K != 99 && c.K > N) return 1;   // tiles larger than the boundary
+            const int want[4] = {c.K, c.R, c.TH, c.P};
+            if (!bc || std::memcmp(bc->variant, want, sizeof want) != 0) {
+                if (make_brick_cache(E, l, fp32, c.K, c.R, c.TH, c.P, bc) != FP_OK) return 1;
+                if (bc->extra_per_pair) CK(E->d_states.reserve(nt * (2 * ((size_t)1 << N) * celem + bc->extra_per_pair)));
             }
-            if (ms_sum < best_ms) { best_ms = ms_sum; bestK = c.K; bestR = c.R; bestT = c.TH; bestP = c.P; }
-            if (c.P >= 3 && ms_sum < best_tc_ms) { best_tc_ms = ms_sum; best_tc = c; }
+            CK(cudaEventRecord(E->ev0, E->st));
+            int nl = 0;
+            if (launch_brick(bc->hp.dev, bc->hp.passes.data(), bc->dp, E->d_pairs.as<PairInfo>(), (int)nt,
+                             haar ? nullptr : E->d_raw.as<double2>(), E->d_maps.p, E->d_states.p, fp32, 0.0, E->d_tr.as<double>(),
+                             nullptr, nullptr, E->st, &nl) != cudaSuccess) {
+                cudaGetLastError();   // a variant this device cannot launch: skip it
+                return 1;
+            }
+            CK(cudaEventRecord(E->ev1, E->st));
+            CK(cudaEventSynchronize(E->ev1));
+            CK(cudaEventElapsedTime(&ms, E->ev0, E->ev1));
+            return bc->dp.err_flag ? check_flag(E) : FP_OK;
+        };
+        std::vector<float> ms;
+        const int ts = time_variants((int)cands.size(), ms, run);
+        if (ts < 0) return (fp_status)ts;
+        // FP_PREC_TF32X3: the fastest tensor-core variant when one runs, else the fastest of all
+        float best_ms = kNoTime, best_tc_ms = kNoTime;
+        Cand best_tc{0, 0, 0, 0};
+        for (size_t i = 0; i < cands.size(); ++i) {
+            const Cand &c = cands[i];
+            if (ms[i] < best_ms) { best_ms = ms[i]; bestK = c.K; bestR = c.R; bestT = c.TH; bestP = c.P; }
+            if (c.P >= 3 && ms[i] < best_tc_ms) { best_tc_ms = ms[i]; best_tc = c; }
         }
-        if (prec == FP_PREC_TF32X3 && best_tc_ms < 1e30f) {
+        if (prec == FP_PREC_TF32X3 && best_tc_ms < kNoTime) {
             bestK = best_tc.K; bestR = best_tc.R; bestT = best_tc.TH; bestP = best_tc.P;
         }
         if (cache) {
