@@ -57,7 +57,8 @@
  * returns after its results are in the caller's arrays.
  *
  * Environment.  FP_AUTOTUNE_CACHE names a file in which the brickwork
- * autotuner keeps its choices; FP_SWEEP_CLUSTER (1, 4, 8 or 16) fixes the
+ * autotuner keeps its choices and from which it takes them (not where there is
+ * nothing to choose: the HEA's boundaries up to 14 bits); FP_SWEEP_CLUSTER (1, 4, 8 or 16) fixes the
  * number of CTAs that share one pair on the generic sweep (default: by
  * boundary size); FP_SPIRAL_WIN (0, 4 or 5) fixes the register-window width
  * of the spiral sweep of FP_HEA_PAULI (0: one map per pass; default: by

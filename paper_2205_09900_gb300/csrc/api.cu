@@ -780,6 +780,9 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
             fclose(f);
         }
     }
+    // where one variant alone is in question, the file's word does not count: entries of before
+    // the HEA sweep would keep a boundary on passes some 7 times slower
+    if (have && N > kmin && cands.size() == 1 && bestP != cands[0].P) have = false;
     std::unique_ptr<BrickCache> cached;
     if (have && N > kmin && make_brick_cache(E, l, fp32, bestK, bestR, bestT, bestP, cached) != FP_OK) {
         have = false;   // a cache entry this depth cannot run (another build's file): tune instead
