@@ -99,7 +99,8 @@ typedef enum {
     FP_PREC_FP32 = 1,         /* boundary tensors and gate maps in FP32, FP64 meet
                                  and reduction; the brickwork autotuner takes the
                                  faster of the FFMA tile passes and the TF32 x 3
-                                 tensor-core passes per depth; a pair whose
+                                 tensor-core passes per depth (the latter, less
+                                 accurate, where they gain 2 %); a pair whose
                                  estimated error exceeds fp32_tol, or whose
                                  cancellation ratio exceeds kappa_max, is
                                  recontracted in FP64 */

@@ -670,8 +670,9 @@ int brick_key(int l, int prec) {
     return 4 * l + (prec == FP_PREC_FP64 ? 0 : prec == FP_PREC_TF32X3 ? 2 : 1);
 }
 
-fp_status make_brick_cache(fp_ensemble *E, int l, bool fp32, int K, int R, int TH, int persist,
+fp_status make_brick_cache(fp_ensemble *E, int l, int prec, int K, int R, int TH, int persist,
                            std::unique_ptr<BrickCache> &out) {
+    const bool fp32 = prec != FP_PREC_FP64;
     auto bc = std::make_unique<BrickCache>();
     if (persist == 5) {   // the HEA sweep: its shape follows from the boundary
         K = 99;
@@ -682,9 +683,12 @@ fp_status make_brick_cache(fp_ensemble *E, int l, bool fp32, int K, int R, int T
     // K > N: shared-memory sweep, K == N: one tile
     // arcs hold the 5 (FP32) or 4 (FP64) lowest bits, so that tile loads read contiguous runs;
     // the tensor-core pass (12-bit tiles) holds 3: at l = 10 a 12-bit arc through the 5
-    // lowest bits would need 49 passes instead of 20; from 20 bits up 2 (27 passes at l = 11
-    // instead of 49: a run of 4 amplitudes is one 32-byte sector)
-    const int low = persist >= 3 ? (2 * (l - 1) >= 20 ? 2 : 3) : (fp32 ? 5 : 4);
+    // lowest bits would need 49 passes instead of 20.  FP_PREC_TF32X3 from 20 bits up: 2 (27 passes
+    // at l = 11 instead of 49, a run of 4 amplitudes is one 32-byte sector; 2 % at 22 and 24 bits).
+    // FP_PREC_FP32 keeps 3, with which the FFMA passes are the faster ones at 20 bits (n = 50, 96
+    // pairs: 34.8 ms against 35.7): with 2 the tensor cores would win there (26.6 ms) with 9
+    // times the error (1.1e-5 of a trace against 1.3e-6, their accumulators truncate).
+    const int low = persist >= 3 ? (prec == FP_PREC_TF32X3 && 2 * (l - 1) >= 20 ? 2 : 3) : (fp32 ? 5 : 4);
     bc->hp = make_brick_plan(E->d.n, l, K, low, R, E->d.kind == FP_HEA ? 1 : 0);
     for (const auto &ps : bc->hp.passes) {
         if (ps.n_gates > 255) return fail(FP_ERR_ARG, "tile pass with %d gates exceeds 255", ps.n_gates);
@@ -744,11 +748,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
     // P = 4: tensor-core windows (TF32 x 3 tcgen05 MMAs) with the tile's operand in tensor memory,
     // boundaries of more than two 12-bit tiles.  P = 3 (the operand in shared memory) runs when the
     // cache file asks for it; it was 20-25 % slower at every depth, and planning it took seconds.
-    // At 20 bits FP_PREC_FP32 stays with the FFMA passes, which timed fastest there before the
-    // tensor-core plans held 2 low bits (35 ms per 96 pairs at n = 50, against 26.8 now): they are
-    // 9 times more accurate (1.2e-6 of a trace against 1.1e-5: the tensor cores' accumulators
-    // truncate).  FP_PREC_TF32X3 asks for the tensor cores.
-    if (fp32 && N >= kTcTile + 2 && (N != 20 || prec == FP_PREC_TF32X3)) cands.push_back({kTcTile, kMaxWin, 256, 4});
+    if (fp32 && N >= kTcTile + 2) cands.push_back({kTcTile, kMaxWin, 256, 4});
     // P = 5: the HEA's own sweep, the fastest of all wherever it applies (kernels_hea.cu), so
     // there is nothing to time; FP_PREC_TF32X3 keeps to the tensor cores where they apply
     int heaR = 0, heaT = 0;
@@ -784,7 +784,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
     // the HEA sweep would keep a boundary on passes some 7 times slower
     if (have && N > kmin && cands.size() == 1 && bestP != cands[0].P) have = false;
     std::unique_ptr<BrickCache> cached;
-    if (have && N > kmin && make_brick_cache(E, l, fp32, bestK, bestR, bestT, bestP, cached) != FP_OK) {
+    if (have && N > kmin && make_brick_cache(E, l, prec, bestK, bestR, bestT, bestP, cached) != FP_OK) {
         have = false;   // a cache entry this depth cannot run (another build's file): tune instead
         cached.reset();
     }
@@ -825,7 +825,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
             if (c.K != 99 && c.K > N) return 1;   // tiles larger than the boundary
             const int want[4] = {c.K, c.R, c.TH, c.P};
             if (!bc || std::memcmp(bc->variant, want, sizeof want) != 0) {
-                if (make_brick_cache(E, l, fp32, c.K, c.R, c.TH, c.P, bc) != FP_OK) return 1;
+                if (make_brick_cache(E, l, prec, c.K, c.R, c.TH, c.P, bc) != FP_OK) return 1;
                 if (bc->extra_per_pair) CK(E->d_states.reserve(nt * (2 * ((size_t)1 << N) * celem + bc->extra_per_pair)));
             }
             CK(cudaEventRecord(E->ev0, E->st));
@@ -845,10 +845,15 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
         const int ts = time_variants((int)cands.size(), ms, run);
         if (ts < 0) return (fp_status)ts;
         // FP_PREC_TF32X3: the fastest tensor-core variant when one runs, else the fastest of all
+        // The others take the tensor cores where they gain 2 %: their traces have 7 to 11 times the
+        // error, which noise in the timing (half a percent) should not decide.  (n = 50, fastest FFMA
+        // variant over tensor cores in a trial of up to 192 pairs: l = 8 1.04, 9 1.35, 10 1.48,
+        // 11 0.89 to 0.98, 12 1.29, 13 1.21.)
         float best_ms = kNoTime, best_tc_ms = kNoTime;
         Cand best_tc{0, 0, 0, 0};
         for (size_t i = 0; i < cands.size(); ++i) {
             const Cand &c = cands[i];
+            if (c.P >= 3 && prec != FP_PREC_TF32X3) ms[i] *= 1.02f;
             if (ms[i] < best_ms) { best_ms = ms[i]; bestK = c.K; bestR = c.R; bestT = c.TH; bestP = c.P; }
             if (c.P >= 3 && ms[i] < best_tc_ms) { best_tc_ms = ms[i]; best_tc = c; }
         }
@@ -862,7 +867,7 @@ fp_status tune_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t>
     }
     std::unique_ptr<BrickCache> bc = std::move(cached);
     if (!bc) {
-        fp_status s = make_brick_cache(E, l, fp32, bestK, bestR, bestT, bestP, bc);
+        fp_status s = make_brick_cache(E, l, prec, bestK, bestR, bestT, bestP, bc);
         if (s != FP_OK) return s;
     }
     E->brick_plans.emplace(key, std::move(bc));
