@@ -26,6 +26,7 @@
 #include "kernels.h"
 #include "brick.h"
 #include "planner.h"
+#include "side_stream.h"
 #include "tune.h"
 
 using namespace fpk;
@@ -124,11 +125,6 @@ struct SpiralCache {        // one depth of the paper's HEA on the spiral sweep
     int nwins[kFp32 + 1] = {}, base = 0;
     int resident[kFp32] = {};        // FP64 clusters of variant p on the device at a time
     SpiralCut cut[kFp32 + 1];
-};
-
-struct SideStream {   // beside an ensemble's own stream, joined before its call goes on
-    cudaStream_t st = nullptr;
-    cudaEvent_t ev = nullptr;
 };
 
 struct fp_ensemble {
@@ -1190,12 +1186,7 @@ fp_status run_spiral(fp_ensemble *E, uint64_t first, const std::map<int, std::ve
         }
         fp_status s = reserve(jobs.back(), jobs.back().idx->size());
         if (s != FP_OK) return s;
-        while (E->side.size() < std::min(jobs.size(), fp_ensemble::kSideStreams)) {
-            SideStream x;
-            CK(cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking));
-            E->side.push_back(x);
-            CK(cudaEventCreateWithFlags(&E->side.back().ev, cudaEventDisableTiming));
-        }
+        while (E->side.size() < std::min(jobs.size(), fp_ensemble::kSideStreams)) CK(add_side_stream(E->side));
         CK(cudaEventRecord(E->ev0, E->st));
         for (SideStream &x : E->side) CK(cudaStreamWaitEvent(x.st, E->ev0, 0));
         for (size_t k = 0; k < jobs.size() && s == FP_OK; ++k)
