@@ -356,6 +356,16 @@ void step_sides(const HostPlan &h, size_t *left, size_t *right) {
     *right = std::max<size_t>(16, (size_t)1 << b[1]);
 }
 
+// log2 of a block's units in a step of `items` operations and about `total` units: 10, or fewer (down to 6,
+// two warps) until the step has two blocks per SM.  A batch of a few pairs is as fast as the number of
+// SM quarters that share it, in FP64 above all (an instruction per 77 cycles and quarter): 2 pairs of n = 14,
+// T = 70 take 0.93 ms in FP64; 1.55 with 10 throughout, 1.30 on clusters of 16 CTAs.
+int step_log_units(uint64_t items, uint64_t total, int sms) {
+    int lg = 10;
+    while (lg > 6 && items + (total >> lg) < 2 * (uint64_t)sms) --lg;
+    return lg;
+}
+
 // Work lists of a lock-step batch, uploaded; plans: the uploaded DevPlans by pinfo[i].plan.
 template <typename F>
 fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<PairInfo> &pinfo,
@@ -364,11 +374,19 @@ fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<Pai
     size_t n_steps = 0, at = 0, n_items = 0;
     for (uint64_t i = 0; i < nb; ++i) n_steps = std::max(n_steps, (size_t)std::max(plan(i).n_left, plan(i).n_right));
     std::vector<uint32_t> count(n_steps + 1, 0), blocks(n_steps, 0);
+    std::vector<uint64_t> quads(n_steps, 0);   // amplitudes first
     for (uint64_t i = 0; i < nb; ++i)
         for (int s = 0; s < 2; ++s)
-            for (int k = 0; k < (s ? plan(i).n_right : plan(i).n_left); ++k) ++count[k + 1];
+            for (int k = 0; k < (s ? plan(i).n_right : plan(i).n_left); ++k) {
+                ++count[k + 1];
+                const DevOp &op = plan(i).ops[s ? plan(i).n_left + k : k];
+                quads[k] += 1ull << std::max<int>(op.b_in, op.b_out);
+            }
     for (size_t k = 0; k < n_steps; ++k) count[k + 1] += count[k];   // first item of each step
     n_items = count[n_steps];
+    std::vector<uint8_t> log_units(n_steps);
+    for (size_t k = 0; k < n_steps; ++k)
+        log_units[k] = (uint8_t)step_log_units(count[k + 1] - count[k], quads[k] >> 2, E->sms);
     std::vector<uint32_t> fill(count.begin(), count.end() - 1);
     std::vector<StepItem> items(n_items);
     uint32_t meet = 0;
@@ -395,7 +413,7 @@ fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<Pai
                         : flat && op.nc == 4 && op.nn == 0 ? STEP_4_0 : STEP_ANY;
                 it.units = it.form == STEP_IN_PLACE ? 1u << (op.b_out - 2)
                          : it.form == STEP_ANY ? 1u << op.b_out : 1u << (op.b_in - op.nc);
-                it.log_units = it.units >= (1u << 16) ? 12 : 10;
+                it.log_units = it.units >= (1u << 16) ? 12 : log_units[k];
                 it.in = buf[cur];
                 if (it.form != STEP_IN_PLACE) cur ^= 1;
                 it.out = buf[cur];
@@ -531,9 +549,12 @@ fp_status run_generic(fp_ensemble *E, uint64_t first, const std::vector<uint64_t
         return std::make_pair(1, E->sms * 2);
     };
     // local-circuit pairs of 2^14 amplitudes and more go in lock-step (kernels_step.cu), each with
-    // its own boundaries; they are the last ones in the order by size
+    // its own boundaries; they are the last ones in the order by size.  A batch of fewer pairs than SMs with a large
+    // one among them goes in lock-step as a whole: apart, the small ones, a CTA each, take their time before
+    // the large ones (5 pairs of n = 18, T = 60 in FP64: 0.69 ms together, 1.20 apart).
     const bool lockstep = local && !sweep_cluster_forced();
-    auto in_steps = [&](uint64_t i) { return lockstep && hp(i).bits_max >= kStepBits; };
+    const int step_bits = lockstep && count < (uint64_t)E->sms && hp(count - 1).bits_max >= kStepBits ? 0 : kStepBits;
+    auto in_steps = [&](uint64_t i) { return lockstep && hp(i).bits_max >= step_bits; };
     uint64_t done = 0;
     while (done < count) {
         uint64_t nb = 0;
