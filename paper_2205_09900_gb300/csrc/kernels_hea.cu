@@ -410,25 +410,75 @@ __global__ void __launch_bounds__((Hea<N, R, CLB>::kCta), (512 / Hea<N, R, CLB>:
     if (t == 0 && rank == 0 && pw < npairs) write_meet(pairs[pw], s, err_scale, tr, kappa, err);
 }
 
-// Boundaries of 2 and 4 bits: a thread per pair, the whole boundary in registers,
+// Boundaries of 2 and 4 bits in FP64: a lane per amplitude, the Hadamards by shuffles.  An FP64
+// instruction takes an SM quarter about 77 cycles per warp whatever its lanes do, so this takes as many
+// of them per pair as a thread per pair and 2^N times fewer one after another: one pair of n = 50, L = 3
+// 95 us with its call against 669 with a thread per pair (548 as dense maps on a warp).
+template <int N>
+__global__ void __launch_bounds__(128) hea_lane_kernel(int n, int cut, const PairInfo *__restrict__ pairs, int npairs,
+                                                       const double2 *__restrict__ slots, double err_scale,
+                                                       double *__restrict__ tr, double *__restrict__ kappa,
+                                                       double *__restrict__ err) {
+    constexpr int V = 1 << N;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x, pw = id / V, i = id % V;
+    const int p = pw < npairs ? pw : npairs - 1;   // spare lanes repeat the last pair and write nothing
+    const double2 *gs = slots + (size_t)p * n * N * 4;
+    auto load = [&](int k, double2 (&m)[N]) {
+        const int q = k < cut ? k : n - 1 - (k - cut);
+#pragma unroll
+        for (int s = 0; s < N; ++s) m[s] = gs[((size_t)q * N + s) * 4 + 2 * ((i >> s) & 1) + ((i >> ((s + N - 1) % N)) & 1)];
+    };
+    double2 v = make_double2(1, 0), left = v, next[N];
+    load(0, next);
+    for (int k = 0; k < n; ++k) {
+        double2 m[N];
+#pragma unroll
+        for (int s = 0; s < N; ++s) m[s] = next[s];
+        if (k + 1 < n) load(k + 1, next);   // arrives while this qubit computes
+#pragma unroll
+        for (int s = 0; s < N; ++s) v = cmul(v, m[s]);
+        if (k + 1 < n) {
+#pragma unroll
+            for (int b = 0; b < N; ++b) {
+                const double2 u = make_double2(__shfl_xor_sync(0xffffffffu, v.x, 1 << b), __shfl_xor_sync(0xffffffffu, v.y, 1 << b));
+                const double sign = (i >> b) & 1 ? -1.0 : 1.0;
+                v = make_double2(fma(sign, v.x, u.x), fma(sign, v.y, u.y));   // (exact products)
+            }
+        }
+        if (k == cut - 1) {
+            left = v;
+            v = make_double2(1, 0);
+        }
+    }
+    MeetAcc<double2> acc;
+    acc.add(left, v);
+    double s[4] = {acc.sr, acc.si, acc.sa, acc.s2};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int d = V / 2; d > 0; d >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], d);
+    if (i == 0 && pw < npairs) write_meet(pairs[pw], s, err_scale, tr, kappa, err);
+}
+
+// The same in FP32: a thread per pair, the whole boundary in registers,
 // every slot applied by itself.
-template <typename C, int N>
+template <int N>
 __global__ void __launch_bounds__(128) hea_thread_kernel(int n, int cut, const PairInfo *__restrict__ pairs, int npairs,
-                                                         const C *__restrict__ slots, double err_scale,
+                                                         const float2 *__restrict__ slots, double err_scale,
                                                          double *__restrict__ tr, double *__restrict__ kappa,
                                                          double *__restrict__ err) {
     constexpr int V = 1 << N;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= npairs) return;
-    const C *gs = slots + (size_t)p * n * N * 4;
-    C v[V], left[V];
+    const float2 *gs = slots + (size_t)p * n * N * 4;
+    float2 v[V], left[V];
 #pragma unroll
     for (int i = 0; i < V; ++i) v[i].x = 1, v[i].y = 0;
     for (int k = 0; k < n; ++k) {
         const int q = k < cut ? k : n - 1 - (k - cut);
 #pragma unroll
         for (int s = 0; s < N; ++s) {
-            C m[4];
+            float2 m[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) m[e] = gs[((size_t)q * N + s) * 4 + e];
 #pragma unroll
@@ -450,7 +500,7 @@ __global__ void __launch_bounds__(128) hea_thread_kernel(int n, int cut, const P
             }
         }
     }
-    MeetAcc<C> acc;
+    MeetAcc<float2> acc;
 #pragma unroll
     for (int i = 0; i < V; ++i) {
         acc.add(left[i], v[i]);
@@ -462,10 +512,14 @@ __global__ void __launch_bounds__(128) hea_thread_kernel(int n, int cut, const P
 }
 
 template <typename C, int N>
-cudaError_t run_thread(const BrickDev &d, const PairInfo *pairs, int npairs, const C *slots, double err_scale, double *tr,
-                       double *kappa, double *err, cudaStream_t st) {
-    hea_thread_kernel<C, N><<<(npairs + 127) / 128, 128, 0, st>>>(d.n, d.cut, pairs, npairs, slots, err_scale, tr, kappa,
-                                                                 err);
+cudaError_t run_few_bits(const BrickDev &d, const PairInfo *pairs, int npairs, const C *slots, double err_scale, double *tr,
+                         double *kappa, double *err, cudaStream_t st) {
+    if constexpr (std::is_same<C, double2>::value) {
+        constexpr int per = 128 >> N;   // pairs per CTA
+        hea_lane_kernel<N><<<(npairs + per - 1) / per, 128, 0, st>>>(d.n, d.cut, pairs, npairs, slots, err_scale, tr, kappa, err);
+    } else {
+        hea_thread_kernel<N><<<(npairs + 127) / 128, 128, 0, st>>>(d.n, d.cut, pairs, npairs, slots, err_scale, tr, kappa, err);
+    }
     return cudaGetLastError();
 }
 
@@ -494,7 +548,7 @@ cudaError_t run_sweep(const BrickDev &d, const PairInfo *pairs, int npairs, cons
     return cudaLaunchKernelEx(&cfg, k, d.n, d.cut, pairs, npairs, slots, lscr, err_scale, tr, kappa, err);
 }
 
-// C: FP32, or FP64 in its thread kernels; W: what the wider sweeps compute in
+// C: FP32, or FP64 up to 4 bits; W: what the wider sweeps compute in
 template <typename C, typename W>
 cudaError_t launch_t(const BrickDev &d, const PairInfo *pairs, int npairs, const void *slots, void *lscr, double err_scale,
                      double *tr, double *kappa, double *err, cudaStream_t st) {
@@ -502,8 +556,8 @@ cudaError_t launch_t(const BrickDev &d, const PairInfo *pairs, int npairs, const
     const auto *ws = (const typename HeaNum<W>::Coef *)slots;
     auto *ls = (typename HeaNum<W>::Out *)lscr;
     switch (d.N) {
-        case 2: return run_thread<C, 2>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
-        case 4: return run_thread<C, 4>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
+        case 2: return run_few_bits<C, 2>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
+        case 4: return run_few_bits<C, 4>(d, pairs, npairs, ts, err_scale, tr, kappa, err, st);
         case 6: return run_sweep<W, 6>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
         case 8: return run_sweep<W, 8>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
         case 10: return run_sweep<W, 10>(d, pairs, npairs, ws, ls, err_scale, tr, kappa, err, st);
