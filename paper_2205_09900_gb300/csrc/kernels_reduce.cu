@@ -79,7 +79,7 @@ __global__ void moments_pass2(const double *__restrict__ partials, int nblocks, 
     out[t] = s + c;
 }
 
-// Members of every group in increasing pair order, on the device: counts per chunk of
+// Members of every group in increasing pair order, on the device (up to 16 groups): counts per chunk of
 // pairs, offsets, and xs = |Tr|^2 of the members group by group.  A CTA takes one (chunk,
 // group) and places its members by a scan; the group ids stay in L2 (one CTA per group
 // over all 200,000 pairs took 520 us, a counting sort on the host and its copies as much).
@@ -114,39 +114,88 @@ __global__ void __launch_bounds__(GT) group_count_kernel(const int32_t *__restri
     if (threadIdx.x == 0) cnt[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = all;
 }
 
-// off[g] = first member of group g, off[n_groups] = all members; xoff: the same over the
-// groups of at most max_n members (the ones that are counted in shared memory); cnt: from
-// counts to the chunk's first position in its group; exp2 and the list `redo` cleared
+// cnt, the same with many groups: a pass over the pairs with an atomic each (cleared before)
+__global__ void group_count_many_kernel(const int32_t *__restrict__ group, uint64_t count, uint64_t per, int nchunks,
+                                        int n_groups, uint32_t *__restrict__ cnt) {
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (i >= count) return;
+    const int g = group[i];
+    if (g >= 0 && g < n_groups) atomicAdd(&cnt[(size_t)g * nchunks + i / per], 1u);
+}
+
+// cnt: from counts to each chunk's first position in its group; off[g + 1] = members of group
+// g; exp2 cleared.  A warp per group.
 constexpr int kNoScale = 1 << 20;
-__global__ void __launch_bounds__(1024) group_offsets_kernel(uint32_t *__restrict__ cnt, int nchunks, int n_groups,
-                                                             uint32_t max_n, uint64_t *__restrict__ off,
-                                                             uint64_t *__restrict__ xoff, int *__restrict__ exp2,
-                                                             unsigned long long *__restrict__ redo) {
+__device__ __forceinline__ void group_prefix(uint32_t *__restrict__ cnt, int nchunks, int g, uint64_t *__restrict__ off,
+                                             int *__restrict__ exp2) {
     const int lane = threadIdx.x & 31;
-    for (int g = threadIdx.x >> 5; g < n_groups; g += 32) {   // a warp per group
-        uint64_t s = 0;
-        for (int c = lane; c - lane < nchunks; c += 32) {
-            const uint32_t v = c < nchunks ? cnt[(size_t)g * nchunks + c] : 0;
-            uint32_t x = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (c < nchunks) cnt[(size_t)g * nchunks + c] = (uint32_t)s + x - v;
-            s += __shfl_sync(0xffffffffu, x, 31);
+    uint64_t s = 0;
+    for (int c = lane; c - lane < nchunks; c += 32) {
+        const uint32_t v = c < nchunks ? cnt[(size_t)g * nchunks + c] : 0;
+        uint32_t x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        if (lane == 0) off[g + 1] = s, exp2[g] = -kNoScale;
+        if (c < nchunks) cnt[(size_t)g * nchunks + c] = (uint32_t)s + x - v;
+        s += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) off[g + 1] = s, exp2[g] = -kNoScale;
+}
+__global__ void __launch_bounds__(256) group_prefix_kernel(uint32_t *__restrict__ cnt, int nchunks, int n_groups,
+                                                           uint64_t *__restrict__ off, int *__restrict__ exp2) {
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g < n_groups) group_prefix(cnt, nchunks, g, off, exp2);
+}
+
+// inclusive sums over a CTA of 1024 threads
+__device__ __forceinline__ uint64_t scan_1024(uint64_t v, uint64_t (&sh)[32]) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    *redo = 0;
-    uint64_t s = 0, x = 0;
-    off[0] = xoff[0] = 0;
-    for (int g = 0; g < n_groups; ++g) {
-        const uint64_t n = off[g + 1];
-        off[g + 1] = s += n;
-        xoff[g + 1] = x += n <= max_n ? n : 0;
+    if (lane == 31) sh[wid] = v;
+    __syncthreads();
+    uint64_t before = 0;
+    for (int w = 0; w < wid; ++w) before += sh[w];
+    return v + before;
+}
+
+// off[g] = first member of group g, off[n_groups] = all members; xoff: the same over the
+// groups of at most max_n members (the ones that are counted in shared memory); the list
+// `redo` cleared.  prefix: the groups' prefixes first (a few groups), else they are in place.
+__global__ void __launch_bounds__(1024) group_offsets_kernel(uint32_t *__restrict__ cnt, int nchunks, int n_groups,
+                                                             uint32_t max_n, bool prefix, uint64_t *__restrict__ off,
+                                                             uint64_t *__restrict__ xoff, int *__restrict__ exp2,
+                                                             unsigned long long *__restrict__ redo) {
+    __shared__ uint64_t sh[2][32], base[2];
+    if (prefix) {
+        for (int g = threadIdx.x >> 5; g < n_groups; g += 32) group_prefix(cnt, nchunks, g, off, exp2);
+        __syncthreads();
     }
+    if (threadIdx.x == 0) {
+        *redo = 0;
+        off[0] = xoff[0] = base[0] = base[1] = 0;
+    }
+    __syncthreads();
+    for (int g0 = 0; g0 < n_groups; g0 += 1024) {
+        const int g = g0 + (int)threadIdx.x;
+        const uint64_t n = g < n_groups ? off[g + 1] : 0;
+        const uint64_t s = base[0] + scan_1024(n, sh[0]), x = base[1] + scan_1024(n <= max_n ? n : 0, sh[1]);
+        if (g < n_groups) off[g + 1] = s, xoff[g + 1] = x;
+        __syncthreads();
+        if (threadIdx.x == 1023) base[0] = s, base[1] = x;
+        __syncthreads();
+    }
+}
+
+// scale of |t|^2 = x: e with x < 2^e, kNoScale when x^k_max is not finite
+__device__ __forceinline__ int scale_of(double x, int k_max) {
+    double p = x;
+    for (int k = 1; k < k_max; ++k) p *= x;
+    return isfinite(p) ? (x > 0 ? ilogb(x) + 1 : -kNoScale) : kNoScale;
 }
 
 // xs of the members, and the group's scale: exp2[g] = e with every x < 2^e, or kNoScale
@@ -174,14 +223,82 @@ __global__ void __launch_bounds__(GT) group_place_kernel(const double *__restric
             if (!in[j]) continue;
             const double a = tr[2 * (i + j)], b = tr[2 * (i + j) + 1], x = a * a + b * b;
             xs[at + pos++] = x;
-            double p = x;
-            for (int k = 1; k < k_max; ++k) p *= x;
-            e = max(e, isfinite(p) ? (x > 0 ? ilogb(x) + 1 : -kNoScale) : kNoScale);
+            e = max(e, scale_of(x, k_max));
         }
         at += all;
     }
     e = __reduce_max_sync(0xffffffffu, e);
     if ((threadIdx.x & 31) == 0 && e > -kNoScale) atomicMax(&exp2[blockIdx.y], e);
+}
+
+// The same with many groups: a warp per chunk, 32 pairs at a time, the lanes of one group
+// ranked among themselves (in lane order) and placed from the chunk's running position.  A CTA per
+// (chunk, group) as above would be 200,000 CTAs for 200,000 pairs in 1,000 groups: 10 resamples of
+// them take 272 us this way, 840 that way; at 16 and 17 groups the two take the same.
+__global__ void __launch_bounds__(32) group_place_many_kernel(const double *__restrict__ tr, const int32_t *__restrict__ group,
+                                                              uint64_t count, uint64_t per, int nchunks, int n_groups,
+                                                              const uint64_t *__restrict__ off, uint32_t *__restrict__ cnt,
+                                                              int k_max, double *__restrict__ xs, int *__restrict__ exp2) {
+    const uint64_t lo = blockIdx.x * per, hi = lo + per < count ? lo + per : count;
+    const int lane = threadIdx.x;
+    for (uint64_t i0 = lo; i0 < hi; i0 += 32) {
+        const uint64_t i = i0 + lane;
+        const int id = i < hi ? group[i] : -1, g = id >= 0 && id < n_groups ? id : -1;
+        const uint32_t mine = __match_any_sync(0xffffffffu, g), lead = __ffs(mine) - 1;
+        uint32_t at = 0;
+        if (g >= 0 && lane == (int)lead) at = atomicAdd(&cnt[(size_t)g * nchunks + blockIdx.x], (uint32_t)__popc(mine));
+        at = __shfl_sync(0xffffffffu, at, lead) + __popc(mine & ((1u << lane) - 1u));
+        if (g >= 0) {
+            const double a = tr[2 * i], b = tr[2 * i + 1], x = a * a + b * b;
+            xs[off[g] + at] = x;
+            const int e = scale_of(x, k_max);
+            if (e > exp2[g]) atomicMax(&exp2[g], e);   // (exp2 only grows: a stale read costs an atomic)
+        }
+        __syncwarp();   // the next 32 see these positions
+    }
+}
+
+// All of it for a small batch, in one CTA: off and xs, group ids and positions in shared memory.
+constexpr int kSmallPairs = 4096, kSmallGroups = 2048;
+__global__ void __launch_bounds__(1024) group_small_kernel(const double *__restrict__ tr, const int32_t *__restrict__ group,
+                                                           int count, int n_groups, uint64_t *__restrict__ off,
+                                                           double *__restrict__ xs) {
+    __shared__ int at[kSmallPairs];
+    __shared__ uint32_t next[kSmallGroups];
+    __shared__ uint64_t sh[32];
+    for (int g = threadIdx.x; g < n_groups; g += 1024) next[g] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < count; i += 1024) {
+        const int g = group[i];
+        at[i] = g >= 0 && g < n_groups ? g : -1;
+        if (at[i] >= 0) atomicAdd(&next[at[i]], 1u);
+    }
+    __syncthreads();
+    uint64_t base = 0;
+    for (int g0 = 0; g0 < n_groups; g0 += 1024) {
+        const int g = g0 + (int)threadIdx.x;
+        const uint32_t n = g < n_groups ? next[g] : 0;
+        const uint64_t s = base + scan_1024(n, sh);
+        if (g < n_groups) off[g + 1] = s, next[g] = (uint32_t)(s - n);
+        for (int w = 0; w < 32; ++w) base += sh[w];
+    }
+    if (threadIdx.x == 0) off[0] = 0;
+    __syncthreads();
+    if (threadIdx.x < 32)
+        for (int i0 = 0; i0 < count; i0 += 32) {
+            const int i = i0 + (int)threadIdx.x, g = i < count ? at[i] : -1;
+            const uint32_t mine = __match_any_sync(0xffffffffu, g), before = mine & ((1u << threadIdx.x) - 1u);
+            if (g >= 0) at[i] = (int)(next[g] + __popc(before));
+            __syncwarp();
+            if (g >= 0 && !before) next[g] += __popc(mine);
+            __syncwarp();
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < count; i += 1024)
+        if (at[i] >= 0) {
+            const double a = tr[2 * i], b = tr[2 * i + 1];
+            xs[at[i]] = a * a + b * b;
+        }
 }
 
 // The powers of every member in fixed point: limbs (low first) of x^k 2^(96 - k e), rounded,
@@ -361,6 +478,7 @@ __global__ void __launch_bounds__(BT) bootstrap_kernel(const double *__restrict_
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
         for (int k = 0; k < FP_MAX_KMAX; ++k) {
+            if (k >= k_max || (uint64_t)wid * 32 >= nq) break;   // (a warp without draws adds nothing)
             double v = s[k];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
             if (lane == 0) sh[k][wid] = v;
@@ -369,7 +487,7 @@ __global__ void __launch_bounds__(BT) bootstrap_kernel(const double *__restrict_
         if (threadIdx.x < k_max && (ks >> threadIdx.x & 1)) {
             const int k = threadIdx.x;
             double v = 0;
-            for (int w = 0; w < BT / 32; ++w) v += sh[k][w];
+            for (int w = 0; w < BT / 32 && (uint64_t)w * 32 < nq; ++w) v += sh[k][w];
             out[((size_t)g * k_max + k) * B + b] = N ? v / (double)N : __longlong_as_double(0x7ff8000000000000LL);
         }
         __syncthreads();
@@ -386,6 +504,11 @@ uint64_t counted_members(uint64_t count, int n_groups) {
 size_t up16(size_t b) { return (b + 15) / 16 * 16; }
 // pairs per chunk: whole passes of a CTA, at most 4096 chunks
 uint64_t chunk_pairs(uint64_t count) { return ((count + 4095) / 4096 + kChunk - 1) / kChunk * kChunk; }
+constexpr int kFewGroups = 16;   // a CTA per (chunk, group) up to here
+constexpr uint64_t kNoWait = 12800;
+// small batches: the FP64 sums of this many draws and powers take 20 us, the launches that the
+// counts need before they start as much
+constexpr uint64_t kSmallSums = 1ull << 22;
 int chunks(uint64_t count) { return count ? (int)((count + chunk_pairs(count) - 1) / chunk_pairs(count)) : 0; }
 }  // namespace
 
@@ -411,31 +534,52 @@ cudaError_t launch_bootstrap(const double *tr, const int32_t *group, uint64_t co
     uint32_t *xf = (uint32_t *)at;
     unsigned long long *redo = (unsigned long long *)(at + up16((size_t)nx * k_max * 12));
     cudaError_t e;
-    const dim3 cg((unsigned)nc, (unsigned)n_groups);
     if (n_groups > 65535) return cudaErrorInvalidValue;
-    if (nc > 0) {
-        group_count_kernel<<<cg, GT, 0, st>>>(group, count, chunk_pairs(count), cnt);
+    const uint64_t entries = (uint64_t)B * n_groups;
+    const unsigned fgrid = (unsigned)std::min<uint64_t>(entries, 152 * 8);
+    if (count <= kSmallPairs && n_groups <= kSmallGroups && count * B * k_max <= kSmallSums) {
+        group_small_kernel<<<1, 1024, 0, st>>>(tr, group, (int)count, n_groups, off, xs);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        bootstrap_kernel<<<fgrid, BT, 0, st>>>(xs, off, n_groups, k_max, B, seed, nullptr, out);
+        return cudaGetLastError();
     }
-    group_offsets_kernel<<<1, 1024, 0, st>>>(cnt, nc, n_groups, kMaxCounted, off, xoff, exp2, redo);
-    if (nc > 0) group_place_kernel<<<cg, GT, 0, st>>>(tr, group, count, chunk_pairs(count), off, cnt, k_max, xs, exp2);
+    const bool many = n_groups > kFewGroups;
+    const uint64_t per = chunk_pairs(count);
+    const dim3 cg((unsigned)nc, (unsigned)n_groups);
+    if (many) {
+        if ((e = cudaMemsetAsync(cnt, 0, (size_t)n_groups * nc * 4, st)) != cudaSuccess) return e;
+        if (nc > 0)
+            group_count_many_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(group, count, per, nc, n_groups, cnt);
+        group_prefix_kernel<<<(unsigned)((n_groups + 7) / 8), 256, 0, st>>>(cnt, nc, n_groups, off, exp2);
+    } else if (nc > 0) {
+        group_count_kernel<<<cg, GT, 0, st>>>(group, count, per, cnt);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    uint64_t largest = 0;   // of the groups that are counted
-    if (nx > 0) {
-        // the largest counted group's size sets the shared memory (two CTAs per SM up to 25,600 members)
+    group_offsets_kernel<<<1, 1024, 0, st>>>(cnt, nc, n_groups, kMaxCounted, !many, off, xoff, exp2, redo);
+    if (nc > 0 && many)
+        group_place_many_kernel<<<(unsigned)nc, 32, 0, st>>>(tr, group, count, per, nc, n_groups, off, cnt, k_max, xs, exp2);
+    else if (nc > 0)
+        group_place_kernel<<<cg, GT, 0, st>>>(tr, group, count, per, off, cnt, k_max, xs, exp2);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // The largest counted group's size sets the shared memory: two CTAs per SM up to 25,600 members, four,
+    // which is what their threads allow, up to kNoWait.  A batch of that many pairs in all does not wait for the sizes.
+    uint64_t largest = count;
+    if (nx > 0) powers_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(xs, off, xoff, n_groups, k_max, exp2, xf);
+    if (count > kNoWait) {
         std::vector<uint64_t> h((size_t)n_groups + 1);
         if ((e = cudaMemcpyAsync(h.data(), off, h.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-        powers_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(xs, off, xoff, n_groups, k_max, exp2, xf);
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        largest = 0;
         for (int g = 0; g < n_groups; ++g)
             if (h[g + 1] - h[g] <= kMaxCounted) largest = std::max(largest, h[g + 1] - h[g]);
-        const size_t smem = (size_t)((largest + 3) / 4) * 4 * RB;
-        if ((e = allow_smem(bootstrap_count_kernel, kMaxCounted * RB)) != cudaSuccess) return e;
-        if (largest > 0)
-            bootstrap_count_kernel<<<dim3((unsigned)((B + RB - 1) / RB), (unsigned)n_groups), CT, smem, st>>>(
-                xf, off, xoff, n_groups, k_max, B, seed, exp2, kMaxCounted, redo, out);
     }
-    const unsigned fgrid = (unsigned)std::min<uint64_t>((uint64_t)B * n_groups, 152 * 8);
+    if (largest > 0) {
+        if ((e = allow_smem(bootstrap_count_kernel, kMaxCounted * RB)) != cudaSuccess) return e;
+        bootstrap_count_kernel<<<dim3((unsigned)((B + RB - 1) / RB), (unsigned)n_groups), CT,
+                                 (size_t)((largest + 3) / 4) * 4 * RB, st>>>(xf, off, xoff, n_groups, k_max, B, seed, exp2,
+                                                                             kMaxCounted, redo, out);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     bootstrap_kernel<<<fgrid, BT, 0, st>>>(xs, off, n_groups, k_max, B, seed, largest > 0 ? redo : nullptr, out);
     return cudaGetLastError();
 }
