@@ -12,15 +12,16 @@
 // place.  Bound: HBM (the boundaries of a batch exceed L2), one read and one write of
 // the boundary per operation.
 //
-// The meet forms its terms from exact FP32 products (a product and its rounding error)
-// and adds them in three-word FP32 sums, which carry more bits than a double: in FP64,
-// 35 operations per term on a pipe 77 times slower, it took longer than the sweep.
+// The meet (exact_meet.h) takes FP32 operations whose products and sums of Re and Im are
+// exact to more bits than a double's: in FP64, 35 operations per term on a pipe 77 times
+// slower, it took longer than the sweep.
 // 4,000 pairs at n = 20, T = 20..100 (1,792 of them here): 17 ms of sweeps and meet against 93.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "kernels.h"
+#include "exact_meet.h"
 #include "meet.h"
 
 namespace fpk {
@@ -183,69 +184,6 @@ __global__ void step_init_kernel(const StepPair *__restrict__ sp, int npairs, C 
     one.y = 0;
     ws[sp[i >> 1].base[i & 1]] = one;
 }
-
-// A sum of floats in three words, each step exact to the last word's rounding (2^-72 of the sum).
-struct Sum3 {
-    float a = 0, b = 0, c = 0;
-    __device__ __forceinline__ static float two(float &s, float x) {   // s <- s + x rounded; returns the rest, exactly
-        const float t = __fadd_rn(s, x), u = __fsub_rn(t, s), r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, u)), __fsub_rn(x, u));
-        s = t;
-        return r;
-    }
-    __device__ __forceinline__ void add(float x) { c += two(b, two(a, x)); }
-    __device__ __forceinline__ void low(float x) { c += two(b, x); }   // |x| of the size of rounding errors
-    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
-};
-
-// Sums over a thread's terms t = L R: Re, Im, |t|, |t|^2.
-template <typename C> struct ExactMeet;
-template <> struct ExactMeet<double2> {
-    double s[4] = {0, 0, 0, 0};
-    __device__ __forceinline__ void add(double2 l, double2 r) {
-        const double px = l.x * r.x - l.y * r.y, py = l.x * r.y + l.y * r.x, q = px * px + py * py;
-        s[0] += px;
-        s[1] += py;
-        s[2] += sqrt(q);
-        s[3] += q;
-    }
-    __device__ __forceinline__ double total(int c) const { return s[c]; }
-};
-template <> struct ExactMeet<float2> {
-    Sum3 re, im, ab, sq;
-    ExactMeet<double2> far;   // terms whose squares or rounding errors leave the range of float
-    __device__ __forceinline__ void add(float2 l, float2 r) {
-        // (__fmul_rn: the products must not be fused into the sums)
-        const float p1 = __fmul_rn(l.x, r.x), p2 = __fmul_rn(-l.y, r.y), p3 = __fmul_rn(l.x, r.y), p4 = __fmul_rn(l.y, r.x);
-        const float m = fmaxf(fmaxf(fabsf(p1), fabsf(p2)), fmaxf(fabsf(p3), fabsf(p4)));
-        if (!(m <= 0x1p60f && m >= 0x1p-46f)) {   // also NaN, and zero
-            if (m != 0.f || !(l.x == 0.f && l.y == 0.f) || !(r.x == 0.f && r.y == 0.f))
-                far.add(make_double2(l.x, l.y), make_double2(r.x, r.y));
-            return;
-        }
-        const float e1 = fmaf(l.x, r.x, -p1), e2 = fmaf(-l.y, r.y, -p2), e3 = fmaf(l.x, r.y, -p3), e4 = fmaf(l.y, r.x, -p4);
-        re.add(p1);
-        re.add(p2);
-        re.low(e1 + e2);   // (rounded at 2^-48 of the products)
-        im.add(p3);
-        im.add(p4);
-        im.low(e3 + e4);
-        // |t|^2 and |t| to about 2^-45
-        float x = p1, y = p3;
-        const float xl = Sum3::two(x, p2) + (e1 + e2), yl = Sum3::two(y, p4) + (e3 + e4);
-        const float qx = __fmul_rn(x, x), qy = __fmul_rn(y, y);
-        float q = qx;
-        const float ql = Sum3::two(q, qy) + (fmaf(x, x, -qx) + fmaf(y, y, -qy)) + 2.f * (x * xl + y * yl);
-        sq.add(q);
-        sq.low(ql);
-        const float s = sqrtf(q);
-        ab.add(s);
-        if (s > 0.f) ab.low((fmaf(-s, s, q) + ql) * (0.5f / s));
-    }
-    __device__ __forceinline__ double total(int c) const {
-        const Sum3 &v = c == 0 ? re : c == 1 ? im : c == 2 ? ab : sq;
-        return v.value() + far.s[c];
-    }
-};
 
 struct Sums { double v[4]; };
 
