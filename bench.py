@@ -504,6 +504,8 @@ def roofline(fp, ks, ms_total, prec, peaks, clocks):
                             f"SMs x {mhz:.0f} MHz (median SM clock of the timed region); "
                             f"{pk['tflops']:.1f} TFLOP/s at {pk['sm_mhz']:.0f} MHz in the microbenchmark"),
             "kernel_ms_share": ks.ms[cls] / ms_total if ms_total else None,
+            "note": ("the FP64 sweeps of boundaries in shared memory and of the HEA run in 64-bit integers: the FP64 "
+                     "rate is a yardstick, not the pipe in use") if prec == fp.PREC_FP64 else None,
             "tensor_view": tensor_view(ks, cls, peaks)}
 
 

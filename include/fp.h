@@ -62,9 +62,9 @@
  * number of CTAs that share one pair on the generic sweep (default: by
  * boundary size); FP_SPIRAL_WIN (0, 4 or 5) fixes the register-window width
  * of the spiral sweep of FP_HEA_PAULI (0: one map per pass; default: by
- * state size) and FP_SPIRAL_SPLIT (0, 1 or 2) the least number of cluster
- * bits its state is split over (default 0: as the state size needs); both are
- * read when an ensemble first contracts a depth.
+ * state size) and FP_SPIRAL_SPLIT (0 to 4, in FP32 at most 2) the least number of
+ * cluster bits its state is split over (default 0: as the state size and the
+ * number of pairs need); both are read when an ensemble first contracts a depth.
  *
  * Errors.  Calls return an fp_status; nothing is thrown across the ABI.
  * fp_last_error() gives a thread-local message for the last failing call on
@@ -193,7 +193,9 @@ typedef struct {
     double ms[FP_K_CLASSES];          /* device milliseconds (CUDA events on the ensemble's stream) */
     uint64_t launches[FP_K_CLASSES];  /* kernel launches */
     double work[FP_K_CLASSES];        /* algorithmic work: complex multiply-adds for the sweep
-                                         classes, pairs for the others */
+                                         classes (the HEA's own sweep: its window products, and
+                                         its Hadamard additions at 2 real operations in 8),
+                                         pairs for the others */
     uint64_t pairs;                   /* pairs contracted */
     uint64_t graph_replays;           /* sub-batches run by CUDA-graph replay (counted always) */
     double mma_flops;                 /* flops issued to the tensor cores by the brickwork

@@ -922,8 +922,14 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
     const size_t per_state = bd.tile_bits ? 2 * S * celem + it->second->extra_per_pair : (both ? 0 : S * celem);
     const size_t per_pair = per_raw + per_map + per_state;
     uint64_t cap = std::max<uint64_t>(1, std::min<uint64_t>(65535, E->ws_budget / per_pair));
-    // flop count of the sweep (complex multiply-adds): 4 per amplitude per gate
-    const double cmac_pair = 4.0 * (double)S * (double)maps_per_pair(bd);
+    // work of the sweep (complex multiply-adds): 4 per amplitude per gate; the HEA's own sweep, per qubit
+    // and amplitude: a product per register window (per factor up to 4 bits) and N Hadamards, 2 real
+    // additions of an 8-flop multiply-add each
+    double cmac_pair = 4.0 * (double)S * (double)maps_per_pair(bd);
+    if (hea) {
+        const int R = it->second->variant[1];
+        cmac_pair = (double)S * d.n * ((N <= 4 ? N : (N + R - 1) / R) + N / 4.0);
+    }
     SampleParams sp;
     sp.seed = d.seed;
     sp.n = d.n;
@@ -944,6 +950,9 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         CK(E->d_maps.reserve(nb * per_map));
         CK(E->d_states.reserve(std::max<size_t>(16, nb * per_state)));
         const double G = (double)std::max(bd.n_layers[0], bd.n_layers[1]) * bd.m;
+        // (FP64 in 64-bit integers, fixed.h: alignment, product and settling each round a component within
+        // half a unit, 2^-57 to 2^-56 of its block's largest: together rms 2^-53.9 of the norm of a block of 16
+        // amplitudes at most, 2^-54.9 of a quad's, where the estimate takes 2^-53 an operation)
         const double err_scale = FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53) * std::sqrt(G);
         // CUDA graph replay: the launch sequence of a sub-batch (sampler, maps,
         // init, passes, meet) is captured once per (depth, precision, size,

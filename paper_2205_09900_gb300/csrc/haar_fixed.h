@@ -6,7 +6,9 @@
 // of 2^-60); a product takes 30-bit halves, three 32 x 32 -> 64 multiply-adds (the
 // product of the low halves, below the last place, is left out and its mean added
 // where sums would collect it) and sums of products share their shifts.  The errors
-// are a few 2^-58, where a double carries 2^-53.
+// are a few 2^-58, where a double carries 2^-53: of a column of length 1, so that an entry
+// below 2^-7 has fewer significant bits than a double, and an error still below the 2^-53 of
+// its column that FP64 Gram-Schmidt or Householder leaves it.
 //
 // The same functions compile for the host (tests/cpp/haar_fixed_check.cpp measures
 // their errors against extended precision).

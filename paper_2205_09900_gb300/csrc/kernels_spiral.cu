@@ -11,7 +11,7 @@
 //                        state bits run on 2^R amplitudes per thread in
 //                        registers, one barrier per window.  The state sits
 //                        in shared memory (swizzled), in one CTA or split
-//                        over a 2- or 4-CTA cluster (distributed shared memory);
+//                        over a cluster of 2 to 16 CTAs (distributed shared memory);
 //   spiral_sweep_kernel  one map per pass (small states, or states too large
 //                        for four CTAs: a per-pair global slice).
 // Both sweeps start from delta(aux, first bit) and end with the FP64 sum of
@@ -371,7 +371,7 @@ template <int CL> struct CtaParts {
 // ("cross" window) reads and writes other CTAs' parts through distributed
 // shared memory and is fenced by cluster barriers; the other windows stay in
 // their own CTA.  Addressing: SpiralWin.  8 and 16 CTAs serve FP64 batches of a few pairs
-// (spiral_split): an FP64 instruction occupies its SM quarter for about 77 cycles, so a
+// (spiral_variant in api.cu chooses): an FP64 instruction occupies its SM quarter for about 77 cycles, so a
 // pair is as fast as the number of quarters that share it.
 // Threads per CTA: the FP32 two-CTA form runs one CTA per SM (its half of the
 // state fills the shared memory), so it takes as many warps as its registers allow.
