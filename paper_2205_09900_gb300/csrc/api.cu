@@ -951,8 +951,8 @@ fp_status run_brick(fp_ensemble *E, uint64_t first, const std::vector<uint64_t> 
         CK(E->d_states.reserve(std::max<size_t>(16, nb * per_state)));
         const double G = (double)std::max(bd.n_layers[0], bd.n_layers[1]) * bd.m;
         // (FP64 in 64-bit integers, fixed.h: alignment, product and settling each round a component within
-        // half a unit, 2^-57 to 2^-56 of its block's largest: together rms 2^-53.9 of the norm of a block of 16
-        // amplitudes at most, 2^-54.9 of a quad's, where the estimate takes 2^-53 an operation)
+        // half a unit, 2^-58 to 2^-57 of its block's largest: together rms 2^-54.5 of the norm of a block of 16
+        // amplitudes at most, 2^-55.5 of a quad's, where the estimate takes 2^-53 an operation)
         const double err_scale = FP_ERR_SAFETY * (fp32 ? 0x1.0p-24 : 0x1.0p-53) * std::sqrt(G);
         // CUDA graph replay: the launch sequence of a sub-batch (sampler, maps,
         // init, passes, meet) is captured once per (depth, precision, size,
