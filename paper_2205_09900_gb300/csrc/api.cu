@@ -374,11 +374,13 @@ fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<Pai
     size_t n_steps = 0, at = 0, n_items = 0;
     for (uint64_t i = 0; i < nb; ++i) n_steps = std::max(n_steps, (size_t)std::max(plan(i).n_left, plan(i).n_right));
     std::vector<uint32_t> count(n_steps + 1, 0), blocks(n_steps, 0);
+    const bool few = nb < 2 * (uint64_t)E->sms;   // else the operations alone make two blocks per SM
     std::vector<uint64_t> quads(n_steps, 0);   // amplitudes first
     for (uint64_t i = 0; i < nb; ++i)
         for (int s = 0; s < 2; ++s)
             for (int k = 0; k < (s ? plan(i).n_right : plan(i).n_left); ++k) {
                 ++count[k + 1];
+                if (!few) continue;
                 const DevOp &op = plan(i).ops[s ? plan(i).n_left + k : k];
                 quads[k] += 1ull << std::max<int>(op.b_in, op.b_out);
             }
@@ -386,7 +388,7 @@ fp_status build_steps(fp_ensemble *E, uint64_t nb, F plan, const std::vector<Pai
     n_items = count[n_steps];
     std::vector<uint8_t> log_units(n_steps);
     for (size_t k = 0; k < n_steps; ++k)
-        log_units[k] = (uint8_t)step_log_units(count[k + 1] - count[k], quads[k] >> 2, E->sms);
+        log_units[k] = few ? (uint8_t)step_log_units(count[k + 1] - count[k], quads[k] >> 2, E->sms) : 10;
     std::vector<uint32_t> fill(count.begin(), count.end() - 1);
     std::vector<StepItem> items(n_items);
     uint32_t meet = 0;

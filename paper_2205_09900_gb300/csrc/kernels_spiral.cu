@@ -24,7 +24,7 @@
 // 12, DIAG 8).  And no window touches a freed bit's zero half (SpiralWin::half).
 // n = 50, about 2,000 pairs per depth: FP32 L = 8 (two CTAs) 36.8 ms instead of 47, L = 7 (one
 // CTA) 4.5 ms instead of 7.0; FP64 with few pairs (four CTAs) 20.9 ms instead of 44.  The two-CTA
-// form is held back by its cross windows and barriers (31 % of the issue slots, 16 warps).
+// form is held back by its cross windows and barriers (30 % of the issue slots, 16 warps).
 // FP64 L = 8, 4 pairs: 16 CTAs each 4.7 ms, 4 CTAs each 13.9.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>

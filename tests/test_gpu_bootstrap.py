@@ -13,18 +13,6 @@ pytestmark = pytest.mark.gpu
 RTOL = 5e-14
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 def both(fp, groups, k_max, B, seed=7):
     grp = np.repeat(np.arange(len(groups), dtype=np.int32), [len(z) for z in groups])
     z = np.concatenate(groups).astype(np.complex128)

@@ -11,18 +11,6 @@ import oracle as O
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 # (groups, pairs, k_max, B): the smallest; 4,096 pairs and one more; 16, 17, 2,048 and 2,049 groups;
 # more sums than a small batch may have; 12,800 pairs, which wait for no sizes; chunks of 1,024 pairs, whole and ragged
 @pytest.mark.parametrize("ng,count,k_max,B", [(1, 1, 1, 1), (3, 40, 4, 7), (9, 4096, 2, 20), (9, 4097, 2, 20), (16, 13_000, 3, 8), (17, 13_000, 3, 8),

@@ -12,18 +12,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 @pytest.mark.parametrize("M,N,K", [(512, 256, 64), (512, 256, 256), (300, 48, 4096), (512, 512, 4096),
                                    (45000, 256, 1024)])
 def test_wait_runs_out_anywhere(fp, M, N, K):

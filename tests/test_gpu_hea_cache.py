@@ -5,18 +5,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 @pytest.mark.parametrize("L,prec,name,entry", [(7, 1, "fp32", "12 4 256 0"), (8, 1, "fp32", "12 5 256 4"),
                                                (7, 0, "fp64", "99 0 0 0"), (8, 0, "fp64", "13 4 256 0")])
 def test_stale_entry_is_replaced(fp, L, prec, name, entry, tmp_path, monkeypatch):

@@ -8,18 +8,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 @pytest.mark.parametrize("n,L", [(2, 2), (3, 2), (50, 2), (2, 3), (5, 3), (51, 3)])
 @pytest.mark.parametrize("count", [1, 3, 8, 35])
 def test_few_bits(fp, n, L, count):

@@ -10,18 +10,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 # boundaries of a few bits beside ones of 2^14 amplitudes and more
 @pytest.mark.parametrize("n,T", [(18, (20, 60, 20)), (13, (5, 45, 20)), (20, (60, 60, 1)), (10, (60, 60, 1))])
 def test_few_pairs(fp, n, T, monkeypatch):

@@ -6,18 +6,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 # gates per pair that are and are not multiples of a warp's 3 (q = 3) or 2 (q = 4)
 @pytest.mark.parametrize("q,n,l", [(3, 4, 2), (3, 5, 3), (3, 8, 3), (3, 4, 4), (4, 3, 2), (4, 4, 3), (4, 6, 2)])
 def test_trace_does_not_depend_on_the_batch(fp, q, n, l):

@@ -9,18 +9,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 def test_precisions_at_20_bits(fp):
     ens = fp.Ensemble(fp.PARALLEL, 50, 11, 11, seed=5)
     t64 = ens.trace_batch(0, 40, fp.PREC_FP64)[0]

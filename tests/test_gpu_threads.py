@@ -8,18 +8,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def fp():
-    import torch
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_09900_gb300 import build
-    build.build()
-    import paper_2205_09900_gb300 as fpm
-    fpm.load()
-    return fpm
-
-
 def side_by_side(calls, rounds):
     """calls: functions of no argument; each thread repeats its own and compares with its first result.
     (Short calls and many rounds: what a thread sets and what it launches lie a microsecond apart.)"""
