@@ -30,7 +30,7 @@
 // 0.07 against 1.5 (one map per shared-memory pass); L = 8 FP64, 214 pairs, 76 us in FP64
 // arithmetic against 320 (FMA tile passes).  100,000 pairs, L = 1..8, of which about 700 go
 // through FP64: 61.5 ms with FP64 arithmetic, 46.7 with integers, 42.7 with the slots
-// sampled in fixed point too.
+// sampled in fixed point too, 42.2 with a lane per amplitude at 2 and 4 bits in FP64.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

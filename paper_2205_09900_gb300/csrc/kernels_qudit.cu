@@ -12,7 +12,7 @@
 //                     entry.  Bound: the integer pipe.  With FP64 Householder QR by a
 //                     thread per gate (its 9 x 9 arrays in local memory) and a separate
 //                     map kernel 500 pairs of l = 2 at n = 50, q = 3, nearly all of it
-//                     this kernel, took 2.5 ms; they take 0.48.
+//                     this kernel, took 2.5 ms; they take 0.46.
 // K3q  qudit_sweep:   one CTA per pair: the boundary over the 2m segment digits
 //                     of one qudit (q^{2m} amplitudes, in shared memory when it
 //                     fits, else in a per-pair global slot), both chain halves,
@@ -216,8 +216,8 @@ __device__ __forceinline__ void meet_term(C l, C r, double &sr, double &si, doub
 // 81 of 256 threads busy with a group each), or, for BIG boundaries, two groups and all
 // their outputs, which reads every map entry from shared memory once for two products.
 // The next map arrives by cp.async meanwhile.  The left half waits in `lscr`.
-// Bound: FP32 issue.  500 pairs at n = 50, q = 3, FP32, sampler and maps included: l = 5 2.9 ms
-// against 8.0, l = 4 1.1 against 5.0 (a group per thread in place, two barriers per map).
+// Bound: FP32 issue.  500 pairs at n = 50, q = 3, FP32, sampler and maps included: l = 5 2.8 ms
+// against 8.0, l = 4 1.0 against 5.0 (a group per thread in place, two barriers per map).
 template <int Q, typename C, bool BIG>
 __global__ void __launch_bounds__(256) qudit_smem_kernel(BrickDev d, const PairInfo *__restrict__ pairs,
                                                          const EntryT<C> *__restrict__ maps, C *__restrict__ lscr,
