@@ -18,7 +18,8 @@ int main() {
     const float load[4] = {2.0f, 0.0f, 5.0f, 1.0f};   // variant 1's code is loaded already
     int runs[4] = {0, 0, 0, 0};
     std::vector<float> ms;
-    auto clock = [&](int i, float &t) {
+    auto clock = [&](int i, bool counted, float &t) {
+        if (counted != (runs[i] == 1)) return -1;
         t = warm[i] + (runs[i]++ ? 0.0f : load[i]);
         return 0;
     };
@@ -27,7 +28,7 @@ int main() {
 
     // one that cannot run here, and one that fails on its second run only
     int n = 0;
-    EXPECT(time_variants(3, ms, [&](int i, float &t) {
+    EXPECT(time_variants(3, ms, [&](int i, bool, float &t) {
                t = 1.0f;
                return i == 0 ? 1 : i == 1 ? n++ : 0;
            }) == 0);
@@ -35,7 +36,7 @@ int main() {
 
     // an error ends it
     int calls = 0;
-    EXPECT(time_variants(3, ms, [&](int i, float &t) {
+    EXPECT(time_variants(3, ms, [&](int i, bool, float &t) {
                ++calls;
                t = 1.0f;
                return i == 1 ? -4 : 0;
